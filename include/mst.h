@@ -85,8 +85,8 @@ mst_status_t mst_layer_destroy(mst_layer_t* layer);
  *   MST_PATH_CUDA_CORE    the sparse kernels (work proportional to nnz, fp32 FMA pipe)
  *   MST_PATH_TENSOR_CORE  dense-tile kernels: W.M is expanded on the fly to a dense bf16 image and contracted on the
  *                         tensor cores (work proportional to O*I, about 18x the FMA pipe's rate); the weight gradient
- *                         is the dense contraction sampled on the mask in its epilogue.  Needs 16-byte-aligned rows
- *                         (leading dimensions multiple of 8), otherwise the CUDA-core kernels are used.
+ *                         is the dense contraction sampled on the mask in its epilogue.  Rows that do not start on
+ *                         16-byte boundaries (leading dimensions that are no multiple of 8) are copied to ones that do.
  *   MST_PATH_SPARSE_TC    forward and input gradient on the 2:4 structured-sparse tensor-core instruction: W.M is
  *                         split into the first two entries of every group of four consecutive contraction indices
  *                         (run at twice the dense tensor rate) and the few third and fourth entries, which the
@@ -96,13 +96,15 @@ mst_status_t mst_layer_destroy(mst_layer_t* layer);
  *                         The weight gradient stays the dense contraction sampled on the mask.
  *   MST_PATH_AUTO         (default) bf16 layers with aligned operands: the structured-sparse instruction at densities
  *                         where it was measured faster than dense tiles, dense tiles above; CUDA cores otherwise.
- * fp32 layers always use the CUDA-core kernels.  Results of the paths agree within the stated tolerance, not
+ * fp32 layers keep single-precision arithmetic whatever the path: on MST_PATH_CUDA_CORE in FMA chains, otherwise as sums of
+ * products of exact bf16 pieces on the tensor cores (three pieces per operand, rounded fp32 sums every 64 terms; at
+ * least as close to the exact product as the FMA chains).  Results of the paths agree within the stated tolerance, not
  * bit for bit (different summation order). */
 typedef enum { MST_PATH_AUTO = 0, MST_PATH_CUDA_CORE = 1, MST_PATH_TENSOR_CORE = 2, MST_PATH_SPARSE_TC = 3 } mst_compute_path_t;
 mst_status_t mst_set_compute_path(mst_layer_t* layer, mst_compute_path_t path);
 
-/* The kernels forward and input gradient of this layer run on for aligned operands, with MST_PATH_AUTO resolved
- * (unaligned operands always fall back to the CUDA-core kernels). */
+/* The kernels forward and input gradient of this layer run on, with MST_PATH_AUTO resolved.  fp32 layers report
+ * MST_PATH_CUDA_CORE: none of the bf16 paths applies to them. */
 mst_status_t mst_layer_path_in_use(const mst_layer_t* layer, mst_compute_path_t* path);
 
 /* Kernels the library has enqueued in this process so far (all layers, all streams): for launch accounting. */

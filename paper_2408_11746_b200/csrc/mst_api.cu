@@ -172,8 +172,8 @@ mst_status_t mst_alloc_csc(mst_layer* L) {
 }
 
 mst_status_t mst_alloc_dense(mst_layer* L) {
-  if (L->dense_w || L->dtype != MST_BF16) return MST_OK;
-  MST_CUDA_TRY(cudaMalloc((void**)&L->dense_w, 2 * (size_t)L->N));
+  if (L->dense_w) return MST_OK;
+  MST_CUDA_TRY(cudaMalloc((void**)&L->dense_w, mst_image_bytes(L)));
   L->dense_version = L->dense_epoch = -1;
   return MST_OK;
 }
@@ -206,12 +206,17 @@ extern "C" mst_status_t mst_set_compute_path(mst_layer_t* L, mst_compute_path_t 
 
 // On B200 the dense-tile tensor-core kernels beat the CUDA-core sparse kernels at every density the method visits
 // (measured down to 2 %: the tensor pipe is about 18x the fp32 FMA pipe and the sparse kernels pay a staging cost
-// that does not shrink with nnz), so AUTO means tensor cores whenever the layer is bf16; the launchers fall back to
-// the CUDA-core kernels when an operand is not 16-byte aligned.
+// that does not shrink with nnz), so AUTO means tensor cores whenever the layer is bf16; operands that are not 16-byte
+// aligned are copied to rows that are.
 bool mst_use_tensor_path(const mst_layer* L) {
   if (L->dtype != MST_BF16 || L->path == MST_PATH_CUDA_CORE) return false;
   return true;
 }
+
+// fp32 layers multiply on the tensor cores in bf16 pieces (mst_tc_split.cu) unless the CUDA-core kernels are asked for.
+bool mst_use_split_path(const mst_layer* L) { return L->dtype == MST_F32 && L->path != MST_PATH_CUDA_CORE; }
+
+bool mst_use_csc(const mst_layer* L) { return L->path == MST_PATH_CUDA_CORE; }
 
 // Forward and input gradient on the structured-sparse instruction: on request, or under AUTO up to the density where
 // it was measured faster than dense tiles.

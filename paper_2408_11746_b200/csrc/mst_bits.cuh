@@ -9,6 +9,26 @@ __device__ __forceinline__ unsigned mst_lanemask_lt() {
   return m;
 }
 
+// x = p[0] + p[1] + p[2] exactly, as bf16 bit patterns: two roundings to nearest leave a remainder of at most 8 bits.  A
+// value that would round to infinity is truncated instead; a non-finite one keeps its pattern and has no remainder.
+__device__ __forceinline__ uint32_t mst_bf16_nearest(float x) {
+  const uint32_t u = __float_as_uint(x);
+  const uint32_t r = (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;
+  return (r & 0x7F80u) == 0x7F80u ? u >> 16 : r;
+}
+__device__ __forceinline__ void mst_split3(float x, uint32_t (&p)[3]) {
+  const uint32_t u = __float_as_uint(x);
+  if ((u & 0x7F800000u) == 0x7F800000u) {
+    p[0] = (u & 0x007FFFFFu) ? (u >> 16) | 0x40u : u >> 16;   // a NaN stays a NaN when its low bits go
+    p[1] = p[2] = 0u;
+    return;
+  }
+  p[0] = mst_bf16_nearest(x);
+  const float r1 = x - __uint_as_float(p[0] << 16);
+  p[1] = mst_bf16_nearest(r1);
+  p[2] = mst_bf16_nearest(r1 - __uint_as_float(p[1] << 16));
+}
+
 // CSR entries of mask word w.  Source of a value: dense W (pack) or the previous structure (update: an entry present
 // before and after keeps its value, a new entry starts at +0).
 template <typename V>

@@ -135,8 +135,9 @@ struct mst_layer {
   mutable int64_t longest_row_version;  // structure version flags[2] belongs to
   unsigned int* counter;  // [1] block-completion counter
 
-  // dense bf16 image of W.M for the tensor-core path (bf16 layers only): [O x I]; the input gradient reads it as an
-  // MN-major operand, so no transposed copy is kept.  Allocated on first use (mst_alloc_dense).
+  // dense image of W.M for the tensor-core paths, kept with value tracking: [O x ldp] bf16, or three bf16 pieces of it
+  // for fp32 layers (mst_densify); the input gradient reads it as an MN-major operand, so no transposed copy is kept.
+  // Allocated on first use (mst_alloc_dense).
   uint16_t* dense_w;
   int path;  // mst_compute_path_t
   // 2:4 split of W.M (forward) and of its transpose (input gradient) for the structured-sparse tensor-core path;
@@ -167,17 +168,24 @@ mst_status_t mst_alloc_dense(mst_layer* L);   // no-op when the dense image exis
 mst_status_t mst_build_csc(mst_layer* L, cudaStream_t s);
 mst_status_t mst_ensure_csc(const mst_layer* L, cudaStream_t s);  // builds the CSC view if it is stale
 mst_status_t mst_combine_update_bits(mst_layer* L, int new_set, cudaStream_t s);
-mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image);
+mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image, int64_t* ld);
+static inline size_t mst_image_bytes(const mst_layer* L) {
+  return (L->dtype == MST_F32 ? 6 : 2) * (size_t)L->O * (size_t)((L->I + 7) & ~7);
+}
 // strided attention forward on warp-level products (mst_attention_fwd_mma.cu); the caller has checked pointers and
 // leading dimensions
 mst_status_t mst_attention_fwd_mma(const void* Q, const void* K, const void* V, int64_t ld, int32_t batch, int32_t seq_len,
                                    int32_t heads, int32_t stride, void* Out, int64_t ldo, float* lse, cudaStream_t s);
 bool mst_use_tensor_path(const mst_layer* L);
+bool mst_use_split_path(const mst_layer* L);
+bool mst_use_csc(const mst_layer* L);   // the input gradient walks the CSC view (CUDA-core kernels)
 bool mst_use_sparse_tc_path(const mst_layer* L);
 
 // sticky error word of the CUDA-core SpMM's bounded waits (mst_spmm.cu)
 mst_status_t mst_spmm_error_flags(int32_t* flags);
 mst_status_t mst_sddmm_error_flags(int32_t* flags);
+// and of the fp32 contraction's (mst_tc_split.cu)
+mst_status_t mst_split_error_flags(int32_t* flags);
 // sticky error word of the attention kernel's bounded waits (mst_attention.cu)
 mst_status_t mst_attention_error_flags(int32_t* flags);
 

@@ -249,17 +249,14 @@ mst_status_t mst_launch_sddmm(const mst_layer* L, const void* dY, int64_t lddy, 
   }
   // Tensor-core path: the dense contraction dY^T X with an epilogue that keeps only the entries under the mask and
   // writes them to their CSR positions; the token range is split when the output has few tiles.
-  if (mst_use_tensor_path(L) && mst_tc_gemm_usable(dY, lddy, X, ldx)) {
+  if (mst_use_tensor_path(L) || mst_use_split_path(L)) {
     const int c = L->cur;
     mst_tc_gemm_args a = {};
-    a.A = dY; a.lda = lddy; a.a_mn_major = 1;
-    a.B = X; a.ldb = ldx; a.b_mn_major = 1;
     a.M = L->O; a.N = L->I; a.K = T;
     a.epilogue = MST_TC_OUT_SAMPLED;
     a.out = dW;
     a.bits = L->bits[c]; a.wscan = L->wscan[c]; a.wpr = L->wpr; a.nnz = L->nnz;
-    a.splits = 0;
-    return mst_tc_gemm(a, s);
+    return mst_tc_gradient(a, L->dtype, dY, lddy, X, ldx, s);
   }
   if (L->dtype == MST_F32) return launch<float>(L, dY, lddy, X, ldx, T, dW, s);
   return launch<uint16_t>(L, dY, lddy, X, ldx, T, dW, s);

@@ -423,21 +423,6 @@ spmm_stream_kernel(const __grid_constant__ CUtensorMap tmIn, const int32_t* __re
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn spmm_encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
 }  // namespace
 mst_status_t mst_feature_major_copy(const void* in, int64_t ldin, int64_t T, int C, mst_dtype_t dtype, void* out, int64_t ldt,
                                     cudaStream_t s);
@@ -539,7 +524,7 @@ mst_status_t mst_feature_major_copy(const void* in, int64_t ldin, int64_t T, int
 }
 bool mst_feature_major_map(CUtensorMap* tm, const void* base, int64_t T, int C, int64_t ldt, mst_dtype_t dtype, int box_tokens,
                            int box_features) {
-  EncodeTiledFn enc = spmm_encode_fn();
+  mst_encode_tiled_fn enc = mst_encode_tiled();
   if (!enc) return false;
   const size_t es = dtype == MST_F32 ? 4 : 2;
   cuuint64_t dims[2] = {(cuuint64_t)T, (cuuint64_t)C};
@@ -563,25 +548,43 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
   if (T == 0) return MST_OK;
   const int c = L->cur;
   const int rows = transpose ? L->I : L->O, cols = transpose ? L->O : L->I;
-  // Dense-tile tensor-core path: expand W.M to a dense bf16 image [O x I].  Forward: out = in * image^T, the image a
-  // K-major operand.  Input gradient: out = in * image, the same image read as an MN-major operand ([K = O] rows of
-  // I contiguous columns), so no transposed copy and no CSC view are needed.
+  // Dense-tile tensor-core path: expand W.M to a dense image [O x I] (three bf16 pieces of it for fp32 layers).  Forward:
+  // out = in * image^T, the image a K-major operand.  Input gradient: out = in * image, the same image read as an MN-major
+  // operand ([K = O] rows of I contiguous columns), so no transposed copy and no CSC view are needed.
   if (act == MST_ACT_NONE && mst_use_sparse_tc_path(L) && mst_sp24_usable(L, transpose ? 1 : 0, in, ldin, out, ldout))
     return mst_sp24_product(const_cast<mst_layer*>(L), transpose ? 1 : 0, in, ldin, T, out, ldout, s);
-  if (mst_use_tensor_path(L) && (ldout % 8 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15u) == 0)) {
-    // the image is 256-byte aligned by construction: only the activations and the row length decide
-    if (mst_tc_gemm_usable(in, ldin, in, L->I)) {
-      const uint16_t* image = nullptr;
-      MST_TRY(mst_densify(L, s, &image));
-      mst_tc_gemm_args a = {};
-      a.A = in; a.lda = ldin; a.a_mn_major = 0;
-      a.B = image; a.ldb = L->I; a.b_mn_major = transpose ? 1 : 0;
-      a.M = T; a.N = rows; a.K = cols;
-      a.epilogue = MST_TC_OUT_BF16;
-      a.out = out; a.ldc = ldout; a.splits = 1;
-      a.act = act; a.pre = pre; a.ldpre = ldpre;
-      return mst_tc_gemm(a, s);
+  if (mst_use_tensor_path(L) || mst_use_split_path(L)) {
+    const uint16_t* image = nullptr;
+    int64_t ldimage = 0;
+    MST_TRY(mst_densify(L, s, &image, &ldimage));
+    mst_tc_gemm_args a = {};
+    a.A = in; a.lda = ldin; a.a_mn_major = 0;
+    a.B = image; a.ldb = ldimage; a.b_mn_major = transpose ? 1 : 0;
+    a.M = T; a.N = rows; a.K = cols;
+    a.out = out; a.ldc = ldout;
+    if (L->dtype == MST_F32) {
+      void* pieces = nullptr;
+      a.lda = (cols + 7) & ~7;
+      MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 6 * (size_t)T * a.lda, &pieces));
+      MST_TRY(mst_split_rows(in, ldin, T, cols, pieces, s));
+      a.A = pieces;
+      a.epilogue = MST_TC_OUT_F32;
+      // the product lands in the pre-activation buffer when the caller keeps one; the activation is a pass of its own
+      if (act == MST_ACT_GELU && pre) { a.out = pre; a.ldc = ldpre; }
+      MST_TRY(mst_tc_split(a, s));
+      return act == MST_ACT_NONE ? MST_OK : launch_act<float>(out, ldout, pre, ldpre, T, rows, act, s);
     }
+    if (!mst_tc_gemm_usable(in, ldin, image, ldimage)) {   // rows that do not start on 16-byte boundaries: an aligned copy
+      void* copy = nullptr;
+      a.lda = (cols + 7) & ~7;
+      MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 2 * (size_t)T * a.lda, &copy));
+      MST_TRY(mst_pad_rows(in, ldin, T, cols, copy, s));
+      a.A = copy;
+    }
+    a.epilogue = MST_TC_OUT_BF16;
+    a.splits = 1;
+    a.act = act; a.pre = pre; a.ldpre = ldpre;
+    return mst_tc_gemm(a, s);
   }
   // CUDA cores: the product lands in the pre-activation buffer when the caller keeps one, else in the output
   void* prod = (act == MST_ACT_GELU && pre) ? pre : out;

@@ -182,40 +182,51 @@ __global__ void fill_csc(const uint32_t* __restrict__ bitsT, const int32_t* __re
   mst_fill_csc_word(w, threadIdx.x & 31, bitsT, wscanT, O, I, wpr, wpc, bits, wscan, row_idx, perm, col_ptr);
 }
 
-// ---- dense bf16 image of W.M (or its transpose) for the tensor-core path ----------------------------------------------
-// One thread per 8 consecutive columns: the stored values of those columns are consecutive in CSR (or CSC) order, so
-// the thread reads them in one run and writes one 16-byte vector (value or +0 per column).  Every element is written,
-// no separate clear.  Needs C % 8 == 0 (the tensor-core path requires it anyway).
-__global__ void densify_from_bits(const uint32_t* __restrict__ bits, const int32_t* __restrict__ wscan, int R, int C,
-                                  int wpr, const uint16_t* __restrict__ vals, const int32_t* __restrict__ perm,
-                                  uint16_t* __restrict__ dense) {
+// ---- dense image of W.M for the tensor-core paths ----------------------------------------------------------------------
+// bf16 values: one bf16 image; fp32 values: three bf16 pieces (mst_split3) one image apart.  One thread per 8 consecutive
+// columns: the stored values of those columns are consecutive in CSR order, so the thread reads them in one run and writes
+// one 16-byte vector per image (value or +0 per column).  Every element is written, no separate clear.  Rows are ldp
+// elements apart, ldp = I rounded up to a multiple of 8 (what the TMA unit asks for); mask bits beyond I are zero.
+template <typename V>
+__global__ void densify_from_bits(const uint32_t* __restrict__ bits, const int32_t* __restrict__ wscan, int R, int ldp,
+                                  int wpr, const V* __restrict__ vals, uint16_t* __restrict__ dense) {
+  constexpr int PIECES = sizeof(V) == 4 ? 3 : 1;
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
   const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;  // group of 8 columns
-  const unsigned gpr = (unsigned)C >> 3;                     // groups per row
+  const unsigned gpr = (unsigned)ldp >> 3;                   // groups per row
   if (g >= (unsigned)R * gpr) return;
   const unsigned r = g / gpr, c8 = g - r * gpr;
   const unsigned w = r * (unsigned)wpr + (c8 >> 2);
   const uint32_t word = bits[w];
   const unsigned sh = (c8 & 3u) * 8u;
   uint32_t m = (word >> sh) & 0xFFu;
-  uint16_t out[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  uint32_t out[PIECES][8];
+#pragma unroll
+  for (int k = 0; k < PIECES; ++k)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) out[k][j] = 0u;
   if (m) {
     int32_t pos = wscan[w] + __popc(word & ((1u << sh) - 1u));
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       if ((m >> j) & 1u) {
-        out[j] = vals[perm ? perm[pos] : pos];
+        if (sizeof(V) == 4) {
+          uint32_t p[3];
+          mst_split3((float)vals[pos], p);
+#pragma unroll
+          for (int k = 0; k < PIECES; ++k) out[k][j] = p[k];
+        } else {
+          out[0][j] = (uint32_t)vals[pos];
+        }
         ++pos;
       }
     }
   }
-  uint4 v;
-  v.x = (uint32_t)out[0] | ((uint32_t)out[1] << 16);
-  v.y = (uint32_t)out[2] | ((uint32_t)out[3] << 16);
-  v.z = (uint32_t)out[4] | ((uint32_t)out[5] << 16);
-  v.w = (uint32_t)out[6] | ((uint32_t)out[7] << 16);
-  *reinterpret_cast<uint4*>(dense + (size_t)r * C + (size_t)c8 * 8) = v;
+#pragma unroll
+  for (int k = 0; k < PIECES; ++k)
+    *reinterpret_cast<uint4*>(dense + ((size_t)k * R + r) * ldp + (size_t)c8 * 8) =
+        make_uint4(out[k][0] | (out[k][1] << 16), out[k][2] | (out[k][3] << 16), out[k][4] | (out[k][5] << 16), out[k][6] | (out[k][7] << 16));
 }
 
 // ---- export / validate ---------------------------------------------------------------------------
@@ -338,13 +349,15 @@ mst_status_t mst_ensure_csc(const mst_layer* L, cudaStream_t s) {
   return mst_build_csc(const_cast<mst_layer*>(L), s);
 }
 
-// Dense bf16 image of W.M for the dense-tile kernels.  Without value tracking the image is rebuilt at every call
-// anyway, so it lives in a per-device scratch buffer shared by all layers (no per-layer memory; like the other
-// scratch kinds, calls that use it must not overlap on the GPU).  With value tracking the layer keeps its own image
-// and reuses it until the mask or the values change.
-mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image) {
+// Dense image of W.M for the tensor-core kernels (see densify_from_bits), *ld elements between its rows.  Without value
+// tracking the image is rebuilt at every call anyway, so it lives in a per-device scratch buffer shared by all layers (no
+// per-layer memory; like the other scratch kinds, calls that use it must not overlap on the GPU).  With value tracking the
+// layer keeps its own image and reuses it until the mask or the values change.
+mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image, int64_t* ld) {
   const int c = L->cur;
-  if (L->nnz == L->N) {  // every entry kept: the CSR values in row-major order are the dense matrix
+  const int ldp = (L->I + 7) & ~7;
+  *ld = ldp;
+  if (L->nnz == L->N && L->dtype == MST_BF16 && ldp == L->I) {  // every entry kept: the CSR values are the dense matrix
     *image = (const uint16_t*)L->vals[c];
     return MST_OK;
   }
@@ -358,15 +371,19 @@ mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** im
     L->dense_epoch = L->values_epoch;
   } else {
     void* ws = nullptr;
-    MST_TRY(mst_workspace_kind(MST_WS_IMAGE, 2 * (size_t)L->N, &ws));
+    MST_TRY(mst_workspace_kind(MST_WS_IMAGE, mst_image_bytes(L), &ws));
     dst = (uint16_t*)ws;
     *image = dst;
   }
-  const int64_t groups = L->N / 8;  // callers guarantee I % 8 == 0
-  MST_CUDA_TRY(mst_launch_overlapped(densify_from_bits, dim3(blocks_for(groups, 256)), dim3(256), 0, s,
-                                     (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, L->I, L->wpr,
-                                     (const uint16_t*)L->vals[c], (const int32_t*)nullptr, dst));
-  MST_CUDA_TRY(cudaGetLastError());
+  const int64_t groups = (int64_t)L->O * (ldp / 8);
+  if (L->dtype == MST_F32)
+    MST_CUDA_TRY(mst_launch_overlapped(densify_from_bits<float>, dim3(blocks_for(groups, 256)), dim3(256), 0, s,
+                                       (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, ldp, L->wpr,
+                                       (const float*)L->vals[c], dst));
+  else
+    MST_CUDA_TRY(mst_launch_overlapped(densify_from_bits<uint16_t>, dim3(blocks_for(groups, 256)), dim3(256), 0, s,
+                                       (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, ldp, L->wpr,
+                                       (const uint16_t*)L->vals[c], dst));
   return MST_OK;
 }
 
@@ -395,10 +412,9 @@ extern "C" mst_status_t mst_pack(mst_layer_t* L, const void* W_dense, int64_t ld
   MST_TRY(mst_rebuild_from_bits(L, set, W_dense, ldw, set, s));
   L->nnz = total;
   ++L->version;
-  // the CSC view serves the CUDA-core input gradient, the CSC export and the structure check: layers on the tensor
-  // path get it on demand
-  if (mst_use_tensor_path(L)) L->csc_valid = 0;
-  else MST_TRY(mst_build_csc(L, s));
+  // the CSC view serves the CUDA-core input gradient, the CSC export and the structure check: other layers get it on demand
+  L->csc_valid = 0;
+  if (mst_use_csc(L)) MST_TRY(mst_build_csc(L, s));
   MST_CUDA_TRY(cudaStreamSynchronize(s));
   return MST_OK;
 }

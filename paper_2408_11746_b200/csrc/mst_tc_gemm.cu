@@ -148,13 +148,19 @@ __device__ __forceinline__ void act_chunk(const Params& P, uint32_t (&r)[32], ui
   }
 }
 
-// One 128 x BN accumulator (tensor-memory lanes = rows) -> global memory, 32 columns at a time, each thread storing
-// its own row.  q = lane quarter this warp may read, m0/n0 = first row / column of this block's tile.
-// c0 = first chunk this warp takes; the warps of one lane quarter interleave their chunks.
-__device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t tmem_base, int acc, int q, int c0, int lane,
+// One 128 x BN accumulator (tensor-memory lanes = rows) -> rows of any leading dimension and alignment, for outputs the TMA
+// unit cannot describe.  q = lane quarter this warp may read, m0/n0 = first row / column of this block's tile, c0 = first
+// 32-column chunk this warp takes (the warps of one lane quarter interleave their chunks).  A chunk goes through the warp's
+// staging box, so that a store instruction writes 32 neighbours of one row; stores by the row-owning lanes touch 32 lines
+// each (2051 x 1999 bf16 outputs: 4.1 M two-byte stores to as many sectors).
+__device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, uint32_t tmem_base, int acc, int q, int c0, int lane,
                                               int64_t m0, int n0, int split) {
-  const int64_t m = (int64_t)m0 + q * 32 + lane;
+  const int64_t row0 = (int64_t)m0 + q * 32;
+  const int64_t m = row0 + lane;
   const bool row_ok = m < P.M;
+  const uint32_t my_row = stage + (uint32_t)lane * 128u;
+  const uint32_t sw = (uint32_t)(lane & 7);
+  const int rows = P.M - row0 < 32 ? (int)(P.M - row0) : 32;
 #pragma unroll 1
   for (int c = c0; c < BN / 32; c += EPI_WARPS / 4) {
     const int n = n0 + c * 32;
@@ -169,57 +175,29 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t tmem_bas
       for (int v = 0; v < 4; ++v) p4[v] = __ldg(reinterpret_cast<const uint4*>(pre) + v);
     }
     tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
-    if (!row_ok) continue;
-    if (P.epilogue == MST_TC_OUT_BF16) {
-      if (P.act) act_chunk(P, r, pre, pre_vec, p4, n);
-      uint16_t* dst = reinterpret_cast<uint16_t*>(P.out) + m * P.ldc + n;
-      if (n + 32 <= P.N && ((P.ldc & 7) == 0) && ((reinterpret_cast<uintptr_t>(P.out) & 15u) == 0)) {
+    if (P.act && row_ok) act_chunk(P, r, pre, pre_vec, p4, n);
+    __syncwarp();  // the previous chunk has been read out of the box
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          uint4 o;
-          o.x = pack_bf16(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1]));
-          o.y = pack_bf16(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3]));
-          o.z = pack_bf16(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5]));
-          o.w = pack_bf16(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7]));
-          reinterpret_cast<uint4*>(dst)[v] = o;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (n + j < P.N) dst[j] = (uint16_t)(pack_bf16(__uint_as_float(r[j]), 0.f) & 0xFFFFu);
-      }
-    } else if (P.epilogue == MST_TC_OUT_F32) {
-      float* base = P.splits > 1 ? P.partial + (int64_t)split * P.M * P.N + m * P.N : reinterpret_cast<float*>(P.out) + m * P.ldc;
-      float* dst = base + n;
-      const int64_t ld = P.splits > 1 ? P.N : P.ldc;
-      if (n + 32 <= P.N && ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(base) & 15u) == 0)) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v)
-          reinterpret_cast<uint4*>(dst)[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (n + j < P.N) dst[j] = __uint_as_float(r[j]);
-      }
-    } else {
-      // sampled: the 32 columns of this chunk are one mask word of row m
-      const int64_t wi = m * P.wpr + (n >> 5);
-      const uint32_t word = P.bits[wi];
-      float* dst = (P.splits > 1 ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out)) + P.wscan[wi];
-      if (word == 0xFFFFFFFFu) {
-        // dense stretch (a restored layer, a saturated row): the 32 values are contiguous in CSR order
-#pragma unroll
-        for (int j = 0; j < 32; ++j) dst[j] = __uint_as_float(r[j]);
-      } else {
-        int rank = 0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if ((word >> j) & 1u) {
-            dst[rank] = __uint_as_float(r[j]);
-            ++rank;
-          }
-        }
-      }
+    for (int v = 0; v < 8; ++v) {
+      const uint32_t piece = (uint32_t)v ^ sw;
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(my_row + piece * 16u), "r"(r[4 * v]), "r"(r[4 * v + 1]),
+                   "r"(r[4 * v + 2]), "r"(r[4 * v + 3])
+                   : "memory");
+    }
+    __syncwarp();
+    const bool col_ok = n + lane < P.N;
+    const bool bf16 = P.epilogue == MST_TC_OUT_BF16;
+    float* f32 = P.splits > 1 ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
+    const int64_t ld = bf16 || P.splits == 1 ? P.ldc : P.N;
+#pragma unroll 4
+    for (int rr = 0; rr < rows; ++rr) {
+      const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)(rr & 7);
+      float v;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(stage + (uint32_t)rr * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
+      const int64_t at = (row0 + rr) * ld + n + lane;
+      if (!col_ok) continue;
+      if (bf16) reinterpret_cast<uint16_t*>(P.out)[at] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
+      else f32[at] = v;
     }
   }
 }
@@ -493,7 +471,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                               n0, split);
       else
-        epilogue_tile(P, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
+        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
@@ -700,7 +678,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                               n0, split);
       else
-        epilogue_tile(P, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
+        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(in_even_block(tempty0 + 8 * acc));
@@ -748,25 +726,9 @@ __global__ void tc_reduce4_kernel(const float4* __restrict__ partial, int splits
 }
 
 // ------------------------------------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
 // rows x cols (cols contiguous, ld elements between rows) bf16 matrix; box = box_rows x 64 columns
 bool make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-  EncodeTiledFn fn = encode_fn();
+  mst_encode_tiled_fn fn = mst_encode_tiled();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
@@ -780,7 +742,7 @@ bool make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int
 // Output maps for the staged epilogue.  bf16 [M x N] (ld elements between rows), box 64 columns x 32 rows;
 // fp32 [splits x M x N], box 32 columns x 32 rows x 1.  Both boxes are 128 bytes wide (128-byte swizzle).
 bool make_out_map_bf16(CUtensorMap* tm, void* base, int64_t M, int64_t N, int64_t ld) {
-  EncodeTiledFn fn = encode_fn();
+  mst_encode_tiled_fn fn = mst_encode_tiled();
   if (!fn || (ld % 8) != 0 || (reinterpret_cast<uintptr_t>(base) & 15u) != 0) return false;
   cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
@@ -790,7 +752,7 @@ bool make_out_map_bf16(CUtensorMap* tm, void* base, int64_t M, int64_t N, int64_
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 bool make_out_map_f32(CUtensorMap* tm, void* base, int64_t M, int64_t N, int64_t ld, int64_t slab_elems, int splits) {
-  EncodeTiledFn fn = encode_fn();
+  mst_encode_tiled_fn fn = mst_encode_tiled();
   if (!fn || (ld % 4) != 0 || (slab_elems % 4) != 0 || (reinterpret_cast<uintptr_t>(base) & 15u) != 0) return false;
   cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)splits};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)slab_elems * 4};
@@ -800,7 +762,21 @@ bool make_out_map_f32(CUtensorMap* tm, void* base, int64_t M, int64_t N, int64_t
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int sm_count() {
+}  // namespace
+
+mst_encode_tiled_fn mst_encode_tiled() {
+  static mst_encode_tiled_fn fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = (mst_encode_tiled_fn)p;
+  }
+  return fn;
+}
+
+int mst_sm_count() {
   static int n[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -810,8 +786,6 @@ int sm_count() {
   }
   return n[dev];
 }
-
-}  // namespace
 
 // Number of K ranges for a contraction whose output has few tiles: minimise a simple time model
 //   waves * (k-blocks per range * t_kblock + t_tile) + traffic of the partial sums
@@ -869,7 +843,7 @@ mst_status_t mst_workspace(size_t bytes, void** ptr) { return mst_workspace_kind
 
 bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb) {
   return (lda % 8 == 0) && (ldb % 8 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15u) == 0) &&
-         ((reinterpret_cast<uintptr_t>(B) & 15u) == 0) && encode_fn() != nullptr;
+         ((reinterpret_cast<uintptr_t>(B) & 15u) == 0) && mst_encode_tiled() != nullptr;
 }
 
 mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
@@ -910,7 +884,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.epilogue != MST_TC_OUT_BF16) {
     // few output tiles: cut the contraction range so that all SMs work; partial sums go to the shared scratch buffer
     const int64_t works1 = pair ? (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles : (int64_t)P.m_tiles * P.n_tiles;
-    const int64_t slots = pair ? sm_count() / 2 : sm_count();
+    const int64_t slots = pair ? mst_sm_count() / 2 : mst_sm_count();
     const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
     P.splits = a.splits > 0 ? a.splits : mst_tc_pick_splits(works1, slots, P.kblocks, out_bytes);
     if (const char* e = getenv("MST_TC_SPLITS")) {  // measurement override
@@ -942,13 +916,13 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (pair) {
     MST_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P_SMEM_BYTES));
     const int64_t works = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits;
-    const int64_t max_pairs = sm_count() / 2;
+    const int64_t max_pairs = mst_sm_count() / 2;
     const int grid = 2 * (int)(works < max_pairs ? works : max_pairs);
     MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel, dim3(grid), dim3(NUM_THREADS), P_SMEM_BYTES, s, tmA, tmB, tmC, P));
   } else {
     MST_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
     const int64_t works = (int64_t)P.m_tiles * P.n_tiles * P.splits;
-    const int grid = (int)(works < sm_count() ? works : sm_count());
+    const int grid = (int)(works < mst_sm_count() ? works : mst_sm_count());
     MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_kernel, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, s, tmA, tmB, tmC, P));
   }
   MST_CUDA_TRY(cudaGetLastError());
@@ -978,6 +952,9 @@ extern "C" mst_status_t mst_device_error_flags(int32_t* flags) {
   int32_t sd = 0;
   MST_TRY(mst_sddmm_error_flags(&sd));
   cc |= sd;
+  int32_t f32 = 0;
+  MST_TRY(mst_split_error_flags(&f32));
+  v |= f32;
   *flags = v | (att << 1) | (sp << 2) | (cc << 3);
   return MST_OK;
 }

@@ -1,6 +1,7 @@
 // Interface of the tcgen05 (5th-generation tensor core) bf16 contraction used for the dense gradient,
 // the dense-tile SpMM path and the sampled weight gradient.  Internal to libmst.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -51,10 +52,31 @@ struct mst_tc_gemm_args {
   int64_t ldpre;
 };
 
+// C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_split_rows; lda / ldb are the pieces'
+// leading dimensions, M / N / K the matrix sizes).  Epilogues F32 (rows) and SAMPLED.
+mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s);
+// Operand preparation (leading dimension of the result: C rounded up to a multiple of 8):
+//   split_rows  fp32 [R x C] -> three bf16 pieces [3][R][ldp] whose sum is the operand
+//   pad_rows    bf16 [R x C] -> the same rows, 16-byte aligned
+mst_status_t mst_split_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s);
+mst_status_t mst_pad_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s);
+
+// dY^T X over T tokens with the sizes and the epilogue in `a` (M = O, N = I, K = T; F32 or SAMPLED), operands as the caller
+// has them (mst_dense_grad.cu)
+mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* dY, int64_t lddy, const void* X, int64_t ldx,
+                             cudaStream_t s);
+
 // Returns MST_ERR_SHAPE when the operands cannot be described to the TMA unit (leading dimension or base address
 // not 16-byte aligned); the caller then falls back to the CUDA-core kernel.
 mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s);
 bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb);
+
+// cuTensorMapEncodeTiled of the loaded driver (nullptr when it has none) and the SM count of the current device
+typedef CUresult (*mst_encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                        const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                        CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+mst_encode_tiled_fn mst_encode_tiled();
+int mst_sm_count();
 
 int mst_tc_pick_splits(int64_t works1, int64_t slots, int64_t kblocks, double out_bytes);
 

@@ -1,0 +1,425 @@
+// fp32 contraction on the 5th-generation tensor cores: every fp32 operand is cut into three bf16 pieces whose sum is
+// exactly the operand (8 + 8 + 8 significand bits), and the product is the sum of the six piece products down to
+// 2^-18 of the leading one.  The three products left out are below 2^-26 of |a b| together, less than the rounding of
+// one fp32 multiplication.
+//
+// Sums.  The tensor core adds into an fp32 accumulator with truncation, so a long chain of additions would drift by
+// more than an fp32 FMA chain does.  Therefore the leading products (a0 b0) and the five small ones go to accumulators
+// of their own, and both are emptied into registers, with ordinary rounded fp32 additions, every 64 contraction
+// indices: at most four truncating additions meet a sum of full size.  Error against fp64 (2-norm, normal operands):
+// 0.7-0.9e-7 for the 3072 x 768 layer at 256 tokens, 1.0-1.6e-7 for 2048 x 4096 at 1024 tokens, where the FMA chains of the
+// CUDA-core kernels leave 2.5-5e-7 and 6-12e-7 (emptied every 256 indices: 2.3e-7, all of it drift).
+//
+// What bounds it: six bf16 MMAs per fp32 product, so 1654 / 6 = 276 TFLOP/s of the measured bf16 peak against 74 for the
+// fp32 FMA pipe; at the few hundred tokens of the fp32 workloads the launch, the pipeline fill and the drain of one tile
+// cost as much as the products.  Hence small tiles (128 x 64) when the output has few of them, and a split of the
+// contraction range whose last block adds the partial sums in a fixed order (no second launch).  3072 x 768, d = 0.25, 256
+// tokens: forward, input gradient and dense gradient with their operand preparation took 65 + 118 + 51 us on the CUDA
+// cores (69 / 123 / 51 with their transposes), about 20 us each here.
+//
+// One block per tile and range, 320 threads: one lane of warp 0 fetches [3 pieces x rows x 64] boxes with TMA, one lane of
+// warp 1 issues the MMAs, warps 2-9 own the sums (one row and BN / 2 columns per thread).  Every wait is bounded.
+#include <cuda.h>
+
+#include "mst_bits.cuh"
+#include "mst_internal.cuh"
+#include "mst_tc_gemm.cuh"
+#include "mst_tc_ptx.cuh"
+
+namespace {
+
+using namespace mst_ptx;
+
+__device__ int g_split_error = 0;  // sticky: a bounded wait expired
+
+constexpr int SBM = 128, SBK = 64;
+constexpr int PIECES = 3;
+constexpr int S_EPI_WARPS = 8;
+constexpr int S_THREADS = 64 + 32 * S_EPI_WARPS;
+constexpr int CHUNK_KB = 1;                 // k-blocks summed inside the tensor core before the sums move to registers
+constexpr int MAX_SPLIT_TILES = 1024;
+constexpr int BOX64 = 64 * SBK * 2;         // one piece of one 64-wide MN-major box
+
+__device__ unsigned int g_split_arrivals[MAX_SPLIT_TILES];  // blocks of a tile that have stored their partial sums; wraps to 0
+
+template <int BN>
+struct SplitCfg {
+  static constexpr int A_BYTES = PIECES * SBM * SBK * 2;
+  static constexpr int B_BYTES = PIECES * BN * SBK * 2;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = BN == 64 ? 3 : 2;
+  static constexpr int TMEM = 4 * BN;       // two chunk buffers x (leading, small)
+  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 128;
+};
+
+struct SplitParams {
+  int64_t M, N;
+  int kblocks, splits, m_tiles, n_tiles;
+  int a_mn, b_mn;
+  int sampled;
+  float* out;
+  int64_t ldc;
+  const uint32_t* bits;
+  const int32_t* wscan;
+  int wpr;
+  float* partial;   // [splits][tiles][8 warps][BN / 8 vectors][32 lanes] float4
+};
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+
+template <int BN>
+__global__ void __launch_bounds__(S_THREADS, 1)
+tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
+  typedef SplitCfg<BN> C;
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t tiles_base = (raw + 1023u) & ~1023u;
+  const uint32_t bar_base = tiles_base + C::STAGES * C::STAGE_BYTES;
+  const uint32_t full0 = bar_base, empty0 = full0 + 8 * C::STAGES, tfull0 = empty0 + 8 * C::STAGES, tempty0 = tfull0 + 16;
+  __shared__ uint32_t tmem_base_holder;
+  __shared__ int abort_sh;
+  __shared__ unsigned int arrived_sh;
+  volatile int* abort_flag = &abort_sh;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    abort_sh = 0;
+    for (int s = 0; s < C::STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(tfull0 + 8 * a, 1);
+      mbar_init(tempty0 + 8 * a, S_EPI_WARPS);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)), "r"(C::TMEM)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_holder;
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+
+  const int tiles = P.m_tiles * P.n_tiles;
+  const int split = blockIdx.x / tiles, tile = blockIdx.x % tiles;
+  const int m0 = (tile / P.n_tiles) * SBM, n0 = (tile % P.n_tiles) * BN;
+  const int kb0 = (int)((int64_t)split * P.kblocks / P.splits), kb1 = (int)((int64_t)(split + 1) * P.kblocks / P.splits);
+  const int chunks = (kb1 - kb0 + CHUNK_KB - 1) / CHUNK_KB;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, &g_split_error)) break;
+        const uint32_t fb = full0 + 8 * s, sa = tiles_base + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+        mbar_expect_tx(fb, C::STAGE_BYTES);
+        if (P.a_mn) {
+          for (int j = 0; j < SBM / 64; ++j) tma_load_3d(sa + j * PIECES * BOX64, &tmA, m0 + j * 64, kb * SBK, 0, fb);
+        } else {
+          tma_load_3d(sa, &tmA, kb * SBK, m0, 0, fb);
+        }
+        if (P.b_mn) {
+          for (int j = 0; j < BN / 64; ++j) tma_load_3d(sb + j * PIECES * BOX64, &tmB, n0 + j * 64, kb * SBK, 0, fb);
+        } else {
+          tma_load_3d(sb, &tmB, kb * SBK, n0, 0, fb);
+        }
+        if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
+                             ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
+      // K-major: the three pieces of a stage lie one after the other; MN-major: 64-wide blocks, each with its three pieces
+      const uint64_t ad0 = smem_desc(tiles_base, P.a_mn ? PIECES * BOX64 : 16, 1024);
+      const uint64_t bd0 = smem_desc(tiles_base + C::A_BYTES, P.b_mn ? PIECES * BOX64 : 16, 1024);
+      const uint32_t a_piece = (uint32_t)(P.a_mn ? BOX64 : SBM * SBK * 2) >> 4, b_piece = (uint32_t)(P.b_mn ? BOX64 : BN * SBK * 2) >> 4;
+      const uint32_t a_k = (uint32_t)(P.a_mn ? 16 * 128 : 32) >> 4, b_k = (uint32_t)(P.b_mn ? 16 * 128 : 32) >> 4;
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int c = 0; c < chunks && ok; ++c) {
+        const int buf = c & 1;
+        if (!mbar_wait(tempty0 + 8 * buf, ((c >> 1) & 1) ^ 1u, abort_flag, &g_split_error)) break;
+        tc_fence_after();
+        const uint32_t d_hi = tmem_base + (uint32_t)(buf * 2 * BN), d_lo = d_hi + BN;
+        const int first = kb0 + c * CHUNK_KB, last = first + CHUNK_KB < kb1 ? first + CHUNK_KB : kb1;
+        for (int kb = first; kb < last; ++kb) {
+          if (!mbar_wait(full0 + 8 * s, ph, abort_flag, &g_split_error)) { ok = false; break; }
+          tc_fence_after();
+          const uint64_t ad = ad0 + (uint64_t)(uint32_t)(s * (C::STAGE_BYTES >> 4)), bd = bd0 + (uint64_t)(uint32_t)(s * (C::STAGE_BYTES >> 4));
+#pragma unroll
+          for (int k = 0; k < SBK / 16; ++k) {
+            const uint32_t more = (kb > first || k > 0) ? 1u : 0u;
+            const uint64_t a0 = ad + (uint64_t)(k * a_k), b0 = bd + (uint64_t)(k * b_k);
+            const uint64_t a1 = a0 + a_piece, a2 = a1 + a_piece, b1 = b0 + b_piece, b2 = b1 + b_piece;
+            tc_mma(d_lo, a2, b0, idesc, more);
+            tc_mma(d_lo, a0, b2, idesc, 1u);
+            tc_mma(d_lo, a1, b1, idesc, 1u);
+            tc_mma(d_lo, a1, b0, idesc, 1u);
+            tc_mma(d_lo, a0, b1, idesc, 1u);
+            tc_mma(d_hi, a0, b0, idesc, more);
+          }
+          tc_commit(empty0 + 8 * s);
+          if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+        }
+        if (ok) tc_commit(tfull0 + 8 * buf);
+      }
+    }
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    constexpr int COLS = BN / 2;   // columns of this thread's row
+    float acc[COLS];
+#pragma unroll
+    for (int j = 0; j < COLS; ++j) acc[j] = 0.f;
+    for (int c = 0; c < chunks; ++c) {
+      const int buf = c & 1;
+      if (!mbar_wait(tfull0 + 8 * buf, (c >> 1) & 1, abort_flag, &g_split_error)) break;
+      tc_fence_after();
+      const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BN + half * COLS);
+#pragma unroll
+      for (int g = 0; g < COLS / 32; ++g) {
+        uint32_t hi[32], lo[32];
+        tmem_ld32_nowait(at + g * 32, hi);
+        tmem_ld32_nowait(at + BN + g * 32, lo);
+        tmem_ld_wait(hi);
+        tmem_ld_wait(lo);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[g * 32 + j] += __uint_as_float(hi[j]) + __uint_as_float(lo[j]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
+    }
+    bool mine = true;
+    if (P.splits > 1) {
+      // partial sums to the scratch buffer; the last block of the tile to arrive adds all of them in range order
+      const size_t slab = (size_t)tiles * S_EPI_WARPS * (COLS / 4) * 32;
+      float4* part = reinterpret_cast<float4*>(P.partial) + ((size_t)tile * S_EPI_WARPS + (warp - 2)) * (COLS / 4) * 32 + lane;
+#pragma unroll
+      for (int v = 0; v < COLS / 4; ++v)
+        __stcg(part + (size_t)split * slab + v * 32, make_float4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]));
+      __threadfence();
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * S_EPI_WARPS) : "memory");
+      if (threadIdx.x == 64) arrived_sh = atomicInc(&g_split_arrivals[tile], (unsigned)P.splits - 1u);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * S_EPI_WARPS) : "memory");
+      mine = arrived_sh == (unsigned)P.splits - 1u;
+      if (mine) {
+        __threadfence();
+#pragma unroll
+        for (int j = 0; j < COLS; ++j) acc[j] = 0.f;
+        for (int sp = 0; sp < P.splits; ++sp) {
+#pragma unroll
+          for (int v = 0; v < COLS / 4; ++v) {
+            const float4 t = __ldcg(part + (size_t)sp * slab + v * 32);
+            acc[4 * v] += t.x; acc[4 * v + 1] += t.y; acc[4 * v + 2] += t.z; acc[4 * v + 3] += t.w;
+          }
+        }
+      }
+    }
+    if (mine && !*abort_flag) {
+      // every MMA of the block has completed, so the operand stages serve as staging: a 32 x 32 square per warp, turned
+      // from rows to columns so that a store instruction writes neighbours
+      float* box = reinterpret_cast<float*>(smem_raw + (tiles_base - raw)) + (warp - 2) * (32 * 33);
+      const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+      for (int g = 0; g < COLS / 32; ++g) {
+        const int n = n0 + half * COLS + g * 32;
+        if (n >= P.N) break;   // uniform
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) box[lane * 33 + j] = acc[g * 32 + j];
+        __syncwarp();
+        const int64_t row0 = (int64_t)m0 + q * 32;
+        if (P.sampled) {
+          uint32_t word = 0;
+          int32_t at = 0;
+          if (row0 + lane < P.M) {
+            const int64_t wi = (row0 + lane) * P.wpr + (n >> 5);
+            word = P.bits[wi];
+            at = P.wscan[wi];
+          }
+#pragma unroll 4
+          for (int rr = 0; rr < 32; ++rr) {
+            const uint32_t w = __shfl_sync(0xffffffffu, word, rr);
+            const int32_t base = __shfl_sync(0xffffffffu, at, rr);
+            if ((w >> lane) & 1u) P.out[base + __popc(w & lt)] = box[rr * 33 + lane];
+          }
+        } else {
+          const bool col_ok = n + lane < P.N;
+#pragma unroll 4
+          for (int rr = 0; rr < 32; ++rr) {
+            if (row0 + rr >= P.M) break;  // uniform
+            if (col_ok) P.out[(row0 + rr) * P.ldc + n + lane] = box[rr * 33 + lane];
+          }
+        }
+      }
+    }
+  }
+
+  if (*abort_flag) {
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // copies and MMAs in flight land before memory is given back
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::TMEM) : "memory");
+  }
+}
+
+// ---- operand preparation -----------------------------------------------------------------------------------------------
+// 8 consecutive columns per thread.  fp32 rows -> three bf16 pieces [3][R][ldp]; bf16 rows -> the same rows at a leading
+// dimension and an address the TMA unit accepts.  Columns C .. ldp-1 become +0.  Memory-bound: 4 + 6 (2 + 2) bytes per
+// element.
+__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ in, int64_t ld, int64_t R, int C, int ldp,
+                                                         uint16_t* __restrict__ out, int vec_ok) {
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+  const int gpr = ldp >> 3;
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= R * gpr) return;
+  const int64_t r = g / gpr;
+  const int c = (int)(g - r * gpr) * 8;
+  float x[8];
+  const float* src = in + r * ld + c;
+  if (vec_ok && c + 8 <= C) {
+    const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = c + j < C ? src[j] : 0.f;
+  }
+  uint32_t p[PIECES][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint32_t lo[PIECES], hi[PIECES];
+    mst_split3(x[2 * j], lo);
+    mst_split3(x[2 * j + 1], hi);
+#pragma unroll
+    for (int k = 0; k < PIECES; ++k) p[k][j] = lo[k] | (hi[k] << 16);
+  }
+#pragma unroll
+  for (int k = 0; k < PIECES; ++k)
+    *reinterpret_cast<uint4*>(out + ((size_t)k * R + r) * ldp + c) = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
+}
+
+__global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restrict__ in, int64_t ld, int64_t R, int C, int ldp,
+                                                       uint16_t* __restrict__ out) {
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+  const int gpr = ldp >> 3;
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= R * gpr) return;
+  const int64_t r = g / gpr;
+  const int c = (int)(g - r * gpr) * 8;
+  const uint16_t* src = in + r * ld + c;
+  uint32_t v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t lo = c + 2 * j < C ? src[2 * j] : 0u, hi = c + 2 * j + 1 < C ? src[2 * j + 1] : 0u;
+    v[j] = lo | (hi << 16);
+  }
+  *reinterpret_cast<uint4*>(out + (size_t)r * ldp + c) = make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// pieces [3][rows][ld] as a 3-d map: rows and columns beyond the matrix read as zero inside every piece
+bool make_piece_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+  mst_encode_tiled_fn fn = mst_encode_tiled();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, PIECES};
+  cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)(ld * rows) * 2};
+  cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, PIECES};
+  cuuint32_t estr[3] = {1u, 1u, 1u};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int BN>
+mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
+  MST_CUDA_TRY(cudaFuncSetAttribute(tc_split_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SplitCfg<BN>::SMEM));
+  MST_CUDA_TRY(mst_launch_overlapped(tc_split_kernel<BN>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)), dim3(S_THREADS),
+                                     SplitCfg<BN>::SMEM, s, tmA, tmB, P));
+  return MST_OK;
+}
+
+}  // namespace
+
+mst_status_t mst_split_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s) {
+  const int ldp = (C + 7) & ~7;
+  const int vec_ok = (ld % 4 == 0 && (reinterpret_cast<uintptr_t>(in) & 15u) == 0) ? 1 : 0;
+  const int64_t n = R * (ldp / 8);
+  MST_CUDA_TRY(mst_launch_overlapped(split_rows_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, (const float*)in, ld, R, C,
+                                     ldp, (uint16_t*)out, vec_ok));
+  return MST_OK;
+}
+
+mst_status_t mst_pad_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s) {
+  const int ldp = (C + 7) & ~7;
+  const int64_t n = R * (ldp / 8);
+  MST_CUDA_TRY(mst_launch_overlapped(pad_rows_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, (const uint16_t*)in, ld, R, C,
+                                     ldp, (uint16_t*)out));
+  return MST_OK;
+}
+
+mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s) {
+  SplitParams P = {};
+  P.M = a.M;
+  P.N = a.N;
+  P.kblocks = (int)((a.K + SBK - 1) / SBK);
+  P.m_tiles = (int)((a.M + SBM - 1) / SBM);
+  P.a_mn = a.a_mn_major;
+  P.b_mn = a.b_mn_major;
+  P.sampled = a.epilogue == MST_TC_OUT_SAMPLED;
+  P.out = (float*)a.out;
+  P.ldc = a.ldc;
+  P.bits = a.bits;
+  P.wscan = a.wscan;
+  P.wpr = a.wpr;
+  // Tile width and number of K ranges from a time model in SM clocks: 24 MMAs per k-block (64 clocks each at 128 columns, 40
+  // at 64, where the A operand's shared-memory reads dominate), about 4000 for launch, fill and drain of a block, and the
+  // last block's read of the partial sums.
+  const int sms = mst_sm_count();
+  int bn = 128, splits = 1;
+  double best = 1e30;
+  for (int w = 64; w <= 128; w += 64) {
+    const int64_t tiles = (int64_t)P.m_tiles * ((a.N + w - 1) / w);
+    for (int sp = 1; sp <= 8 && sp <= P.kblocks && (sp == 1 || tiles <= MAX_SPLIT_TILES); ++sp) {
+      const int64_t waves = (tiles * sp + sms - 1) / sms;
+      const int kb = (P.kblocks + sp - 1) / sp;
+      const double t = (double)waves * (kb * (w == 64 ? 960.0 : 1536.0) + 4000.0) + (sp > 1 ? 2000.0 + sp * 5.0 * w : 0.0);
+      if (t < best * 0.97) { best = t; bn = w; splits = sp; }
+    }
+  }
+  P.splits = splits;
+  P.n_tiles = (int)((a.N + bn - 1) / bn);
+  CUtensorMap tmA, tmB;
+  const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, a.M, a.K, a.lda, SBM);
+  const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, a.N, a.K, a.ldb, bn);
+  if (!okA || !okB) return MST_ERR_SHAPE;
+  if (splits > 1) {
+    void* ws = nullptr;
+    MST_TRY(mst_workspace(sizeof(float) * (size_t)splits * P.m_tiles * P.n_tiles * SBM * bn, &ws));
+    P.partial = (float*)ws;
+  }
+  return bn == 64 ? launch_split<64>(tmA, tmB, P, s) : launch_split<128>(tmA, tmB, P, s);
+}
+
+mst_status_t mst_split_error_flags(int32_t* flags) {
+  int v = 0;
+  MST_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_split_error, sizeof(int)));
+  *flags = v;
+  return MST_OK;
+}

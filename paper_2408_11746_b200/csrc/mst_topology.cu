@@ -2077,7 +2077,7 @@ void fill_fused_params(const UpdatePlan& pl, FusedParams& F) {
   F.new_wscan = L->wscan[n]; F.new_row_ptr = L->row_ptr[n]; F.new_col = L->col_idx[n]; F.new_vals = L->vals[n];
   F.bitsT = L->bitsT; F.wscanT = L->wscanT; F.col_ptr = L->col_ptr; F.row_idx = L->row_idx; F.perm = L->perm;
   F.wpc = L->wpc; F.nwordsT = L->nwordsT;
-  F.build_csc = mst_use_tensor_path(L) ? 0 : 1;
+  F.build_csc = mst_use_csc(L) ? 1 : 0;
   F.smem_keys = 0;
   F.dual = 0;
   F.g_bulk = 0;
@@ -2234,7 +2234,7 @@ mst_status_t launch_single_update(const UpdatePlan& pl, cudaStream_t s, bool* fu
       MST_CUDA_TRY(cudaMemsetAsync(L->hist, 0, sizeof(unsigned int) * 3 * HSTRIDE, s));
       MST_CUDA_TRY(cudaMemsetAsync(L->rand_ctr, 0, 2 * sizeof(unsigned long long), s));
     }
-    if (!mst_use_tensor_path(L)) MST_TRY(mst_alloc_csc(L));   // the kernel fills the view's arrays for such layers
+    if (mst_use_csc(L)) MST_TRY(mst_alloc_csc(L));   // the kernel fills the view's arrays for such layers
     FusedParams F;
     fill_fused_params(pl, F);
     F.smem_keys = smem_keys;
@@ -2322,7 +2322,7 @@ extern "C" mst_status_t mst_topology_update_many(int32_t n_layers, mst_layer_t* 
     while (batching && i < n_layers && B.n < BATCH_MAX) {
       mst_layer* L = plans[i].L;
       const size_t per = (size_t)((L->nwords + grid_limit - 1) / grid_limit);
-      const bool ok = mst_use_tensor_path(L) && 2 * (int64_t)grid_limit <= mst_scan_block_sums_len(L->nwords) + 1024 &&
+      const bool ok = !mst_use_csc(L) && 2 * (int64_t)grid_limit <= mst_scan_block_sums_len(L->nwords) + 1024 &&
                       (words + 3 * per) * 4 <= 40 * 1024;
       if (!ok) break;
       B.smem_off[B.n] = (int)words;

@@ -1,0 +1,71 @@
+"""fp32 layers on the tensor cores (three exact bf16 pieces per operand) and bf16 layers whose rows start anywhere:
+edges of the 128 x 64 / 128 x 128 tiles and of the 64-wide contraction blocks, against an fp64 product."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import paper_2408_11746_b200 as mst  # noqa: E402
+
+
+def _rel(got, ref):
+    return float((got.double() - ref).norm() / ref.norm().clamp_min(1e-300))
+
+
+def _layer_case(O, I, T, dtype, density, seed, pad=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    dt, mdt = (torch.float32, mst.MST_F32) if dtype == "f32" else (torch.bfloat16, mst.MST_BF16)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda").to(dt)
+    X, dY, W = n(T, I + pad), n(T, O + pad), n(O, I)
+    M = (torch.rand(O, I, generator=g, device="cuda") < density).to(torch.uint8)
+    M[0, 0] = 1
+    L = mst.Layer(0, O, I, mdt)
+    L.pack(W, M)
+    Y = torch.full((T, O + pad), float("nan"), dtype=dt, device="cuda")
+    dX = torch.full((T, I + pad), float("nan"), dtype=dt, device="cuda")
+    dW = torch.full((L.nnz,), float("nan"), device="cuda")
+    G = torch.full((O, I), float("nan"), device="cuda")
+    mst.mst_spmm_fwd(L.handle, X, I + pad, T, Y, O + pad)
+    mst.mst_spmm_bwd_x(L.handle, dY, O + pad, T, dX, I + pad)
+    mst.mst_sddmm_dw(L.handle, dY, O + pad, X, I + pad, T, dW)
+    mst.mst_dense_grad(dY, O + pad, X, I + pad, T, O, I, mdt, G)
+    assert mst.mst_device_error_flags() == 0
+    Xr, dYr, Wr = X[:, :I].double(), dY[:, :O].double(), (W * M.to(dt)).double()
+    Gr = dYr.T @ Xr
+    if pad:                                     # columns beyond the matrix are not written
+        assert bool(Y[:, O:].isnan().all()) and bool(dX[:, I:].isnan().all())
+    out = (_rel(Y[:, :O], Xr @ Wr.T), _rel(dX[:, :I], dYr @ Wr), _rel(dW, Gr[M.bool()]), _rel(G, Gr))
+    L.close()
+    return out
+
+
+@pytest.mark.parametrize("O,I,T", [(1, 1, 1), (64, 64, 64), (65, 63, 129), (128, 128, 128), (127, 257, 65), (300, 40, 1000),
+                                   (40, 2050, 33), (2051, 130, 257)])
+def test_fp32_products_are_single_precision(O, I, T):
+    for err in _layer_case(O, I, T, "f32", 0.3, O + I + T):
+        assert err <= 5e-7
+
+
+def test_fp32_extreme_magnitudes():
+    # pieces of values near the top and the bottom of the normal range; sums stay finite
+    O, I, T = 70, 66, 40
+    X = torch.zeros(T, I, device="cuda")
+    X[:, 0], X[:, 1] = 3.4028234e38, 1e-30
+    W = torch.zeros(O, I, device="cuda")
+    W[:, 0], W[:, 1] = 0.99999994, 1.0
+    L = mst.Layer(0, O, I, mst.MST_F32)
+    L.pack(W, torch.ones(O, I, dtype=torch.uint8, device="cuda"))
+    Y = torch.empty(T, O, device="cuda")
+    L.fwd(X, Y, T)
+    ref = X.double() @ W.double().T
+    assert bool(torch.isfinite(Y).all()) and float(((Y.double() - ref) / ref).abs().max()) <= 3e-7
+    L.close()
+
+
+@pytest.mark.parametrize("O,I,T,pad", [(65, 63, 129, 0), (255, 257, 300, 0), (64, 128, 130, 3), (513, 31, 520, 5), (1, 3, 1, 0)])
+def test_bf16_rows_at_any_address(O, I, T, pad):
+    y, dx, dw, g = _layer_case(O, I, T, "bf16", 0.3, O + I + T, pad)
+    assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
