@@ -474,14 +474,9 @@ def run_profile_case(args) -> None:
         lib = ctypes.CDLL(os.path.join(ROOT, "paper_2408_11746_b200", "libmst.so"))
         if not hasattr(lib, "mst_update_profile"):
             raise SystemExit("libmst.so was built without -DMST_UPD_PROFILE")
-        names = {2: "slice loaded", 4: "hash test of the inactive entries", 3: "keys and first histogram", 40: "tie ranking",
-                 41: "marking sweep", 42: "bracket list + barrier", 43: "threshold among the listed", 44: "random marks + new mask",
-                 49: "-", 51: "-", 52: "scan of the new mask (barrier inside)", 53: "CSR fill", 54: "scratch cleared",
-                 60: "prune selection (sequential form)", 61: "gradient selection (sequential form)", 62: "random selection (general form)"}
-        for p in range(3):
-            names[10 + p] = "histogram sweep %d" % p
-            names[20 + p] = "flush + barrier %d" % p
-            names[30 + p] = "digit picks %d" % p
+        names = {2: "samples", 18: "hashes of the inactive entries", 3: "barrier 0", 4: "brackets", 5: "sweep", 6: "bins of the listed",
+                 7: "barrier 1", 8: "bin of the threshold, its entries listed", 9: "barrier 2", 10: "thresholds", 11: "random threshold",
+                 12: "listed entries grown", 13: "pruned entries", 14: "new mask", 15: "barrier 3", 16: "scan", 17: "CSR fill"}
         O, I = 4096, 1024                                # fc1 of GPT-2 medium
         nnz = mst_inputs.exact_nnz(O, I, 0.1)
         Wd = (torch.randn(O, I, device=dev, generator=gen) * 0.02).to(torch.bfloat16)
@@ -820,7 +815,7 @@ def main() -> None:
     roof = dict(rooflines[dom])
     paths = sorted({mst.path_name(s.L.path_in_use()) for s in slots})
     if dom_family == "update":
-        roof["kernel"] = "mg_update_fused_kernel"
+        roof["kernel"] = "mg_update_kernel"
     elif dom in ("sddmm_dw", "dense_grad"):
         roof["kernel"] = "tc_gemm_pair_kernel as " + dom
     else:

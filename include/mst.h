@@ -257,9 +257,7 @@ mst_status_t mst_topology_update(mst_layer_t* layer, double prune_frac, const ms
  * results, bit for bit, to calling mst_topology_update on each layer in turn.  prune_frac[i], rules[i], G_dense[i]
  * belong to layers[i]; stats is NULL or an array of n_layers entries (same meaning as above, the call then
  * synchronises once per layer).  A layer may appear once.  All arguments are validated before anything is launched.
- * With MST_UPDATE_BATCH=1 in the environment up to 8 tensor-path layers share one cooperative launch and its grid-wide
- * barriers; measured slower than one launch per layer on GPT-2 shapes (the shared launch cannot keep the layers'
- * keys on chip between passes), so it is off by default.
+ * Up to 8 layers share one cooperative launch: each has its own blocks, and the layers' phases run side by side.
  * Returns the first error met; layers before and after it are still completed. */
 mst_status_t mst_topology_update_many(int32_t n_layers, mst_layer_t* const* layers, const double* prune_frac,
                                       const mst_regrow_rule_t* rules, const float* const* G_dense,

@@ -89,12 +89,14 @@ extern "C" mst_status_t mst_layer_create(mst_layer_t** out, int32_t layer_id, in
   const size_t o_cnt = cv.take(4 * (size_t)(wmax + 1));
   const size_t o_scan = cv.take(4 * (size_t)(wmax + 1));
   const size_t o_bsum = cv.take(4 * (size_t)(mst_scan_block_sums_len(wmax) + 1024));
-  const size_t o_hist = cv.take(4 * (size_t)MST_SELECT_BINS * 2 * 3);
+  const size_t o_hist = cv.take(4 * (size_t)MST_SELECT_BINS * 5);
   int64_t rand_cap = N / 64;
-  if (rand_cap < 1024) rand_cap = 1024;
-  if (rand_cap > 32768) rand_cap = 32768;
+  if (rand_cap < 2048) rand_cap = 2048;
+  if (rand_cap > 65536) rand_cap = 65536;
   const size_t o_rlist = cv.take(16 * (size_t)rand_cap);
-  const size_t o_rctr = cv.take(16);
+  const size_t o_uctr = cv.take(4 * 64);
+  const size_t o_usmp = cv.take(4 * 2 * 4096);
+  const size_t o_ulst = cv.take(8 * 2 * 4096);
   const size_t o_sel = cv.take(sizeof(mst_select_state));
   const size_t o_flags = cv.take(4 * 4);
   const size_t o_counter = cv.take(4);
@@ -130,7 +132,9 @@ extern "C" mst_status_t mst_layer_create(mst_layer_t** out, int32_t layer_id, in
   L->block_sums = (int32_t*)(base + o_bsum);
   L->hist = (unsigned int*)(base + o_hist);
   L->rand_list = (unsigned long long*)(base + o_rlist);
-  L->rand_ctr = (unsigned long long*)(base + o_rctr);
+  L->upd_ctr = (unsigned int*)(base + o_uctr);
+  L->upd_samples = (uint32_t*)(base + o_usmp);
+  L->upd_list = (unsigned long long*)(base + o_ulst);
   L->rand_cap = (int)rand_cap;
   L->scratch_clean = 1;   // the allocation was cleared above
   L->longest_row_version = -1;

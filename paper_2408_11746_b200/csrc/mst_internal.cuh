@@ -125,11 +125,13 @@ struct mst_layer {
   int32_t* word_cnt;      // [max(nwords, nwordsT)+1]
   int32_t* word_scan;     // [max(nwords, nwordsT)+1]
   int32_t* block_sums;    // scan partials
-  unsigned int* hist;     // [3][2 * MST_SELECT_BINS]: rotating global histograms of the radix select (two selections side by side)
-  unsigned long long* rand_list;  // [rand_cap][2]: hash key and flat index of the random-growth candidates inside the bracket
-  unsigned long long* rand_ctr;   // [2]: candidates below the bracket, list length
+  unsigned int* hist;     // [5][MST_SELECT_BINS]: global histograms of the selections
+  unsigned long long* rand_list;  // [rand_cap][2]: hash key, gradient key and slot of the listed random-growth candidates
+  unsigned int* upd_ctr;          // [64]: barrier, exit and list counters of the update kernel
+  uint32_t* upd_samples;          // [2][4096]: sampled selection keys
+  unsigned long long* upd_list;   // [2][4096]: entries of the bin that holds a selection's threshold
   int rand_cap;
-  int scratch_clean;      // hist and rand_ctr are known to be zero (the fused update kernel leaves them so)
+  int scratch_clean;      // hist and upd_ctr are known to be zero (the update kernel leaves them so)
   mst_select_state* sel;  // [1]
   int32_t* flags;         // [4]: error bits, max row nnz of the last update, longest row (CUDA-core forward), spare
   mutable int64_t longest_row_version;  // structure version flags[2] belongs to
