@@ -284,7 +284,7 @@ mst_status_t mst_layer_step_host(mst_layer_t* layer, const void* X_host, const v
  *   row_ptr  device int32 [O+1]; row_ptr[O] receives the true number of active entries
  *   col_idx  device int32 [nnz_capacity];  vals device [nnz_capacity] in `dtype`
  * Entries at CSR positions >= nnz_capacity are not written (compare row_ptr[O] with the capacity afterwards).
- * Work space is a fixed array inside the library (about 3 MB of device memory on every GPU that loads the library,
+ * Work space is a fixed array inside the library (about 1 MB of device memory on every GPU that loads the library,
  * held until the process ends), which limits the layer to O*I <= 4 194 304 entries and O*ceil(I/32) <= 262 144 mask
  * words; larger layers return MST_ERR_CAPACITY.  The call itself allocates nothing and frees nothing.
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress); make that first call

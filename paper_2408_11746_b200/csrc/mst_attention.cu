@@ -580,7 +580,7 @@ extern "C" mst_status_t mst_strided_attention_fwd(const void* Q, const void* K, 
   if (tiles > 0x7FFFFFFF) return MST_ERR_SHAPE;
   P.tiles = (int)tiles;
   const size_t smem = (size_t)(1 + 4 * P.nkb) * TILE_BYTES + RED_BYTES + 1024 + 128;
-  MST_CUDA_TRY(cudaFuncSetAttribute(strided_attention_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MST_CUDA_TRY(cudaFuncSetAttribute(strided_attention_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // depends on the stride
   int dev = 0, sms = 0;
   MST_CUDA_TRY(cudaGetDevice(&dev));
   MST_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

@@ -429,8 +429,8 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
   static_assert(2 * TS * LDF * 4 <= 4 * TS * LDB * 2, "the staged gradients must fit the tile buffers");
   const size_t smem_q = (size_t)(6 * TS * LDB) * 2 + 128;
   const size_t smem_kv = (size_t)(6 * TS * LDB) * 2 + 128;
-  MST_CUDA_TRY(cudaFuncSetAttribute(attn_bwd_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_q));
-  MST_CUDA_TRY(cudaFuncSetAttribute(attn_bwd_dkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kv));
+  MST_SMEM_LIMIT((attn_bwd_dq_kernel), smem_q);
+  MST_SMEM_LIMIT((attn_bwd_dkv_kernel), smem_kv);
   dim3 grid((unsigned)(seq_len / TS), (unsigned)heads, (unsigned)batch);
   attn_bwd_dq_kernel<<<grid, BW_THREADS, smem_q, s>>>(P); MST_COUNT_LAUNCH();
   attn_bwd_dkv_kernel<<<grid, BW_THREADS, smem_kv, s>>>(P); MST_COUNT_LAUNCH();

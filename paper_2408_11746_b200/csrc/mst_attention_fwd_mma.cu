@@ -321,7 +321,7 @@ mst_status_t mst_attention_fwd_mma(const void* Q, const void* K, const void* V, 
   dim3 grid((unsigned)(seq_len / (64 * halves)), (unsigned)heads, (unsigned)batch);
 #define MST_ATTN_LAUNCH(NS_, H_)                                                                                              \
   do {                                                                                                                        \
-    MST_CUDA_TRY(cudaFuncSetAttribute(attn_fwd_mma_kernel<NS_, H_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  \
+    MST_SMEM_LIMIT((attn_fwd_mma_kernel<NS_, H_>), smem);  \
     attn_fwd_mma_kernel<NS_, H_><<<grid, 128 * H_ / NS_, smem, s>>>(P); MST_COUNT_LAUNCH();                                    \
   } while (0)
   if (halves == 2 && strips == 2) MST_ATTN_LAUNCH(2, 2);

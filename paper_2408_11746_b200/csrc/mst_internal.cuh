@@ -63,6 +63,27 @@ inline cudaError_t mst_launch_overlapped(void (*kernel)(KArgs...), dim3 grid, di
 }
 #endif
 
+// Raises a kernel's dynamic shared-memory limit once per device instead of at every launch (about 0.7 us of host time each).
+#define MST_SMEM_LIMIT(kernel, bytes)                                                                                 \
+  do {                                                                                                                \
+    static std::atomic<unsigned long long> done__{0};                                                                 \
+    int dev__ = 0;                                                                                                    \
+    MST_CUDA_TRY(cudaGetDevice(&dev__));                                                                              \
+    if (dev__ >= 64 || !((done__.load(std::memory_order_relaxed) >> dev__) & 1ULL)) {                                 \
+      MST_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes)));          \
+      if (dev__ < 64) done__.fetch_or(1ULL << dev__, std::memory_order_relaxed);                                      \
+    }                                                                                                                 \
+  } while (0)
+
+// Measurement switches are read at every call; one pass over the environment tells whether any is set.
+extern "C" char** environ;
+inline const char* mst_getenv(bool any, const char* name) { return any ? getenv(name) : nullptr; }
+inline bool mst_env_any() {
+  for (char** e = environ; e && *e; ++e)
+    if ((*e)[0] == 'M' && (*e)[1] == 'S' && (*e)[2] == 'T' && (*e)[3] == '_') return true;
+  return false;
+}
+
 #define MST_TRY(expr)                   \
   do {                                  \
     mst_status_t s__ = (expr);          \

@@ -445,7 +445,7 @@ mst_status_t launch_rpw(const CUtensorMap& tm, const int32_t* ptr, const uint16_
   const int PANEL = longest_row ? WARPS * RPW - 3 * RPW : WARPS * RPW;
   const size_t smem = spmm_smem<T>();
   // per call: the attribute belongs to the current device's copy of the kernel
-  MST_CUDA_TRY(cudaFuncSetAttribute(spmm_stream_kernel<T, PERM, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MST_SMEM_LIMIT((spmm_stream_kernel<T, PERM, RPW>), smem);
   dim3 grid((unsigned)((R_total + PANEL - 1) / PANEL), (unsigned)((T_total + TOK - 1) / TOK));
   spmm_stream_kernel<T, PERM, RPW><<<grid, THREADS, smem, s>>>(tm, ptr, idx, (const T*)vals, perm, (T*)out, ldout, T_total, R_total, C, longest_row); MST_COUNT_LAUNCH();
   MST_CUDA_TRY(cudaGetLastError());

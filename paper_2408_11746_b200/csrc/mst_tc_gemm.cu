@@ -849,10 +849,11 @@ bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb) 
 mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
   if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
+  const bool env = mst_env_any();
   CUtensorMap tmA, tmB;
   // Block pairs (256-row tiles) pay off once there are at least two row tiles; MST_TC_PAIR=0/1 overrides.
   bool pair = a.M > BM;
-  if (const char* e = getenv("MST_TC_PAIR")) pair = (e[0] == '1');
+  if (const char* e = mst_getenv(env, "MST_TC_PAIR")) pair = (e[0] == '1');
   // K-major: [rows x K], box 64 (K) x tile rows.  MN-major: [K x rows], box 64 (rows) x BK.
   const bool okA = a.a_mn_major ? make_map(&tmA, a.A, a.K, a.M, a.lda, BK) : make_map(&tmA, a.A, a.M, a.K, a.lda, BM);
   const int b_rows = pair ? BN / 2 : BN;
@@ -880,14 +881,14 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   P.ldpre = a.ldpre;
   if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
   P.sampled_stage_min = 384;  // measured: row-by-row stores pay from a density of about 0.4
-  if (const char* e = getenv("MST_TC_SAMPLED_STAGE")) P.sampled_stage_min = atoi(e);  // measurement override
+  if (const char* e = mst_getenv(env, "MST_TC_SAMPLED_STAGE")) P.sampled_stage_min = atoi(e);  // measurement override
   if (a.epilogue != MST_TC_OUT_BF16) {
     // few output tiles: cut the contraction range so that all SMs work; partial sums go to the shared scratch buffer
     const int64_t works1 = pair ? (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles : (int64_t)P.m_tiles * P.n_tiles;
     const int64_t slots = pair ? mst_sm_count() / 2 : mst_sm_count();
     const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
     P.splits = a.splits > 0 ? a.splits : mst_tc_pick_splits(works1, slots, P.kblocks, out_bytes);
-    if (const char* e = getenv("MST_TC_SPLITS")) {  // measurement override
+    if (const char* e = mst_getenv(env, "MST_TC_SPLITS")) {  // measurement override
       const int v = atoi(e);
       if (v > 0) P.splits = v;
     }
@@ -910,17 +911,17 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
                     ? 1
                     : 0;
   }
-  if (const char* e = getenv("MST_TC_TMA_OUT")) {
+  if (const char* e = mst_getenv(env, "MST_TC_TMA_OUT")) {
     if (e[0] == '0') P.tma_out = 0;
   }
   if (pair) {
-    MST_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P_SMEM_BYTES));
+    MST_SMEM_LIMIT((tc_gemm_pair_kernel), P_SMEM_BYTES);
     const int64_t works = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits;
     const int64_t max_pairs = mst_sm_count() / 2;
     const int grid = 2 * (int)(works < max_pairs ? works : max_pairs);
     MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel, dim3(grid), dim3(NUM_THREADS), P_SMEM_BYTES, s, tmA, tmB, tmC, P));
   } else {
-    MST_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    MST_SMEM_LIMIT((tc_gemm_kernel), SMEM_BYTES);
     const int64_t works = (int64_t)P.m_tiles * P.n_tiles * P.splits;
     const int grid = (int)(works < mst_sm_count() ? works : mst_sm_count());
     MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_kernel, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, s, tmA, tmB, tmC, P));

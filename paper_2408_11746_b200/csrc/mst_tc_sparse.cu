@@ -822,7 +822,7 @@ mst_status_t mst_sp24_product(mst_layer* L, int dir, const void* in, int64_t ldi
   P.spill = S.spill;
   P.xr = (const uint16_t*)xr;
   P.ldxr = ldxr;
-  MST_CUDA_TRY(cudaFuncSetAttribute(tc_sp24_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S_SMEM_BYTES));
+  MST_SMEM_LIMIT((tc_sp24_pair_kernel), S_SMEM_BYTES);
   const int64_t works = (int64_t)P.m_tiles * P.n_tiles;
   const int64_t max_pairs = sp_sm_count() / 2;
   const int grid = 2 * (int)(works < max_pairs ? works : max_pairs);

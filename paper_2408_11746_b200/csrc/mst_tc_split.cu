@@ -349,7 +349,7 @@ bool make_piece_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t col
 
 template <int BN>
 mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
-  MST_CUDA_TRY(cudaFuncSetAttribute(tc_split_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SplitCfg<BN>::SMEM));
+  MST_SMEM_LIMIT((tc_split_kernel<BN>), SplitCfg<BN>::SMEM);
   MST_CUDA_TRY(mst_launch_overlapped(tc_split_kernel<BN>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)), dim3(S_THREADS),
                                      SplitCfg<BN>::SMEM, s, tmA, tmB, P));
   return MST_OK;

@@ -900,6 +900,7 @@ __global__ void __launch_bounds__(UT, 1) mg_update_kernel(const __grid_constant_
   int barriers = 0, gpass = 0;
   bool alive = true, okR = false;
 
+  __syncthreads();   // the slice is in shared memory
   int cnt[2] = {0, 0};   // listed entries of this warp: prune, gradient
   if (tryA || tryB || tryR) {
     if (tryA || tryB) {
