@@ -581,6 +581,10 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
       MST_TRY(mst_pad_rows(in, ldin, T, cols, copy, s));
       a.A = copy;
     }
+    // A few tokens: the latency kernel (16 tokens: 3 us a layer of GPT-2-small width against 5 for the smallest tiles; at 32 its
+    // blocks read the activations too often and it loses).  Columns beyond the row must be zero in the activations too.
+    if (!transpose && T <= MST_SMALL_FWD_TOKENS && (cols % 8 == 0 || a.A != in))
+      return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, s);
     a.epilogue = MST_TC_OUT_BF16;
     a.splits = 1;
     a.act = act; a.pre = pre; a.ldpre = ldpre;

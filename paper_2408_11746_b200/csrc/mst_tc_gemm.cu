@@ -850,6 +850,16 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
   if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
   const bool env = mst_env_any();
+  // Few tiles: compare one wave of this kernel (about 6000 clocks of fill, last epilogue and launch, 512 per k-block of a pair's
+  // tile, and for the gradients a second launch that adds the ranges) with the small-tile kernel's estimate.
+  if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
+    const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
+    if (tiles <= pairs) {
+      double here = 6000.0 + (double)kb * 512.0;
+      if (a.epilogue != MST_TC_OUT_BF16 && kb > 8 && tiles * 2 <= pairs) here = here / (double)(pairs / tiles) + 8000.0;
+      if (mst_tc_small_clocks(a) < 0.9 * here) return mst_tc_small(a, s);
+    }
+  }
   CUtensorMap tmA, tmB;
   // Block pairs (256-row tiles) pay off once there are at least two row tiles; MST_TC_PAIR=0/1 overrides.
   bool pair = a.M > BM;

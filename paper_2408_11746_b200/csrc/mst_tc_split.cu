@@ -13,9 +13,13 @@
 // What bounds it: six bf16 MMAs per fp32 product, so 1654 / 6 = 276 TFLOP/s of the measured bf16 peak against 74 for the
 // fp32 FMA pipe; at the few hundred tokens of the fp32 workloads the launch, the pipeline fill and the drain of one tile
 // cost as much as the products.  Hence small tiles (128 x 64) when the output has few of them, and a split of the
-// contraction range whose last block adds the partial sums in a fixed order (no second launch).  3072 x 768, d = 0.25, 256
+// contraction range over the blocks of a cluster, which add their sums through distributed shared memory in a fixed order
+// (partial sums through global memory with the last block adding them cost 4 us more).  3072 x 768, d = 0.25, 256
 // tokens: forward, input gradient and dense gradient with their operand preparation took 65 + 118 + 51 us on the CUDA
 // cores (69 / 123 / 51 with their transposes), about 20 us each here.
+//
+// The same kernel with one piece serves bf16 contractions whose output has too few 256 x 256 tiles to occupy the GPU
+// (mst_tc_small): small tiles and a split of the contraction range inside one launch.
 //
 // One block per tile and range, 320 threads: one lane of warp 0 fetches [3 pieces x rows x 64] boxes with TMA, one lane of
 // warp 1 issues the MMAs, warps 2-9 own the sums (one row and BN / 2 columns per thread).  Every wait is bounded.
@@ -33,36 +37,38 @@ using namespace mst_ptx;
 __device__ int g_split_error = 0;  // sticky: a bounded wait expired
 
 constexpr int SBM = 128, SBK = 64;
-constexpr int PIECES = 3;
 constexpr int S_EPI_WARPS = 8;
 constexpr int S_THREADS = 64 + 32 * S_EPI_WARPS;
-constexpr int CHUNK_KB = 1;                 // k-blocks summed inside the tensor core before the sums move to registers
-constexpr int MAX_SPLIT_TILES = 1024;
 constexpr int BOX64 = 64 * SBK * 2;         // one piece of one 64-wide MN-major box
 
-__device__ unsigned int g_split_arrivals[MAX_SPLIT_TILES];  // blocks of a tile that have stored their partial sums; wraps to 0
-
-template <int BN>
+template <int BN, int PIECES>
 struct SplitCfg {
+  static constexpr int CHUNK_KB = PIECES == 3 ? 1 : 1 << 20;   // k-blocks summed inside the tensor core before the sums move to registers
   static constexpr int A_BYTES = PIECES * SBM * SBK * 2;
   static constexpr int B_BYTES = PIECES * BN * SBK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = BN == 64 ? 3 : 2;
-  static constexpr int TMEM = 4 * BN;       // two chunk buffers x (leading, small)
-  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 128;
+  // one piece: at most half of an SM's shared memory, so that the next launch's blocks can be set up while this one drains
+  static constexpr int STAGES = PIECES == 1 ? 4 : BN == 64 ? 3 : 2;
+  static constexpr int TMEM = PIECES == 3 ? 4 * BN : BN;       // three pieces: two chunk buffers x (leading, small)
+  // after the last MMA the stages hold the warps' turning squares and the block's sums
+  static constexpr int STAGING = S_EPI_WARPS * 32 * 33 * 4 + SBM * BN * 4;
+  static constexpr int TILES = STAGES * STAGE_BYTES > STAGING ? STAGES * STAGE_BYTES : STAGING;
+  static constexpr size_t SMEM = (size_t)TILES + 1024 /*align*/ + 128 /*barriers*/;
 };
 
 struct SplitParams {
   int64_t M, N;
   int kblocks, splits, m_tiles, n_tiles;
   int a_mn, b_mn;
-  int sampled;
-  float* out;
+  int epilogue;
+  void* out;
+  int act;
+  uint16_t* pre;
+  int64_t ldpre;
   int64_t ldc;
   const uint32_t* bits;
   const int32_t* wscan;
   int wpr;
-  float* partial;   // [splits][tiles][8 warps][BN / 8 vectors][32 lanes] float4
 };
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
@@ -72,18 +78,25 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm,
       : "memory");
 }
 
-template <int BN>
-__global__ void __launch_bounds__(S_THREADS, 1)
+// all warps of all blocks of the cluster, converged
+__device__ __forceinline__ void split_cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int BN, int PIECES>
+__global__ void __launch_bounds__(S_THREADS, PIECES == 1 ? 2 : 1)
 tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
-  typedef SplitCfg<BN> C;
+  typedef SplitCfg<BN, PIECES> C;
+  constexpr int CHUNK_KB = C::CHUNK_KB;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
-  const uint32_t bar_base = tiles_base + C::STAGES * C::STAGE_BYTES;
+  const uint32_t bar_base = tiles_base + C::TILES;
   const uint32_t full0 = bar_base, empty0 = full0 + 8 * C::STAGES, tfull0 = empty0 + 8 * C::STAGES, tempty0 = tfull0 + 16;
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_sh;
-  __shared__ unsigned int arrived_sh;
   volatile int* abort_flag = &abort_sh;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -99,6 +112,10 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 0 && lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)), "r"(C::TMEM)
                  : "memory");
@@ -111,8 +128,7 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
 
-  const int tiles = P.m_tiles * P.n_tiles;
-  const int split = blockIdx.x / tiles, tile = blockIdx.x % tiles;
+  const int split = P.splits > 1 ? (int)(blockIdx.x % (unsigned)P.splits) : 0, tile = (int)(blockIdx.x / (unsigned)P.splits);   // rank in the cluster
   const int m0 = (tile / P.n_tiles) * SBM, n0 = (tile % P.n_tiles) * BN;
   const int kb0 = (int)((int64_t)split * P.kblocks / P.splits), kb1 = (int)((int64_t)(split + 1) * P.kblocks / P.splits);
   const int chunks = (kb1 - kb0 + CHUNK_KB - 1) / CHUNK_KB;
@@ -164,6 +180,10 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           for (int k = 0; k < SBK / 16; ++k) {
             const uint32_t more = (kb > first || k > 0) ? 1u : 0u;
             const uint64_t a0 = ad + (uint64_t)(k * a_k), b0 = bd + (uint64_t)(k * b_k);
+            if (PIECES == 1) {
+              tc_mma(d_hi, a0, b0, idesc, more);
+              continue;
+            }
             const uint64_t a1 = a0 + a_piece, a2 = a1 + a_piece, b1 = b0 + b_piece, b2 = b1 + b_piece;
             tc_mma(d_lo, a2, b0, idesc, more);
             tc_mma(d_lo, a0, b2, idesc, 1u);
@@ -193,57 +213,62 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       for (int g = 0; g < COLS / 32; ++g) {
         uint32_t hi[32], lo[32];
         tmem_ld32_nowait(at + g * 32, hi);
-        tmem_ld32_nowait(at + BN + g * 32, lo);
+        if (PIECES == 3) tmem_ld32_nowait(at + BN + g * 32, lo);
         tmem_ld_wait(hi);
-        tmem_ld_wait(lo);
+        if (PIECES == 3) tmem_ld_wait(lo);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[g * 32 + j] += __uint_as_float(hi[j]) + __uint_as_float(lo[j]);
+        for (int j = 0; j < 32; ++j) acc[g * 32 + j] += PIECES == 3 ? __uint_as_float(hi[j]) + __uint_as_float(lo[j]) : __uint_as_float(hi[j]);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
     }
-    bool mine = true;
+    // Every MMA of the block has completed, so the operand stages serve as staging.
+    float* box = reinterpret_cast<float*>(smem_raw + (tiles_base - raw)) + (warp - 2) * (32 * 33);
+    const uint32_t part = tiles_base + S_EPI_WARPS * 32 * 33 * 4 + (uint32_t)((warp - 2) * (COLS / 4) * 32 + lane) * 16u;
+    int rr0 = 0, rr1 = 32;   // rows of the warp's 32 this block stores
     if (P.splits > 1) {
-      // partial sums to the scratch buffer; the last block of the tile to arrive adds all of them in range order
-      const size_t slab = (size_t)tiles * S_EPI_WARPS * (COLS / 4) * 32;
-      float4* part = reinterpret_cast<float4*>(P.partial) + ((size_t)tile * S_EPI_WARPS + (warp - 2)) * (COLS / 4) * 32 + lane;
+      // The blocks of a cluster hold the sums of one tile over different parts of the contraction range: each leaves its sums in
+      // its shared memory, then adds up and stores 32 / splits of every 32 rows, in range order.
 #pragma unroll
       for (int v = 0; v < COLS / 4; ++v)
-        __stcg(part + (size_t)split * slab + v * 32, make_float4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]));
-      __threadfence();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * S_EPI_WARPS) : "memory");
-      if (threadIdx.x == 64) arrived_sh = atomicInc(&g_split_arrivals[tile], (unsigned)P.splits - 1u);
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * S_EPI_WARPS) : "memory");
-      mine = arrived_sh == (unsigned)P.splits - 1u;
-      if (mine) {
-        __threadfence();
-#pragma unroll
-        for (int j = 0; j < COLS; ++j) acc[j] = 0.f;
-        for (int sp = 0; sp < P.splits; ++sp) {
-#pragma unroll
-          for (int v = 0; v < COLS / 4; ++v) {
-            const float4 t = __ldcg(part + (size_t)sp * slab + v * 32);
-            acc[4 * v] += t.x; acc[4 * v + 1] += t.y; acc[4 * v + 2] += t.z; acc[4 * v + 3] += t.w;
-          }
-        }
-      }
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(part + v * 512u), "f"(acc[4 * v]), "f"(acc[4 * v + 1]), "f"(acc[4 * v + 2]),
+                     "f"(acc[4 * v + 3])
+                     : "memory");
+      split_cluster_sync();
+      rr0 = split * (32 / P.splits);
+      rr1 = rr0 + 32 / P.splits;
     }
-    if (mine && !*abort_flag) {
-      // every MMA of the block has completed, so the operand stages serve as staging: a 32 x 32 square per warp, turned
-      // from rows to columns so that a store instruction writes neighbours
-      float* box = reinterpret_cast<float*>(smem_raw + (tiles_base - raw)) + (warp - 2) * (32 * 33);
+    if (!*abort_flag) {
+      // a 32 x 32 square per warp, turned from rows to columns so that a store instruction writes neighbours
       const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
       for (int g = 0; g < COLS / 32; ++g) {
         const int n = n0 + half * COLS + g * 32;
         if (n >= P.N) break;   // uniform
         __syncwarp();
+        if (P.splits > 1) {
+          for (int i = lane; i < 8 * (rr1 - rr0); i += 32) {   // four columns of one row
+            const int v = i & 7, row = rr0 + (i >> 3);
+            const uint32_t at = part - (uint32_t)lane * 16u + (uint32_t)((g * 8 + v) * 32 + row) * 16u;
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int sp = 0; sp < P.splits; ++sp) {
+              uint32_t peer;
+              float4 x;
+              asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(sp));
+              asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(peer) : "memory");
+              sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+            }
+            float* d = box + row * 33 + 4 * v;
+            d[0] = sum.x; d[1] = sum.y; d[2] = sum.z; d[3] = sum.w;
+          }
+        } else {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) box[lane * 33 + j] = acc[g * 32 + j];
+          for (int j = 0; j < 32; ++j) box[lane * 33 + j] = acc[g * 32 + j];
+        }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
-        if (P.sampled) {
+        if (P.epilogue == MST_TC_OUT_SAMPLED) {
           uint32_t word = 0;
           int32_t at = 0;
           if (row0 + lane < P.M) {
@@ -252,23 +277,45 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             at = P.wscan[wi];
           }
 #pragma unroll 4
-          for (int rr = 0; rr < 32; ++rr) {
+          for (int rr = rr0; rr < rr1; ++rr) {
             const uint32_t w = __shfl_sync(0xffffffffu, word, rr);
             const int32_t base = __shfl_sync(0xffffffffu, at, rr);
-            if ((w >> lane) & 1u) P.out[base + __popc(w & lt)] = box[rr * 33 + lane];
+            if ((w >> lane) & 1u) reinterpret_cast<float*>(P.out)[base + __popc(w & lt)] = box[rr * 33 + lane];
+          }
+        } else if (PIECES == 1 && P.epilogue == MST_TC_OUT_BF16) {
+          const bool col_ok = n + lane < P.N;
+          uint16_t* out = reinterpret_cast<uint16_t*>(P.out);
+#pragma unroll 4
+          for (int rr = rr0; rr < rr1; ++rr) {
+            if (row0 + rr >= P.M) break;  // uniform
+            if (!col_ok) continue;
+            float v = box[rr * 33 + lane];
+            uint16_t* pre = P.pre + (row0 + rr) * P.ldpre + n + lane;
+            if (P.act == MST_ACT_GELU) {
+              if (P.pre) *pre = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
+              v = mst_gelu(v);
+            } else if (P.act == MST_ACT_GELU_GRAD) {
+              v *= mst_gelu_grad(__uint_as_float((uint32_t)*pre << 16));
+            }
+            out[(row0 + rr) * P.ldc + n + lane] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
           }
         } else {
           const bool col_ok = n + lane < P.N;
+          float* out = reinterpret_cast<float*>(P.out);
 #pragma unroll 4
-          for (int rr = 0; rr < 32; ++rr) {
+          for (int rr = rr0; rr < rr1; ++rr) {
             if (row0 + rr >= P.M) break;  // uniform
-            if (col_ok) P.out[(row0 + rr) * P.ldc + n + lane] = box[rr * 33 + lane];
+            if (col_ok) out[(row0 + rr) * P.ldc + n + lane] = box[rr * 33 + lane];
           }
         }
       }
     }
   }
 
+  if (P.splits > 1) {
+    if (warp < 2) split_cluster_sync();   // the barrier above, for the warps without sums
+    split_cluster_sync();                 // no block leaves while another still reads its sums
+  }
   if (*abort_flag) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // copies and MMAs in flight land before memory is given back
   }
@@ -302,6 +349,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict
 #pragma unroll
     for (int j = 0; j < 8; ++j) x[j] = c + j < C ? src[j] : 0.f;
   }
+  constexpr int PIECES = 3;
   uint32_t p[PIECES][4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -335,24 +383,76 @@ __global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restric
   *reinterpret_cast<uint4*>(out + (size_t)r * ldp + c) = make_uint4(v[0], v[1], v[2], v[3]);
 }
 
-// pieces [3][rows][ld] as a 3-d map: rows and columns beyond the matrix read as zero inside every piece
-bool make_piece_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+// pieces [1 or 3][rows][ld] as a 3-d map: rows and columns beyond the matrix read as zero inside every piece
+bool make_piece_map(CUtensorMap* tm, const void* base, int pieces, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
   mst_encode_tiled_fn fn = mst_encode_tiled();
   if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, PIECES};
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)pieces};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)(ld * rows) * 2};
-  cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, PIECES};
+  cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, (cuuint32_t)pieces};
   cuuint32_t estr[3] = {1u, 1u, 1u};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
+template <int BN, int PIECES>
 mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
-  MST_SMEM_LIMIT((tc_split_kernel<BN>), SplitCfg<BN>::SMEM);
-  MST_CUDA_TRY(mst_launch_overlapped(tc_split_kernel<BN>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)), dim3(S_THREADS),
-                                     SplitCfg<BN>::SMEM, s, tmA, tmB, P));
+  typedef SplitCfg<BN, PIECES> C;
+  MST_SMEM_LIMIT((tc_split_kernel<BN, PIECES>), C::SMEM);
+  MST_CUDA_TRY(mst_launch_overlapped_cluster(tc_split_kernel<BN, PIECES>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)), dim3(S_THREADS),
+                                             P.splits, C::SMEM, s, tmA, tmB, P));
   return MST_OK;
+}
+
+// Tile width and number of K ranges from a time model in SM clocks.  Three pieces: 24 MMAs per k-block (64 clocks each at 128
+// columns, 40 at 64, where the A operand's shared-memory reads dominate).  One piece: its 24 KB of operands per k-block at the 54
+// bytes per clock that an SM gets from L2 (128 columns were no faster).  Both: about 4000 for launch, fill and drain of a block, and 1500 for the sums of a
+// cluster.
+double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
+  const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
+  const int64_t m_tiles = (a.M + SBM - 1) / SBM;
+  double best = 1e30;
+  *bn = 128;
+  *splits = 1;
+  for (int w = 64; w <= (pieces == 3 ? 128 : 64); w += 64) {
+    const int64_t tiles = m_tiles * ((a.N + w - 1) / w);
+    const double t_kb = pieces == 1 ? 450.0 : w == 64 ? 960.0 : 1536.0;
+    for (int sp = 1; sp <= 8 && sp <= kblocks; sp *= 2) {   // cluster sizes
+      const int64_t waves = (tiles * sp + sms - 1) / sms;
+      const int kb = (kblocks + sp - 1) / sp;
+      const double t = (double)waves * (kb * t_kb + 4000.0) + (sp > 1 ? 1500.0 : 0.0);
+      if (t < best * 0.97) { best = t; *bn = w; *splits = sp; }
+    }
+  }
+  return best;
+}
+
+mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits, cudaStream_t s) {
+  SplitParams P = {};
+  P.M = a.M;
+  P.N = a.N;
+  P.kblocks = (int)((a.K + SBK - 1) / SBK);
+  P.m_tiles = (int)((a.M + SBM - 1) / SBM);
+  P.n_tiles = (int)((a.N + bn - 1) / bn);
+  P.splits = splits;
+  P.a_mn = a.a_mn_major;
+  P.b_mn = a.b_mn_major;
+  P.epilogue = a.epilogue;
+  P.out = a.out;
+  P.ldc = a.ldc;
+  P.act = a.epilogue == MST_TC_OUT_BF16 ? a.act : 0;
+  P.pre = (uint16_t*)a.pre;
+  P.ldpre = a.ldpre;
+  P.bits = a.bits;
+  P.wscan = a.wscan;
+  P.wpr = a.wpr;
+  if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
+  CUtensorMap tmA, tmB;
+  const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, pieces, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, pieces, a.M, a.K, a.lda, SBM);
+  const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, pieces, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, pieces, a.N, a.K, a.ldb, bn);
+  if (!okA || !okB) return MST_ERR_SHAPE;
+  if (pieces == 3) return bn == 64 ? launch_split<64, 3>(tmA, tmB, P, s) : launch_split<128, 3>(tmA, tmB, P, s);
+  return launch_split<64, 1>(tmA, tmB, P, s);
 }
 
 }  // namespace
@@ -375,46 +475,20 @@ mst_status_t mst_pad_rows(const void* in, int64_t ld, int64_t R, int C, void* ou
 }
 
 mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s) {
-  SplitParams P = {};
-  P.M = a.M;
-  P.N = a.N;
-  P.kblocks = (int)((a.K + SBK - 1) / SBK);
-  P.m_tiles = (int)((a.M + SBM - 1) / SBM);
-  P.a_mn = a.a_mn_major;
-  P.b_mn = a.b_mn_major;
-  P.sampled = a.epilogue == MST_TC_OUT_SAMPLED;
-  P.out = (float*)a.out;
-  P.ldc = a.ldc;
-  P.bits = a.bits;
-  P.wscan = a.wscan;
-  P.wpr = a.wpr;
-  // Tile width and number of K ranges from a time model in SM clocks: 24 MMAs per k-block (64 clocks each at 128 columns, 40
-  // at 64, where the A operand's shared-memory reads dominate), about 4000 for launch, fill and drain of a block, and the
-  // last block's read of the partial sums.
-  const int sms = mst_sm_count();
-  int bn = 128, splits = 1;
-  double best = 1e30;
-  for (int w = 64; w <= 128; w += 64) {
-    const int64_t tiles = (int64_t)P.m_tiles * ((a.N + w - 1) / w);
-    for (int sp = 1; sp <= 8 && sp <= P.kblocks && (sp == 1 || tiles <= MAX_SPLIT_TILES); ++sp) {
-      const int64_t waves = (tiles * sp + sms - 1) / sms;
-      const int kb = (P.kblocks + sp - 1) / sp;
-      const double t = (double)waves * (kb * (w == 64 ? 960.0 : 1536.0) + 4000.0) + (sp > 1 ? 2000.0 + sp * 5.0 * w : 0.0);
-      if (t < best * 0.97) { best = t; bn = w; splits = sp; }
-    }
-  }
-  P.splits = splits;
-  P.n_tiles = (int)((a.N + bn - 1) / bn);
-  CUtensorMap tmA, tmB;
-  const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, a.M, a.K, a.lda, SBM);
-  const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, a.N, a.K, a.ldb, bn);
-  if (!okA || !okB) return MST_ERR_SHAPE;
-  if (splits > 1) {
-    void* ws = nullptr;
-    MST_TRY(mst_workspace(sizeof(float) * (size_t)splits * P.m_tiles * P.n_tiles * SBM * bn, &ws));
-    P.partial = (float*)ws;
-  }
-  return bn == 64 ? launch_split<64>(tmA, tmB, P, s) : launch_split<128>(tmA, tmB, P, s);
+  int bn, splits;
+  plan_split(a, 3, &bn, &splits);
+  return run_split(a, 3, bn, splits, s);
+}
+
+double mst_tc_small_clocks(const mst_tc_gemm_args& a) {
+  int bn, splits;
+  return plan_split(a, 1, &bn, &splits);
+}
+
+mst_status_t mst_tc_small(const mst_tc_gemm_args& a, cudaStream_t s) {
+  int bn, splits;
+  plan_split(a, 1, &bn, &splits);
+  return run_split(a, 1, bn, splits, s);
 }
 
 mst_status_t mst_split_error_flags(int32_t* flags) {

@@ -1,4 +1,4 @@
-"""fp32 layers on the tensor cores (three exact bf16 pieces per operand) and bf16 layers whose rows start anywhere:
+"""fp32 layers on the tensor cores (three exact bf16 pieces per operand) and bf16 layers whose rows start anywhere or whose outputs have few tiles:
 edges of the 128 x 64 / 128 x 128 tiles and of the 64-wide contraction blocks, against an fp64 product."""
 import numpy as np
 import pytest
@@ -68,4 +68,11 @@ def test_fp32_extreme_magnitudes():
 @pytest.mark.parametrize("O,I,T,pad", [(65, 63, 129, 0), (255, 257, 300, 0), (64, 128, 130, 3), (513, 31, 520, 5), (1, 3, 1, 0)])
 def test_bf16_rows_at_any_address(O, I, T, pad):
     y, dx, dw, g = _layer_case(O, I, T, "bf16", 0.3, O + I + T, pad)
+    assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
+
+
+@pytest.mark.parametrize("O,I,T", [(2304, 768, 8), (2304, 768, 9), (770, 3080, 16), (768, 3072, 17), (136, 200, 128), (1280, 1288, 40), (16, 8, 3)])
+def test_bf16_products_of_few_tiles(O, I, T):
+    # the latency kernel up to 16 tokens, small tiles with the contraction range split over a cluster above
+    y, dx, dw, g = _layer_case(O, I, T, "bf16", 0.2, O + I + T)
     assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
