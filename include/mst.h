@@ -196,7 +196,7 @@ mst_status_t mst_strided_attention_fwd(const void* Q, const void* K, const void*
  * dQ, dK, dV: device bf16, ldg elements between tokens, head h in columns h*head_dim .. (three column slices of one
  * fused gradient buffer may be passed).  Supported: head_dim = 64, seq_len and stride multiples of 64, leading
  * dimensions multiples of 8, 16-byte aligned pointers; anything else MST_ERR_SHAPE.  Deterministic (no atomics).
- * Keeps one float per (token, head) in a per-device scratch buffer: calls must not overlap on the GPU. */
+ * Keeps two floats per (token, head) in a per-device scratch buffer: calls must not overlap on the GPU. */
 mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, const void* V, int64_t ld, const void* Out,
                                        int64_t ldo, const void* dOut, int64_t lddo, const float* lse, int32_t batch,
                                        int32_t seq_len, int32_t heads, int32_t head_dim, int32_t stride, void* dQ,

@@ -529,7 +529,9 @@ bool att_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int6
 mst_status_t mst_attention_error_flags(int32_t* flags) {
   int v = 0;
   MST_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_attn_error, sizeof(int)));
-  *flags = v;
+  int32_t bwd = 0;
+  MST_TRY(mst_attention_bwd_error_flags(&bwd));
+  *flags = v | bwd;
   return MST_OK;
 }
 

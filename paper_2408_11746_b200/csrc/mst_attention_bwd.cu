@@ -6,395 +6,614 @@
 //   P_ij    = exp(q_i . k_j / sqrt(d) - lse_i)   dP_ij = dOut_i . v_j      dS_ij = P_ij (dP_ij - delta_i)
 //   dV_j = sum_i P_ij dOut_i      dK_j = sum_i dS_ij q_i / sqrt(d)      dQ_i = sum_j dS_ij k_j / sqrt(d)
 //
-// Three launches, no atomics (every output element has one owner and a fixed summation order):
-//   1. delta: eight lanes per (token, head) row, 16-byte loads.
-//   2. dQ, query-centric: a block owns 64 queries of one (sequence, head) and walks the key tiles of their window
-//      (stride / 64 + 1 tiles of 64 keys; the tile that starts `stride` positions back also holds the first strided
-//      key of every query).  Per tile: S = Q K^T and dP = dOut V^T on the tensor cores (warp-level mma.sync
-//      m16n8k16, bf16 operands fetched with ldmatrix, fp32 accumulators), the softmax algebra on the accumulator
-//      registers, then dQ += dS K with dS rounded to bf16 and used as the next A operand straight from the registers
-//      (the accumulator layout of two neighbouring 16 x 8 tiles is the A layout).  The strided keys further back (i - 2l, i - 3l, ...) are
-//      visited as further tiles of which only the diagonal is kept.
-//   3. dK and dV, key-centric: a block owns 64 keys and walks the query tiles that can see them, with the
-//      transposed products (S^T = K Q^T, dP^T = V dOut^T), dV += P^T dOut and dK += dS^T Q; far queries
-//      (j + 2l, j + 3l, ...) as further tiles, diagonal only.
-// Every warp owns a 16-row strip of each tile, so the element-wise steps need no block-wide barrier; the barriers
-// are around the cooperative tile loads only.  Scores, sums and deltas are fp32; P and dS are rounded to bf16 where
-// they enter a tensor-core product (as the forward kernel does with P).
+// Two launches, no atomics (every output element has one owner and a fixed summation order):
+//   1. dQ, query-centric: a block owns 128 queries of one (sequence, head) and walks 64-key tiles.  It forms delta first and
+//      leaves (-lse log2 e, delta) of its rows in the scratch buffer for the second launch.
+//   2. dK and dV, key-centric: a block owns 128 keys and walks the 64-query tiles that see them, on the transposed scores.
+// Roles of a block's eighteen warps:
+//   warps 0-15 algebra: thread = own row (tensor-memory lane), the four warps of a lane quarter share the tile's 64 columns.
+//              Scores and dP come from tensor memory, dS (and P) go back as bf16 and are the A operand of the second products
+//              where they lie, so nothing score-shaped passes through shared memory;
+//   warp 16    one lane feeds a four-tile ring by TMA;
+//   warp 17    one lane issues tcgen05.mma: S = Q K^T, dP = dOut V^T (128 x 64), then dQ += dS K, or dV += P^T dOut, dK += dS^T Q.
+// 256 columns of tensor memory and 102 KiB of shared memory: two blocks per SM, so that one block's products run while
+// the other's algebra does.  The far strided positions (i - 2l, i - 3l, ...: one key per query and distance) are visited
+// after the window as tiles of which only the diagonal counts: warp-level mma.sync products of 16 rows each, whose sums are
+// added to the accumulators when the rows leave.
+// Measured at 16 x 1024 tokens, 12 heads: l = 256 148 us, l = 128 (8 x 1024, 16 heads) 112 us; the two mma.sync kernels and the delta
+// kernel before took 219 and 117 us.  Leaving out the far tiles gives 124 and 75 us, the window's tiles beyond the first as well 67
+// and 47 us (300 and 200 MB of compulsory traffic in two passes: 46 and 31 us); the exponentials cost 2 us.
+#include <cuda.h>
 #include <cuda_bf16.h>
 
-#include "mst_attention_mma.cuh"
+#include "mst_attention_tile.cuh"
 #include "mst_internal.cuh"
-#include "mst_tc_gemm.cuh"
 
 namespace {
-using namespace mst_attn;
+using namespace mst_att;
+
+constexpr int CW = 8;                              // algebra warps (16 x 1024 tokens, 12 heads, l = 256, the call: 4 - 165 us, 8 - 148, 16 - 171)
+constexpr int PARTS = CW / 4;                      // warps of a lane quarter: they share a tile's 64 columns
+constexpr int COLS = TS / PARTS;                   // columns of one warp ...
+constexpr int PIECES = COLS / 16;                  // ... in pieces of sixteen
+constexpr int STRIPS = ROWS / 16 / CW;             // 16-row strips of a warp in the far tiles' products
+constexpr int THREADS = 32 * (CW + 2);
+constexpr int STAGES = 4;
+constexpr int STAT_BYTES = TS * 8;                 // -lse log2 e of a tile's queries, then their -delta
+constexpr int RING_BYTES = STAGES * 2 * TILE_BYTES;
+constexpr int TMEM_COLS = 256;
+
+__device__ int g_bwd_error = 0;
 
 struct BwdParams {
   const __nv_bfloat16 *Q, *K, *V, *Out, *dOut;
-  int64_t ld, ldo, lddo;
+  int64_t ldo;
   const float* lse;    // [batch, heads, seq]
-  float* delta;        // [batch, heads, seq]
+  float* stat;         // [batch, heads, seq / 64][2][64]: -lse log2 e, -delta
   __nv_bfloat16 *dQ, *dK, *dV;
   int64_t ldg;
-  int batch, seq, heads, stride;
+  int batch, seq, heads, stride, tiles;   // tiles of 128 rows per sequence
+  uint32_t magic;
 };
 
-// delta[b, h, i] = dOut_i . Out_i per head: eight lanes per (token, head) row of 64 elements, 16 bytes per lane and
-// tensor, four rows per warp and trip
-__global__ void __launch_bounds__(256) attn_delta_kernel(BwdParams P) {
-  const int lane = threadIdx.x & 31, grp = lane >> 3, piece = lane & 7;
-  const int64_t rows = (int64_t)P.batch * P.seq * P.heads;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t w0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; w0 < rows; w0 += warps * 4) {
-    const int64_t w = w0 + grp;          // (token, head)
-    float s = 0.f;
-    int64_t t = 0;
-    int h = 0;
-    if (w < rows) {
-      t = w / P.heads;
-      h = (int)(w - t * P.heads);
-      const uint4 o = *reinterpret_cast<const uint4*>(P.Out + t * P.ldo + h * D + piece * 8);
-      const uint4 g = *reinterpret_cast<const uint4*>(P.dOut + t * P.lddo + h * D + piece * 8);
-      const uint32_t ow[4] = {o.x, o.y, o.z, o.w}, gw[4] = {g.x, g.y, g.z, g.w};
+// shared memory of a block, 1024-byte aligned: the own rows of two operands, the ring, the ring's statistics, barriers
+struct Smem {
+  uint32_t own0, own1, ring, stat, full, empty, own_full, s_full, s_free, w_full, w_free, acc_full, dp_full, p_full, far_done;
+  unsigned char* base;
+  __device__ __forceinline__ explicit Smem(unsigned char* raw) {
+    const uint32_t a = (smem_u32(raw) + 1023u) & ~1023u;
+    base = raw + (a - smem_u32(raw));
+    own0 = a;
+    own1 = own0 + 2 * TILE_BYTES;
+    ring = own1 + 2 * TILE_BYTES;
+    stat = ring + RING_BYTES;
+    full = stat + STAGES * STAT_BYTES + PARTS * ROWS * 4 + ROWS * 8;
+    empty = full + 8 * STAGES;
+    own_full = empty + 8 * STAGES;
+    s_full = own_full + 8;
+    s_free = s_full + 8;
+    w_full = s_free + 8;
+    w_free = w_full + 8;
+    acc_full = w_free + 8;
+    dp_full = acc_full + 8;
+    p_full = dp_full + 8;
+    far_done = p_full + 8;
+  }
+  template <typename T>
+  __device__ __forceinline__ T* at(uint32_t addr) const {
+    return reinterpret_cast<T*>(base + (addr - own0));
+  }
+};
+constexpr size_t SMEM_BYTES = 4 * TILE_BYTES + RING_BYTES + STAGES * STAT_BYTES + PARTS * ROWS * 4 + ROWS * 8 + 24 * STAGES + 80 + 1024;
+static_assert(ROWS * LDF * 4 <= RING_BYTES, "staged sums must fit the ring");
+static_assert(ROWS * LDO * 2 <= 4 * TILE_BYTES, "staged results must fit the own tiles");
+
+__device__ __forceinline__ bool wait_on(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return mbar_wait_suspended(bar, parity, abort_flag, &g_bwd_error);
+}
+
+__device__ __forceinline__ uint32_t block_setup(const Smem& S, uint32_t* holder, int* abort_sh, int warp) {
+  if (threadIdx.x == 0) {
+    *abort_sh = 0;
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(S.full + 8 * s, 1);
+      mbar_init(S.empty + 8 * s, 1);
+      mbar_init(S.far_done + 8 * s, CW / 2);
+    }
+    mbar_init(S.own_full, 1);
+    mbar_init(S.s_full, 1);
+    mbar_init(S.dp_full, 1);
+    mbar_init(S.s_free, CW);
+    mbar_init(S.w_full, CW);
+    mbar_init(S.p_full, CW);
+    mbar_init(S.w_free, 1);
+    mbar_init(S.acc_full, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == CW + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(holder)), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  return *holder;
+}
+__device__ __forceinline__ void block_teardown(uint32_t tmem, int warp, volatile int* abort_flag) {
+  if (*abort_flag) {
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);   // let copies and products in flight land
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == CW + 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+// The lane that feeds the ring: the block's own rows of two operands, then tile after tile of two others (and, for the
+// keys' pass, the statistics of the tile's queries).
+template <typename W>
+__device__ __forceinline__ void feed(const Smem& S, const W& walk, const CUtensorMap* own_a, const CUtensorMap* own_b,
+                                     const CUtensorMap* tile_a, const CUtensorMap* tile_b, int col, int row0, const float* stat,
+                                     volatile int* abort_flag) {
+  mbar_expect_tx(S.own_full, 4 * TILE_BYTES);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        s = fmaf(__uint_as_float(ow[j] << 16), __uint_as_float(gw[j] << 16), s);
-        s = fmaf(__uint_as_float(ow[j] & 0xFFFF0000u), __uint_as_float(gw[j] & 0xFFFF0000u), s);
-      }
+  for (int t = 0; t < 2; ++t) {
+    tma_load_2d(S.own0 + t * TILE_BYTES, own_a, col, row0 + walk.r0 + t * TS, S.own_full);
+    tma_load_2d(S.own1 + t * TILE_BYTES, own_b, col, row0 + walk.r0 + t * TS, S.own_full);
+  }
+  int s = 0;
+  uint32_t lap = 0;
+  for (int j = 0; j < walk.total; ++j) {
+    // what the stage held one lap ago: a near tile is given back by the second products' commit, a far one by its four warps
+    const int before = j - STAGES;
+    if (before >= 0) {
+      const bool far = before >= walk.near;
+      const uint32_t use = far ? (uint32_t)((before - walk.near) / STAGES) : lap - 1;
+      if (!wait_on((far ? S.far_done : S.empty) + 8 * s, use & 1u, abort_flag)) return;
     }
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 4);
-    if (piece == 0 && w < rows) {
-      const int64_t b = t / P.seq;
-      const int i = (int)(t - b * P.seq);
-      P.delta[(b * P.heads + h) * P.seq + i] = s;
-    }
+    const int at = walk.start(j);
+    const uint32_t bar = S.full + 8 * s, dst = S.ring + s * 2 * TILE_BYTES;
+    mbar_expect_tx(bar, 2 * TILE_BYTES + (stat ? STAT_BYTES : 0));
+    tma_load_2d(dst, tile_a, col, row0 + at, bar);
+    tma_load_2d(dst + TILE_BYTES, tile_b, col, row0 + at, bar);
+    if (stat) bulk_load(S.stat + s * STAT_BYTES, stat + 2 * at, STAT_BYTES, bar);
+    if (++s == STAGES) { s = 0; ++lap; }
   }
 }
 
 // ------------------------------------------------------------------------------------------- dQ
-__global__ void __launch_bounds__(BW_THREADS, 4) attn_bwd_dq_kernel(BwdParams P) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __nv_bfloat16* Qs = reinterpret_cast<__nv_bfloat16*>(smem);   // [64][LDB]
-  __nv_bfloat16* Gs = Qs + TS * LDB;                             // dOut tile
-  __nv_bfloat16* KV = Gs + TS * LDB;                             // two (K tile, V tile) buffers: the next pair is fetched
-  float* Sf = reinterpret_cast<float*>(KV);                      //   while the current one is used; dQ [64][LDF] is staged
-                                                                 //   over them when the last tile has been consumed
-  __shared__ float lse_s[TS], del_s[TS];
-
-  const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int q0 = qt * TS, l = P.stride;
-  const int64_t row0 = (int64_t)b * P.seq;
+// Tensor memory: S in columns 0-63, dP 64-127, dQ 128-191, dS (bf16) 192-223.  S and dP are free as soon as they are in
+// registers, so the next tile's scores are formed during this tile's algebra.
+__global__ void __launch_bounds__(THREADS, 2)
+attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const BwdParams P) {
+  extern __shared__ unsigned char smem_raw[];
+  const Smem S(smem_raw);
+  __shared__ uint32_t holder;
+  __shared__ int abort_sh;
+  volatile int* abort_flag = &abort_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, t = lane & 3;
-  const int64_t stat0 = ((int64_t)b * P.heads + h) * P.seq;
-  load_tile_async(Qs, P.Q + h * D, P.ld, row0 + q0);       // all first loads in flight together
-  load_tile_async(Gs, P.dOut + h * D, P.lddo, row0 + q0);
-  if (threadIdx.x < TS) {
-    lse_s[threadIdx.x] = P.lse[stat0 + q0 + threadIdx.x];
-    del_s[threadIdx.x] = P.delta[stat0 + q0 + threadIdx.x];
-  }
-  const int r_base = warp * 16;
-  // key tiles: the window's tiles, then one tile per strided position further back (i - 2l, i - 3l, ...), of which
-  // only the diagonal (query r, key r) is attended
-  const int k_first = q0 - l > 0 ? q0 - l : 0;
-  const int n_near = (q0 - k_first) / TS + 1;
-  const int n_tiles = n_near + (q0 / l > 1 ? q0 / l - 1 : 0);
-  auto tile_start = [&](int ti) { return ti < n_near ? k_first + ti * TS : q0 - (ti - n_near + 2) * l; };
-  load_tile_async(KV, P.K + h * D, P.ld, row0 + k_first);
-  load_tile_async(KV + TS * LDB, P.V + h * D, P.ld, row0 + k_first);
-  async_commit();
-  async_wait_all();
-  __syncthreads();   // Q, dOut, the statistics and the first key tile are in place
-  uint32_t qa[4][4], ga[4][4];
-#pragma unroll
-  for (int kb = 0; kb < 4; ++kb) {
-    load_a(qa[kb], Qs, r_base, kb, lane);
-    load_a(ga[kb], Gs, r_base, kb, lane);
-  }
-  const float nl0 = -lse_s[r_base + g] * 1.4426950408889634f, nl1 = -lse_s[r_base + g + 8] * 1.4426950408889634f;
-  const float del0 = del_s[r_base + g], del1 = del_s[r_base + g + 8];
-  float acc[8][4];
-#pragma unroll
-  for (int nb = 0; nb < 8; ++nb) acc[nb][0] = acc[nb][1] = acc[nb][2] = acc[nb][3] = 0.f;
-  int buf = 0;
-  for (int ti = 0; ti < n_tiles; ++ti, buf ^= 1) {
-    const int k0 = tile_start(ti);
-    async_wait_all();
-    __syncthreads();   // this tile has landed for everyone; the other buffer's tile has been consumed
-    const __nv_bfloat16* Ks = KV + buf * 2 * TS * LDB;
-    const __nv_bfloat16* Vs = Ks + TS * LDB;
-    if (ti + 1 < n_tiles) {
-      const int kn = tile_start(ti + 1);
-      load_tile_async(KV + (buf ^ 1) * 2 * TS * LDB, P.K + h * D, P.ld, row0 + kn);
-      load_tile_async(KV + (buf ^ 1) * 2 * TS * LDB + TS * LDB, P.V + h * D, P.ld, row0 + kn);
-      async_commit();
-    }
-    // a window tile lies within l + 64 positions behind the queries: a pair is kept iff 0 <= i - j <= l (the window,
-    // and the first strided position i - l); in a tile further back iff i - j is the tile's own distance
-    const int back_lo = ti < n_near ? 0 : q0 - k0, back_hi = ti < n_near ? l : q0 - k0;
-    const int back0 = q0 - k0 + r_base + g - 2 * t;   // i - j of this lane's first element of key column 0
-    if (ti >= n_near) {
-      // a tile further back: query r sees key r of the tile only, so of the 64 keys just the 16 in line with this
-      // warp's rows matter (two score tiles of 16 x 8, one 16-key step of the second product)
-      const int c0 = r_base;                            // first of those keys
-      float sc[2][4], dp[2][4];
-#pragma unroll
-      for (int nb = 0; nb < 2; ++nb) {
-        sc[nb][0] = sc[nb][1] = sc[nb][2] = sc[nb][3] = 0.f;
-        dp[nb][0] = dp[nb][1] = dp[nb][2] = dp[nb][3] = 0.f;
+  const int h = blockIdx.y, b = blockIdx.z, q0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * ROWS, l = P.stride;
+  const int row0 = b * P.seq;
+  const Walk<true> walk(q0, l, P.seq, P.magic);
+  if (warp == CW && lane < 4) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : &tmG);
+  const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+
+  if (warp == CW) {
+    if (lane == 0) feed(S, walk, &tmQ, &tmG, &tmK, &tmV, h * D, row0, nullptr, abort_flag);
+  } else if (warp == CW + 1) {
+    if (lane == 0) {
+      const uint64_t qd = smem_desc(S.own0, 16, 1024), gd = smem_desc(S.own1, 16, 1024), kd0 = smem_desc(S.ring, 16, 1024);
+      const uint64_t step = (2 * TILE_BYTES) >> 4, vofs = TILE_BYTES >> 4;
+      bool ok = wait_on(S.own_full, 0, abort_flag);
+      int s = 0, sp = 0;
+      uint32_t ph = 0;
+      for (int j = 0; j <= walk.near && ok; ++j) {
+        if (j < walk.near) {
+          ok = wait_on(S.full + 8 * s, ph, abort_flag) && (j == 0 || wait_on(S.s_free, (uint32_t)(j - 1) & 1u, abort_flag));
+          if (!ok) break;
+          tc_fence_after();
+          mma_scores(tmem, qd, kd0 + step * (uint32_t)s);
+          mma_scores(tmem + 64, gd, kd0 + step * (uint32_t)s + vofs);
+          tc_commit(S.s_full);
+        }
+        if (j > 0) {
+          ok = wait_on(S.w_full, (uint32_t)(j - 1) & 1u, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          mma_weights(tmem + 128, tmem + 192, 8, kd0 + step * (uint32_t)sp, j > 1 ? 1u : 0u);
+          tc_commit(S.empty + 8 * sp);
+          tc_commit(j == walk.near ? S.acc_full : S.w_free);
+        }
+        sp = s;
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      mma_rows_wide<2>(sc, qa, Ks, c0, lane);
-      mma_rows_wide<2>(dp, ga, Vs, c0, lane);
+    }
+  } else {
+    const int quarter = warp & 3, c = (warp >> 2) * COLS;    // this warp's lanes, and its share of a tile's 64 columns
+    const int r = quarter * 32 + lane, i = q0 + r;
+    const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
+    float* part = S.at<float>(S.stat + STAGES * STAT_BYTES);                  // [PARTS][128] partial sums of delta
+    float2* stat_s = reinterpret_cast<float2*>(part + PARTS * ROWS);              // the rows' -lse log2 e and delta
+    // delta of this row: the threads of a row take COLS dimensions each
+    const bool row_ok = i < P.seq;
+    const int64_t st = ((int64_t)b * P.heads + h) * P.seq + i;
+    uint4 o[COLS / 8];
+    float nl = 0.f;
+    if (row_ok) {
+      const uint4* src = reinterpret_cast<const uint4*>(P.Out + ((int64_t)row0 + i) * P.ldo + h * D + c);
 #pragma unroll
-      for (int nb = 0; nb < 2; ++nb) {
+      for (int p = 0; p < COLS / 8; ++p) o[p] = __ldg(src + p);
+      nl = -__ldg(P.lse + st) * LOG2E;
+    }
+    bool ok = wait_on(S.own_full, 0, abort_flag);
+    float del = 0.f;
+    if (row_ok) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          // row r_base + g + 8 (i >> 1) against key c0 + 8 nb + 2 t + (i & 1): kept on the diagonal
-          float ds = 0.f;
-          if (g + (i >> 1) * 8 == nb * 8 + 2 * t + (i & 1)) {
-            const float p = ex2_approx(fmaf(sc[nb][i], SCALE_LOG2E, (i >> 1) ? nl1 : nl0));
-            ds = p * (dp[nb][i] - ((i >> 1) ? del1 : del0));
-          }
-          sc[nb][i] = ds;
+      for (int p = 0; p < COLS / 8; ++p) {
+        const uint4 g = lds128(piece_addr(S.own1, r, c / 8 + p));
+        const uint32_t ow[4] = {o[p].x, o[p].y, o[p].z, o[p].w}, gw[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          del = fmaf(bf_lo(ow[e]), bf_lo(gw[e]), del);
+          del = fmaf(bf_hi(ow[e]), bf_hi(gw[e]), del);
         }
       }
-      uint32_t a[4];
-      a[0] = pack_bf16(sc[0][0], sc[0][1]);
-      a[1] = pack_bf16(sc[0][2], sc[0][3]);
-      a[2] = pack_bf16(sc[1][0], sc[1][1]);
-      a[3] = pack_bf16(sc[1][2], sc[1][3]);
-      mma_cols(acc, a, Ks, c0, lane);
-      continue;
     }
-    // every pair of this warp's rows with the tile's keys is kept: no mask arithmetic (uniform over the warp)
-    const bool full = q0 - k0 + r_base - 63 >= back_lo && q0 - k0 + r_base + 15 <= back_hi;
+    part[c / COLS * ROWS + r] = del;
+    compute_sync<32 * CW>();
+    del = 0.f;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {            // 32 keys at a time
-      float sc[4][4], dp[4][4];
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb) {
-        sc[nb][0] = sc[nb][1] = sc[nb][2] = sc[nb][3] = 0.f;
-        dp[nb][0] = dp[nb][1] = dp[nb][2] = dp[nb][3] = 0.f;
+    for (int p = 0; p < PARTS; ++p) del += part[p * ROWS + r];
+    if (c == 0) {
+      stat_s[r] = make_float2(nl, del);
+      if (row_ok) {
+        float* out = P.stat + (st / TS) * (2 * TS) + r % TS;   // st = r modulo 64
+        out[0] = nl;
+        out[TS] = -del;
       }
-      mma_rows_wide<4>(sc, qa, Ks, half * 32, lane);
-      mma_rows_wide<4>(dp, ga, Vs, half * 32, lane);
-      if (full) {
+    }
+
+    const uint64_t scale2 = pack2(SCALE_LOG2E, SCALE_LOG2E), nl2 = pack2(nl, nl), ndel2 = pack2(-del, -del);
+    const int i_lo = q0 + quarter * 32;                      // this warp's rows: i_lo .. i_lo + 31
+    for (int j = 0; j < walk.near && ok; ++j) {
+      ok = wait_on(S.s_full, (uint32_t)j & 1u, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t s[PIECES][16], dp[PIECES][16], w[PIECES][8];
 #pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
+      for (int pc = 0; pc < PIECES; ++pc) {
+        tmem_ld16_nowait(t_row + (uint32_t)(c + pc * 16), s[pc]);
+        tmem_ld16_nowait(t_row + (uint32_t)(64 + c + pc * 16), dp[pc]);
+      }
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float p = ex2_approx(fmaf(sc[nb][i], SCALE_LOG2E, (i >> 1) ? nl1 : nl0));
-            sc[nb][i] = p * (dp[nb][i] - ((i >> 1) ? del1 : del0));
+      for (int pc = 0; pc < PIECES; ++pc) {
+        tmem_ld16_wait(s[pc]);
+        tmem_ld16_wait(dp[pc]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(S.s_free);
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) {
+        const int k0 = walk.first + j * TS + c + pc * 16;    // the piece's keys: k0 .. k0 + 15
+        if (i_lo + 31 >= k0 && i_lo - (k0 + 15) <= l) {      // some pair is attended
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const uint64_t pp = ex2_2(fma2(pack2(s[pc][2 * e], s[pc][2 * e + 1]), scale2, nl2));
+            w[pc][e] = pack_bf16_2(mul2(pp, add2(pack2(dp[pc][2 * e], dp[pc][2 * e + 1]), ndel2)));
           }
-        }
-      } else {
+          if (!(i_lo >= k0 + 15 && i_lo + 31 - k0 <= l)) {   // some pair is not
+            const int back0 = i - k0;
 #pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int back = back0 + (i >> 1) * 8 - (half * 32 + nb * 8 + (i & 1));
-            float ds = 0.f;
-            if ((unsigned)(back - back_lo) <= (unsigned)(back_hi - back_lo)) {
-              const float p = ex2_approx(fmaf(sc[nb][i], SCALE_LOG2E, (i >> 1) ? nl1 : nl0));
-              ds = p * (dp[nb][i] - ((i >> 1) ? del1 : del0));
+            for (int e = 0; e < 8; ++e) {
+              if ((unsigned)(back0 - 2 * e) > (unsigned)l) w[pc][e] &= 0xFFFF0000u;
+              if ((unsigned)(back0 - 2 * e - 1) > (unsigned)l) w[pc][e] &= 0x0000FFFFu;
             }
-            sc[nb][i] = ds;
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {                   // 16 keys per step
-        uint32_t a[4];
-        a[0] = pack_bf16(sc[2 * j][0], sc[2 * j][1]);
-        a[1] = pack_bf16(sc[2 * j][2], sc[2 * j][3]);
-        a[2] = pack_bf16(sc[2 * j + 1][0], sc[2 * j + 1][1]);
-        a[3] = pack_bf16(sc[2 * j + 1][2], sc[2 * j + 1][3]);
-        mma_cols(acc, a, Ks, half * 32 + j * 16, lane);
-      }
-    }
-  }
-  __syncthreads();   // every warp is done with the key tiles: their storage takes dQ
-  store_acc(Sf, acc, r_base, lane);
-  __syncwarp();
-  for (int r = r_base; r < r_base + 16; ++r) {   // lane = two head dimensions
-    const float ox = Sf[r * LDF + 2 * lane] * SCALE, oy = Sf[r * LDF + 2 * lane + 1] * SCALE;
-    *reinterpret_cast<__nv_bfloat162*>(P.dQ + (row0 + q0 + r) * P.ldg + h * D + 2 * lane) = __floats2bfloat162_rn(ox, oy);
-  }
-}
-
-// ------------------------------------------------------------------------------------------- dK, dV
-__global__ void __launch_bounds__(BW_THREADS, 3) attn_bwd_dkv_kernel(BwdParams P) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(smem);
-  __nv_bfloat16* Vs = Ks + TS * LDB;
-  __nv_bfloat16* QG = Vs + TS * LDB;                             // two (Q tile, dOut tile) buffers
-  float* Sf = reinterpret_cast<float*>(QG);                      // dK [64][LDF] and dV are staged over the query buffers
-  float* Pf = Sf + TS * LDF;                                     //   when the last tile has been consumed
-  __shared__ float stat_s[2][2 * TS];   // per buffer: log-sum-exp and delta of the tile's queries
-
-  const int kt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int k0 = kt * TS, l = P.stride;
-  const int64_t row0 = (int64_t)b * P.seq;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, t = lane & 3;
-  const int64_t stat0 = ((int64_t)b * P.heads + h) * P.seq;
-  load_tile_async(Ks, P.K + h * D, P.ld, row0 + k0);         // all first loads in flight together
-  load_tile_async(Vs, P.V + h * D, P.ld, row0 + k0);
-  const int r_base = warp * 16;   // this warp's keys
-  // query tiles: those whose window reaches these keys, then one tile per strided position further on
-  // (j + 2l, j + 3l, ...), of which only the diagonal is attended
-  const int q_last = k0 + l < P.seq - TS ? k0 + l : P.seq - TS;
-  const int n_near = (q_last - k0) / TS + 1;
-  const int m_max = (P.seq - TS - k0) / l;
-  const int n_tiles = n_near + (m_max > 1 ? m_max - 1 : 0);
-  auto tile_start = [&](int ti) { return ti < n_near ? k0 + ti * TS : k0 + (ti - n_near + 2) * l; };
-  auto fetch = [&](int q0, int bf) {
-    load_tile_async(QG + bf * 2 * TS * LDB, P.Q + h * D, P.ld, row0 + q0);
-    load_tile_async(QG + bf * 2 * TS * LDB + TS * LDB, P.dOut + h * D, P.lddo, row0 + q0);
-    load_floats_async(stat_s[bf], P.lse + stat0 + q0, TS);
-    load_floats_async(stat_s[bf] + TS, P.delta + stat0 + q0, TS);
-    async_commit();
-  };
-  fetch(k0, 0);
-  async_wait_all();
-  __syncthreads();   // K, V and the first query tile are in place
-  uint32_t ka[4][4], va[4][4];
-#pragma unroll
-  for (int kb = 0; kb < 4; ++kb) {
-    load_a(ka[kb], Ks, r_base, kb, lane);
-    load_a(va[kb], Vs, r_base, kb, lane);
-  }
-  float acc_k[8][4], acc_v[8][4];
-#pragma unroll
-  for (int nb = 0; nb < 8; ++nb) {
-    acc_k[nb][0] = acc_k[nb][1] = acc_k[nb][2] = acc_k[nb][3] = 0.f;
-    acc_v[nb][0] = acc_v[nb][1] = acc_v[nb][2] = acc_v[nb][3] = 0.f;
-  }
-  int buf = 0;
-  for (int ti = 0; ti < n_tiles; ++ti, buf ^= 1) {
-    const int q0 = tile_start(ti);
-    async_wait_all();
-    __syncthreads();   // this query tile has landed for everyone; the other buffer has been consumed
-    const __nv_bfloat16* Qs = QG + buf * 2 * TS * LDB;
-    const __nv_bfloat16* Gs = Qs + TS * LDB;
-    const float* lse_s = stat_s[buf];
-    const float* del_s = stat_s[buf] + TS;
-    if (ti + 1 < n_tiles) fetch(tile_start(ti + 1), buf ^ 1);
-    // a window tile lies within l + 64 positions ahead of the keys: a pair is kept iff 0 <= i - j <= l; in a tile
-    // further on iff i - j is the tile's own distance
-    const int back_lo = ti < n_near ? 0 : q0 - k0, back_hi = ti < n_near ? l : q0 - k0;
-    const int back0 = q0 - k0 - (r_base + g) + 2 * t;   // i - j of this lane's first element of query column 0
-    if (ti >= n_near) {
-      // a tile further on: key r is seen by query r of the tile only, so just the 16 queries in line with this warp's
-      // keys matter
-      const int c0 = r_base;
-      float st[2][4], dp[2][4];
-#pragma unroll
-      for (int nb = 0; nb < 2; ++nb) {
-        st[nb][0] = st[nb][1] = st[nb][2] = st[nb][3] = 0.f;
-        dp[nb][0] = dp[nb][1] = dp[nb][2] = dp[nb][3] = 0.f;
-      }
-      mma_rows_wide<2>(st, ka, Qs, c0, lane);
-      mma_rows_wide<2>(dp, va, Gs, c0, lane);
-#pragma unroll
-      for (int nb = 0; nb < 2; ++nb) {
-        const int c = c0 + nb * 8 + 2 * t;
-        const float2 ls = *reinterpret_cast<const float2*>(lse_s + c), dl = *reinterpret_cast<const float2*>(del_s + c);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float p = 0.f, ds = 0.f;
-          if (g + (i >> 1) * 8 == nb * 8 + 2 * t + (i & 1)) {
-            p = ex2_approx(fmaf(st[nb][i], SCALE_LOG2E, -1.4426950408889634f * ((i & 1) ? ls.y : ls.x)));
-            ds = p * (dp[nb][i] - ((i & 1) ? dl.y : dl.x));
-          }
-          st[nb][i] = p;
-          dp[nb][i] = ds;
-        }
-      }
-      uint32_t pa[4], da[4];
-      pa[0] = pack_bf16(st[0][0], st[0][1]);
-      pa[1] = pack_bf16(st[0][2], st[0][3]);
-      pa[2] = pack_bf16(st[1][0], st[1][1]);
-      pa[3] = pack_bf16(st[1][2], st[1][3]);
-      da[0] = pack_bf16(dp[0][0], dp[0][1]);
-      da[1] = pack_bf16(dp[0][2], dp[0][3]);
-      da[2] = pack_bf16(dp[1][0], dp[1][1]);
-      da[3] = pack_bf16(dp[1][2], dp[1][3]);
-      mma_cols(acc_v, pa, Gs, c0, lane);
-      mma_cols(acc_k, da, Qs, c0, lane);
-      continue;
-    }
-    // every pair of the tile's queries with this warp's keys is kept: no mask arithmetic (uniform over the warp)
-    const bool full = q0 - k0 - r_base - 15 >= back_lo && q0 - k0 - r_base + 63 <= back_hi;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {              // 32 queries at a time
-      float st[4][4], dp[4][4];                         // S^T and dP^T: rows = keys, columns = queries
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb) {
-        st[nb][0] = st[nb][1] = st[nb][2] = st[nb][3] = 0.f;
-        dp[nb][0] = dp[nb][1] = dp[nb][2] = dp[nb][3] = 0.f;
-      }
-      mma_rows_wide<4>(st, ka, Qs, half * 32, lane);
-      mma_rows_wide<4>(dp, va, Gs, half * 32, lane);
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb) {
-        const int c = half * 32 + nb * 8 + 2 * t;
-        float2 ls = *reinterpret_cast<const float2*>(lse_s + c);
-        const float2 dl = *reinterpret_cast<const float2*>(del_s + c);
-        ls.x *= -1.4426950408889634f;
-        ls.y *= -1.4426950408889634f;
-        if (full) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float p = ex2_approx(fmaf(st[nb][i], SCALE_LOG2E, (i & 1) ? ls.y : ls.x));
-            st[nb][i] = p;
-            dp[nb][i] = p * (dp[nb][i] - ((i & 1) ? dl.y : dl.x));
           }
         } else {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int back = back0 + (half * 32 + nb * 8 + (i & 1)) - (i >> 1) * 8;
-            float p = 0.f, ds = 0.f;
-            if ((unsigned)(back - back_lo) <= (unsigned)(back_hi - back_lo)) {
-              p = ex2_approx(fmaf(st[nb][i], SCALE_LOG2E, (i & 1) ? ls.y : ls.x));
-              ds = p * (dp[nb][i] - ((i & 1) ? dl.y : dl.x));
-            }
-            st[nb][i] = p;
-            dp[nb][i] = ds;
-          }
+          for (int e = 0; e < 8; ++e) w[pc][e] = 0u;
         }
       }
+      if (j > 0) {
+        ok = wait_on(S.w_free, (uint32_t)(j - 1) & 1u, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+      }
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {                     // 16 queries per step
-        uint32_t pa[4], da[4];
-        pa[0] = pack_bf16(st[2 * j][0], st[2 * j][1]);
-        pa[1] = pack_bf16(st[2 * j][2], st[2 * j][3]);
-        pa[2] = pack_bf16(st[2 * j + 1][0], st[2 * j + 1][1]);
-        pa[3] = pack_bf16(st[2 * j + 1][2], st[2 * j + 1][3]);
-        da[0] = pack_bf16(dp[2 * j][0], dp[2 * j][1]);
-        da[1] = pack_bf16(dp[2 * j][2], dp[2 * j][3]);
-        da[2] = pack_bf16(dp[2 * j + 1][0], dp[2 * j + 1][1]);
-        da[3] = pack_bf16(dp[2 * j + 1][2], dp[2 * j + 1][3]);
-        mma_cols(acc_v, pa, Gs, half * 32 + j * 16, lane);
-        mma_cols(acc_k, da, Qs, half * 32 + j * 16, lane);
+      for (int pc = 0; pc < PIECES; ++pc) tmem_st8(t_row + (uint32_t)(192 + c / 2 + pc * 8), w[pc]);
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(S.w_full);
+    }
+
+    // far tiles: warp = STRIPS times 16 rows of the block, with the keys in line with them
+    const int far = walk.far0 + walk.far1;
+    const int r0 = warp * 16 * STRIPS;
+    float acc[STRIPS][8][4];
+#pragma unroll
+    for (int sp = 0; sp < STRIPS; ++sp)
+#pragma unroll
+      for (int nb = 0; nb < 8; ++nb) acc[sp][nb][0] = acc[sp][nb][1] = acc[sp][nb][2] = acc[sp][nb][3] = 0.f;
+    if (far > 0) {
+      compute_sync<32 * CW>();                               // the rows' statistics are in place
+      const int g = lane >> 2, t = lane & 3;
+      int s = walk.near % STAGES;
+      uint32_t ph = (uint32_t)(walk.near / STAGES) & 1u;
+      for (int f = 0; f < far && ok; ++f) {
+        if (walk.far_half(f) == r0 >> 6) {
+          ok = wait_on(S.full + 8 * s, ph, abort_flag);
+          if (!ok) break;
+          const uint32_t kt = S.ring + s * 2 * TILE_BYTES;
+#pragma unroll
+          for (int sp = 0; sp < STRIPS; ++sp) {
+            const int rs = r0 + sp * 16, c0 = rs & 63;
+            const float2 st0 = stat_s[rs + g], st1 = stat_s[rs + g + 8];
+            float sc[2][4], dp[2][4];
+            far_scores(sc, S.own0, rs, kt, c0, lane);
+            far_scores(dp, S.own1, rs, kt + TILE_BYTES, c0, lane);
+#pragma unroll
+            for (int nb = 0; nb < 2; ++nb) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                float ds = 0.f;
+                if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
+                  const float p = ex2(fmaf(sc[nb][e], SCALE_LOG2E, (e >> 1) ? st1.x : st0.x));
+                  ds = p * (dp[nb][e] - ((e >> 1) ? st1.y : st0.y));
+                }
+                sc[nb][e] = ds;
+              }
+            }
+            far_accumulate<4>(acc[sp], sc, kt, c0, 0, lane);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+        }
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
     }
+    ok = ok && wait_on(S.acc_full, 0, abort_flag);
+    tc_fence_after();
+    // every product has completed and every tile has been consumed: the ring takes the far sums, the own tiles the results
+    uint32_t v[PIECES][16];
+#pragma unroll
+    for (int pc = 0; pc < PIECES; ++pc) tmem_ld16_nowait(t_row + (uint32_t)(128 + c + pc * 16), v[pc]);
+    compute_sync<32 * CW>();
+    float* sums = far > 0 ? S.at<float>(S.ring) : nullptr;
+    __nv_bfloat16* res = S.at<__nv_bfloat16>(S.own0);
+    if (far > 0) {
+#pragma unroll
+      for (int sp = 0; sp < STRIPS; ++sp) far_stage<8>(sums, acc[sp], r0 + sp * 16, 0, lane);
+      compute_sync<32 * CW>();
+    }
+#pragma unroll
+    for (int pc = 0; pc < PIECES; ++pc) {
+      tmem_ld16_wait(v[pc]);
+      stage_row(res, r, c + pc * 16, v[pc], sums, SCALE);
+    }
+    compute_sync<32 * CW>();
+    constexpr int N = ROWS / CW;   // rows a warp writes
+    if (ok && q0 + warp * N < P.seq) write_rows<N>(res, warp * N, P.dQ + h * D, (int64_t)row0 + q0, P.ldg, lane);
   }
-  __syncthreads();   // every warp is done with the query tiles: their storage takes dK and dV
-  store_acc(Sf, acc_k, r_base, lane);
-  store_acc(Pf, acc_v, r_base, lane);
-  __syncwarp();
-  for (int r = r_base; r < r_base + 16; ++r) {   // lane = two head dimensions
-    const int64_t o = (row0 + k0 + r) * P.ldg + h * D + 2 * lane;
-    *reinterpret_cast<__nv_bfloat162*>(P.dK + o) = __floats2bfloat162_rn(Sf[r * LDF + 2 * lane] * SCALE, Sf[r * LDF + 2 * lane + 1] * SCALE);
-    *reinterpret_cast<__nv_bfloat162*>(P.dV + o) = __floats2bfloat162_rn(Pf[r * LDF + 2 * lane], Pf[r * LDF + 2 * lane + 1]);
+  block_teardown(tmem, warp, abort_flag);
+}
+
+// ------------------------------------------------------------------------------------------- dK, dV
+// Tensor memory: S^T in columns 0-63, dP^T 64-127, dK 128-191, dV 192-255; each warp writes P^T over the scores it has
+// read (eight columns at its sixteen's start) and dS^T over its dP.
+__global__ void __launch_bounds__(THREADS, 2)
+attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const BwdParams P) {
+  extern __shared__ unsigned char smem_raw[];
+  const Smem S(smem_raw);
+  __shared__ uint32_t holder;
+  __shared__ int abort_sh;
+  volatile int* abort_flag = &abort_sh;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = blockIdx.y, b = blockIdx.z, k0 = (int)blockIdx.x * ROWS, l = P.stride;   // early keys have the most tiles
+  const int row0 = b * P.seq;
+  const Walk<false> walk(k0, l, P.seq, P.magic);
+  if (warp == CW && lane < 4) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : &tmG);
+  const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+
+  if (warp == CW) {
+    if (lane == 0)
+      feed(S, walk, &tmK, &tmV, &tmQ, &tmG, h * D, row0, P.stat + 2 * ((int64_t)b * P.heads + h) * P.seq, abort_flag);
+  } else if (warp == CW + 1) {
+    if (lane == 0) {
+      const uint64_t kd = smem_desc(S.own0, 16, 1024), vd = smem_desc(S.own1, 16, 1024), qd0 = smem_desc(S.ring, 16, 1024);
+      const uint64_t step = (2 * TILE_BYTES) >> 4, gofs = TILE_BYTES >> 4;
+      bool ok = wait_on(S.own_full, 0, abort_flag);
+      int s = 0;
+      uint32_t ph = 0;
+      for (int j = 0; j < walk.near && ok; ++j) {
+        ok = wait_on(S.full + 8 * s, ph, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t qd = qd0 + step * (uint32_t)s;
+        // Everything executes in issue order, so the scores may overwrite the P of the tile before (its dV product is issued)
+        // and dP its dS.  S goes ahead of the last tile's dK: the exponentials start while dK and dP are formed.
+        if (j == 0) mma_scores(tmem, kd, qd);
+        if (j == 0) tc_commit(S.s_full);
+        mma_scores(tmem + 64, vd, qd + gofs);
+        tc_commit(S.dp_full);
+        ok = wait_on(S.p_full, (uint32_t)j & 1u, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        mma_weights(tmem + 192, tmem, 16, qd + gofs, j > 0 ? 1u : 0u);
+        if (j + 1 < walk.near) {
+          const int sn = s + 1 == STAGES ? 0 : s + 1;
+          ok = wait_on(S.full + 8 * sn, sn ? ph : ph ^ 1u, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          mma_scores(tmem, kd, qd0 + step * (uint32_t)sn);
+          tc_commit(S.s_full);
+        }
+        ok = wait_on(S.w_full, (uint32_t)j & 1u, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        mma_weights(tmem + 128, tmem + 64, 16, qd, j > 0 ? 1u : 0u);
+        tc_commit(S.empty + 8 * s);
+        if (j + 1 == walk.near) tc_commit(S.acc_full);
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
+      }
+    }
+  } else {
+    const int quarter = warp & 3, c = (warp >> 2) * COLS;    // this warp's lanes, and its share of a tile's 64 columns
+    const int r = quarter * 32 + lane, jk = k0 + r;
+    const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
+    const uint64_t scale2 = pack2(SCALE_LOG2E, SCALE_LOG2E);
+    const int j_lo = k0 + quarter * 32;                      // this warp's keys: j_lo .. j_lo + 31
+    bool ok = wait_on(S.own_full, 0, abort_flag);
+    int s = 0;
+    uint32_t ph = 0;
+    for (int j = 0; j < walk.near && ok; ++j) {
+      const uint32_t sa = S.stat + (uint32_t)(s * STAT_BYTES + c * 4);
+      ok = wait_on(S.full + 8 * s, ph, abort_flag) &&        // the statistics have landed too
+           wait_on(S.s_full, (uint32_t)j & 1u, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t w[PIECES][8], st[PIECES][16];
+      uint64_t p[PIECES][8];                                 // P^T of this row, fp32 pairs
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) tmem_ld16_nowait(t_row + (uint32_t)(c + pc * 16), st[pc]);
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) {
+        const int q0 = walk.first + j * TS + c + pc * 16;    // the piece's queries: q0 .. q0 + 15
+        tmem_ld16_wait(st[pc]);
+        if (q0 + 15 >= j_lo && q0 - (j_lo + 31) <= l) {      // some pair is attended
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {                      // statistics of four queries at a time
+            const uint4 nl = lds128(sa + 64u * pc + 16u * e);
+            p[pc][2 * e] = ex2_2(fma2(pack2(st[pc][4 * e], st[pc][4 * e + 1]), scale2, pack2(nl.x, nl.y)));
+            p[pc][2 * e + 1] = ex2_2(fma2(pack2(st[pc][4 * e + 2], st[pc][4 * e + 3]), scale2, pack2(nl.z, nl.w)));
+          }
+          if (!(q0 >= j_lo + 31 && q0 + 15 - j_lo <= l)) {   // some pair is not
+            const int back0 = q0 - jk;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              float lo, hi;
+              unpack2(p[pc][e], lo, hi);
+              p[pc][e] = pack2((unsigned)(back0 + 2 * e) > (unsigned)l ? 0.f : lo, (unsigned)(back0 + 2 * e + 1) > (unsigned)l ? 0.f : hi);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) p[pc][e] = 0ULL;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[pc][e] = pack_bf16_2(p[pc][e]);
+        tmem_st8(t_row + (uint32_t)(c + pc * 16), w[pc]);
+      }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(S.p_full);
+      ok = wait_on(S.dp_full, (uint32_t)j & 1u, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) tmem_ld16_nowait(t_row + (uint32_t)(64 + c + pc * 16), st[pc]);
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) {
+        const int q0 = walk.first + j * TS + c + pc * 16;
+        tmem_ld16_wait(st[pc]);
+        if (q0 + 15 >= j_lo && q0 - (j_lo + 31) <= l) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const uint4 nd = lds128(sa + (uint32_t)(TS * 4) + 64u * pc + 16u * e);
+            w[pc][2 * e] = pack_bf16_2(mul2(p[pc][2 * e], add2(pack2(st[pc][4 * e], st[pc][4 * e + 1]), pack2(nd.x, nd.y))));
+            w[pc][2 * e + 1] = pack_bf16_2(mul2(p[pc][2 * e + 1], add2(pack2(st[pc][4 * e + 2], st[pc][4 * e + 3]), pack2(nd.z, nd.w))));
+          }
+          if (!(q0 >= j_lo + 31 && q0 + 15 - j_lo <= l)) {
+            const int back0 = q0 - jk;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              w[pc][e] &= ((unsigned)(back0 + 2 * e) > (unsigned)l ? 0u : 0x0000FFFFu) |
+                          ((unsigned)(back0 + 2 * e + 1) > (unsigned)l ? 0u : 0xFFFF0000u);
+          }
+        }
+        tmem_st8(t_row + (uint32_t)(64 + c + pc * 16), w[pc]);   // zeros where nothing is attended
+      }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(S.w_full);
+      if (++s == STAGES) { s = 0; ph ^= 1u; }
+    }
+
+    // far tiles: warp = STRIPS times 16 keys of the block, with the queries in line with them
+    const int far = walk.far0 + walk.far1;
+    const int r0 = warp * 16 * STRIPS;
+    float acc_k[STRIPS][8][4], acc_v[STRIPS][8][4];
+#pragma unroll
+    for (int sp = 0; sp < STRIPS; ++sp)
+#pragma unroll
+      for (int nb = 0; nb < 8; ++nb) {
+        acc_k[sp][nb][0] = acc_k[sp][nb][1] = acc_k[sp][nb][2] = acc_k[sp][nb][3] = 0.f;
+        acc_v[sp][nb][0] = acc_v[sp][nb][1] = acc_v[sp][nb][2] = acc_v[sp][nb][3] = 0.f;
+      }
+    if (far > 0) {
+      const int g = lane >> 2, t = lane & 3;
+      for (int f = 0; f < far && ok; ++f) {
+        if (walk.far_half(f) == r0 >> 6) {
+          ok = wait_on(S.full + 8 * s, ph, abort_flag);
+          if (!ok) break;
+          const uint32_t qt = S.ring + s * 2 * TILE_BYTES;
+#pragma unroll
+          for (int sp = 0; sp < STRIPS; ++sp) {
+            const int rs = r0 + sp * 16, c0 = rs & 63;
+            float st[2][4], dp[2][4];
+            far_scores(st, S.own0, rs, qt, c0, lane);
+            far_scores(dp, S.own1, rs, qt + TILE_BYTES, c0, lane);
+#pragma unroll
+            for (int nb = 0; nb < 2; ++nb) {
+              const float* sq = S.at<float>(S.stat + (uint32_t)(s * STAT_BYTES)) + c0 + nb * 8 + 2 * t;
+              const float2 nl = *reinterpret_cast<const float2*>(sq), nd = *reinterpret_cast<const float2*>(sq + TS);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                float p = 0.f, ds = 0.f;
+                if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
+                  p = ex2(fmaf(st[nb][e], SCALE_LOG2E, (e & 1) ? nl.y : nl.x));
+                  ds = p * (dp[nb][e] + ((e & 1) ? nd.y : nd.x));
+                }
+                st[nb][e] = p;
+                dp[nb][e] = ds;
+              }
+            }
+            far_accumulate<4>(acc_v[sp], st, qt + TILE_BYTES, c0, 0, lane);
+            far_accumulate<4>(acc_k[sp], dp, qt, c0, 0, lane);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+        }
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
+      }
+    }
+    ok = ok && wait_on(S.acc_full, 0, abort_flag);
+    tc_fence_after();
+    compute_sync<32 * CW>();   // every product has completed and every tile has been consumed
+    float* sums = far > 0 ? S.at<float>(S.ring) : nullptr;
+    __nv_bfloat16* res = S.at<__nv_bfloat16>(S.own0);
+    constexpr int N = ROWS / CW;   // rows a warp writes
+#pragma unroll
+    for (int which = 0; which < 2; ++which) {   // dK, then dV
+      uint32_t v[PIECES][16];
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) tmem_ld16_nowait(t_row + (uint32_t)(128 + which * 64 + c + pc * 16), v[pc]);
+      if (far > 0) {
+#pragma unroll
+        for (int sp = 0; sp < STRIPS; ++sp) far_stage<8>(sums, which ? acc_v[sp] : acc_k[sp], r0 + sp * 16, 0, lane);
+      }
+      if (far > 0 || which) compute_sync<32 * CW>();   // the sums are in place, dK's rows have left the staging tile
+#pragma unroll
+      for (int pc = 0; pc < PIECES; ++pc) {
+        tmem_ld16_wait(v[pc]);
+        stage_row(res, r, c + pc * 16, v[pc], sums, which ? 1.f : SCALE);
+      }
+      compute_sync<32 * CW>();
+      if (ok && k0 + warp * N < P.seq) write_rows<N>(res, warp * N, (which ? P.dV : P.dK) + h * D, (int64_t)row0 + k0, P.ldg, lane);
+    }
   }
+  block_teardown(tmem, warp, abort_flag);
 }
 
 }  // namespace
+
+mst_status_t mst_attention_bwd_error_flags(int32_t* flags) {
+  int v = 0;
+  MST_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_bwd_error, sizeof(int)));
+  *flags = v;
+  return MST_OK;
+}
 
 extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, const void* V, int64_t ld, const void* Out,
                                                   int64_t ldo, const void* dOut, int64_t lddo, const float* lse,
@@ -411,29 +630,31 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
         reinterpret_cast<uintptr_t>(dK) | reinterpret_cast<uintptr_t>(dV)) & 15u) != 0)
     return MST_ERR_SHAPE;
   if (batch == 0) return MST_OK;
-  if ((int64_t)batch * seq_len > 0x7FFFFFFF || heads > 65535 || batch > 65535) return MST_ERR_SHAPE;
+  const int64_t rows = (int64_t)batch * seq_len;
+  if (rows > 0x7FFFFFFF || heads > 65535 || batch > 65535) return MST_ERR_SHAPE;
   cudaStream_t s = (cudaStream_t)stream;
+  CUtensorMap tmQ, tmK, tmV, tmG;
+  if (!tile_map(&tmQ, Q, rows, width, ld) || !tile_map(&tmK, K, rows, width, ld) || !tile_map(&tmV, V, rows, width, ld) ||
+      !tile_map(&tmG, dOut, rows, width, lddo))
+    return MST_ERR_SHAPE;
   void* ws = nullptr;
-  MST_TRY(mst_workspace_kind(MST_WS_ATTENTION, sizeof(float) * (size_t)batch * heads * seq_len, &ws));
+  MST_TRY(mst_workspace_kind(MST_WS_ATTENTION, 2 * sizeof(float) * (size_t)rows * heads, &ws));
   BwdParams P;
   P.Q = (const __nv_bfloat16*)Q; P.K = (const __nv_bfloat16*)K; P.V = (const __nv_bfloat16*)V;
   P.Out = (const __nv_bfloat16*)Out; P.dOut = (const __nv_bfloat16*)dOut;
-  P.ld = ld; P.ldo = ldo; P.lddo = lddo;
-  P.lse = lse; P.delta = (float*)ws;
+  P.ldo = ldo;
+  P.lse = lse; P.stat = (float*)ws;
   P.dQ = (__nv_bfloat16*)dQ; P.dK = (__nv_bfloat16*)dK; P.dV = (__nv_bfloat16*)dV;
   P.ldg = ldg;
-  P.batch = batch; P.seq = seq_len; P.heads = heads; P.stride = stride;
-  const int64_t delta_rows = (int64_t)batch * seq_len * heads;
-  const int64_t delta_blocks = (delta_rows / 4 + 7) / 8 + 1;   // eight warps per block, four rows per warp and trip
-  attn_delta_kernel<<<(unsigned)(delta_blocks < 148 * 16 ? delta_blocks : 148 * 16), 256, 0, s>>>(P); MST_COUNT_LAUNCH();
-  static_assert(2 * TS * LDF * 4 <= 4 * TS * LDB * 2, "the staged gradients must fit the tile buffers");
-  const size_t smem_q = (size_t)(6 * TS * LDB) * 2 + 128;
-  const size_t smem_kv = (size_t)(6 * TS * LDB) * 2 + 128;
-  MST_SMEM_LIMIT((attn_bwd_dq_kernel), smem_q);
-  MST_SMEM_LIMIT((attn_bwd_dkv_kernel), smem_kv);
-  dim3 grid((unsigned)(seq_len / TS), (unsigned)heads, (unsigned)batch);
-  attn_bwd_dq_kernel<<<grid, BW_THREADS, smem_q, s>>>(P); MST_COUNT_LAUNCH();
-  attn_bwd_dkv_kernel<<<grid, BW_THREADS, smem_kv, s>>>(P); MST_COUNT_LAUNCH();
+  P.batch = batch; P.seq = seq_len; P.heads = heads;
+  P.stride = stride < seq_len ? stride : seq_len;   // from there on the same pairs: all earlier positions
+  P.magic = stride_magic(P.stride, seq_len);
+  P.tiles = (seq_len + ROWS - 1) / ROWS;
+  MST_SMEM_LIMIT((attn_bwd_dq_kernel), SMEM_BYTES);
+  MST_SMEM_LIMIT((attn_bwd_dkv_kernel), SMEM_BYTES);
+  dim3 grid((unsigned)P.tiles, (unsigned)heads, (unsigned)batch);
+  MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dq_kernel, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, P));
+  MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dkv_kernel, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, P));
   MST_CUDA_TRY(cudaGetLastError());
   return MST_OK;
 }

@@ -219,6 +219,7 @@ mst_status_t mst_sddmm_error_flags(int32_t* flags);
 mst_status_t mst_split_error_flags(int32_t* flags);
 // sticky error word of the attention kernel's bounded waits (mst_attention.cu)
 mst_status_t mst_attention_error_flags(int32_t* flags);
+mst_status_t mst_attention_bwd_error_flags(int32_t* flags);
 
 // bins of one radix-select pass (digit width MST_SELECT_RADIX_BITS)
 constexpr int MST_SELECT_RADIX_BITS = 11;

@@ -106,3 +106,16 @@ def test_attention_bwd_random_shapes():
         got, ref, _ = _run(B, n, H, stride, 1300 + case, pad, float(rng.choice([0.5, 1.0, 1.5])))
         for a, b, name in zip(got, ref, ("dQ", "dK", "dV")):
             assert rel_err(a, b) <= 2e-2, (case, name, B, n, H, stride, pad)
+
+
+@pytest.mark.parametrize("B,n,H,stride", [
+    (2, 64, 1, 64),        # half a tile of own rows, nothing but the window
+    (3, 192, 2, 64),       # the last tile's second half lies outside the sequence; one far tile
+    (2, 448, 1, 192),      # windows that end inside a tile's half
+    (1, 576, 2, 64),       # the halves have different numbers of far tiles, more than the ring holds
+    (1, 320, 1, 1 << 20)])  # stride beyond the sequence: causal attention
+def test_attention_bwd_tile_edges(B, n, H, stride):
+    got, ref, _ = _run(B, n, H, stride, 1500 + n + B)
+    for a, b, name in zip(got, ref, ("dQ", "dK", "dV")):
+        assert np.isfinite(a).all() and rel_err(a, b) <= 2e-2, name
+    assert mst.mst_device_error_flags() == 0
