@@ -11,15 +11,15 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
                              cudaStream_t s) {
   const int O = (int)a.M, I = (int)a.N;
   const int64_t T = a.K;
-  const int ldO = (O + 7) & ~7, ldI = (I + 7) & ~7;
+  const int ldO = mst_row_pitch(O), ldI = mst_row_pitch(I);
   a.A = dY; a.lda = lddy; a.a_mn_major = 1;
   a.B = X; a.ldb = ldx; a.b_mn_major = 1;
   if (dtype == MST_F32) {
     void* ws = nullptr;
     MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 6 * (size_t)T * (ldO + ldI), &ws));
     uint16_t* x = (uint16_t*)ws + 3 * (size_t)T * ldO;
-    MST_TRY(mst_split_rows(dY, lddy, T, O, ws, s));
-    MST_TRY(mst_split_rows(X, ldx, T, I, x, s));
+    const mst_rows_job jobs[2] = {{dY, lddy, T, O, ws}, {X, ldx, T, I, x}};
+    MST_TRY(mst_prepare(dtype, nullptr, jobs, 2, s));
     a.A = ws; a.lda = ldO;
     a.B = x; a.ldb = ldI;
     return mst_tc_split(a, s);
@@ -29,15 +29,18 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
     void* ws = nullptr;
     MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 2 * (size_t)T * ((okY ? 0 : ldO) + (okX ? 0 : ldI)), &ws));
     uint16_t* at = (uint16_t*)ws;
+    mst_rows_job jobs[2];
+    int n = 0;
     if (!okY) {
-      MST_TRY(mst_pad_rows(dY, lddy, T, O, at, s));
+      jobs[n++] = {dY, lddy, T, O, at};
       a.A = at; a.lda = ldO;
       at += (size_t)T * ldO;
     }
     if (!okX) {
-      MST_TRY(mst_pad_rows(X, ldx, T, I, at, s));
+      jobs[n++] = {X, ldx, T, I, at};
       a.B = at; a.ldb = ldI;
     }
+    MST_TRY(mst_prepare(dtype, nullptr, jobs, n, s));
   }
   a.splits = 0;
   return mst_tc_gemm(a, s);

@@ -167,7 +167,7 @@ struct mst_layer {
   unsigned int* counter;  // [1] block-completion counter
 
   // dense image of W.M for the tensor-core paths, kept with value tracking: [O x ldp] bf16, or three bf16 pieces of it
-  // for fp32 layers (mst_densify); the input gradient reads it as an MN-major operand, so no transposed copy is kept.
+  // for fp32 layers (mst_image); the input gradient reads it as an MN-major operand, so no transposed copy is kept.
   // Allocated on first use (mst_alloc_dense).
   uint16_t* dense_w;
   int path;  // mst_compute_path_t
@@ -199,9 +199,22 @@ mst_status_t mst_alloc_dense(mst_layer* L);   // no-op when the dense image exis
 mst_status_t mst_build_csc(mst_layer* L, cudaStream_t s);
 mst_status_t mst_ensure_csc(const mst_layer* L, cudaStream_t s);  // builds the CSC view if it is stale
 mst_status_t mst_combine_update_bits(mst_layer* L, int new_set, cudaStream_t s);
-mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image, int64_t* ld);
+// operand preparation (mst_prepare.cu): the pitch of prepared rows, a layer's dense image, rows of a caller's operand
+static inline int mst_row_pitch(int C) { return C <= 32 ? (C + 7) & ~7 : (C + 63) & ~63; }
+struct mst_image_job {
+  const mst_layer* layer;
+  uint16_t* out;          // NULL: the image is in place
+};
+struct mst_rows_job {
+  const void* in;         // [R x C], ld elements apart
+  int64_t ld, R;
+  int C;
+  void* out;              // bf16 [R][pitch], or three pieces of that for fp32 rows
+};
+mst_status_t mst_image(const mst_layer* L, mst_image_job* job, const uint16_t** image, int64_t* ld);
+mst_status_t mst_prepare(mst_dtype_t dtype, const mst_image_job* image, const mst_rows_job* rows, int n_rows, cudaStream_t s);
 static inline size_t mst_image_bytes(const mst_layer* L) {
-  return (L->dtype == MST_F32 ? 6 : 2) * (size_t)L->O * (size_t)((L->I + 7) & ~7);
+  return (L->dtype == MST_F32 ? 6 : 2) * (size_t)L->O * (size_t)mst_row_pitch(L->I);
 }
 // strided attention forward on warp-level products (mst_attention_fwd_mma.cu); the caller has checked pointers and
 // leading dimensions

@@ -556,7 +556,8 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
   if (mst_use_tensor_path(L) || mst_use_split_path(L)) {
     const uint16_t* image = nullptr;
     int64_t ldimage = 0;
-    MST_TRY(mst_densify(L, s, &image, &ldimage));
+    mst_image_job job;
+    MST_TRY(mst_image(L, &job, &image, &ldimage));
     mst_tc_gemm_args a = {};
     a.A = in; a.lda = ldin; a.a_mn_major = 0;
     a.B = image; a.ldb = ldimage; a.b_mn_major = transpose ? 1 : 0;
@@ -564,9 +565,10 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     a.out = out; a.ldc = ldout;
     if (L->dtype == MST_F32) {
       void* pieces = nullptr;
-      a.lda = (cols + 7) & ~7;
+      a.lda = mst_row_pitch(cols);
       MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 6 * (size_t)T * a.lda, &pieces));
-      MST_TRY(mst_split_rows(in, ldin, T, cols, pieces, s));
+      const mst_rows_job rows_in = {in, ldin, T, cols, pieces};
+      MST_TRY(mst_prepare(L->dtype, &job, &rows_in, 1, s));
       a.A = pieces;
       a.epilogue = MST_TC_OUT_F32;
       // the product lands in the pre-activation buffer when the caller keeps one; the activation is a pass of its own
@@ -576,10 +578,13 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     }
     if (!mst_tc_gemm_usable(in, ldin, image, ldimage)) {   // rows that do not start on 16-byte boundaries: an aligned copy
       void* copy = nullptr;
-      a.lda = (cols + 7) & ~7;
+      a.lda = mst_row_pitch(cols);
       MST_TRY(mst_workspace_kind(MST_WS_COLUMNS, 2 * (size_t)T * a.lda, &copy));
-      MST_TRY(mst_pad_rows(in, ldin, T, cols, copy, s));
+      const mst_rows_job rows_in = {in, ldin, T, cols, copy};
+      MST_TRY(mst_prepare(L->dtype, &job, &rows_in, 1, s));
       a.A = copy;
+    } else {
+      MST_TRY(mst_prepare(L->dtype, &job, nullptr, 0, s));
     }
     // A few tokens: the latency kernel (16 tokens: 3 us a layer of GPT-2-small width against 5 for the smallest tiles; at 32 its
     // blocks read the activations too often and it loses).  Columns beyond the row must be zero in the activations too.

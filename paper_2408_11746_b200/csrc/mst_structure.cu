@@ -296,53 +296,6 @@ __global__ void fill_csc(const uint32_t* __restrict__ bitsT, const int32_t* __re
   mst_fill_csc_word(w, threadIdx.x & 31, bitsT, wscanT, O, I, wpr, wpc, bits, wscan, row_idx, perm, col_ptr);
 }
 
-// ---- dense image of W.M for the tensor-core paths ----------------------------------------------------------------------
-// bf16 values: one bf16 image; fp32 values: three bf16 pieces (mst_split3) one image apart.  One thread per 8 consecutive
-// columns: the stored values of those columns are consecutive in CSR order, so the thread reads them in one run and writes
-// one 16-byte vector per image (value or +0 per column).  Every element is written, no separate clear.  Rows are ldp
-// elements apart, ldp = I rounded up to a multiple of 8 (what the TMA unit asks for); mask bits beyond I are zero.
-template <typename V>
-__global__ void densify_from_bits(const uint32_t* __restrict__ bits, const int32_t* __restrict__ wscan, int R, int ldp,
-                                  int wpr, const V* __restrict__ vals, uint16_t* __restrict__ dense) {
-  constexpr int PIECES = sizeof(V) == 4 ? 3 : 1;
-  mst_grid_launch_dependents();
-  mst_grid_dependency_wait();
-  const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;  // group of 8 columns
-  const unsigned gpr = (unsigned)ldp >> 3;                   // groups per row
-  if (g >= (unsigned)R * gpr) return;
-  const unsigned r = g / gpr, c8 = g - r * gpr;
-  const unsigned w = r * (unsigned)wpr + (c8 >> 2);
-  const uint32_t word = bits[w];
-  const unsigned sh = (c8 & 3u) * 8u;
-  uint32_t m = (word >> sh) & 0xFFu;
-  uint32_t out[PIECES][8];
-#pragma unroll
-  for (int k = 0; k < PIECES; ++k)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) out[k][j] = 0u;
-  if (m) {
-    int32_t pos = wscan[w] + __popc(word & ((1u << sh) - 1u));
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if ((m >> j) & 1u) {
-        if (sizeof(V) == 4) {
-          uint32_t p[3];
-          mst_split3((float)vals[pos], p);
-#pragma unroll
-          for (int k = 0; k < PIECES; ++k) out[k][j] = p[k];
-        } else {
-          out[0][j] = (uint32_t)vals[pos];
-        }
-        ++pos;
-      }
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < PIECES; ++k)
-    *reinterpret_cast<uint4*>(dense + ((size_t)k * R + r) * ldp + (size_t)c8 * 8) =
-        make_uint4(out[k][0] | (out[k][1] << 16), out[k][2] | (out[k][3] << 16), out[k][4] | (out[k][5] << 16), out[k][6] | (out[k][7] << 16));
-}
-
 // ---- export / validate ---------------------------------------------------------------------------
 // row pointers, column indices (widened) and values of the live structure in one launch; any destination may be NULL
 template <typename V>
@@ -487,44 +440,6 @@ mst_status_t mst_build_csc(mst_layer* L, cudaStream_t s) {
 mst_status_t mst_ensure_csc(const mst_layer* L, cudaStream_t s) {
   if (L->csc_valid) return MST_OK;
   return mst_build_csc(const_cast<mst_layer*>(L), s);
-}
-
-// Dense image of W.M for the tensor-core kernels (see densify_from_bits), *ld elements between its rows.  Without value
-// tracking the image is rebuilt at every call anyway, so it lives in a per-device scratch buffer shared by all layers (no
-// per-layer memory; like the other scratch kinds, calls that use it must not overlap on the GPU).  With value tracking the
-// layer keeps its own image and reuses it until the mask or the values change.
-mst_status_t mst_densify(const mst_layer* L, cudaStream_t s, const uint16_t** image, int64_t* ld) {
-  const int c = L->cur;
-  const int ldp = (L->I + 7) & ~7;
-  *ld = ldp;
-  if (L->nnz == L->N && L->dtype == MST_BF16 && ldp == L->I) {  // every entry kept: the CSR values are the dense matrix
-    *image = (const uint16_t*)L->vals[c];
-    return MST_OK;
-  }
-  uint16_t* dst = nullptr;
-  if (L->track_values) {
-    MST_TRY(mst_alloc_dense(const_cast<mst_layer*>(L)));
-    dst = L->dense_w;
-    *image = dst;
-    if (L->dense_version == L->version && L->dense_epoch == L->values_epoch) return MST_OK;
-    L->dense_version = L->version;
-    L->dense_epoch = L->values_epoch;
-  } else {
-    void* ws = nullptr;
-    MST_TRY(mst_workspace_kind(MST_WS_IMAGE, mst_image_bytes(L), &ws));
-    dst = (uint16_t*)ws;
-    *image = dst;
-  }
-  const int64_t groups = (int64_t)L->O * (ldp / 8);
-  if (L->dtype == MST_F32)
-    MST_CUDA_TRY(mst_launch_overlapped(densify_from_bits<float>, dim3(blocks_for(groups, 256)), dim3(256), 0, s,
-                                       (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, ldp, L->wpr,
-                                       (const float*)L->vals[c], dst));
-  else
-    MST_CUDA_TRY(mst_launch_overlapped(densify_from_bits<uint16_t>, dim3(blocks_for(groups, 256)), dim3(256), 0, s,
-                                       (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, ldp, L->wpr,
-                                       (const uint16_t*)L->vals[c], dst));
-  return MST_OK;
 }
 
 // new mask of an update from the three selection results; leaves popcounts in word_cnt

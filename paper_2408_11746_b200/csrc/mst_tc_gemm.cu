@@ -850,14 +850,19 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
   if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
   const bool env = mst_env_any();
-  // Few tiles: compare one wave of this kernel (about 6000 clocks of fill, last epilogue and launch, 512 per k-block of a pair's
-  // tile, and for the gradients a second launch that adds the ranges) with the small-tile kernel's estimate.
+  // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate.  SM clocks, fitted like that one's: 10500 a
+  // launch and 537 per k-block of a pair's tile; the gradients' epilogue, which nothing overlaps in a single wave, 7500, and a
+  // second launch that adds the ranges 6000.
   if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
-      double here = 6000.0 + (double)kb * 512.0;
-      if (a.epilogue != MST_TC_OUT_BF16 && kb > 8 && tiles * 2 <= pairs) here = here / (double)(pairs / tiles) + 8000.0;
-      if (mst_tc_small_clocks(a) < 0.9 * here) return mst_tc_small(a, s);
+      double here = 10500.0 + (double)kb * 537.0;
+      if (a.epilogue != MST_TC_OUT_BF16) {
+        const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
+        const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes);
+        here = 18000.0 + (double)((kb + sp - 1) / sp) * 537.0 + (sp > 1 ? 6000.0 : 0.0);
+      }
+      if (mst_tc_small_clocks(a) < 0.95 * here) return mst_tc_small(a, s);
     }
   }
   CUtensorMap tmA, tmB;

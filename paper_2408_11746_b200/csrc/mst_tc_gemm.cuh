@@ -52,18 +52,12 @@ struct mst_tc_gemm_args {
   int64_t ldpre;
 };
 
-// C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_split_rows; lda / ldb are the pieces'
+// C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_prepare.cu; lda / ldb are the pieces'
 // leading dimensions, M / N / K the matrix sizes).  Epilogues F32 (rows) and SAMPLED.
 mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s);
 // The same kernel for bf16 operands and outputs of few tiles, all epilogues, and its estimated time in SM clocks
 mst_status_t mst_tc_small(const mst_tc_gemm_args& a, cudaStream_t s);
 double mst_tc_small_clocks(const mst_tc_gemm_args& a);
-// Operand preparation (leading dimension of the result: C rounded up to a multiple of 8):
-//   split_rows  fp32 [R x C] -> three bf16 pieces [3][R][ldp] whose sum is the operand
-//   pad_rows    bf16 [R x C] -> the same rows, 16-byte aligned
-mst_status_t mst_split_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s);
-mst_status_t mst_pad_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s);
-
 // forward product for at most MST_SMALL_FWD_TOKENS tokens (mst_small_fwd.cu)
 constexpr int64_t MST_SMALL_FWD_TOKENS = 16;
 mst_status_t mst_small_fwd(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,

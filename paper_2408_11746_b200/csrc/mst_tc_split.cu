@@ -25,7 +25,6 @@
 // warp 1 issues the MMAs, warps 2-9 own the sums (one row and BN / 2 columns per thread).  Every wait is bounded.
 #include <cuda.h>
 
-#include "mst_bits.cuh"
 #include "mst_internal.cuh"
 #include "mst_tc_gemm.cuh"
 #include "mst_tc_ptx.cuh"
@@ -327,62 +326,6 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   }
 }
 
-// ---- operand preparation -----------------------------------------------------------------------------------------------
-// 8 consecutive columns per thread.  fp32 rows -> three bf16 pieces [3][R][ldp]; bf16 rows -> the same rows at a leading
-// dimension and an address the TMA unit accepts.  Columns C .. ldp-1 become +0.  Memory-bound: 4 + 6 (2 + 2) bytes per
-// element.
-__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ in, int64_t ld, int64_t R, int C, int ldp,
-                                                         uint16_t* __restrict__ out, int vec_ok) {
-  mst_grid_launch_dependents();
-  mst_grid_dependency_wait();
-  const int gpr = ldp >> 3;
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= R * gpr) return;
-  const int64_t r = g / gpr;
-  const int c = (int)(g - r * gpr) * 8;
-  float x[8];
-  const float* src = in + r * ld + c;
-  if (vec_ok && c + 8 <= C) {
-    const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = c + j < C ? src[j] : 0.f;
-  }
-  constexpr int PIECES = 3;
-  uint32_t p[PIECES][4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    uint32_t lo[PIECES], hi[PIECES];
-    mst_split3(x[2 * j], lo);
-    mst_split3(x[2 * j + 1], hi);
-#pragma unroll
-    for (int k = 0; k < PIECES; ++k) p[k][j] = lo[k] | (hi[k] << 16);
-  }
-#pragma unroll
-  for (int k = 0; k < PIECES; ++k)
-    *reinterpret_cast<uint4*>(out + ((size_t)k * R + r) * ldp + c) = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
-}
-
-__global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restrict__ in, int64_t ld, int64_t R, int C, int ldp,
-                                                       uint16_t* __restrict__ out) {
-  mst_grid_launch_dependents();
-  mst_grid_dependency_wait();
-  const int gpr = ldp >> 3;
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= R * gpr) return;
-  const int64_t r = g / gpr;
-  const int c = (int)(g - r * gpr) * 8;
-  const uint16_t* src = in + r * ld + c;
-  uint32_t v[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t lo = c + 2 * j < C ? src[2 * j] : 0u, hi = c + 2 * j + 1 < C ? src[2 * j + 1] : 0u;
-    v[j] = lo | (hi << 16);
-  }
-  *reinterpret_cast<uint4*>(out + (size_t)r * ldp + c) = make_uint4(v[0], v[1], v[2], v[3]);
-}
-
 // pieces [1 or 3][rows][ld] as a 3-d map: rows and columns beyond the matrix read as zero inside every piece
 bool make_piece_map(CUtensorMap* tm, const void* base, int pieces, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
   mst_encode_tiled_fn fn = mst_encode_tiled();
@@ -404,23 +347,31 @@ mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
   return MST_OK;
 }
 
-// Tile width and number of K ranges from a time model in SM clocks.  Three pieces: 24 MMAs per k-block (64 clocks each at 128
-// columns, 40 at 64, where the A operand's shared-memory reads dominate).  One piece: its 24 KB of operands per k-block at the 54
-// bytes per clock that an SM gets from L2 (128 columns were no faster).  Both: about 4000 for launch, fill and drain of a block, and 1500 for the sums of a
-// cluster.
+// Tile width and number of K ranges from a time model in SM clocks.
+// Three pieces: 24 MMAs per k-block (64 clocks each at 128 columns, 40 at 64, where the A operand's shared-memory reads dominate),
+// about 4000 for launch, fill and drain of a block, and 1500 for the sums of a cluster.
+// One piece (64 columns; 128 were no faster), fitted to back-to-back calls of 64 to 4096 tokens on layers of 320 to 4096 features, at
+// 1.85 GHz: 9000 a launch, 555 per k-block (its 24 KB of operands), two blocks to an SM (clusters do not pack
+// that way: one); rows of bf16 4500 a wave, a further wave 10000, the sums of a cluster 1500 (5000 when the sampled rows are what the ranks divide).
 double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
   const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
   double best = 1e30;
-  *bn = 128;
+  *bn = pieces == 3 ? 128 : 64;
   *splits = 1;
   for (int w = 64; w <= (pieces == 3 ? 128 : 64); w += 64) {
     const int64_t tiles = m_tiles * ((a.N + w - 1) / w);
-    const double t_kb = pieces == 1 ? 450.0 : w == 64 ? 960.0 : 1536.0;
     for (int sp = 1; sp <= 8 && sp <= kblocks; sp *= 2) {   // cluster sizes
-      const int64_t waves = (tiles * sp + sms - 1) / sms;
       const int kb = (kblocks + sp - 1) / sp;
-      const double t = (double)waves * (kb * t_kb + 4000.0) + (sp > 1 ? 1500.0 : 0.0);
+      double t;
+      if (pieces == 3) {
+        const int64_t waves = (tiles * sp + sms - 1) / sms;
+        t = (double)waves * (kb * (w == 64 ? 960.0 : 1536.0) + 4000.0) + (sp > 1 ? 1500.0 : 0.0);
+      } else {
+        const int64_t slots = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + slots - 1) / slots;
+        const bool rows = a.epilogue == MST_TC_OUT_BF16;
+        t = 9000.0 + (double)waves * (kb * 555.0 + (rows ? 4500.0 : 0.0)) + (double)(waves - 1) * 10000.0 + (sp > 1 ? (rows ? 1500.0 : 5000.0) : 0.0);
+      }
       if (t < best * 0.97) { best = t; *bn = w; *splits = sp; }
     }
   }
@@ -456,23 +407,6 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
 }
 
 }  // namespace
-
-mst_status_t mst_split_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s) {
-  const int ldp = (C + 7) & ~7;
-  const int vec_ok = (ld % 4 == 0 && (reinterpret_cast<uintptr_t>(in) & 15u) == 0) ? 1 : 0;
-  const int64_t n = R * (ldp / 8);
-  MST_CUDA_TRY(mst_launch_overlapped(split_rows_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, (const float*)in, ld, R, C,
-                                     ldp, (uint16_t*)out, vec_ok));
-  return MST_OK;
-}
-
-mst_status_t mst_pad_rows(const void* in, int64_t ld, int64_t R, int C, void* out, cudaStream_t s) {
-  const int ldp = (C + 7) & ~7;
-  const int64_t n = R * (ldp / 8);
-  MST_CUDA_TRY(mst_launch_overlapped(pad_rows_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, (const uint16_t*)in, ld, R, C,
-                                     ldp, (uint16_t*)out));
-  return MST_OK;
-}
 
 mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s) {
   int bn, splits;
