@@ -44,6 +44,7 @@ struct Params {
   int kblocks;        // ceil(K / BK)
   int splits;
   int m_tiles, n_tiles;
+  uint32_t full, cut; // pair kernel: whole jobs, and how many each later one is cut into (rows: two halves; gradients: K ranges)
   int a_mn, b_mn;
   int epilogue;
   void* out;
@@ -154,7 +155,7 @@ __device__ __forceinline__ void act_chunk(const Params& P, uint32_t (&r)[32], ui
 // staging box, so that a store instruction writes 32 neighbours of one row; stores by the row-owning lanes touch 32 lines
 // each (2051 x 1999 bf16 outputs: 4.1 M two-byte stores to as many sectors).
 __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, uint32_t tmem_base, int acc, int q, int c0, int lane,
-                                              int64_t m0, int n0, int split) {
+                                              int64_t m0, int n0, int split, int cols) {
   const int64_t row0 = (int64_t)m0 + q * 32;
   const int64_t m = row0 + lane;
   const bool row_ok = m < P.M;
@@ -162,7 +163,7 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
   const uint32_t sw = (uint32_t)(lane & 7);
   const int rows = P.M - row0 < 32 ? (int)(P.M - row0) : 32;
 #pragma unroll 1
-  for (int c = c0; c < BN / 32; c += EPI_WARPS / 4) {
+  for (int c = c0; c < cols / 32; c += EPI_WARPS / 4) {
     const int n = n0 + c * 32;
     if (n >= P.N) break;  // uniform
     uint32_t r[32];
@@ -187,8 +188,8 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
     __syncwarp();
     const bool col_ok = n + lane < P.N;
     const bool bf16 = P.epilogue == MST_TC_OUT_BF16;
-    float* f32 = P.splits > 1 ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
-    const int64_t ld = bf16 || P.splits == 1 ? P.ldc : P.N;
+    float* f32 = P.partial ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
+    const int64_t ld = bf16 || !P.partial ? P.ldc : P.N;
 #pragma unroll 4
     for (int rr = 0; rr < rows; ++rr) {
       const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)(rr & 7);
@@ -208,13 +209,12 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
 // neighbours in CSR order; a row-per-lane store touches 32 lines per instruction and costs the memory pipeline as many
 // passes, which at high density slows the concurrent main loop.
 __device__ __forceinline__ void epilogue_tile_sampled(const Params& P, uint32_t stage, uint32_t tmem_base, int acc, int q,
-                                                      int c0, int lane, int64_t m0, int n0, int split) {
+                                                      int c0, int lane, int64_t m0, int n0, float* __restrict__ out) {
   const int64_t m = (int64_t)m0 + q * 32 + lane;
   const bool row_ok = m < P.M;
   const uint32_t my_row = stage + (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
   const uint32_t lt = (1u << lane) - 1u;
-  float* out = P.splits > 1 ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out);
 #pragma unroll 1
   for (int c = c0; c < BN / 32; c += EPI_WARPS / 4) {
     const int n = n0 + c * 32;
@@ -270,7 +270,7 @@ __device__ __forceinline__ void epilogue_tile_sampled(const Params& P, uint32_t 
 // K-range index as third coordinate.  Per-thread stores of a row-per-lane layout touch 32 lines per instruction and
 // were measured to slow the concurrent main loop by about 15 %.
 __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtensorMap* tmC, uint32_t stage, uint32_t tmem_base,
-                                                  int acc, int q, int c0, int lane, int64_t m0, int n0, int split) {
+                                                  int acc, int q, int c0, int lane, int64_t m0, int n0, int split, int cols) {
   const int64_t row0 = (int64_t)m0 + q * 32;
   const int64_t m = row0 + lane;
   const bool row_ok = m < P.M;
@@ -278,7 +278,7 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
   const uint32_t sw = (uint32_t)(lane & 7);
   if (P.epilogue == MST_TC_OUT_BF16) {
 #pragma unroll 1
-    for (int g = c0; g < BN / 64; g += EPI_WARPS / 4) {
+    for (int g = c0; g < cols / 64; g += EPI_WARPS / 4) {
       const int n = n0 + g * 64;
       if (n >= P.N) break;  // uniform
       if (lane == 0) bulk_wait_read();  // the box's previous contents have left shared memory
@@ -466,12 +466,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tc_fence_after();
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                          n0, split);
+                          n0, split, BN);
       else if (P.epilogue == MST_TC_OUT_SAMPLED)
         epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                              n0, split);
+                              n0, P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
       else
-        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
+        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, BN);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
@@ -506,6 +506,66 @@ constexpr int P_STAGES = 6;
 constexpr int PB_BYTES = (BN / 2) * BK * 2;        // this block's half of B: 16 KiB
 constexpr int P_STAGE_BYTES = A_BYTES + PB_BYTES;  // 32 KiB
 constexpr size_t P_SMEM_BYTES = (size_t)P_STAGES * P_STAGE_BYTES + EPI_WARPS * OUT_BOX_BYTES + 1024 + 256;
+// The jobs of a pair, one after the other: a tile's rows and columns over one K range.  Jobs beyond P.full, a last wave that would
+// leave at least half of the pairs idle, are cut into P.cut:
+//   products with the weights (rows of bf16)   two halves of the tile's columns; a tile whose columns end within its first half is
+//                                              half as wide in any case;
+//   gradients                                  parts of the job's K range, with sums (`split`) of their own.
+// (The k-blocks of all tiles shared out evenly were slower, 34 -> 40 us for 2304 x 768 at 8192 tokens and 108 -> 144 for 4096 x 1024
+// at 16384: pairs at different places of the K range read the activations at different times, and L2 does not hold them.)
+// One kernel serves all of these: a training step alternates between them, and a second instantiation cost every launch
+// about 2 us more.
+struct PairJobs {
+  uint32_t w, end, step, tiles;
+  int split, m0, n0, cols, kb0, kb1;
+  __device__ __forceinline__ PairJobs(const Params& P, uint32_t pair, uint32_t npairs) {
+    tiles = (uint32_t)((P.m_tiles + 1) / 2) * (uint32_t)P.n_tiles;
+    w = pair;
+    end = P.full + P.cut * (tiles * (uint32_t)P.splits - P.full);
+    step = npairs;
+    split = kb0 = 0;
+    kb1 = P.kblocks;
+  }
+  __device__ __forceinline__ bool next(const Params& P) {
+    while (w < end) {
+      uint32_t job = w, part = 0;
+      const bool cut = w >= P.full;
+      if (cut) {
+        const uint32_t k = w - P.full;
+        job = P.full + k / P.cut;
+        part = k - (job - P.full) * P.cut;
+      }
+      w += step;
+      uint32_t tile = job, range = 0;
+      if (job >= tiles) {
+        range = job / tiles;
+        tile = job - range * tiles;
+      }
+      const uint32_t row = tile / (uint32_t)P.n_tiles;
+      m0 = (int)row * (2 * BM);
+      n0 = (int)(tile - row * (uint32_t)P.n_tiles) * BN;
+      if (P.epilogue == MST_TC_OUT_BF16) {
+        n0 += (int)part * (BN / 2);
+        cols = cut || P.N - n0 <= BN / 2 ? BN / 2 : BN;
+        if (n0 >= P.N) continue;   // that half lies outside the output
+      } else {
+        cols = BN;
+        if (P.splits > 1 || cut) {
+          kb0 = (int)((int64_t)range * P.kblocks / P.splits);
+          kb1 = (int)((int64_t)(range + 1) * P.kblocks / P.splits);
+          split = (int)(range + part);
+          if (cut) {
+            const int n = kb1 - kb0, from = kb0;
+            kb0 = from + (int)((int64_t)part * n / P.cut);
+            kb1 = from + (int)((int64_t)(part + 1) * n / P.cut);
+          }
+        }
+      }
+      return true;
+    }
+    return false;
+  }
+};
 // shared::cluster address of the same shared-memory location in the even block (rank 0) of the pair
 __device__ __forceinline__ uint32_t in_even_block(uint32_t local_addr) {
   uint32_t r;
@@ -550,7 +610,7 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmC, const Params P) {
+                    const __grid_constant__ CUtensorMap tmBn, const __grid_constant__ CUtensorMap tmC, const Params P) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -590,35 +650,34 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
 
-  const int m_pairs = (P.m_tiles + 1) / 2;
-  const int tiles = m_pairs * P.n_tiles;
-  const int64_t works = (int64_t)tiles * P.splits;
-  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const uint32_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (both blocks)
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      for (int64_t w = pair; w < works && !*abort_flag; w += npairs) {
-        const int split = (int)(w / tiles), t = (int)(w % tiles);
-        const int m0 = (t / P.n_tiles) * (2 * BM) + (int)rank * BM;       // this block's rows
-        const int n0 = (t % P.n_tiles) * BN + (int)rank * (BN / 2);       // this block's half of B
-        const int kb0 = (int)((int64_t)split * P.kblocks / P.splits), kb1 = (int)((int64_t)(split + 1) * P.kblocks / P.splits);
+      PairJobs J(P, pair, npairs);
+      while (J.next(P) && !*abort_flag) {
+        const int m0 = J.m0 + (int)rank * BM;              // this block's rows
+        const int n0 = J.n0 + (int)rank * (J.cols / 2);    // this block's half of B
+        const uint32_t bytes = (uint32_t)(A_BYTES + J.cols / 2 * BK * 2);
+        const int kb0 = J.kb0, kb1 = J.kb1;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag)) break;
           const uint32_t fb = in_even_block(full0 + 8 * s);  // the even block's barrier collects both blocks' bytes
           const uint32_t sa = tiles_base + s * P_STAGE_BYTES, sb = sa + A_BYTES;
-          mbar_expect_tx_cluster(fb, P_STAGE_BYTES);
+          mbar_expect_tx_cluster(fb, bytes);
           if (P.a_mn) {
             for (int j = 0; j < BM / 64; ++j) tma_load_2d_pair(sa + j * BOX_BYTES, &tmA, m0 + j * 64, kb * BK, fb);
           } else {
             tma_load_2d_pair(sa, &tmA, kb * BK, m0, fb);
           }
           if (P.b_mn) {
-            for (int j = 0; j < BN / 128; ++j) tma_load_2d_pair(sb + j * BOX_BYTES, &tmB, n0 + j * 64, kb * BK, fb);
+            tma_load_2d_pair(sb, &tmB, n0, kb * BK, fb);
+            if (J.cols == BN) tma_load_2d_pair(sb + BOX_BYTES, &tmB, n0 + 64, kb * BK, fb);
           } else {
-            tma_load_2d_pair(sb, &tmB, kb * BK, n0, fb);
+            tma_load_2d_pair(sb, J.cols == BN ? &tmB : &tmBn, kb * BK, n0, fb);
           }
           if (++s == P_STAGES) { s = 0; ph ^= 1u; }
         }
@@ -627,18 +686,18 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (even block only)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
-                             ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) |
-                             ((uint32_t)((2 * BM) >> 4) << 24);
+      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
+                              ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)((2 * BM) >> 4) << 24);
       const uint64_t adesc0 = smem_desc(tiles_base, P.a_mn ? BOX_BYTES : 16, 1024);
       const uint64_t bdesc0 = smem_desc(tiles_base + A_BYTES, P.b_mn ? BOX_BYTES : 16, 1024);
       const uint32_t a_kstep = (uint32_t)(P.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
       const uint32_t b_kstep = (uint32_t)(P.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
-      for (int64_t w = pair; w < works && !*abort_flag; w += npairs) {
-        const int split = (int)(w / tiles);
-        const int kb0 = (int)((int64_t)split * P.kblocks / P.splits), kb1 = (int)((int64_t)(split + 1) * P.kblocks / P.splits);
+      PairJobs J(P, pair, npairs);
+      while (J.next(P) && !*abort_flag) {
+        const uint32_t idesc = idesc0 | ((uint32_t)(J.cols >> 3) << 17);
+        const int kb0 = J.kb0, kb1 = J.kb1;
         if (!mbar_wait(tempty0 + 8 * acc, acc_ph ^ 1u, abort_flag)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
@@ -666,19 +725,21 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool use_tma = P.tma_out && P.epilogue != MST_TC_OUT_SAMPLED;
     int acc = 0;
     uint32_t acc_ph = 0;
-    for (int64_t w = pair; w < works; w += npairs) {
-      const int split = (int)(w / tiles), t = (int)(w % tiles);
-      const int m0 = (t / P.n_tiles) * (2 * BM) + (int)rank * BM, n0 = (t % P.n_tiles) * BN;
+    PairJobs J(P, pair, npairs);
+    while (J.next(P)) {
+      const int m0 = J.m0 + (int)rank * BM, n0 = J.n0;
+      const int split = J.split;
+      float* sampled = P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out);
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                          n0, split);
+                          n0, split, J.cols);
       else if (P.epilogue == MST_TC_OUT_SAMPLED)
         epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                              n0, split);
+                              n0, sampled);
       else
-        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split);
+        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, J.cols);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(in_even_block(tempty0 + 8 * acc));
@@ -723,6 +784,39 @@ __global__ void tc_reduce4_kernel(const float4* __restrict__ partial, int splits
     s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
   }
   out[i] = s;
+}
+
+// The same where the last jobs were cut, so that tiles have different numbers of sums: a warp per row of a tile.  Sampled output: the
+// row's kept entries are one run.
+__global__ void __launch_bounds__(256) tc_reduce_tiles_kernel(const Params P) {
+  mst_grid_launch_dependents();
+  mst_grid_dependency_wait();
+  const int lane = threadIdx.x & 31;
+  const int64_t m = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int g = blockIdx.y;
+  if (m >= P.M) return;
+  const uint32_t tiles = (uint32_t)((P.m_tiles + 1) / 2) * (uint32_t)P.n_tiles, t = (uint32_t)(m / (2 * BM)) * (uint32_t)P.n_tiles + (uint32_t)g;
+  const int sums = P.splits + (t + (uint32_t)(P.splits - 1) * tiles >= P.full ? (int)P.cut - 1 : 0);
+  int64_t first, last, slab;
+  const float* in = P.partial;
+  float* out = reinterpret_cast<float*>(P.out);
+  if (P.epilogue == MST_TC_OUT_SAMPLED) {
+    const int64_t w0 = m * P.wpr + g * (BN / 32);
+    first = P.wscan[w0];
+    last = P.wscan[(g + 1) * (BN / 32) < P.wpr ? w0 + BN / 32 : (m + 1) * P.wpr];
+    slab = P.nnz;
+  } else {
+    first = (int64_t)g * BN;
+    last = first + BN < P.N ? first + BN : P.N;
+    slab = P.M * P.N;
+    in += m * P.N;
+    out += m * P.ldc;
+  }
+  for (int64_t e = first + lane; e < last; e += 32) {
+    float v = in[e];
+    for (int k = 1; k < sums; ++k) v += in[k * slab + e];
+    out[e] = v;
+  }
 }
 
 // ------------------------------------------------------------------------------------------- host side
@@ -787,22 +881,35 @@ int mst_sm_count() {
   return n[dev];
 }
 
-// Number of K ranges for a contraction whose output has few tiles: minimise a simple time model
+// Number of K ranges for a contraction whose output has few tiles, and into how many parts (*cut, 1: none) the jobs of a last wave
+// that would leave half of the slots idle are cut when there is one range (cutting the last of several ranges lost: 2304 x 768
+// at 8192 tokens 34 -> 41 us, 1280 x 1280 at 16384 70 -> 84): minimise a simple time model
 //   waves * (k-blocks per range * t_kblock + t_tile) + traffic of the partial sums
-// over 1..16 ranges.  `works1` = tile jobs with one range, `slots` = jobs that run at once (blocks or block pairs),
-// `out_bytes` = bytes one range writes as partial sums (and the reduction reads back).
-int mst_tc_pick_splits(int64_t works1, int64_t slots, int64_t kblocks, double out_bytes) {
+// over 1..16 ranges.  `tiles` of the output, `slots` = jobs that run at once (blocks or block pairs), `out_bytes` = bytes one range
+// writes as partial sums (and the reduction reads back).  75 tiles on 74 pairs (3840 x 1280, 16384
+// tokens, d = 0.5) are one wave and a sixteenth, 171 us; without the cut they were three waves of two ranges, 185 us.
+int mst_tc_pick_splits(int64_t tiles, int64_t slots, int64_t kblocks, double out_bytes, int* cut) {
   const double t_kblock = 0.32e-6, t_tile = 1.5e-6, bw = 4.0e12, t_reduce_launch = 3.0e-6;
   int best = 1;
   double best_t = 1e30;
+  *cut = 1;
   for (int sp = 1; sp <= 16 && sp <= kblocks; ++sp) {
-    const int64_t waves = (works1 * sp + slots - 1) / slots;
+    const int64_t jobs = tiles * sp, rest = jobs % slots, waves = (jobs + slots - 1) / slots;
     const double kb = (double)((kblocks + sp - 1) / sp);
     double t = (double)waves * (kb * t_kblock + t_tile);
     if (sp > 1) t += t_reduce_launch + (double)sp * out_bytes * 2.0 / bw;
+    int c = 1;
+    if (sp == 1 && rest > 0 && jobs > slots && rest * 2 <= slots) {
+      int parts = (int)(slots / rest < 16 ? slots / rest : 16);
+      while (parts > 1 && kb / parts < 4.0) --parts;
+      const double sums = 1.0 + (double)rest * (parts - 1) / (double)tiles;
+      const double tc = (double)(waves - 1) * (kb * t_kblock + t_tile) + kb / parts * t_kblock + 3.0 * t_tile + t_reduce_launch + sums * out_bytes * 2.0 / bw;
+      if (parts > 1 && tc < t * 0.95) { t = tc; c = parts; }
+    }
     if (t < best_t * 0.97) {  // prefer fewer ranges unless the gain is clear
       best_t = t;
       best = sp;
+      *cut = c;
     }
   }
   return best;
@@ -859,8 +966,10 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       double here = 10500.0 + (double)kb * 537.0;
       if (a.epilogue != MST_TC_OUT_BF16) {
         const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
-        const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes);
+        int cut;
+        const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes, &cut);
         here = 18000.0 + (double)((kb + sp - 1) / sp) * 537.0 + (sp > 1 ? 6000.0 : 0.0);
+        if (cut > 1) here += (double)((kb + sp - 1) / sp / cut) * 537.0 + 3000.0;
       }
       if (mst_tc_small_clocks(a) < 0.95 * here) return mst_tc_small(a, s);
     }
@@ -879,6 +988,8 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   P.N = a.N;
   P.kblocks = (int)((a.K + BK - 1) / BK);
   P.splits = 1;
+  P.cut = 1;
+  int sums = 1;   // partial sums kept for one output at most
   P.m_tiles = (int)((a.M + BM - 1) / BM);
   P.n_tiles = (int)((a.N + BN - 1) / BN);
   P.a_mn = a.a_mn_major;
@@ -902,16 +1013,19 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
     const int64_t works1 = pair ? (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles : (int64_t)P.m_tiles * P.n_tiles;
     const int64_t slots = pair ? mst_sm_count() / 2 : mst_sm_count();
     const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
-    P.splits = a.splits > 0 ? a.splits : mst_tc_pick_splits(works1, slots, P.kblocks, out_bytes);
+    int cut = 1;
+    P.splits = a.splits > 0 ? a.splits : mst_tc_pick_splits(works1, slots, P.kblocks, out_bytes, &cut);
     if (const char* e = mst_getenv(env, "MST_TC_SPLITS")) {  // measurement override
       const int v = atoi(e);
-      if (v > 0) P.splits = v;
+      if (v > 0) { P.splits = v; cut = 1; }
     }
     if (P.splits > P.kblocks) P.splits = P.kblocks;
-    if (P.splits > 1) {
+    if (pair) P.cut = (uint32_t)cut;
+    sums = P.splits + (int)P.cut - 1;
+    if (sums > 1) {
       const size_t per = a.epilogue == MST_TC_OUT_F32 ? (size_t)a.M * a.N : (size_t)a.nnz;
       void* ws = nullptr;
-      MST_TRY(mst_workspace(sizeof(float) * per * P.splits, &ws));
+      MST_TRY(mst_workspace(sizeof(float) * per * sums, &ws));
       P.partial = (float*)ws;
     }
   }
@@ -921,7 +1035,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.epilogue == MST_TC_OUT_BF16) {
     P.tma_out = make_out_map_bf16(&tmC, a.out, a.M, a.N, a.ldc) ? 1 : 0;
   } else if (a.epilogue == MST_TC_OUT_F32) {
-    P.tma_out = (P.splits > 1 ? make_out_map_f32(&tmC, P.partial, a.M, a.N, a.N, a.M * a.N, P.splits)
+    P.tma_out = (sums > 1 ? make_out_map_f32(&tmC, P.partial, a.M, a.N, a.N, a.M * a.N, sums)
                               : make_out_map_f32(&tmC, a.out, a.M, a.N, a.ldc, a.M * a.ldc, 1))
                     ? 1
                     : 0;
@@ -930,11 +1044,19 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
     if (e[0] == '0') P.tma_out = 0;
   }
   if (pair) {
+    const int64_t jobs = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits, max_pairs = mst_sm_count() / 2, rest = jobs % max_pairs;
+    CUtensorMap tmBn = tmB;
+    if (a.epilogue == MST_TC_OUT_BF16) {
+      // half-wide tiles take about 0.62 of a full one (at most twice as many blocks share the L2 bandwidth that bounds them)
+      if (rest * 2 <= max_pairs) P.cut = 2;
+      if (!a.b_mn_major && !make_map(&tmBn, a.B, a.N, a.K, a.ldb, BN / 4)) return MST_ERR_SHAPE;
+    }
+    P.full = (uint32_t)(P.cut > 1 ? jobs - rest : jobs);
+    const int64_t works = (int64_t)P.full + (int64_t)P.cut * (jobs - (int64_t)P.full);
+    if (works > 0x7FFFFFFF) return MST_ERR_SHAPE;
     MST_SMEM_LIMIT((tc_gemm_pair_kernel), P_SMEM_BYTES);
-    const int64_t works = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits;
-    const int64_t max_pairs = mst_sm_count() / 2;
-    const int grid = 2 * (int)(works < max_pairs ? works : max_pairs);
-    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel, dim3(grid), dim3(NUM_THREADS), P_SMEM_BYTES, s, tmA, tmB, tmC, P));
+    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel, dim3(2 * (unsigned)(works < max_pairs ? works : max_pairs)), dim3(NUM_THREADS),
+                                       P_SMEM_BYTES, s, tmA, tmB, tmBn, tmC, P));
   } else {
     MST_SMEM_LIMIT((tc_gemm_kernel), SMEM_BYTES);
     const int64_t works = (int64_t)P.m_tiles * P.n_tiles * P.splits;
@@ -942,7 +1064,9 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
     MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_kernel, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, s, tmA, tmB, tmC, P));
   }
   MST_CUDA_TRY(cudaGetLastError());
-  if (P.splits > 1) {
+  if (pair && P.cut > 1 && sums > 1) {
+    MST_CUDA_TRY(mst_launch_overlapped(tc_reduce_tiles_kernel, dim3((unsigned)((P.M + 7) / 8), (unsigned)P.n_tiles), dim3(256), 0, s, P));
+  } else if (P.splits > 1) {
     const int64_t n = a.epilogue == MST_TC_OUT_F32 ? a.M * a.N : a.nnz;
     if (n > 0 && (n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0)
       MST_CUDA_TRY(mst_launch_overlapped(tc_reduce4_kernel, dim3((unsigned)((n / 4 + 255) / 256)), dim3(256), 0, s,

@@ -80,7 +80,7 @@ typedef CUresult (*mst_encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuin
 mst_encode_tiled_fn mst_encode_tiled();
 int mst_sm_count();
 
-int mst_tc_pick_splits(int64_t works1, int64_t slots, int64_t kblocks, double out_bytes);
+int mst_tc_pick_splits(int64_t tiles, int64_t slots, int64_t kblocks, double out_bytes, int* cut);
 
 // Process-wide scratch buffer for handle-less entry points (grows on demand; growing synchronises the device).
 // Calls that use it must not overlap on the GPU.

@@ -76,3 +76,24 @@ def test_bf16_products_of_few_tiles(O, I, T):
     # the latency kernel up to 16 tokens, small tiles with the contraction range split over a cluster above
     y, dx, dw, g = _layer_case(O, I, T, "bf16", 0.2, O + I + T)
     assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
+
+
+@pytest.mark.parametrize("O,I,T,density", [
+    (5120, 1280, 8190, 0.1),     # 100 tiles on 74 pairs: 26 cut in two
+    (3840, 1250, 8000, 0.3),     # 75 tiles: one cut, the others whole; ragged columns
+    (1300, 1290, 9000, 0.1)])    # ragged rows and columns, nothing cut
+def test_gradients_with_a_cut_last_wave(O, I, T, density):
+    g = torch.Generator(device="cuda").manual_seed(O + I)
+    mask = (torch.rand((O, I), device="cuda", generator=g) < density).to(torch.uint8)
+    L = mst.Layer(0, O, I, mst.MST_BF16)
+    L.pack(torch.ones((O, I), dtype=torch.bfloat16, device="cuda"), mask)
+    dY = torch.randn((T, O), device="cuda", generator=g).bfloat16()
+    X = torch.randn((T, I), device="cuda", generator=g).bfloat16()
+    dW = torch.full((L.nnz,), float("nan"), device="cuda")
+    G = torch.full((O, I), float("nan"), device="cuda")
+    L.sddmm(dY, X, T, dW)
+    L.dense_grad(dY, X, T, G)
+    ref = dY.double().t() @ X.double()
+    for got, want in ((dW.double(), ref[mask.bool()]), (G.double(), ref)):
+        assert float((got - want).norm() / want.norm()) < 1e-5
+    assert mst.mst_device_error_flags() == 0
