@@ -89,7 +89,7 @@ static_assert(ROWS * LDF * 4 <= RING_BYTES, "staged sums must fit the ring");
 static_assert(ROWS * LDO * 2 <= 4 * TILE_BYTES, "staged results must fit the own tiles");
 
 __device__ __forceinline__ bool wait_on(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return mbar_wait_suspended(bar, parity, abort_flag, &g_bwd_error);
+  return mbar_wait(bar, parity, abort_flag, &g_bwd_error);
 }
 
 __device__ __forceinline__ uint32_t block_setup(const Smem& S, uint32_t* holder, int* abort_sh, int warp) {
@@ -143,24 +143,12 @@ __device__ __forceinline__ void feed(const Smem& S, const W& walk, const CUtenso
     tma_load_2d(S.own0 + t * TILE_BYTES, own_a, col, row0 + walk.r0 + t * TS, S.own_full);
     tma_load_2d(S.own1 + t * TILE_BYTES, own_b, col, row0 + walk.r0 + t * TS, S.own_full);
   }
-  int s = 0;
-  uint32_t lap = 0;
-  for (int j = 0; j < walk.total; ++j) {
-    // what the stage held one lap ago: a near tile is given back by the second products' commit, a far one by its four warps
-    const int before = j - STAGES;
-    if (before >= 0) {
-      const bool far = before >= walk.near;
-      const uint32_t use = far ? (uint32_t)((before - walk.near) / STAGES) : lap - 1;
-      if (!wait_on((far ? S.far_done : S.empty) + 8 * s, use & 1u, abort_flag)) return;
-    }
-    const int at = walk.start(j);
-    const uint32_t bar = S.full + 8 * s, dst = S.ring + s * 2 * TILE_BYTES;
+  feed_ring<STAGES>(walk, S.ring, S.full, S.empty, S.far_done, [&](int s, int at, uint32_t dst, uint32_t bar) {
     mbar_expect_tx(bar, 2 * TILE_BYTES + (stat ? STAT_BYTES : 0));
     tma_load_2d(dst, tile_a, col, row0 + at, bar);
     tma_load_2d(dst + TILE_BYTES, tile_b, col, row0 + at, bar);
     if (stat) bulk_load(S.stat + s * STAT_BYTES, stat + 2 * at, STAT_BYTES, bar);
-    if (++s == STAGES) { s = 0; ++lap; }
-  }
+  }, [&](uint32_t bar, uint32_t parity) { return wait_on(bar, parity, abort_flag); });
 }
 
 // ------------------------------------------------------------------------------------------- dQ

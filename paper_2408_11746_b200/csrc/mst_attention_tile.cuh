@@ -118,7 +118,7 @@ __device__ __forceinline__ void mma_weights(uint32_t tmem_d, uint32_t tmem_a, ui
   for (int ks = 0; ks < TS / 16; ++ks)
     tc_mma_ts(tmem_d, tmem_a + (uint32_t)ks * apart, tile + (uint64_t)(ks * ((16 * 128) >> 4)), IDESC_MN, ks > 0 ? 1u : accum);
 }
-// sixteen fp32 columns of this warp's 32 lanes, and eight packed ones back
+// sixteen fp32 columns of this warp's 32 lanes, and sixteen or eight packed ones back
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -134,6 +134,14 @@ __device__ __forceinline__ void tmem_ld16_wait(uint32_t (&r)[16]) {
                  "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                :
                : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]),
+      "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]),
+      "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+      : "memory");
 }
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]),
@@ -189,6 +197,24 @@ struct Walk {
   }
   __device__ __forceinline__ int start(int j) const { return j < near ? first + j * TS : far_start(j - near); }
 };
+
+// The lane that feeds the ring.  A stage is given back by the commit behind the products of a near tile, or by the four warps that
+// a far tile concerns (a barrier of its own: those warps cannot come to it again before the stage has been filled again).
+template <int STAGES, typename W, typename Load, typename Wait>
+__device__ __forceinline__ void feed_ring(const W& walk, uint32_t ring, uint32_t full, uint32_t empty, uint32_t far_done, Load load, Wait wait) {
+  int s = 0;
+  uint32_t lap = 0;
+  for (int j = 0; j < walk.total; ++j) {
+    const int before = j - STAGES;   // what the stage held one lap ago
+    if (before >= 0) {
+      const bool far = before >= walk.near;
+      const uint32_t use = far ? (uint32_t)((before - walk.near) / STAGES) : lap - 1;
+      if (!wait((far ? far_done : empty) + 8 * s, use & 1u)) return;
+    }
+    load(s, walk.start(j), ring + (uint32_t)(s * 2 * TILE_BYTES), full + 8 * s);
+    if (++s == STAGES) { s = 0; ++lap; }
+  }
+}
 
 // ---------------------------------------------------------------------------------------------- warp-level products (far tiles)
 // mma.sync m16n8k16 with the published fragment layouts: with g = lane / 4 and t = lane % 4, an accumulator tile (16 x 8) holds

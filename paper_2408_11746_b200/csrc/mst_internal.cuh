@@ -216,10 +216,6 @@ mst_status_t mst_prepare(mst_dtype_t dtype, const mst_image_job* image, const ms
 static inline size_t mst_image_bytes(const mst_layer* L) {
   return (L->dtype == MST_F32 ? 6 : 2) * (size_t)L->O * (size_t)mst_row_pitch(L->I);
 }
-// strided attention forward on warp-level products (mst_attention_fwd_mma.cu); the caller has checked pointers and
-// leading dimensions
-mst_status_t mst_attention_fwd_mma(const void* Q, const void* K, const void* V, int64_t ld, int32_t batch, int32_t seq_len,
-                                   int32_t heads, int32_t stride, void* Out, int64_t ldo, float* lse, cudaStream_t s);
 bool mst_use_tensor_path(const mst_layer* L);
 bool mst_use_split_path(const mst_layer* L);
 bool mst_use_csc(const mst_layer* L);   // the input gradient walks the CSC view (CUDA-core kernels)
