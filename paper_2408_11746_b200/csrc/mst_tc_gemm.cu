@@ -203,29 +203,41 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
   }
 }
 
-// The sampled accumulator (weight gradient under the mask).  A chunk is 32 rows x one mask word.  Chunks with few
-// entries are written by the row-owning lanes, entry by entry.  Denser chunks leave through the warp's staging box:
-// the lanes turn from rows to columns, so that each store instruction writes the kept entries of ONE row, which are
-// neighbours in CSR order; a row-per-lane store touches 32 lines per instruction and costs the memory pipeline as many
-// passes, which at high density slows the concurrent main loop.
-__device__ __forceinline__ void epilogue_tile_sampled(const Params& P, uint32_t stage, uint32_t tmem_base, int acc, int q,
-                                                      int c0, int lane, int64_t m0, int n0, float* __restrict__ out) {
-  const int64_t m = (int64_t)m0 + q * 32 + lane;
-  const bool row_ok = m < P.M;
+// The sampled accumulator (weight gradient under the mask).  A chunk is 32 rows x one mask word; a warp's four chunks' words and
+// CSR positions are fetched while the products still run (a wave's last tile has nothing else to hide them behind).  Chunks with
+// few entries are written by the row-owning lanes, entry by entry.  Denser chunks turn from rows to columns through the warp's
+// staging box, so that each store instruction writes the kept entries of ONE row, which are neighbours in CSR order; all 32 rows
+// are read back before the first is stored, or every row would wait for its own round trip.
+constexpr int SAMPLED_CHUNKS = BN / 32 / (EPI_WARPS / 4);
+struct SampledWords {
+  uint32_t word[SAMPLED_CHUNKS];
+  int32_t at[SAMPLED_CHUNKS];
+  __device__ __forceinline__ SampledWords(const Params& P, int q, int c0, int lane, int64_t m0, int n0) {
+    const int64_t m = m0 + q * 32 + lane;
+#pragma unroll
+    for (int k = 0; k < SAMPLED_CHUNKS; ++k) {
+      const int n = n0 + (c0 + k * (EPI_WARPS / 4)) * 32;
+      word[k] = 0;
+      at[k] = 0;
+      if (m < P.M && n < P.N) {
+        const int64_t wi = m * P.wpr + (n >> 5);
+        word[k] = __ldg(P.bits + wi);
+        at[k] = __ldg(P.wscan + wi);
+      }
+    }
+  }
+};
+__device__ __forceinline__ void epilogue_tile_sampled(const Params& P, const SampledWords& W, uint32_t stage, uint32_t tmem_base, int acc,
+                                                      int q, int c0, int lane, int n0, float* __restrict__ out) {
   const uint32_t my_row = stage + (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
   const uint32_t lt = (1u << lane) - 1u;
-#pragma unroll 1
-  for (int c = c0; c < BN / 32; c += EPI_WARPS / 4) {
-    const int n = n0 + c * 32;
-    if (n >= P.N) break;  // uniform
-    uint32_t word = 0;
-    int32_t at = 0;
-    if (row_ok) {
-      const int64_t wi = m * P.wpr + (n >> 5);
-      word = P.bits[wi];
-      at = P.wscan[wi];
-    }
+#pragma unroll
+  for (int k = 0; k < SAMPLED_CHUNKS; ++k) {
+    const int c = c0 + k * (EPI_WARPS / 4);
+    if (n0 + c * 32 >= P.N) break;  // uniform
+    const uint32_t word = W.word[k];
+    const int32_t at = W.at[k];
     uint32_t r[32];
     tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
     const int kept = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
@@ -250,15 +262,16 @@ __device__ __forceinline__ void epilogue_tile_sampled(const Params& P, uint32_t 
                    : "memory");
     }
     __syncwarp();
-#pragma unroll 4
+#pragma unroll
+    for (int rr = 0; rr < 32; ++rr) {
+      const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)(rr & 7);
+      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(r[rr]) : "r"(stage + (uint32_t)rr * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
+    }
+#pragma unroll
     for (int rr = 0; rr < 32; ++rr) {
       const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, rr);
       const int32_t base = __shfl_sync(0xFFFFFFFFu, at, rr);
-      if (w == 0) continue;  // uniform
-      const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)(rr & 7);
-      uint32_t v;
-      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(stage + (uint32_t)rr * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
-      if ((w >> lane) & 1u) out[base + __popc(w & lt)] = __uint_as_float(v);
+      if ((w >> lane) & 1u) out[base + __popc(w & lt)] = __uint_as_float(r[rr]);
     }
   }
 }
@@ -462,14 +475,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int64_t w = blockIdx.x; w < works; w += gridDim.x) {
       const int split = (int)(w / tiles), t = (int)(w % tiles);
       const int m0 = (t / P.n_tiles) * BM, n0 = (t % P.n_tiles) * BN;
+      if (P.epilogue == MST_TC_OUT_SAMPLED) {
+        const SampledWords W(P, q, (warp - 2) >> 2, lane, m0, n0);
+        if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
+        tc_fence_after();
+        epilogue_tile_sampled(P, W, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, n0,
+                              P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
+        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+        continue;
+      }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                           n0, split, BN);
-      else if (P.epilogue == MST_TC_OUT_SAMPLED)
-        epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                              n0, P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
       else
         epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, BN);
       tc_fence_before();
@@ -636,6 +658,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 0 && lane < 4)   // the maps are parameters: fetched while the predecessor drains
+    asm volatile("prefetch.tensormap [%0];" ::"l"(lane == 0 ? &tmA : lane == 1 ? &tmB : lane == 2 ? &tmBn : &tmC) : "memory");
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
                  "r"(TMEM_COLS)
@@ -729,15 +753,23 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     while (J.next(P)) {
       const int m0 = J.m0 + (int)rank * BM, n0 = J.n0;
       const int split = J.split;
-      float* sampled = P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out);
+      if (P.epilogue == MST_TC_OUT_SAMPLED) {
+        const SampledWords W(P, q, (warp - 2) >> 2, lane, m0, n0);
+        if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
+        tc_fence_after();
+        epilogue_tile_sampled(P, W, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, n0,
+                              P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(in_even_block(tempty0 + 8 * acc));
+        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+        continue;
+      }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                           n0, split, J.cols);
-      else if (P.epilogue == MST_TC_OUT_SAMPLED)
-        epilogue_tile_sampled(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                              n0, sampled);
       else
         epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, J.cols);
       tc_fence_before();
@@ -1006,7 +1038,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   P.pre = a.pre;
   P.ldpre = a.ldpre;
   if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
-  P.sampled_stage_min = 384;  // measured: row-by-row stores pay from a density of about 0.4
+  P.sampled_stage_min = 192;  // d of about 0.19; 8192 tokens, 768 x 768: entry by entry 15.5 / 16.6 / 19.3 / 24 us at d = 0.1 / 0.15 / 0.25 / 0.5, row by row 17.0 / 17.0 / 17.2 / 18.3
   if (const char* e = mst_getenv(env, "MST_TC_SAMPLED_STAGE")) P.sampled_stage_min = atoi(e);  // measurement override
   if (a.epilogue != MST_TC_OUT_BF16) {
     // few output tiles: cut the contraction range so that all SMs work; partial sums go to the shared scratch buffer
