@@ -190,15 +190,38 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
     const bool bf16 = P.epilogue == MST_TC_OUT_BF16;
     float* f32 = P.partial ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
     const int64_t ld = bf16 || !P.partial ? P.ldc : P.N;
-#pragma unroll 4
-    for (int rr = 0; rr < rows; ++rr) {
-      const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)(rr & 7);
-      float v;
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(stage + (uint32_t)rr * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
-      const int64_t at = (row0 + rr) * ld + n + lane;
-      if (!col_ok) continue;
-      if (bf16) reinterpret_cast<uint16_t*>(P.out)[at] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
-      else f32[at] = v;
+    // A square inside the output is stored without a test per row (the branches and 64-bit addresses cost four times the stores).
+    const bool inside = rows == 32 && n + 32 <= P.N;
+    const int64_t at0 = row0 * ld + n + lane;
+#pragma unroll 1
+    for (int r8 = 0; r8 < rows; r8 += 8) {
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {   // eight rows are read back before the first is stored
+        const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)k;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[k]) : "r"(stage + (uint32_t)(r8 + k) * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
+      }
+      if (bf16) {
+        uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + at0 + r8 * ld;
+        if (inside) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) out[k * ld] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
+        } else if (col_ok) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (r8 + k < rows) out[k * ld] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
+        }
+      } else {
+        float* out = f32 + at0 + r8 * ld;
+        if (inside) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) out[k * ld] = v[k];
+        } else if (col_ok) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (r8 + k < rows) out[k * ld] = v[k];
+        }
+      }
     }
   }
 }

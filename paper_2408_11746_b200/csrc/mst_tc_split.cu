@@ -84,6 +84,48 @@ __device__ __forceinline__ void split_cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Sums of a 32-column square over the 2^LG blocks of the cluster, this block's 32 / 2^LG rows from rr0 on, into the warp's box: a
+// lane adds four columns of some rows, eight reads whatever the number of blocks, all in flight together, added in range order.
+template <int LG>
+__device__ __forceinline__ void gather_sums(uint32_t sums, int rr0, float* box, int lane) {
+  float4 x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int i = lane + 32 * (j >> LG), row = rr0 + (i >> 3);
+    uint32_t peer;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(sums + (uint32_t)((i & 7) * 32 + row) * 16u), "r"(j & ((1 << LG) - 1)));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[j].x), "=f"(x[j].y), "=f"(x[j].z), "=f"(x[j].w) : "r"(peer) : "memory");
+  }
+#pragma unroll
+  for (int j = 0; j < 8; j += 1 << LG) {
+    float4 sum = x[j];
+#pragma unroll
+    for (int k = 1; k < 1 << LG; ++k) { sum.x += x[j + k].x; sum.y += x[j + k].y; sum.z += x[j + k].z; sum.w += x[j + k].w; }
+    const int i = lane + 32 * (j >> LG);
+    float* d = box + (rr0 + (i >> 3)) * 33 + 4 * (i & 7);
+    d[0] = sum.x; d[1] = sum.y; d[2] = sum.z; d[3] = sum.w;
+  }
+}
+
+// Rows rr0 .. rr1 - 1 (a multiple of four) of the warp's box, four at a time: read back together, then handed on one by one.  `inside`
+// (uniform): the square lies inside the output, so nothing is tested - a test per store, with its branch and its 64-bit address, made
+// 64 KB of stores take 8000 clocks instead of 2200.
+template <typename Store>
+__device__ __forceinline__ void box_rows(const float* box, int rr0, int rr1, bool inside, int64_t rows_left, bool col_ok, int lane, Store store) {
+  if (inside) {
+#pragma unroll 2
+    for (int r = rr0; r < rr1; r += 4) {
+      float v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = box[(r + k) * 33 + lane];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) store(r + k, v[k]);
+    }
+  } else if (col_ok) {
+    for (int r = rr0; r < rr1 && r < rows_left; ++r) store(r, box[r * 33 + lane]);
+  }
+}
+
 template <int BN, int PIECES>
 __global__ void __launch_bounds__(S_THREADS, PIECES == 1 ? 2 : 1)
 tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
@@ -247,26 +289,16 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (n >= P.N) break;   // uniform
         __syncwarp();
         if (P.splits > 1) {
-          for (int i = lane; i < 8 * (rr1 - rr0); i += 32) {   // four columns of one row
-            const int v = i & 7, row = rr0 + (i >> 3);
-            const uint32_t at = part - (uint32_t)lane * 16u + (uint32_t)((g * 8 + v) * 32 + row) * 16u;
-            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int sp = 0; sp < P.splits; ++sp) {
-              uint32_t peer;
-              float4 x;
-              asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(sp));
-              asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(peer) : "memory");
-              sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
-            }
-            float* d = box + row * 33 + 4 * v;
-            d[0] = sum.x; d[1] = sum.y; d[2] = sum.z; d[3] = sum.w;
-          }
+          if (P.splits == 2) gather_sums<1>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
+          else if (P.splits == 4) gather_sums<2>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
+          else gather_sums<3>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) box[lane * 33 + j] = acc[g * 32 + j];
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
+        const bool inside = row0 + 32 <= P.M && n + 32 <= P.N, col_ok = n + lane < P.N;
         if (P.epilogue == MST_TC_OUT_SAMPLED) {
           uint32_t word = 0;
           int32_t at = 0;
@@ -275,37 +307,31 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             word = P.bits[wi];
             at = P.wscan[wi];
           }
-#pragma unroll 4
-          for (int rr = rr0; rr < rr1; ++rr) {
+          float* out = reinterpret_cast<float*>(P.out);
+          box_rows(box, rr0, rr1, true, 0, true, lane, [&](int rr, float v) {   // words beyond the matrix are empty
             const uint32_t w = __shfl_sync(0xffffffffu, word, rr);
             const int32_t base = __shfl_sync(0xffffffffu, at, rr);
-            if ((w >> lane) & 1u) reinterpret_cast<float*>(P.out)[base + __popc(w & lt)] = box[rr * 33 + lane];
-          }
+            if ((w >> lane) & 1u) out[base + __popc(w & lt)] = v;
+          });
         } else if (PIECES == 1 && P.epilogue == MST_TC_OUT_BF16) {
-          const bool col_ok = n + lane < P.N;
-          uint16_t* out = reinterpret_cast<uint16_t*>(P.out);
-#pragma unroll 4
-          for (int rr = rr0; rr < rr1; ++rr) {
-            if (row0 + rr >= P.M) break;  // uniform
-            if (!col_ok) continue;
-            float v = box[rr * 33 + lane];
-            uint16_t* pre = P.pre + (row0 + rr) * P.ldpre + n + lane;
-            if (P.act == MST_ACT_GELU) {
-              if (P.pre) *pre = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
-              v = mst_gelu(v);
-            } else if (P.act == MST_ACT_GELU_GRAD) {
-              v *= mst_gelu_grad(__uint_as_float((uint32_t)*pre << 16));
-            }
-            out[(row0 + rr) * P.ldc + n + lane] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
-          }
+          uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + row0 * P.ldc + n + lane;
+          uint16_t* pre = P.pre + row0 * P.ldpre + n + lane;
+          if (P.act == MST_ACT_NONE)
+            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane,
+                     [&](int rr, float v) { out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu); });
+          else if (P.act == MST_ACT_GELU_GRAD)
+            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) {
+              v *= mst_gelu_grad(__uint_as_float((uint32_t)pre[rr * P.ldpre] << 16));
+              out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
+            });
+          else
+            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) {
+              if (P.pre) pre[rr * P.ldpre] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
+              out[rr * P.ldc] = (uint16_t)(pack_bf16(mst_gelu(v), 0.f) & 0xFFFFu);
+            });
         } else {
-          const bool col_ok = n + lane < P.N;
-          float* out = reinterpret_cast<float*>(P.out);
-#pragma unroll 4
-          for (int rr = rr0; rr < rr1; ++rr) {
-            if (row0 + rr >= P.M) break;  // uniform
-            if (col_ok) out[(row0 + rr) * P.ldc + n + lane] = box[rr * 33 + lane];
-          }
+          float* out = reinterpret_cast<float*>(P.out) + row0 * P.ldc + n + lane;
+          box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) { out[rr * P.ldc] = v; });
         }
       }
     }
