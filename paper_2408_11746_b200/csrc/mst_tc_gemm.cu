@@ -250,17 +250,22 @@ struct SampledWords {
     }
   }
 };
-__device__ __forceinline__ void epilogue_tile_sampled(const Params& P, const SampledWords& W, uint32_t stage, uint32_t tmem_base, int acc,
+__device__ __forceinline__ void epilogue_tile_sampled(const Params& P, SampledWords W, uint32_t stage, uint32_t tmem_base, int acc,
                                                       int q, int c0, int lane, int n0, float* __restrict__ out) {
   const uint32_t my_row = stage + (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
   const uint32_t lt = (1u << lane) - 1u;
-#pragma unroll
-  for (int k = 0; k < SAMPLED_CHUNKS; ++k) {
+#pragma unroll 1
+  for (int k = 0; k < SAMPLED_CHUNKS; ++k) {   // rolled: four copies of this body cost the neighbouring launches instruction fetches
     const int c = c0 + k * (EPI_WARPS / 4);
     if (n0 + c * 32 >= P.N) break;  // uniform
-    const uint32_t word = W.word[k];
-    const int32_t at = W.at[k];
+    const uint32_t word = W.word[0];
+    const int32_t at = W.at[0];
+#pragma unroll
+    for (int j = 1; j < SAMPLED_CHUNKS; ++j) {
+      W.word[j - 1] = W.word[j];
+      W.at[j - 1] = W.at[j];
+    }
     uint32_t r[32];
     tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
     const int kept = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
@@ -319,7 +324,7 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
       if (n >= P.N) break;  // uniform
       if (lane == 0) bulk_wait_read();  // the box's previous contents have left shared memory
       __syncwarp();
-#pragma unroll
+#pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int nn = n + h * 32;
         if (nn >= P.N) break;  // uniform; the TMA store clips these columns
