@@ -3,7 +3,7 @@
 // What bounds it: latency.  The image is read once (14 MB for a GPT-2-small block, from L2 when it is reused) and the sums are
 // a few million, so the time is one launch plus one round trip to memory, if enough loads are in flight.  A 128 x 256 tcgen05
 // tile leaves 139 of 148 SMs idle here and walks through the contraction range one block after the other (11-19 us per layer).
-// Instead a block takes 16 output features and all of its eight warps share their contraction range, 32 indices at a
+// Instead a block takes 16 output features and all of its warps share their contraction range, 32 indices at a
 // time; fragments go from global memory straight to registers: the order of the contraction indices is free as long as both
 // operands agree, so a lane's eight neighbouring values (one 16-byte load) serve as the k-pairs of two m16n8k16 products.  The
 // warps' sums meet in shared memory in a fixed order.  Measured at 16 tokens: 3-4 us per layer of a GPT-2-small block.
@@ -14,8 +14,6 @@
 
 namespace {
 
-constexpr int SF_WARPS = 8;
-
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -24,7 +22,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 }
 
 // NT: groups of 8 tokens per block
-template <int NT>
+template <int NT, int SF_WARPS>
 __global__ void __launch_bounds__(32 * SF_WARPS)
 small_fwd_kernel(const uint16_t* __restrict__ X, int64_t ldx, int T, const uint16_t* __restrict__ W, int64_t ldw, int O, int K,
                  __nv_bfloat16* __restrict__ Y, int64_t ldy, int act, __nv_bfloat16* __restrict__ pre, int64_t ldpre) {
@@ -88,13 +86,22 @@ small_fwd_kernel(const uint16_t* __restrict__ X, int64_t ldx, int T, const uint1
   }
 }
 
-template <int NT>
-mst_status_t launch_small(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
+template <int NT, int SF_WARPS>
+mst_status_t launch_warps(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
                           int act, void* pre, int64_t ldpre, cudaStream_t s) {
-  MST_CUDA_TRY(mst_launch_overlapped(small_fwd_kernel<NT>, dim3((unsigned)((O + 15) / 16), (unsigned)((T + NT * 8 - 1) / (NT * 8))),
+  MST_CUDA_TRY(mst_launch_overlapped(small_fwd_kernel<NT, SF_WARPS>, dim3((unsigned)((O + 15) / 16), (unsigned)((T + NT * 8 - 1) / (NT * 8))),
                                      dim3(32 * SF_WARPS), 0, s, (const uint16_t*)X, ldx, (int)T, image, ldimage, O, K, (__nv_bfloat16*)Y,
                                      ldy, act, (__nv_bfloat16*)pre, ldpre));
   return MST_OK;
+}
+
+// As many warps as give each four chunks of the range, one trip to memory (768 x 3072: 5.8 us with 8 warps and three trips, 4.4 with 24)
+template <int NT>
+mst_status_t launch_small(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
+                          int act, void* pre, int64_t ldpre, cudaStream_t s) {
+  if (K <= 1024) return launch_warps<NT, 8>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
+  if (K <= 2048) return launch_warps<NT, 16>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
+  return launch_warps<NT, 24>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
 }
 
 }  // namespace

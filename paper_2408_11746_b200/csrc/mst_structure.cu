@@ -127,8 +127,9 @@ __global__ void scan_empty(int32_t* out) { out[0] = 0; }
 // ---- pack: byte mask -> bit mask -> CSR in two launches ----------------------------------------------------------------------
 // Launch 1 turns 256 mask words per block into bits and leaves the block's entry count; launch 2 adds up the counts of the
 // blocks before its own, scans its words and writes their part of the structure, one warp per word (lane = bit: reads of
-// W and writes of the compacted arrays are coalesced), eight words in flight.  4096 x 1024 bf16, d = 0.1: 3 + 14 us where the
-// separate bits / popcount / three-kernel scan (twice) / one-word-per-warp fill took 46 us in eleven launches.
+// W and writes of the compacted arrays are coalesced), eight words in flight, or half a word per thread where there are few entries.
+// 4096 x 1024 bf16, d = 0.1, with its export: 31 us with whole words only (a warp instruction per word and array, a tenth of its lanes at
+// work), 24 us with half words; separate bits, popcounts, three-kernel scans (twice) and one-word-per-warp fill, eleven launches, 106 us.
 constexpr int PACK_THREADS = 256;
 constexpr int PACK_WORDS = PACK_THREADS;       // mask words per block
 
@@ -224,7 +225,39 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_fill_kernel(const uint32_t*
       if (total) *total = at;
     }
   }
-  __syncthreads();
+  // Few entries: half a word per thread, four entries at a time; a store then touches many lines, but there are few stores.
+  if (__syncthreads_count(mine > 8) < PACK_THREADS / 8) {
+    for (int i = threadIdx.x; i < 2 * PACK_WORDS; i += PACK_THREADS) {
+      const int li = i >> 1;
+      const uint32_t word = word_sh[li];
+      uint32_t m = (i & 1) ? word & 0xFFFF0000u : word & 0xFFFFu;
+      if (m == 0u) continue;
+      const unsigned w = (unsigned)(w0 + li), o = w / (unsigned)wpr;
+      const int c0 = (int)(w - o * (unsigned)wpr) * 32;
+      const V* src = W + (int64_t)o * ldw + c0;
+      int64_t pos = (int64_t)at_sh[li] + ((i & 1) ? __popc(word & 0xFFFFu) : 0);
+      while (m) {
+        int b[4];
+        V v[4];
+        const int n = __popc(m);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          b[j] = m ? __ffs(m) - 1 : 0;
+          m &= m - 1u;
+          v[j] = src[b[j]];   // without an entry column 0 of the word, inside the row
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (j < n && pos + j < cap) {
+            col_idx[pos + j] = (COL)(c0 + b[j]);
+            vals[pos + j] = v[j];
+          }
+        }
+        pos += 4;
+      }
+    }
+    return;
+  }
   const int lane = threadIdx.x & 31;
   constexpr int U = 8;
   for (int l0 = threadIdx.x >> 5; l0 < PACK_WORDS; l0 += (PACK_THREADS / 32) * U) {

@@ -97,3 +97,42 @@ def test_gradients_with_a_cut_last_wave(O, I, T, density):
     for got, want in ((dW.double(), ref[mask.bool()]), (G.double(), ref)):
         assert float((got - want).norm() / want.norm()) < 1e-5
     assert mst.mst_device_error_flags() == 0
+
+
+@pytest.mark.parametrize("O,I,density,rows", [
+    (64, 96, 0.02, None),        # few entries: half a word per thread
+    (70, 1030, 0.27, None),      # blocks on either side of the choice, ragged rows
+    (130, 200, 0.05, 3)])        # three full rows among sparse ones
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_pack_few_and_many_entries(O, I, density, rows, dtype):
+    g = torch.Generator(device="cuda").manual_seed(O * I)
+    mask = (torch.rand((O, I), device="cuda", generator=g) < density).to(torch.uint8)
+    if rows:
+        mask[5:5 + rows] = 1
+    dt, mdt = (torch.float32, mst.MST_F32) if dtype == "f32" else (torch.bfloat16, mst.MST_BF16)
+    W = torch.randn((O, I), device="cuda", generator=g).to(dt)
+    L = mst.Layer(0, O, I, mdt)
+    L.pack(W, mask)
+    nnz = int(mask.sum())
+    assert L.nnz == nnz
+    ptr = torch.zeros(O + 1, dtype=torch.int32, device="cuda")
+    col = torch.zeros(nnz, dtype=torch.int32, device="cuda")
+    val = torch.zeros(nnz, dtype=dt, device="cuda")
+    mst.mst_export_csr(L.handle, ptr, col, val)
+    at = mask.bool().nonzero()
+    assert torch.equal(col.long(), at[:, 1]) and torch.equal(val, W[mask.bool()])
+    assert torch.equal(ptr[1:].long(), mask.sum(1).cumsum(0))
+
+
+@pytest.mark.parametrize("T,O,I", [(1, 40, 1025), (9, 17, 2049), (16, 33, 3072), (7, 24, 2040)])   # 8, 16 and 24 warps, partial chunks
+def test_few_tokens_long_rows(T, O, I):
+    g = torch.Generator(device="cuda").manual_seed(T + O + I)
+    W = torch.randn((O, I), device="cuda", generator=g).bfloat16()
+    mask = (torch.rand((O, I), device="cuda", generator=g) < 0.2).to(torch.uint8)
+    mask[0, 0] = 1
+    L = mst.Layer(0, O, I, mst.MST_BF16)
+    L.pack(W, mask)
+    X = torch.randn((T, I), device="cuda", generator=g).bfloat16()
+    Y = torch.full((T, O), float("nan"), dtype=torch.bfloat16, device="cuda")
+    L.fwd(X, Y, T)
+    assert _rel(Y, X.double() @ (W.double() * mask.double()).t()) < 4e-3
