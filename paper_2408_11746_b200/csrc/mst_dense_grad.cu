@@ -46,13 +46,14 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
   return mst_tc_gemm(a, s);
 }
 
-extern "C" mst_status_t mst_dense_grad(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64_t T,
-                                       int32_t out_features, int32_t in_features, mst_dtype_t dtype, float* G,
-                                       mst_stream_t stream) {
+namespace {
+
+// with a layer: its entries of G go to dW as well, *sampled when the contraction has seen to that
+mst_status_t dense_grad(const mst_layer* L, const void* dY, int64_t lddy, const void* X, int64_t ldx, int64_t T, int32_t out_features,
+                        int32_t in_features, mst_dtype_t dtype, float* G, float* dW, bool* sampled, cudaStream_t s) {
   if (!G || T < 0 || out_features <= 0 || in_features <= 0 || (T > 0 && (!dY || !X))) return MST_ERR_INVALID_ARG;
   if (dtype != MST_F32 && dtype != MST_BF16) return MST_ERR_DTYPE;
   if (lddy < out_features || ldx < in_features) return MST_ERR_SHAPE;
-  cudaStream_t s = (cudaStream_t)stream;
   if (T == 0) {
     MST_CUDA_TRY(cudaMemsetAsync(G, 0, sizeof(float) * (size_t)out_features * in_features, s));
     return MST_OK;
@@ -61,5 +62,29 @@ extern "C" mst_status_t mst_dense_grad(const void* dY, int64_t lddy, const void*
   a.M = out_features; a.N = in_features; a.K = T;
   a.epilogue = MST_TC_OUT_F32;
   a.out = G; a.ldc = in_features;
+  if (L) {
+    a.bits = L->bits[L->cur];
+    a.wscan = L->wscan[L->cur];
+    a.wpr = L->wpr;
+    a.also_sampled = dW;
+    a.sampled = sampled;
+  }
   return mst_tc_gradient(a, dtype, dY, lddy, X, ldx, s);
+}
+
+}  // namespace
+
+extern "C" mst_status_t mst_dense_grad(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64_t T,
+                                       int32_t out_features, int32_t in_features, mst_dtype_t dtype, float* G,
+                                       mst_stream_t stream) {
+  return dense_grad(nullptr, dY, lddy, X, ldx, T, out_features, in_features, dtype, G, nullptr, nullptr, (cudaStream_t)stream);
+}
+
+extern "C" mst_status_t mst_dense_grad_dw(const mst_layer_t* L, const void* dY, int64_t lddy, const void* X, int64_t ldx,
+                                          int64_t T, float* G_dense, float* dW_vals, mst_stream_t stream) {
+  if (!L || !G_dense || !dW_vals) return MST_ERR_INVALID_ARG;
+  if (L->nnz < 0) return MST_ERR_NOT_PACKED;
+  bool sampled = false;
+  MST_TRY(dense_grad(L, dY, lddy, X, ldx, T, L->O, L->I, L->dtype, G_dense, dW_vals, &sampled, (cudaStream_t)stream));
+  return sampled ? MST_OK : mst_sddmm_from_dense(L, G_dense, dW_vals, stream);
 }

@@ -298,11 +298,3 @@ extern "C" mst_status_t mst_sddmm_from_dense(const mst_layer_t* L, const float* 
                                      (const uint32_t*)L->bits[c], (const int32_t*)L->wscan[c], L->O, L->I, L->wpr, G_dense, dW_vals));
   return MST_OK;
 }
-
-extern "C" mst_status_t mst_dense_grad_dw(const mst_layer_t* L, const void* dY, int64_t lddy, const void* X, int64_t ldx,
-                                          int64_t T, float* G_dense, float* dW_vals, mst_stream_t stream) {
-  if (!L || !G_dense || !dW_vals) return MST_ERR_INVALID_ARG;
-  if (L->nnz < 0) return MST_ERR_NOT_PACKED;
-  MST_TRY(mst_dense_grad(dY, lddy, X, ldx, T, L->O, L->I, L->dtype, G_dense, stream));
-  return mst_sddmm_from_dense(L, G_dense, dW_vals, stream);
-}

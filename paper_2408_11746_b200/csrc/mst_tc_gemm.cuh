@@ -50,6 +50,8 @@ struct mst_tc_gemm_args {
   void* pre;             // GELU: optional bf16 output for the pre-activation (may be NULL);
                          // GELU_GRAD: bf16 input holding the pre-activation the derivative is taken at
   int64_t ldpre;
+  float* also_sampled;   // F32: the entries under the mask (bits, wscan, wpr) as well, where partial sums are added up anyway;
+  bool* sampled;         //      set to true when that was done
 };
 
 // C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_prepare.cu; lda / ldb are the pieces'

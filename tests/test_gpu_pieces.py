@@ -136,3 +136,22 @@ def test_few_tokens_long_rows(T, O, I):
     Y = torch.full((T, O), float("nan"), dtype=torch.bfloat16, device="cuda")
     L.fwd(X, Y, T)
     assert _rel(Y, X.double() @ (W.double() * mask.double()).t()) < 4e-3
+
+
+@pytest.mark.parametrize("O,I,T,density", [
+    (96, 264, 700, 0.1),         # small tiles: a pass over the dense gradient
+    (768, 1284, 4096, 0.06),     # two or more ranges: both results from the partial sums; half a word at the end of a row
+    (3840, 1280, 8190, 0.1),     # one tile of the last wave cut
+    (515, 770, 3000, 0.2)])      # columns that four do not divide
+def test_dense_gradient_and_its_entries(O, I, T, density):
+    g = torch.Generator(device="cuda").manual_seed(O * 7 + I)
+    mask = (torch.rand((O, I), device="cuda", generator=g) < density).to(torch.uint8)
+    L = mst.Layer(0, O, I, mst.MST_BF16)
+    L.pack(torch.ones((O, I), dtype=torch.bfloat16, device="cuda"), mask)
+    dY = torch.randn((T, O), device="cuda", generator=g).bfloat16()
+    X = torch.randn((T, I), device="cuda", generator=g).bfloat16()
+    dW = torch.full((L.nnz,), float("nan"), device="cuda")
+    G = torch.full((O, I), float("nan"), device="cuda")
+    L.dense_grad_dw(dY, X, T, G, dW)
+    assert _rel(G, dY.double().t() @ X.double()) < 1e-5
+    assert torch.equal(dW, G[mask.bool()])
