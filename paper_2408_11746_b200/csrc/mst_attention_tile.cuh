@@ -188,8 +188,13 @@ struct Walk {
     both = 2 * (far0 < far1 ? far0 : far1);
     total = near + far0 + far1;
   }
-  // far tile f: which half of the own rows, and where the tile starts; the halves take turns while both have tiles left
-  __device__ __forceinline__ int far_half(int f) const { return f < both ? f & 1 : (far0 > far1 ? 0 : 1); }
+  // far tile f: which half of the own rows, and where the tile starts.  The halves take turns while both have tiles left, the one
+  // with more of them first: the ring has an even number of stages, so each half keeps to stages of its own, sees every filling
+  // of those and cannot take one for the next but one.
+  __device__ __forceinline__ int far_half(int f) const {
+    const int longer = far1 > far0 ? 1 : 0;
+    return f < both ? (f & 1) ^ longer : longer;
+  }
   __device__ __forceinline__ int far_start(int f) const {
     const int m = f < both ? (f >> 1) + 2 : (both >> 1) + (f - both) + 2;
     const int own = r0 + TS * far_half(f);
@@ -202,6 +207,7 @@ struct Walk {
 // a far tile concerns (a barrier of its own: those warps cannot come to it again before the stage has been filled again).
 template <int STAGES, typename W, typename Load, typename Wait>
 __device__ __forceinline__ void feed_ring(const W& walk, uint32_t ring, uint32_t full, uint32_t empty, uint32_t far_done, Load load, Wait wait) {
+  static_assert(STAGES % 2 == 0, "the halves' far tiles take turns");
   int s = 0;
   uint32_t lap = 0;
   for (int j = 0; j < walk.total; ++j) {
