@@ -230,51 +230,48 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
     if (far > 0) {
       const int g = lane >> 2, t = lane & 3, c0 = rs & 63;
       float fm[2] = {-INFINITY, -INFINITY}, fs[2] = {0.f, 0.f};   // rows rs + g and rs + g + 8; sums: this lane's columns only
-      int s = walk.near % STAGES;
-      uint32_t ph = (uint32_t)(walk.near / STAGES) & 1u;
-      for (int f = 0; f < far && ok; ++f) {
-        if (walk.far_half(f) == rs >> 6) {
-          ok = wait_on(full + 8 * s, ph, abort_flag);
-          if (!ok) break;
-          const uint32_t kt = ring + s * 2 * TILE_BYTES;
-          float x[2][4];
-          far_scores(x, own, rs, kt, c0, lane);
+      const int step = walk.far_step();
+      for (int place = walk.near + walk.far_first(rs >> 6); place < walk.total; place += step) {
+        const int s = place % STAGES;
+        ok = wait_on(full + 8 * s, (uint32_t)(place / STAGES) & 1u, abort_flag);
+        if (!ok) break;
+        const uint32_t kt = ring + s * 2 * TILE_BYTES;
+        float x[2][4];
+        far_scores(x, own, rs, kt, c0, lane);
 #pragma unroll
-          for (int rr = 0; rr < 2; ++rr) {
-            float v = -INFINITY;
+        for (int rr = 0; rr < 2; ++rr) {
+          float v = -INFINITY;
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb)
+          for (int nb = 0; nb < 2; ++nb)
 #pragma unroll
-              for (int e = 2 * rr; e < 2 * rr + 2; ++e) {
-                if (g + rr * 8 != nb * 8 + 2 * t + (e & 1)) x[nb][e] = -INFINITY;
-                v = fmaxf(v, x[nb][e]);
-              }
-            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
-            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2)) * SCALE_LOG2E;
-            if (v > fm[rr] + LAZY) {
-              const float c = ex2(fm[rr] - v);
-              fm[rr] = v;
-              fs[rr] *= c;
-#pragma unroll
-              for (int nb = 0; nb < 8; ++nb) {
-                acc[nb][2 * rr] *= c;
-                acc[nb][2 * rr + 1] *= c;
-              }
+            for (int e = 2 * rr; e < 2 * rr + 2; ++e) {
+              if (g + rr * 8 != nb * 8 + 2 * t + (e & 1)) x[nb][e] = -INFINITY;
+              v = fmaxf(v, x[nb][e]);
             }
-            const float nm = -reference(fm[rr]);
+          v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
+          v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2)) * SCALE_LOG2E;
+          if (v > fm[rr] + LAZY) {
+            const float c = ex2(fm[rr] - v);
+            fm[rr] = v;
+            fs[rr] *= c;
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb)
-#pragma unroll
-              for (int e = 2 * rr; e < 2 * rr + 2; ++e) {
-                x[nb][e] = ex2(fmaf(x[nb][e], SCALE_LOG2E, nm));
-                fs[rr] += x[nb][e];
-              }
+            for (int nb = 0; nb < 8; ++nb) {
+              acc[nb][2 * rr] *= c;
+              acc[nb][2 * rr + 1] *= c;
+            }
           }
-          far_accumulate<4>(acc, x, kt + TILE_BYTES, c0, 0, lane);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(far_done + 8 * s);
+          const float nm = -reference(fm[rr]);
+#pragma unroll
+          for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+            for (int e = 2 * rr; e < 2 * rr + 2; ++e) {
+              x[nb][e] = ex2(fmaf(x[nb][e], SCALE_LOG2E, nm));
+              fs[rr] += x[nb][e];
+            }
         }
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        far_accumulate<4>(acc, x, kt + TILE_BYTES, c0, 0, lane);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(far_done + 8 * s);
       }
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {

@@ -312,38 +312,35 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     if (far > 0) {
       compute_sync<32 * CW>();                               // the rows' statistics are in place
       const int g = lane >> 2, t = lane & 3;
-      int s = walk.near % STAGES;
-      uint32_t ph = (uint32_t)(walk.near / STAGES) & 1u;
-      for (int f = 0; f < far && ok; ++f) {
-        if (walk.far_half(f) == r0 >> 6) {
-          ok = wait_on(S.full + 8 * s, ph, abort_flag);
-          if (!ok) break;
-          const uint32_t kt = S.ring + s * 2 * TILE_BYTES;
+      const int step = walk.far_step();
+      for (int place = walk.near + walk.far_first(r0 >> 6); place < walk.total; place += step) {
+        const int s = place % STAGES;
+        ok = wait_on(S.full + 8 * s, (uint32_t)(place / STAGES) & 1u, abort_flag);
+        if (!ok) break;
+        const uint32_t kt = S.ring + s * 2 * TILE_BYTES;
 #pragma unroll
-          for (int sp = 0; sp < STRIPS; ++sp) {
-            const int rs = r0 + sp * 16, c0 = rs & 63;
-            const float2 st0 = stat_s[rs + g], st1 = stat_s[rs + g + 8];
-            float sc[2][4], dp[2][4];
-            far_scores(sc, S.own0, rs, kt, c0, lane);
-            far_scores(dp, S.own1, rs, kt + TILE_BYTES, c0, lane);
+        for (int sp = 0; sp < STRIPS; ++sp) {
+          const int rs = r0 + sp * 16, c0 = rs & 63;
+          const float2 st0 = stat_s[rs + g], st1 = stat_s[rs + g + 8];
+          float sc[2][4], dp[2][4];
+          far_scores(sc, S.own0, rs, kt, c0, lane);
+          far_scores(dp, S.own1, rs, kt + TILE_BYTES, c0, lane);
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb) {
+          for (int nb = 0; nb < 2; ++nb) {
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float ds = 0.f;
-                if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
-                  const float p = ex2(fmaf(sc[nb][e], SCALE_LOG2E, (e >> 1) ? st1.x : st0.x));
-                  ds = p * (dp[nb][e] - ((e >> 1) ? st1.y : st0.y));
-                }
-                sc[nb][e] = ds;
+            for (int e = 0; e < 4; ++e) {
+              float ds = 0.f;
+              if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
+                const float p = ex2(fmaf(sc[nb][e], SCALE_LOG2E, (e >> 1) ? st1.x : st0.x));
+                ds = p * (dp[nb][e] - ((e >> 1) ? st1.y : st0.y));
               }
+              sc[nb][e] = ds;
             }
-            far_accumulate<4>(acc[sp], sc, kt, c0, 0, lane);
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+          far_accumulate<4>(acc[sp], sc, kt, c0, 0, lane);
         }
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(S.far_done + 8 * s);
       }
     }
     ok = ok && wait_on(S.acc_full, 0, abort_flag);
@@ -531,39 +528,38 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       }
     if (far > 0) {
       const int g = lane >> 2, t = lane & 3;
-      for (int f = 0; f < far && ok; ++f) {
-        if (walk.far_half(f) == r0 >> 6) {
-          ok = wait_on(S.full + 8 * s, ph, abort_flag);
-          if (!ok) break;
-          const uint32_t qt = S.ring + s * 2 * TILE_BYTES;
+      const int step = walk.far_step();
+      for (int place = walk.near + walk.far_first(r0 >> 6); place < walk.total; place += step) {
+        const int s = place % STAGES;
+        ok = wait_on(S.full + 8 * s, (uint32_t)(place / STAGES) & 1u, abort_flag);
+        if (!ok) break;
+        const uint32_t qt = S.ring + s * 2 * TILE_BYTES;
 #pragma unroll
-          for (int sp = 0; sp < STRIPS; ++sp) {
-            const int rs = r0 + sp * 16, c0 = rs & 63;
-            float st[2][4], dp[2][4];
-            far_scores(st, S.own0, rs, qt, c0, lane);
-            far_scores(dp, S.own1, rs, qt + TILE_BYTES, c0, lane);
+        for (int sp = 0; sp < STRIPS; ++sp) {
+          const int rs = r0 + sp * 16, c0 = rs & 63;
+          float st[2][4], dp[2][4];
+          far_scores(st, S.own0, rs, qt, c0, lane);
+          far_scores(dp, S.own1, rs, qt + TILE_BYTES, c0, lane);
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb) {
-              const float* sq = S.at<float>(S.stat + (uint32_t)(s * STAT_BYTES)) + c0 + nb * 8 + 2 * t;
-              const float2 nl = *reinterpret_cast<const float2*>(sq), nd = *reinterpret_cast<const float2*>(sq + TS);
+          for (int nb = 0; nb < 2; ++nb) {
+            const float* sq = S.at<float>(S.stat + (uint32_t)(s * STAT_BYTES)) + c0 + nb * 8 + 2 * t;
+            const float2 nl = *reinterpret_cast<const float2*>(sq), nd = *reinterpret_cast<const float2*>(sq + TS);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float p = 0.f, ds = 0.f;
-                if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
-                  p = ex2(fmaf(st[nb][e], SCALE_LOG2E, (e & 1) ? nl.y : nl.x));
-                  ds = p * (dp[nb][e] + ((e & 1) ? nd.y : nd.x));
-                }
-                st[nb][e] = p;
-                dp[nb][e] = ds;
+            for (int e = 0; e < 4; ++e) {
+              float p = 0.f, ds = 0.f;
+              if (g + (e >> 1) * 8 == nb * 8 + 2 * t + (e & 1)) {
+                p = ex2(fmaf(st[nb][e], SCALE_LOG2E, (e & 1) ? nl.y : nl.x));
+                ds = p * (dp[nb][e] + ((e & 1) ? nd.y : nd.x));
               }
+              st[nb][e] = p;
+              dp[nb][e] = ds;
             }
-            far_accumulate<4>(acc_v[sp], st, qt + TILE_BYTES, c0, 0, lane);
-            far_accumulate<4>(acc_k[sp], dp, qt, c0, 0, lane);
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+          far_accumulate<4>(acc_v[sp], st, qt + TILE_BYTES, c0, 0, lane);
+          far_accumulate<4>(acc_k[sp], dp, qt, c0, 0, lane);
         }
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(S.far_done + 8 * s);
       }
     }
     ok = ok && wait_on(S.acc_full, 0, abort_flag);

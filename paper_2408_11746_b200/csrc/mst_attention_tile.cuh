@@ -195,6 +195,12 @@ struct Walk {
     const int longer = far1 > far0 ? 1 : 0;
     return f < both ? (f & 1) ^ longer : longer;
   }
+  // one half's far tiles: first, first + step, .. below far0 + far1
+  __device__ __forceinline__ int far_step() const { return both > 0 ? 2 : 1; }
+  __device__ __forceinline__ int far_first(int half) const {
+    const int longer = far1 > far0 ? 1 : 0;
+    return both > 0 ? half ^ longer : half == longer ? 0 : far0 + far1;
+  }
   __device__ __forceinline__ int far_start(int f) const {
     const int m = f < both ? (f >> 1) + 2 : (both >> 1) + (f - both) + 2;
     const int own = r0 + TS * far_half(f);
