@@ -232,6 +232,9 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
 // staging box, so that each store instruction writes the kept entries of ONE row, which are neighbours in CSR order; all 32 rows
 // are read back before the first is stored, or every row would wait for its own round trip.
 constexpr int SAMPLED_CHUNKS = BN / 32 / (EPI_WARPS / 4);
+// Entries of a 1024-output chunk from which rows win: d of about 0.19.  8192 tokens, 768 x 768: entry by entry 15.5 / 16.6 / 19.3 /
+// 24 us at d = 0.1 / 0.15 / 0.25 / 0.5, row by row 17.0 / 17.0 / 17.2 / 18.3.
+constexpr int SAMPLED_STAGE_MIN = 192;
 struct SampledWords {
   uint32_t word[SAMPLED_CHUNKS];
   int32_t at[SAMPLED_CHUNKS];
@@ -1045,21 +1048,29 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
   if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
   const bool env = mst_env_any();
-  // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate.  SM clocks, fitted like that one's: 10500 a
-  // launch and 537 per k-block of a pair's tile; the gradients' epilogue, which nothing overlaps in a single wave, 7500, and a
-  // second launch that adds the ranges 6000.
+  // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
+  // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
+  // The entries under the mask are fitted to widths 320..768 x 4, 600..4096 tokens, d = 0.026..0.4 (the two epilogues change over at
+  // P.sampled_stage_min); of 160 such calls 159 get the faster kernel to within 0.4 us.  1280 x 320 at 2046 tokens, d = 0.05: 10.0 us
+  // in seven ranges here, 12.3 in the small-tile kernel.  Rows are fitted to widths 192..1280 x 4 (each way), 64..4096 tokens:
+  // 3072 -> 768 at 1024 tokens 17.3 us in the small-tile kernel, 19.6 here.
   if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
-      double here = 10500.0 + (double)kb * 537.0;
+      double here = (!a.act ? 9100.0 : a.M > BM ? 13000.0 : 18000.0) + (double)kb * 564.0;   // one token tile: single blocks
       if (a.epilogue != MST_TC_OUT_BF16) {
-        const double out_bytes = a.epilogue == MST_TC_OUT_F32 ? 4.0 * (double)a.M * (double)a.N : 4.0 * (double)a.nnz;
+        const bool entries = a.epilogue == MST_TC_OUT_SAMPLED;
+        const double out_bytes = entries ? 4.0 * (double)a.nnz : 4.0 * (double)a.M * (double)a.N;
         int cut;
-        const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes, &cut);
-        here = 18000.0 + (double)((kb + sp - 1) / sp) * 537.0 + (sp > 1 ? 6000.0 : 0.0);
-        if (cut > 1) here += (double)((kb + sp - 1) / sp / cut) * 537.0 + 3000.0;
+        const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes, &cut), per = (kb + sp - 1) / sp;
+        if (entries) {
+          here = ((double)a.nnz * 1024.0 < SAMPLED_STAGE_MIN * (double)a.M * (double)a.N ? 12000.0 : 14000.0) + (double)per * 574.0;
+          if (sp > 1) here += 3500.0 + (double)sp * out_bytes * 7.4e-4;   // written and read, 5 TB/s at 1.85 GHz
+        } else {
+          here = 17100.0 + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0);
+        }
       }
-      if (mst_tc_small_clocks(a) < 0.95 * here) return mst_tc_small(a, s);
+      if (mst_tc_small_clocks(a) < here) return mst_tc_small(a, s);
     }
   }
   CUtensorMap tmA, tmB;
@@ -1094,7 +1105,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   P.pre = a.pre;
   P.ldpre = a.ldpre;
   if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
-  P.sampled_stage_min = 192;  // d of about 0.19; 8192 tokens, 768 x 768: entry by entry 15.5 / 16.6 / 19.3 / 24 us at d = 0.1 / 0.15 / 0.25 / 0.5, row by row 17.0 / 17.0 / 17.2 / 18.3
+  P.sampled_stage_min = SAMPLED_STAGE_MIN;
   if (const char* e = mst_getenv(env, "MST_TC_SAMPLED_STAGE")) P.sampled_stage_min = atoi(e);  // measurement override
   if (a.epilogue != MST_TC_OUT_BF16) {
     // few output tiles: cut the contraction range so that all SMs work; partial sums go to the shared scratch buffer

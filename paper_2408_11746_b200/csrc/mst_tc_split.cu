@@ -107,23 +107,22 @@ __device__ __forceinline__ void gather_sums(uint32_t sums, int rr0, float* box, 
   }
 }
 
-// Rows rr0 .. rr1 - 1 (a multiple of four) of the warp's box, four at a time: read back together, then handed on one by one.  `inside`
-// (uniform): the square lies inside the output, so nothing is tested - a test per store, with its branch and its 64-bit address, made
-// 64 KB of stores take 8000 clocks instead of 2200.
+// Rows rr0 .. end - 1 of this lane's column of the warp's box, four at a time: read back together, then handed on one by one.  Nothing
+// is tested per store - a test, with its branch and its 64-bit address, made 64 KB of stores take 8000 clocks instead of 2200, and
+// the last token tile of 600 tokens, whose rows went one by one, cost each call 1.6 us.
 template <typename Store>
-__device__ __forceinline__ void box_rows(const float* box, int rr0, int rr1, bool inside, int64_t rows_left, bool col_ok, int lane, Store store) {
-  if (inside) {
+__device__ __forceinline__ void box_rows(const float* box, int rr0, int end, int lane, Store store) {
+  int r = rr0;
 #pragma unroll 2
-    for (int r = rr0; r < rr1; r += 4) {
-      float v[4];
+  for (; r + 4 <= end; r += 4) {
+    float v[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = box[(r + k) * 33 + lane];
+    for (int k = 0; k < 4; ++k) v[k] = box[(r + k) * 33 + lane];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) store(r + k, v[k]);
-    }
-  } else if (col_ok) {
-    for (int r = rr0; r < rr1 && r < rows_left; ++r) store(r, box[r * 33 + lane]);
+    for (int k = 0; k < 4; ++k) store(r + k, v[k]);
   }
+#pragma unroll 1
+  for (; r < end; ++r) store(r, box[r * 33 + lane]);
 }
 
 template <int BN, int PIECES>
@@ -298,7 +297,7 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
-        const bool inside = row0 + 32 <= P.M && n + 32 <= P.N, col_ok = n + lane < P.N;
+        const int end = n + lane >= P.N ? 0 : (int)(P.M - row0 < rr1 ? P.M - row0 : rr1);   // rows of this lane's column
         if (P.epilogue == MST_TC_OUT_SAMPLED) {
           uint32_t word = 0;
           int32_t at = 0;
@@ -308,7 +307,7 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             at = P.wscan[wi];
           }
           float* out = reinterpret_cast<float*>(P.out);
-          box_rows(box, rr0, rr1, true, 0, true, lane, [&](int rr, float v) {   // words beyond the matrix are empty
+          box_rows(box, rr0, rr1, lane, [&](int rr, float v) {   // words beyond the matrix are empty
             const uint32_t w = __shfl_sync(0xffffffffu, word, rr);
             const int32_t base = __shfl_sync(0xffffffffu, at, rr);
             if ((w >> lane) & 1u) out[base + __popc(w & lt)] = v;
@@ -317,21 +316,33 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + row0 * P.ldc + n + lane;
           uint16_t* pre = P.pre + row0 * P.ldpre + n + lane;
           if (P.act == MST_ACT_NONE)
-            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane,
+            box_rows(box, rr0, end, lane,
                      [&](int rr, float v) { out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu); });
-          else if (P.act == MST_ACT_GELU_GRAD)
-            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) {
-              v *= mst_gelu_grad(__uint_as_float((uint32_t)pre[rr * P.ldpre] << 16));
-              out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
-            });
-          else
-            box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) {
+          else if (P.act == MST_ACT_GELU_GRAD) {
+            // sixteen rows' inputs at a time, before any of their results leaves: row by row each waits out its load (64 tokens,
+            // 192 x 768: 11.6 us).  Rows past the end repeat the last one, so that only the stores are conditional and the sixteen
+            // derivatives overlap.
+#pragma unroll 1
+            for (int r = rr0; r < end; r += 16) {
+              uint16_t x[16];
+              float y[16];
+#pragma unroll
+              for (int k = 0; k < 16; ++k) x[k] = pre[(r + k < end ? r + k : end - 1) * P.ldpre];
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                y[k] = box[(r + k < end ? r + k : end - 1) * 33 + lane] * mst_gelu_grad(__uint_as_float((uint32_t)x[k] << 16));
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                if (r + k < end) out[(r + k) * P.ldc] = (uint16_t)(pack_bf16(y[k], 0.f) & 0xFFFFu);
+            }
+          } else
+            box_rows(box, rr0, end, lane, [&](int rr, float v) {
               if (P.pre) pre[rr * P.ldpre] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
               out[rr * P.ldc] = (uint16_t)(pack_bf16(mst_gelu(v), 0.f) & 0xFFFFu);
             });
         } else {
           float* out = reinterpret_cast<float*>(P.out) + row0 * P.ldc + n + lane;
-          box_rows(box, rr0, rr1, inside, P.M - row0, col_ok, lane, [&](int rr, float v) { out[rr * P.ldc] = v; });
+          box_rows(box, rr0, end, lane, [&](int rr, float v) { out[rr * P.ldc] = v; });
         }
       }
     }
@@ -376,9 +387,9 @@ mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
 // Tile width and number of K ranges from a time model in SM clocks.
 // Three pieces: 24 MMAs per k-block (64 clocks each at 128 columns, 40 at 64, where the A operand's shared-memory reads dominate),
 // about 4000 for launch, fill and drain of a block, and 1500 for the sums of a cluster.
-// One piece (64 columns; 128 were no faster), fitted to back-to-back calls of 64 to 4096 tokens on layers of 320 to 4096 features, at
-// 1.85 GHz: 9000 a launch, 555 per k-block (its 24 KB of operands), two blocks to an SM (clusters do not pack
-// that way: one); rows of bf16 4500 a wave, a further wave 10000, the sums of a cluster 1500 (5000 when the sampled rows are what the ranks divide).
+// One piece (64 columns; 128 were no faster), fitted to back-to-back calls of 64 to 4096 tokens on layers of 192 to 4096 features, at
+// 1.85 GHz: a launch, the k-blocks (24 KB of operands each), two blocks to an SM (clusters do not pack that way: one), a further
+// wave, the sums of a cluster.  GELU adds 1500 a wave and its derivative 8000, and 3000 where two such blocks share an SM.
 double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
   const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
@@ -395,8 +406,11 @@ double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
         t = (double)waves * (kb * (w == 64 ? 960.0 : 1536.0) + 4000.0) + (sp > 1 ? 1500.0 : 0.0);
       } else {
         const int64_t slots = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + slots - 1) / slots;
-        const bool rows = a.epilogue == MST_TC_OUT_BF16;
-        t = 9000.0 + (double)waves * (kb * 555.0 + (rows ? 4500.0 : 0.0)) + (double)(waves - 1) * 10000.0 + (sp > 1 ? (rows ? 1500.0 : 5000.0) : 0.0);
+        if (a.epilogue == MST_TC_OUT_BF16)
+          t = 9300.0 + (double)waves * (kb * 480.0 + (a.act == MST_ACT_GELU_GRAD ? 8000.0 : a.act ? 1500.0 : 0.0)) +
+              (double)(waves - 1) * 8000.0 + (sp > 1 ? 5000.0 : a.act && tiles > sms ? 3000.0 : 0.0);
+        else
+          t = 9000.0 + (double)waves * kb * 555.0 + (double)(waves - 1) * 10000.0 + (sp > 1 ? 5000.0 : 0.0);
       }
       if (t < best * 0.97) { best = t; *bn = w; *splits = sp; }
     }

@@ -155,3 +155,22 @@ def test_dense_gradient_and_its_entries(O, I, T, density):
     L.dense_grad_dw(dY, X, T, G, dW)
     assert _rel(G, dY.double().t() @ X.double()) < 1e-5
     assert torch.equal(dW, G[mask.bool()])
+
+
+@pytest.mark.parametrize("O,I,T", [(192, 200, 34), (256, 192, 130), (72, 320, 60), (40, 1032, 67), (24, 2056, 129)])   # last rows of a tile 1 to 31, clusters of 1 to 8
+def test_activation_rows_of_a_partial_tile(O, I, T):
+    g = torch.Generator(device="cuda").manual_seed(O + I + T)
+    W = (torch.randn((O, I), device="cuda", generator=g) / I ** 0.5).bfloat16()
+    mask = (torch.rand((O, I), device="cuda", generator=g) < 0.3).to(torch.uint8)
+    mask[0, 0] = 1
+    L, Lt = mst.Layer(0, O, I, mst.MST_BF16), mst.Layer(1, I, O, mst.MST_BF16)
+    L.pack(W, mask)
+    Lt.pack(W.t().contiguous(), mask.t().contiguous())
+    X, pre = torch.randn((T, I), device="cuda", generator=g).bfloat16(), torch.randn((T, O), device="cuda", generator=g).bfloat16()
+    H, Y, D = (torch.full((T, O), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(3))
+    L.fwd_gelu(X, H, T, Y_pre=Y)
+    Lt.bwd_x_gelu(X, pre, D, T)
+    product = X.double() @ (W.double() * mask.double()).t()
+    p = pre.double().requires_grad_(True)
+    torch.nn.functional.gelu(p).sum().backward()
+    assert _rel(Y, product) < 4e-3 and _rel(H, torch.nn.functional.gelu(product)) < 4e-3 and _rel(D, product * p.grad) < 4e-3
