@@ -270,8 +270,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
             }
         }
         far_accumulate<4>(acc, x, kt + TILE_BYTES, c0, 0, lane);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(far_done + 8 * s);
+        far_release(far_done + 8 * s, lane);
       }
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {

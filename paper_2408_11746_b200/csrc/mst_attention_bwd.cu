@@ -339,8 +339,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           }
           far_accumulate<4>(acc[sp], sc, kt, c0, 0, lane);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+        far_release(S.far_done + 8 * s, lane);
       }
     }
     ok = ok && wait_on(S.acc_full, 0, abort_flag);
@@ -558,8 +557,7 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           far_accumulate<4>(acc_v[sp], st, qt + TILE_BYTES, c0, 0, lane);
           far_accumulate<4>(acc_k[sp], dp, qt, c0, 0, lane);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(S.far_done + 8 * s);
+        far_release(S.far_done + 8 * s, lane);
       }
     }
     ok = ok && wait_on(S.acc_full, 0, abort_flag);

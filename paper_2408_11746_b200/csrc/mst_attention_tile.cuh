@@ -232,10 +232,16 @@ __device__ __forceinline__ void feed_ring(const W& walk, uint32_t ring, uint32_t
 // mma.sync m16n8k16 with the published fragment layouts: with g = lane / 4 and t = lane % 4, an accumulator tile (16 x 8) holds
 // rows g, g + 8 and columns 2t, 2t + 1; two neighbouring accumulator tiles, rounded to bf16, are the A operand of the next one.
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t a) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
 }
 __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t a) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
 }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -271,6 +277,15 @@ __device__ __forceinline__ void far_accumulate(float (&acc)[2 * N2][4], const fl
     mma_bf16(acc[2 * n2], a, b[0], b[1]);
     mma_bf16(acc[2 * n2 + 1], a, b[2], b[3]);
   }
+}
+// This warp has read its rows of a far tile: its stage may be filled again.  The reads went through the generic proxy and the next
+// copy into the stage goes through the async proxy, which an arrival alone does not order: without the proxy fence a read that was
+// still under way now and then saw rows of the tile that came next (dQ at l = 128 differed from run to run in one of three calls;
+// up to three tiles per half, as at l = 256, no stage is filled twice).
+__device__ __forceinline__ void far_release(uint32_t far_done, int lane) {
+  fence_async_smem();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(far_done);
 }
 // this strip's accumulators -> fp32 rows r0 .. r0 + 15, columns d0 .., in shared memory (pitch LDF)
 template <int NB>

@@ -119,3 +119,58 @@ def test_attention_bwd_tile_edges(B, n, H, stride):
     for a, b, name in zip(got, ref, ("dQ", "dK", "dV")):
         assert np.isfinite(a).all() and rel_err(a, b) <= 2e-2, name
     assert mst.mst_device_error_flags() == 0
+
+
+def _row_bounds(qkv, dO, B, n, H, stride):
+    """Forward and backward results in fp64 and, element by element, the largest error that bf16 weights, score gradients and results
+    allow (bf16 has 8 significant bits, so a rounding to nearest moves a value by up to u = 2^-8 of it; fp32 sums and exponentials
+    are a hundredth of that, within the 5 % on top)."""
+    u = 1.05 * 2.0 ** -8
+    x = qkv.double().view(B, n, 3, H, 64).permute(2, 0, 3, 1, 4)
+    g = dO.double().view(B, n, H, 64).transpose(1, 2)
+    back = torch.arange(n, device=qkv.device)
+    back = back[:, None] - back[None, :]
+    keep = (back >= 0) & ((back < stride) | (back % stride == 0))
+    ref, bound = [], []
+    for b in range(B):
+        q, k, v, go = x[0, b], x[1, b], x[2, b], g[b]
+        P = torch.softmax((q @ k.mT / 8).masked_fill(~keep, float("-inf")), -1)
+        out = P @ v
+        e_out = u * (out.abs() + P @ v.abs())
+        dS = P * (go @ v.mT - (go * out).sum(-1, keepdim=True))
+        e_dS = u * dS.abs() + P * (go.abs() * e_out).sum(-1, keepdim=True)     # its own rounding, and delta from the rounded output
+        dq, dk, dv = dS @ k / 8, dS.mT @ q / 8, P.mT @ go
+        ref.append(torch.stack([out, dq, dk, dv]))
+        bound.append(torch.stack([e_out, u * dq.abs() + e_dS @ k.abs() / 8, u * dk.abs() + e_dS.mT @ q.abs() / 8,
+                                  u * (dv.abs() + P.mT @ go.abs())]))
+    return torch.stack(ref, 1), torch.stack(bound, 1)     # [4, B, H, n, 64]
+
+
+@pytest.mark.parametrize("B,n,H,stride", [
+    (8, 1024, 16, 128),     # up to twelve far tiles: the ring's stages are filled with far tiles again and again
+    (8, 1024, 8, 64),       # up to twenty-eight of them
+    (2, 1024, 12, 256)])    # four: none is filled twice
+def test_every_element_and_every_repetition(B, n, H, stride):
+    """Repeated calls agree bit for bit, and each element lies within what the data types give for it, so that a single wrong row
+    cannot hide behind the largest values."""
+    gen = torch.Generator(device="cuda").manual_seed(stride)
+    C = 64 * H
+    qkv = torch.randn(B * n, 3 * C, generator=gen, device="cuda").bfloat16()
+    dO = torch.randn(B * n, C, generator=gen, device="cuda").bfloat16()
+    first = None
+    for _ in range(40):
+        out, dqkv = torch.zeros_like(dO), torch.zeros_like(qkv)
+        lse = torch.zeros(B, H, n, device="cuda")
+        a, d = qkv.data_ptr(), dqkv.data_ptr()
+        mst.mst_strided_attention_fwd(a, a + 2 * C, a + 4 * C, 3 * C, B, n, H, 64, stride, out, C, lse)
+        mst.mst_strided_attention_bwd(a, a + 2 * C, a + 4 * C, 3 * C, out, C, dO, C, lse, B, n, H, 64, stride, d, d + 2 * C, d + 4 * C, 3 * C)
+        got = [out, lse, dqkv]
+        if first is None:
+            first = got
+        else:
+            assert all(torch.equal(p, q) for p, q in zip(got, first))
+    ref, bound = _row_bounds(qkv, dO, B, n, H, stride)
+    for name, t, r, e in zip(("out", "dQ", "dK", "dV"), [first[0]] + list(first[2].view(B * n, 3, C).unbind(1)), ref, bound):
+        over = (t.double().view(B, n, H, 64).transpose(1, 2) - r).abs() - e
+        # dS of the first positions is a difference of fp32 products that cancel: 64 truncated terms of size |dOut||v|
+        assert float(over.max()) <= 64 * 2.0 ** -23 * 8, (name, float(over.max()), int(over.argmax()))
