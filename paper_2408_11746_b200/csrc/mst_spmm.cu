@@ -385,6 +385,7 @@ spmm_stream_kernel(const __grid_constant__ CUtensorMap tmIn, const int32_t* __re
           load_window(rr);
         }
       }
+      mst_ptx::fence_async_smem();   // the reads of this stage are done before TMA may fill it again
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0 + 8 * s);
       if (++s == STAGES) { s = 0; ph ^= 1u; }
