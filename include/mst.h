@@ -99,7 +99,11 @@ mst_status_t mst_layer_destroy(mst_layer_t* layer);
  * fp32 layers keep single-precision arithmetic whatever the path: on MST_PATH_CUDA_CORE in FMA chains, otherwise as sums of
  * products of exact bf16 pieces on the tensor cores (three pieces per operand, rounded fp32 sums every 64 terms; at
  * least as close to the exact product as the FMA chains).  Results of the paths agree within the stated tolerance, not
- * bit for bit (different summation order). */
+ * bit for bit (different summation order).
+ * Infinite and NaN operands: an fp32 layer, a bf16 layer on MST_PATH_CUDA_CORE, and a bf16 call with rows (of the activations or
+ * of the result) that do not start on 16-byte boundaries or with in_features that is no multiple of 8, go by the stored entries
+ * alone: such a value reaches the outputs connected to it and no others.  Dense tiles over aligned bf16 rows multiply it by the
+ * masked zeros as well, so that it makes a NaN of every output of its token. */
 typedef enum { MST_PATH_AUTO = 0, MST_PATH_CUDA_CORE = 1, MST_PATH_TENSOR_CORE = 2, MST_PATH_SPARSE_TC = 3 } mst_compute_path_t;
 mst_status_t mst_set_compute_path(mst_layer_t* layer, mst_compute_path_t path);
 

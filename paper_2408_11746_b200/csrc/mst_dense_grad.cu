@@ -22,6 +22,10 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
     MST_TRY(mst_prepare(dtype, nullptr, jobs, 2, s));
     a.A = ws; a.lda = ldO;
     a.B = x; a.ldb = ldI;
+    a.redo.kind = MST_REDO_GRADIENT;
+    a.redo.A = dY; a.redo.lda = lddy;
+    a.redo.B = X; a.redo.ldb = ldx;
+    a.redo.K = T;
     return mst_tc_split(a, s);
   }
   const bool okY = mst_tc_gemm_usable(dY, lddy, dY, lddy), okX = mst_tc_gemm_usable(X, ldx, X, ldx);

@@ -8,6 +8,7 @@
 // operands agree, so a lane's eight neighbouring values (one 16-byte load) serve as the k-pairs of two m16n8k16 products.  The
 // warps' sums meet in shared memory in a fixed order.  Measured at 16 tokens: 3-4 us per layer of a GPT-2-small block.
 #include "mst_internal.cuh"
+#include "mst_redo.cuh"
 #include "mst_tc_gemm.cuh"
 
 #include <cuda_bf16.h>
@@ -25,7 +26,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 template <int NT, int SF_WARPS>
 __global__ void __launch_bounds__(32 * SF_WARPS)
 small_fwd_kernel(const uint16_t* __restrict__ X, int64_t ldx, int T, const uint16_t* __restrict__ W, int64_t ldw, int O, int K,
-                 __nv_bfloat16* __restrict__ Y, int64_t ldy, int act, __nv_bfloat16* __restrict__ pre, int64_t ldpre) {
+                 __nv_bfloat16* __restrict__ Y, int64_t ldy, int act, __nv_bfloat16* __restrict__ pre, int64_t ldpre, const mst_redo redo) {
   __shared__ float red[SF_WARPS][NT * 8][17];
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
@@ -78,6 +79,7 @@ small_fwd_kernel(const uint16_t* __restrict__ X, int64_t ldx, int T, const uint1
     float v = red[0][n][f];
 #pragma unroll
     for (int w = 1; w < SF_WARPS; ++w) v += red[w][n][f];
+    if (redo.kind && mst_redo_needed(v)) v = mst_redo_one<uint16_t>(redo, tok, o);
     if (act == MST_ACT_GELU) {
       if (pre) pre[(int64_t)tok * ldpre + o] = __float2bfloat16_rn(v);
       v = mst_gelu(v);
@@ -88,27 +90,27 @@ small_fwd_kernel(const uint16_t* __restrict__ X, int64_t ldx, int T, const uint1
 
 template <int NT, int SF_WARPS>
 mst_status_t launch_warps(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
-                          int act, void* pre, int64_t ldpre, cudaStream_t s) {
+                          int act, void* pre, int64_t ldpre, const mst_redo& redo, cudaStream_t s) {
   MST_CUDA_TRY(mst_launch_overlapped(small_fwd_kernel<NT, SF_WARPS>, dim3((unsigned)((O + 15) / 16), (unsigned)((T + NT * 8 - 1) / (NT * 8))),
                                      dim3(32 * SF_WARPS), 0, s, (const uint16_t*)X, ldx, (int)T, image, ldimage, O, K, (__nv_bfloat16*)Y,
-                                     ldy, act, (__nv_bfloat16*)pre, ldpre));
+                                     ldy, act, (__nv_bfloat16*)pre, ldpre, redo));
   return MST_OK;
 }
 
 // As many warps as give each four chunks of the range, one trip to memory (768 x 3072: 5.8 us with 8 warps and three trips, 4.4 with 24)
 template <int NT>
 mst_status_t launch_small(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
-                          int act, void* pre, int64_t ldpre, cudaStream_t s) {
-  if (K <= 1024) return launch_warps<NT, 8>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
-  if (K <= 2048) return launch_warps<NT, 16>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
-  return launch_warps<NT, 24>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
+                          int act, void* pre, int64_t ldpre, const mst_redo& redo, cudaStream_t s) {
+  if (K <= 1024) return launch_warps<NT, 8>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, redo, s);
+  if (K <= 2048) return launch_warps<NT, 16>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, redo, s);
+  return launch_warps<NT, 24>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, redo, s);
 }
 
 }  // namespace
 
 // X rows 16-byte aligned, columns K .. multiple of 8 zero in X and in the image; act NONE or GELU
 mst_status_t mst_small_fwd(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
-                           int act, void* pre, int64_t ldpre, cudaStream_t s) {
-  if (T <= 8) return launch_small<1>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
-  return launch_small<2>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, s);
+                           int act, void* pre, int64_t ldpre, const mst_redo& redo, cudaStream_t s) {
+  if (T <= 8) return launch_small<1>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, redo, s);
+  return launch_small<2>(X, ldx, T, image, ldimage, O, K, Y, ldy, act, pre, ldpre, redo, s);
 }

@@ -564,6 +564,14 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     a.B = image; a.ldb = ldimage; a.b_mn_major = transpose ? 1 : 0;
     a.M = T; a.N = rows; a.K = cols;
     a.out = out; a.ldc = ldout;
+    // fp32 layers and bf16 rows that TMA does not take (here or on their way out) go by the stored entries alone where sums are not finite
+    if (L->dtype == MST_F32 || ldout % 8 != 0 || (reinterpret_cast<uintptr_t>(out) & 15u) != 0 || !mst_tc_gemm_usable(in, ldin, in, L->I)) {
+      a.redo.kind = transpose ? MST_REDO_BACKWARD : MST_REDO_FORWARD;
+      a.redo.bits = L->bits[c]; a.redo.wscan = L->wscan[c]; a.redo.wpr = L->wpr;
+      a.redo.A = in; a.redo.lda = ldin;
+      a.redo.B = L->vals[c];
+      a.redo.K = cols;
+    }
     if (L->dtype == MST_F32) {
       void* pieces = nullptr;
       a.lda = mst_row_pitch(cols);
@@ -590,7 +598,7 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     // A few tokens: the latency kernel (16 tokens: 3 us a layer of GPT-2-small width against 5 for the smallest tiles; at 32 its
     // blocks read the activations too often and it loses).  Columns beyond the row must be zero in the activations too.
     if (!transpose && T <= MST_SMALL_FWD_TOKENS && (cols % 8 == 0 || a.A != in))
-      return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, s);
+      return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, a.redo, s);
     a.epilogue = MST_TC_OUT_BF16;
     a.splits = 1;
     a.act = act; a.pre = pre; a.ldpre = ldpre;

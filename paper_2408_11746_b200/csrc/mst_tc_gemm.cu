@@ -22,6 +22,7 @@
 #include <cstdlib>
 
 #include "mst_internal.cuh"
+#include "mst_redo.cuh"
 #include "mst_tc_ptx.cuh"
 
 namespace {
@@ -58,6 +59,7 @@ struct Params {
   void* pre;
   int64_t ldpre;
   int tma_out;  // rows leave through shared memory and TMA stores (tensor map tmC) instead of per-thread stores
+  mst_redo redo;          // rows of bf16: sums that are not finite are formed again
   int sampled_stage_min;  // sampled output: a 32 x 32 chunk with at least this many kept entries leaves row by row
 };
 
@@ -102,6 +104,33 @@ __device__ __forceinline__ float gelu_grad_fast(float x) {
   float cdf, e;
   phi_fast(x, cdf, e);
   return fmaf(x * 0.39894228040143268f, e, cdf);
+}
+
+// For calls that want sums that are not finite formed again: this warp's share of the accumulator, ahead of the epilogue that stores it
+// and into the same places.  A pass of its own (a launch with such rows pays 0.1-1.2 us for it: 770 -> 3072 at 8192 tokens 38.8 -> 39.9): the test inside the epilogues cost the
+// fused activation of calls that have no use for it 2 %, and sending these calls through the row-by-row epilogue cost them 14 %.
+__device__ __forceinline__ void redo_tile(const Params& P, uint32_t tmem_base, int acc, int q, int c0, int step, int lane, int64_t m0, int n0, int cols) {
+  const int64_t row0 = m0 + q * 32;
+  const bool row_ok = row0 + lane < P.M;
+#pragma unroll 1
+  for (int c = c0; c < cols / 32; c += step) {
+    const int n = n0 + c * 32;
+    if (n >= P.N) break;  // uniform
+    const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32);
+    uint32_t r[32];
+    tmem_ld32(at, r);
+    float zero = 0.f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(r[j]), 0.f, zero);
+    if (!__any_sync(0xffffffffu, row_ok && zero != 0.f)) continue;
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    mst_redo_square<uint16_t>(P.redo, v, row0 + lane, row_ok, n, P.N);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
+    tmem_st32(at, r);
+  }
 }
 
 // Activation step of one 32-column chunk held in registers (row m, columns n..n+31).  GELU: r <- gelu(r), the
@@ -520,6 +549,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
+      if (P.redo.kind) {   // the chunks this warp stores: pairs of them through the bf16 box
+        const int c0 = (warp - 2) >> 2, pairs = use_tma ? 2 : 1;
+        for (int h = 0; h < pairs; ++h) redo_tile(P, tmem_base, acc, q, c0 * pairs + h, EPI_WARPS / 4 * pairs, lane, m0, n0, BN);
+      }
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                           n0, split, BN);
@@ -798,6 +831,10 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
+      if (P.redo.kind) {   // the chunks this warp stores: pairs of them through the bf16 box
+        const int c0 = (warp - 2) >> 2, pairs = use_tma ? 2 : 1;
+        for (int h = 0; h < pairs; ++h) redo_tile(P, tmem_base, acc, q, c0 * pairs + h, EPI_WARPS / 4 * pairs, lane, m0, n0, J.cols);
+      }
       if (use_tma)
         epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
                           n0, split, J.cols);
@@ -1104,6 +1141,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   P.act = a.epilogue == MST_TC_OUT_BF16 ? a.act : 0;
   P.pre = a.pre;
   P.ldpre = a.ldpre;
+  P.redo = a.redo;
   if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
   P.sampled_stage_min = SAMPLED_STAGE_MIN;
   if (const char* e = mst_getenv(env, "MST_TC_SAMPLED_STAGE")) P.sampled_stage_min = atoi(e);  // measurement override

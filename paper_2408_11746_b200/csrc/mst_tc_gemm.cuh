@@ -29,6 +29,20 @@ __host__ __device__ inline float mst_gelu_grad(float x) {
   return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
+// Operands from which sums that are not finite are formed again (mst_redo.cuh); kind 0: they stay
+enum { MST_REDO_FORWARD = 1, MST_REDO_BACKWARD = 2, MST_REDO_GRADIENT = 3 };
+struct mst_redo {
+  int kind;
+  int wpr;               // products: mask words per row, and the mask
+  const uint32_t* bits;
+  const int32_t* wscan;
+  const void* A;         // products: activations [M x K]; gradient: dY [K x M]
+  int64_t lda;
+  const void* B;         // products: stored values; gradient: X [K x N]
+  int64_t ldb;
+  int64_t K;
+};
+
 struct mst_tc_gemm_args {
   const void* A;
   int64_t lda;
@@ -52,6 +66,7 @@ struct mst_tc_gemm_args {
   int64_t ldpre;
   float* also_sampled;   // F32: the entries under the mask (bits, wscan, wpr) as well, where partial sums are added up anyway;
   bool* sampled;         //      set to true when that was done
+  mst_redo redo;         // BF16 epilogue and mst_tc_split: sums that are not finite are formed again
 };
 
 // C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_prepare.cu; lda / ldb are the pieces'
@@ -63,7 +78,7 @@ double mst_tc_small_clocks(const mst_tc_gemm_args& a);
 // forward product for at most MST_SMALL_FWD_TOKENS tokens (mst_small_fwd.cu)
 constexpr int64_t MST_SMALL_FWD_TOKENS = 16;
 mst_status_t mst_small_fwd(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
-                           int act, void* pre, int64_t ldpre, cudaStream_t s);
+                           int act, void* pre, int64_t ldpre, const mst_redo& redo, cudaStream_t s);
 
 // dY^T X over T tokens with the sizes and the epilogue in `a` (M = O, N = I, K = T; F32 or SAMPLED), operands as the caller
 // has them (mst_dense_grad.cu)

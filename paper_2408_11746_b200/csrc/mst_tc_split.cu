@@ -26,6 +26,7 @@
 #include <cuda.h>
 
 #include "mst_internal.cuh"
+#include "mst_redo.cuh"
 #include "mst_tc_gemm.cuh"
 #include "mst_tc_ptx.cuh"
 
@@ -68,6 +69,7 @@ struct SplitParams {
   const uint32_t* bits;
   const int32_t* wscan;
   int wpr;
+  mst_redo redo;
 };
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
@@ -297,6 +299,19 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
+        if (P.redo.kind) {
+          const bool mine = lane >= rr0 && lane < rr1 && row0 + lane < P.M;
+          float zero = 0.f;
+          if (mine) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) zero = fmaf(box[lane * 33 + j], 0.f, zero);
+          }
+          if (__any_sync(0xffffffffu, zero != 0.f)) {
+            if (PIECES == 3) mst_redo_square<float>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
+            else mst_redo_square<uint16_t>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
+          }
+          __syncwarp();
+        }
         const int end = n + lane >= P.N ? 0 : (int)(P.M - row0 < rr1 ? P.M - row0 : rr1);   // rows of this lane's column
         if (P.epilogue == MST_TC_OUT_SAMPLED) {
           uint32_t word = 0;
@@ -437,6 +452,7 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
   P.bits = a.bits;
   P.wscan = a.wscan;
   P.wpr = a.wpr;
+  P.redo = a.redo;
   if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
   CUtensorMap tmA, tmB;
   const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, pieces, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, pieces, a.M, a.K, a.lda, SBM);
