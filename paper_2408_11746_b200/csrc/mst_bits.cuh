@@ -9,14 +9,19 @@ __device__ __forceinline__ unsigned mst_lanemask_lt() {
   return m;
 }
 
-// x = p[0] + p[1] + p[2] exactly, as bf16 bit patterns: two roundings to nearest leave a remainder of at most 8 bits.  A
-// value that would round to infinity is truncated instead; a non-finite one keeps its pattern and has no remainder.
+// 2^16 x = p[0] + p[1] + p[2] exactly, as bf16 bit patterns: two roundings to nearest leave a remainder of at most 8 bits.  bf16
+// reaches down to 2^-133 only: unscaled, the third piece of an x below 2^-110 would lose bits, with the factor every fp32 value down to
+// the last subnormal (2^-149) has its pieces.  The product of two operands takes MST_SPLIT_UNSCALE off again; values from 2^112 on
+// become infinite here, as sums from 2^95 on do on the way, and those sums are formed again from the operands (mst_redo.cuh).
+// A value that would round to infinity is truncated instead; a non-finite one keeps its pattern and has no remainder.
+constexpr float MST_SPLIT_SCALE = 65536.f, MST_SPLIT_UNSCALE = 1.f / (65536.f * 65536.f);
 __device__ __forceinline__ uint32_t mst_bf16_nearest(float x) {
   const uint32_t u = __float_as_uint(x);
   const uint32_t r = (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;
   return (r & 0x7F80u) == 0x7F80u ? u >> 16 : r;
 }
 __device__ __forceinline__ void mst_split3(float x, uint32_t (&p)[3]) {
+  x *= MST_SPLIT_SCALE;
   const uint32_t u = __float_as_uint(x);
   if ((u & 0x7F800000u) == 0x7F800000u) {
     p[0] = (u & 0x007FFFFFu) ? (u >> 16) | 0x40u : u >> 16;   // a NaN stays a NaN when its low bits go

@@ -6,8 +6,8 @@
 // take (the calls that have always gone over stored entries) therefore look at their sums on the way out: a sum that is not finite
 // is formed again, term by term in fp32, over the stored entries (products) or over the tokens (gradients).  Sums that are finite
 // had only finite terms and are left as they are.
-// The test is one multiply-add per sum by the thread that holds it (3072 x 768 fp32 step at 256 tokens 131.8 -> 134.0 us, 2051 x 1023
-// bf16 at 1999 tokens, all three products, 57.2 -> 58.0).  What follows a find is far slower than the tensor cores (one
+// The test is one multiply-add per sum by the thread that holds it (2051 x 1023 bf16 at 1999 tokens, all three
+// products: 57.1 -> 57.9 us; 3072 x 768 fp32 step at 256 tokens, with the scaled pieces: 131.8 -> 135.0).  What follows a find is far slower than the tensor cores (one
 // warp per 32 x 32 square, from global memory) and bounded by the work of the CUDA-core kernels times a small factor.
 #pragma once
 #include <stdint.h>

@@ -1,5 +1,5 @@
 // fp32 contraction on the 5th-generation tensor cores: every fp32 operand is cut into three bf16 pieces whose sum is
-// exactly the operand (8 + 8 + 8 significand bits), and the product is the sum of the six piece products down to
+// exactly the operand (8 + 8 + 8 significand bits; times 2^16, so that bf16's range holds the last bits of small values), and the product is the sum of the six piece products down to
 // 2^-18 of the leading one.  The three products left out are below 2^-26 of |a b| together, less than the rounding of
 // one fp32 multiplication.
 //
@@ -25,6 +25,7 @@
 // warp 1 issues the MMAs, warps 2-9 own the sums (one row and BN / 2 columns per thread).  Every wait is bounded.
 #include <cuda.h>
 
+#include "mst_bits.cuh"
 #include "mst_internal.cuh"
 #include "mst_redo.cuh"
 #include "mst_tc_gemm.cuh"
@@ -88,9 +89,11 @@ __device__ __forceinline__ void split_cluster_sync() {
 
 // Sums of a 32-column square over the 2^LG blocks of the cluster, this block's 32 / 2^LG rows from rr0 on, into the warp's box: a
 // lane adds four columns of some rows, eight reads whatever the number of blocks, all in flight together, added in range order.
-template <int LG>
-__device__ __forceinline__ void gather_sums(uint32_t sums, int rr0, float* box, int lane) {
+// Returns 0 if this lane's sums are finite, else NaN.
+template <int LG, int PIECES>
+__device__ __forceinline__ float gather_sums(uint32_t sums, int rr0, float* box, int lane) {
   float4 x[8];
+  float zero = 0.f;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int i = lane + 32 * (j >> LG), row = rr0 + (i >> 3);
@@ -103,10 +106,13 @@ __device__ __forceinline__ void gather_sums(uint32_t sums, int rr0, float* box, 
     float4 sum = x[j];
 #pragma unroll
     for (int k = 1; k < 1 << LG; ++k) { sum.x += x[j + k].x; sum.y += x[j + k].y; sum.z += x[j + k].z; sum.w += x[j + k].w; }
+    if (PIECES == 3) { sum.x *= MST_SPLIT_UNSCALE; sum.y *= MST_SPLIT_UNSCALE; sum.z *= MST_SPLIT_UNSCALE; sum.w *= MST_SPLIT_UNSCALE; }
     const int i = lane + 32 * (j >> LG);
     float* d = box + (rr0 + (i >> 3)) * 33 + 4 * (i & 7);
     d[0] = sum.x; d[1] = sum.y; d[2] = sum.z; d[3] = sum.w;
+    zero = fmaf(sum.x, 0.f, fmaf(sum.y, 0.f, fmaf(sum.z, 0.f, fmaf(sum.w, 0.f, zero))));
   }
+  return zero;
 }
 
 // Rows rr0 .. end - 1 of this lane's column of the warp's box, four at a time: read back together, then handed on one by one.  Nothing
@@ -289,27 +295,23 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const int n = n0 + half * COLS + g * 32;
         if (n >= P.N) break;   // uniform
         __syncwarp();
+        float zero = 0.f;   // NaN where a sum is not finite
         if (P.splits > 1) {
-          if (P.splits == 2) gather_sums<1>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
-          else if (P.splits == 4) gather_sums<2>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
-          else gather_sums<3>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
+          if (P.splits == 2) zero = gather_sums<1, PIECES>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
+          else if (P.splits == 4) zero = gather_sums<2, PIECES>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
+          else zero = gather_sums<3, PIECES>(part - (uint32_t)lane * 16u + (uint32_t)(g * 8 * 32) * 16u, rr0, box, lane);
         } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) box[lane * 33 + j] = acc[g * 32 + j];
+          for (int j = 0; j < 32; ++j) zero = fmaf(acc[g * 32 + j], 0.f, zero);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) box[lane * 33 + j] = PIECES == 3 ? acc[g * 32 + j] * MST_SPLIT_UNSCALE : acc[g * 32 + j];
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
-        if (P.redo.kind) {
+        if (P.redo.kind && __any_sync(0xffffffffu, zero != 0.f)) {
           const bool mine = lane >= rr0 && lane < rr1 && row0 + lane < P.M;
-          float zero = 0.f;
-          if (mine) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) zero = fmaf(box[lane * 33 + j], 0.f, zero);
-          }
-          if (__any_sync(0xffffffffu, zero != 0.f)) {
-            if (PIECES == 3) mst_redo_square<float>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
-            else mst_redo_square<uint16_t>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
-          }
+          if (PIECES == 3) mst_redo_square<float>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
+          else mst_redo_square<uint16_t>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
           __syncwarp();
         }
         const int end = n + lane >= P.N ? 0 : (int)(P.M - row0 < rr1 ? P.M - row0 : rr1);   // rows of this lane's column

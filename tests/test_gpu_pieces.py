@@ -49,6 +49,30 @@ def test_fp32_products_are_single_precision(O, I, T):
         assert err <= 5e-7
 
 
+@pytest.mark.parametrize("x,w", [(-118, 0), (0, -118), (-142, 60), (60, -142), (-60, -58), (116, -20), (-20, 116), (100, 10)])
+def test_fp32_pieces_over_the_whole_range(x, w):
+    # operands of size 2^x (activations, upstream gradients) and 2^w (weights; the other gradient operand), down to subnormal ones and
+    # up to where sums pass 2^95; results stay in the normal range and keep single precision relative to the sum of their terms' sizes
+    O, I, T = 130, 200, 140
+    g = torch.Generator(device="cuda").manual_seed(x - w)
+    n = lambda e, *s: (torch.randn(*s, generator=g, device="cuda", dtype=torch.double) * 2.0 ** e).float()
+    X, dY, W, V = n(x, T, I), n(x, T, O), n(w, O, I), n(w, T, I)
+    M = (torch.rand(O, I, generator=g, device="cuda") < 0.4).to(torch.uint8)
+    L = mst.Layer(0, O, I, mst.MST_F32)
+    L.pack(W, M)
+    Y, dX = torch.zeros(T, O, device="cuda"), torch.zeros(T, I, device="cuda")
+    dW, G = torch.zeros(L.nnz, device="cuda"), torch.zeros(O, I, device="cuda")
+    L.fwd(X, Y, T)
+    L.bwd_x(dY, dX, T)
+    L.sddmm(dY, V, T, dW)
+    L.dense_grad(dY, V, T, G)
+    Wr = (W * M).double()
+    Gr = dY.double().T @ V.double()
+    for got, ref in ((Y, X.double() @ Wr.T), (dX, dY.double() @ Wr), (G, Gr), (dW, Gr[M.bool()])):
+        assert _rel(got, ref) <= 5e-7
+    L.close()
+
+
 def test_fp32_extreme_magnitudes():
     # pieces of values near the top and the bottom of the normal range; sums stay finite
     O, I, T = 70, 66, 40
