@@ -88,8 +88,7 @@ extern "C" mst_status_t mst_layer_create(mst_layer_t** out, int32_t layer_id, in
   const size_t o_rand = cv.take(4 * (size_t)L->nwords);
   const size_t o_cnt = cv.take(4 * (size_t)(wmax + 1));
   const size_t o_scan = cv.take(4 * (size_t)(wmax + 1));
-  const int64_t n_bsum = mst_scan_block_sums_len(wmax) + 1024, n_pack = L->nwords / 256 + 2;   // scan partials; counts of pack's blocks
-  const size_t o_bsum = cv.take(4 * (size_t)(n_bsum > n_pack ? n_bsum : n_pack));
+  const size_t o_bsum = cv.take(4 * (size_t)(mst_scan_block_sums_len(wmax) + 1024));
   const size_t o_hist = cv.take(4 * (size_t)MST_SELECT_BINS * 5);
   int64_t rand_cap = N / 64;
   if (rand_cap < 2048) rand_cap = 2048;

@@ -126,7 +126,7 @@ __global__ void scan_empty(int32_t* out) { out[0] = 0; }
 
 // ---- pack: byte mask -> bit mask -> CSR in two launches ----------------------------------------------------------------------
 // Launch 1 turns 256 mask words per block into bits and leaves the block's entry count; launch 2 adds up the counts of the
-// blocks before its own, scans its words and writes their part of the structure, one warp per word (lane = bit: reads of
+// blocks before its own (of many blocks: reads their scan), scans its words and writes their part of the structure, one warp per word (lane = bit: reads of
 // W and writes of the compacted arrays are coalesced), eight words in flight, or half a word per thread where there are few entries.
 // 4096 x 1024 bf16, d = 0.1, with its export: 31 us with whole words only (a warp instruction per word and array, a tenth of its lanes at
 // work), 24 us with half words; separate bits, popcounts, three-kernel scans (twice) and one-word-per-warp fill, eleven launches, 106 us.
@@ -181,10 +181,10 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_bits_kernel(const uint8_t* 
   if (threadIdx.x == 0) sums[blockIdx.x] = r;
 }
 
-// Entries at positions >= cap are counted but not written.  *total receives the number of entries (device memory or mapped host
+// sums: the blocks' counts, or with `scanned` the counts before each of them.  Entries at positions >= cap are counted but not written.  *total receives the number of entries (device memory or mapped host
 // memory); wscan may be NULL.
 template <typename V, typename COL>
-__global__ void __launch_bounds__(PACK_THREADS) pack_fill_kernel(const uint32_t* __restrict__ bits, const int32_t* __restrict__ sums, int O,
+__global__ void __launch_bounds__(PACK_THREADS) pack_fill_kernel(const uint32_t* __restrict__ bits, const int32_t* __restrict__ sums, int scanned, int O,
                                                                  int wpr, const V* __restrict__ W, int64_t ldw, int64_t cap,
                                                                  int32_t* __restrict__ wscan, int32_t* __restrict__ row_ptr,
                                                                  COL* __restrict__ col_idx, V* __restrict__ vals, volatile int32_t* total) {
@@ -196,8 +196,12 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_fill_kernel(const uint32_t*
   mst_grid_dependency_wait();
   const int64_t nwords = (int64_t)O * wpr, w0 = (int64_t)blockIdx.x * PACK_WORDS;
   int before = 0;
-  for (int j = threadIdx.x; j < (int)blockIdx.x; j += PACK_THREADS) before += sums[j];
-  before = block_reduce_sum(before, sh);
+  if (scanned) {
+    before = sums[blockIdx.x];
+  } else {
+    for (int j = threadIdx.x; j < (int)blockIdx.x; j += PACK_THREADS) before += sums[j];
+    before = block_reduce_sum(before, sh);
+  }
   if (threadIdx.x == 0) before_sh = before;
   const int64_t my_w = w0 + threadIdx.x;
   const uint32_t my_bits = my_w < nwords ? bits[my_w] : 0u;
@@ -499,14 +503,22 @@ struct PinnedWord {
 };
 thread_local PinnedWord t_pack_total;
 
+// Blocks from which their counts are scanned by launches of their own: each block adding up what lies before it saves those launches,
+// but its reads grow with the square of the blocks.  bf16, d = 0.05, added up / scanned: 26 / 36 us at 1120 blocks, 87 / 90 at 8192,
+// 164 / 149 at 16384, 792 / 498 at 65536, 6650 / 1892 at 262140.
+constexpr unsigned PACK_SCAN_BLOCKS = 10240;
+
+// counts, scan: room for a word per block and one more (scan may be NULL below PACK_SCAN_BLOCKS); partials: for the scan
 template <typename V, typename COL>
-mst_status_t launch_pack(const uint8_t* mask, int O, int I, int wpr, const void* W, int64_t ldw, int64_t cap, uint32_t* bits, int32_t* sums,
-                         int32_t* wscan, int32_t* row_ptr, COL* col_idx, void* vals, int32_t* total, cudaStream_t s) {
+mst_status_t launch_pack(const uint8_t* mask, int O, int I, int wpr, const void* W, int64_t ldw, int64_t cap, uint32_t* bits, int32_t* counts,
+                         int32_t* scan, int32_t* partials, int32_t* wscan, int32_t* row_ptr, COL* col_idx, void* vals, int32_t* total, cudaStream_t s) {
   const unsigned blocks = blocks_for((int64_t)O * wpr, PACK_WORDS);
   const int vec = (I % 32 == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0) ? 1 : 0;
-  MST_CUDA_TRY(mst_launch_overlapped(pack_bits_kernel, dim3(blocks), dim3(PACK_THREADS), 0, s, mask, O, I, wpr, vec, bits, sums));
+  MST_CUDA_TRY(mst_launch_overlapped(pack_bits_kernel, dim3(blocks), dim3(PACK_THREADS), 0, s, mask, O, I, wpr, vec, bits, counts));
+  const int scanned = scan && blocks >= PACK_SCAN_BLOCKS ? 1 : 0;
+  if (scanned) MST_TRY(mst_scan_i32(counts, scan, blocks, partials, s));
   MST_CUDA_TRY(mst_launch_overlapped(pack_fill_kernel<V, COL>, dim3(blocks), dim3(PACK_THREADS), 0, s, (const uint32_t*)bits,
-                                     (const int32_t*)sums, O, wpr, (const V*)W, ldw, cap, wscan, row_ptr, col_idx, (V*)vals,
+                                     (const int32_t*)(scanned ? scan : counts), scanned, O, wpr, (const V*)W, ldw, cap, wscan, row_ptr, col_idx, (V*)vals,
                                      (volatile int32_t*)total));
   return MST_OK;
 }
@@ -534,11 +546,11 @@ extern "C" mst_status_t mst_pack(mst_layer_t* L, const void* W_dense, int64_t ld
   int32_t* total = t_pack_total.get();
   if (!total) return MST_ERR_CUDA;
   if (L->dtype == MST_F32)
-    MST_TRY((launch_pack<float, uint16_t>(mask, L->O, L->I, L->wpr, W_dense, ldw, L->cap, L->bits[set], L->block_sums, L->wscan[set],
-                                          L->row_ptr[set], L->col_idx[set], L->vals[set], total, s)));
+    MST_TRY((launch_pack<float, uint16_t>(mask, L->O, L->I, L->wpr, W_dense, ldw, L->cap, L->bits[set], L->word_cnt, L->word_scan,
+                                          L->block_sums, L->wscan[set], L->row_ptr[set], L->col_idx[set], L->vals[set], total, s)));
   else
-    MST_TRY((launch_pack<uint16_t, uint16_t>(mask, L->O, L->I, L->wpr, W_dense, ldw, L->cap, L->bits[set], L->block_sums, L->wscan[set],
-                                             L->row_ptr[set], L->col_idx[set], L->vals[set], total, s)));
+    MST_TRY((launch_pack<uint16_t, uint16_t>(mask, L->O, L->I, L->wpr, W_dense, ldw, L->cap, L->bits[set], L->word_cnt, L->word_scan,
+                                             L->block_sums, L->wscan[set], L->row_ptr[set], L->col_idx[set], L->vals[set], total, s)));
   MST_CUDA_TRY(cudaStreamSynchronize(s));
   const int32_t n = *(volatile int32_t*)total;
   if (n > L->cap) return MST_ERR_CAPACITY;
@@ -601,6 +613,7 @@ namespace {
 constexpr int64_t NOALLOC_MAX_NUMEL = (int64_t)1 << 22;  // 4 194 304 entries, e.g. a 4096 x 1024 layer
 constexpr int64_t NOALLOC_MAX_WORDS = (int64_t)1 << 18;  // >= numel/32 + rows for every shape accepted below
 constexpr int64_t NOALLOC_SUMS = NOALLOC_MAX_WORDS / PACK_WORDS + 2;
+static_assert(NOALLOC_MAX_WORDS / PACK_WORDS < PACK_SCAN_BLOCKS, "the counts are added up without a scan");
 constexpr size_t NOALLOC_OFF_BITS = 0;
 constexpr size_t NOALLOC_OFF_SUMS = NOALLOC_OFF_BITS + 4 * (size_t)NOALLOC_MAX_WORDS;
 constexpr size_t NOALLOC_BYTES = NOALLOC_OFF_SUMS + 4 * (size_t)(NOALLOC_SUMS + 62);
@@ -644,6 +657,6 @@ extern "C" mst_status_t mst_mask_to_csr_noalloc(int32_t O, int32_t I, mst_dtype_
   cudaStream_t s = (cudaStream_t)stream;
   // every word of the scratch that the second launch reads is written by the first: nothing needs clearing
   if (dtype == MST_F32)
-    return launch_pack<float, int32_t>(mask, O, I, wpr, W_dense, ldw, nnz_capacity, bits, sums, nullptr, row_ptr, col_idx, vals, nullptr, s);
-  return launch_pack<uint16_t, int32_t>(mask, O, I, wpr, W_dense, ldw, nnz_capacity, bits, sums, nullptr, row_ptr, col_idx, vals, nullptr, s);
+    return launch_pack<float, int32_t>(mask, O, I, wpr, W_dense, ldw, nnz_capacity, bits, sums, nullptr, nullptr, nullptr, row_ptr, col_idx, vals, nullptr, s);
+  return launch_pack<uint16_t, int32_t>(mask, O, I, wpr, W_dense, ldw, nnz_capacity, bits, sums, nullptr, nullptr, nullptr, row_ptr, col_idx, vals, nullptr, s);
 }

@@ -725,3 +725,23 @@ def test_update_many_checks_every_layer_first():
     for x, y in zip(before, export_csr(L1, "bf16")):
         np.testing.assert_array_equal(x, y)
     L1.close(); L2.close()
+
+
+# ------------------------------------------------------------ layers whose blocks are too many to add up one another's counts
+@pytest.mark.parametrize("O,I", [(20478, 4096), (20480, 4096), (41000, 2050)])     # 10239, 10240 and 10410 blocks
+def test_pack_of_a_large_layer(O, I):
+    g = torch.Generator(device="cuda").manual_seed(O)
+    M = (torch.randint(0, 100, (O, I), generator=g, device="cuda", dtype=torch.uint8) == 0).to(torch.uint8)
+    W = torch.randn(O, I, generator=g, device="cuda", dtype=torch.bfloat16)
+    nnz = int(M.sum(dtype=torch.int64))
+    L = mst.Layer(0, O, I, mst.MST_BF16, nnz)
+    L.pack(W, M)
+    rp = torch.zeros(O + 1, dtype=torch.int32, device="cuda")
+    ci = torch.zeros(nnz, dtype=torch.int32, device="cuda")
+    vv = torch.zeros(nnz, dtype=torch.bfloat16, device="cuda")
+    mst.mst_export_csr(L.handle, rp, ci, vv)
+    at = M.nonzero()
+    assert L.nnz == nnz and int(rp[0]) == 0
+    assert torch.equal(rp[1:].long(), M.sum(1, dtype=torch.int64).cumsum(0))
+    assert torch.equal(ci.long(), at[:, 1]) and torch.equal(vv, W[at[:, 0], at[:, 1]])
+    L.close()
