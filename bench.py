@@ -536,7 +536,7 @@ def run_profile_case(args) -> None:
 
 # ------------------------------------------------------------------------------------------ other workloads
 def other_legs(reps: int, dev):
-    """Timed legs of the workloads the headline does not cover: the single fp32 layer (CUDA-core kernels), the
+    """Timed legs of the workloads the headline does not cover: the single fp32 layer (bf16 pieces on the tensor cores), the
     GPT-2-small block at density 0.25, and one block of the ultra-sparse Zipf workload with an update every step."""
     import torch
     import paper_2408_11746_b200 as mst
@@ -575,7 +575,7 @@ def other_legs(reps: int, dev):
         t_prod, _ = median_ms(products, reps)
         useful = sum(6.0 * p.tokens * p.nnz for _, p, *_ in slots)
         res = {"workload": label, "fwd_bwd_ms": round(t_prod, 4), "fwd_bwd_useful_tflops": round(useful / (t_prod * 1e-3) / 1e12, 3),
-               "paths": sorted({mst.path_name(s[0].path_in_use()) for s in slots})}
+               "paths": sorted({mst.path_name(s[0].path_in_use()) if s[1].dtype == "bf16" else "bf16_pieces" for s in slots})}
         if update:
             t_all, _ = median_ms(whole, reps)
             res["step_with_dense_grad_and_update_ms"] = round(t_all, 4)
@@ -592,7 +592,7 @@ def other_legs(reps: int, dev):
             s[0].close()
         return res
 
-    legs = [leg(mst_inputs.config1(), True, 0.3, "single fp32 layer 768->3072, T=256, d=0.25 (CUDA-core kernels)"),
+    legs = [leg(mst_inputs.config1(), True, 0.3, "single fp32 layer 768->3072, T=256, d=0.25 (bf16 pieces on the tensor cores)"),
             leg(mst_inputs.config2(), True, 0.3, "gpt2-small block, T=8192, bf16, uniform d=0.25"),
             leg(mst_inputs.config3(blocks=1), True, 0.1,
                 "ultra-sparse gpt2-small block 0, T=8192, bf16, Zipf(1.1) rows, d in [0.03, 0.10], update every step")]

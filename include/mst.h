@@ -76,12 +76,13 @@ typedef struct {
 } mst_update_stats_t;
 
 /* Create an empty layer.  out_features, in_features in [1, 65535]; nnz_capacity in [1, O*I].
- * Allocates all device memory the layer will ever use on the current device. */
+ * Allocates the structure and the update's scratch on the current device; the CSC view, the dense image that value tracking
+ * keeps and the structured-sparse operands are allocated when a call first needs them. */
 mst_status_t mst_layer_create(mst_layer_t** layer, int32_t layer_id, int32_t out_features, int32_t in_features,
                               mst_dtype_t dtype, int64_t nnz_capacity);
 mst_status_t mst_layer_destroy(mst_layer_t* layer);
 
-/* Which kernels serve forward, input gradient and weight gradient of a bf16 layer:
+/* Which kernels serve forward, input gradient and weight gradient of a bf16 layer (fp32 layers: below):
  *   MST_PATH_CUDA_CORE    the sparse kernels (work proportional to nnz, fp32 FMA pipe)
  *   MST_PATH_TENSOR_CORE  dense-tile kernels: W.M is expanded on the fly to a dense bf16 image and contracted on the
  *                         tensor cores (work proportional to O*I, about 18x the FMA pipe's rate); the weight gradient
@@ -94,8 +95,7 @@ mst_status_t mst_layer_destroy(mst_layer_t* layer);
  *                         Exact for any mask; pays off while few groups hold more than two entries (density up to
  *                         about 0.25).  Needs nnz <= O*I/4 and aligned operands, otherwise the dense tiles are used.
  *                         The weight gradient stays the dense contraction sampled on the mask.
- *   MST_PATH_AUTO         (default) bf16 layers with aligned operands: the structured-sparse instruction at densities
- *                         where it was measured faster than dense tiles, dense tiles above; CUDA cores otherwise.
+ *   MST_PATH_AUTO         (default) the dense tiles, whatever the density and the alignment of the operands.
  * fp32 layers keep single-precision arithmetic whatever the path: on MST_PATH_CUDA_CORE in FMA chains, otherwise as sums of
  * products of exact bf16 pieces on the tensor cores (three pieces per operand, rounded fp32 sums every 64 terms; at
  * least as close to the exact product as the FMA chains).  Results of the paths agree within the stated tolerance, not
@@ -107,8 +107,8 @@ mst_status_t mst_layer_destroy(mst_layer_t* layer);
 typedef enum { MST_PATH_AUTO = 0, MST_PATH_CUDA_CORE = 1, MST_PATH_TENSOR_CORE = 2, MST_PATH_SPARSE_TC = 3 } mst_compute_path_t;
 mst_status_t mst_set_compute_path(mst_layer_t* layer, mst_compute_path_t path);
 
-/* The kernels forward and input gradient of this layer run on, with MST_PATH_AUTO resolved.  fp32 layers report
- * MST_PATH_CUDA_CORE: none of the bf16 paths applies to them. */
+/* Which of the bf16 kernel families forward and input gradient of this layer run on, with MST_PATH_AUTO resolved.  fp32
+ * layers run on none of them and always report MST_PATH_CUDA_CORE, also where they multiply on the tensor cores (above). */
 mst_status_t mst_layer_path_in_use(const mst_layer_t* layer, mst_compute_path_t* path);
 
 /* Kernels the library has enqueued in this process so far (all layers, all streams): for launch accounting. */
@@ -120,7 +120,7 @@ mst_status_t mst_layer_nnz(const mst_layer_t* layer, int64_t* nnz);
 /* Dense mask -> sparse structure (Sec. 3.2: the binary mask M_theta; Algorithm 1: theta <- theta . M).
  *   W_dense  device, [O x ldw] in the layer's dtype; only entries under the mask are read
  *   mask     device, uint8 [O x I] contiguous, non-zero = active
- * Builds CSR, the CSC view and the bit mask.  Synchronises the stream (returns nnz to the host);
+ * Builds CSR and the bit mask (the CSC view when something needs it: MST_PATH_CUDA_CORE, mst_export_csc, mst_validate).  Synchronises the stream (returns nnz to the host);
  * MST_ERR_CAPACITY if the mask holds more than nnz_capacity entries (layer left unpacked). */
 mst_status_t mst_pack(mst_layer_t* layer, const void* W_dense, int64_t ldw, const uint8_t* mask, mst_stream_t stream);
 
@@ -157,7 +157,7 @@ mst_status_t mst_spmm_fwd(const mst_layer_t* layer, const void* X, int64_t ldx, 
                           mst_stream_t stream);
 
 /* Input gradient, dX[t,i] = sum_{o:(o,i) in M} dY[t,o] W[o,i]   (App. "FLOP Calculation": backward = 2 x forward).
- * dY device [T x lddy], dX device [T x lddx].  Uses the CSC view: a gather, no floating-point atomics. */
+ * dY device [T x lddy], dX device [T x lddx].  No floating-point atomics on any path (CUDA cores: a gather over the CSC view). */
 mst_status_t mst_spmm_bwd_x(const mst_layer_t* layer, const void* dY, int64_t lddy, int64_t T, void* dX, int64_t lddx,
                             mst_stream_t stream);
 

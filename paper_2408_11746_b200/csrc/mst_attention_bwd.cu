@@ -10,12 +10,12 @@
 //   1. dQ, query-centric: a block owns 128 queries of one (sequence, head) and walks 64-key tiles.  It forms delta first and
 //      leaves (-lse log2 e, delta) of its rows in the scratch buffer for the second launch.
 //   2. dK and dV, key-centric: a block owns 128 keys and walks the 64-query tiles that see them, on the transposed scores.
-// Roles of a block's eighteen warps:
-//   warps 0-15 algebra: thread = own row (tensor-memory lane), the four warps of a lane quarter share the tile's 64 columns.
+// Roles of a block's ten warps:
+//   warps 0-7  algebra: thread = own row (tensor-memory lane), the two warps of a lane quarter take 32 of a tile's 64 columns each.
 //              Scores and dP come from tensor memory, dS (and P) go back as bf16 and are the A operand of the second products
 //              where they lie, so nothing score-shaped passes through shared memory;
-//   warp 16    one lane feeds a four-tile ring by TMA;
-//   warp 17    one lane issues tcgen05.mma: S = Q K^T, dP = dOut V^T (128 x 64), then dQ += dS K, or dV += P^T dOut, dK += dS^T Q.
+//   warp 8     one lane feeds a four-tile ring by TMA;
+//   warp 9     one lane issues tcgen05.mma: S = Q K^T, dP = dOut V^T (128 x 64), then dQ += dS K, or dV += P^T dOut, dK += dS^T Q.
 // 256 columns of tensor memory and 102 KiB of shared memory: two blocks per SM, so that one block's products run while
 // the other's algebra does.  The far strided positions (i - 2l, i - 3l, ...: one key per query and distance) are visited
 // after the window as tiles of which only the diagonal counts: warp-level mma.sync products of 16 rows each, whose sums are
@@ -46,13 +46,13 @@ constexpr int TMEM_COLS = 256;
 __device__ int g_bwd_error = 0;
 
 struct BwdParams {
-  const __nv_bfloat16 *Q, *K, *V, *Out, *dOut;
+  const __nv_bfloat16* Out;
   int64_t ldo;
   const float* lse;    // [batch, heads, seq]
   float* stat;         // [batch, heads, seq / 64][2][64]: -lse log2 e, -delta
   __nv_bfloat16 *dQ, *dK, *dV;
   int64_t ldg;
-  int batch, seq, heads, stride, tiles;   // tiles of 128 rows per sequence
+  int seq, heads, stride;
   uint32_t magic;
 };
 
@@ -622,19 +622,17 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
   void* ws = nullptr;
   MST_TRY(mst_workspace_kind(MST_WS_ATTENTION, 2 * sizeof(float) * (size_t)rows * heads, &ws));
   BwdParams P;
-  P.Q = (const __nv_bfloat16*)Q; P.K = (const __nv_bfloat16*)K; P.V = (const __nv_bfloat16*)V;
-  P.Out = (const __nv_bfloat16*)Out; P.dOut = (const __nv_bfloat16*)dOut;
+  P.Out = (const __nv_bfloat16*)Out;
   P.ldo = ldo;
   P.lse = lse; P.stat = (float*)ws;
   P.dQ = (__nv_bfloat16*)dQ; P.dK = (__nv_bfloat16*)dK; P.dV = (__nv_bfloat16*)dV;
   P.ldg = ldg;
-  P.batch = batch; P.seq = seq_len; P.heads = heads;
+  P.seq = seq_len; P.heads = heads;
   P.stride = stride < seq_len ? stride : seq_len;   // from there on the same pairs: all earlier positions
   P.magic = stride_magic(P.stride, seq_len);
-  P.tiles = (seq_len + ROWS - 1) / ROWS;
   MST_SMEM_LIMIT((attn_bwd_dq_kernel), SMEM_BYTES);
   MST_SMEM_LIMIT((attn_bwd_dkv_kernel), SMEM_BYTES);
-  dim3 grid((unsigned)P.tiles, (unsigned)heads, (unsigned)batch);
+  dim3 grid((unsigned)((seq_len + ROWS - 1) / ROWS), (unsigned)heads, (unsigned)batch);
   MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dq_kernel, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, P));
   MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dkv_kernel, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, P));
   MST_CUDA_TRY(cudaGetLastError());

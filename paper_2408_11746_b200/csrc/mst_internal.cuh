@@ -136,9 +136,8 @@ struct mst_layer {
   uint16_t* col_idx[2];  // [cap]
   void* vals[2];         // [cap] layer dtype
 
-  // CSC view of the live structure.  Built at pack; the fused update skips it for layers whose input gradient runs
-  // on the tensor path (which reads the dense image, not the CSC view) and it is then rebuilt on first use.
-  // Allocated on first use (mst_alloc_csc): layers that never leave the tensor path never pay for it.
+  // CSC view of the live structure.  Pack and the update build it for layers on the CUDA-core path only (the tensor paths read
+  // the dense image); otherwise it is built, and allocated (mst_alloc_csc), on first use.
   mutable int csc_valid;
   unsigned char* csc_base;  // the view's own allocation, nullptr until it is needed
   uint32_t* bitsT;       // [nwordsT]

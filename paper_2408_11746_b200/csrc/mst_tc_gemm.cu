@@ -1,6 +1,6 @@
 // bf16 contraction on the 5th-generation tensor cores (tcgen05) with fp32 accumulators in tensor memory.
 //
-// One persistent block per SM, 192 threads in three roles:
+// One persistent block per SM, 320 threads in three roles:
 //   warp 0     producer: one lane issues TMA tile loads (cp.async.bulk.tensor, 128-byte swizzle) into a 4-stage
 //              shared-memory ring, signalling "full" mbarriers by transaction bytes;
 //   warp 1     one lane issues tcgen05.mma (M=128, N=256, K=16 per instruction) from shared-memory descriptors
@@ -1048,11 +1048,11 @@ int mst_tc_pick_splits(int64_t tiles, int64_t slots, int64_t kblocks, double out
 //                   buffer, so two such calls must not overlap on the GPU (mst_dense_grad, mst_dense_grad_dw,
 //                   mst_sddmm_dw and the host-step calls on the tensor path): keep them on one stream or order them
 //                   with events.
-//   MST_WS_COLUMNS  feature-major copies of activations for the structured-sparse path and the CUDA-core kernels
-//                   (same rule).
+//   MST_WS_COLUMNS  operands prepared for one call: pieces of fp32 rows, aligned copies of bf16 rows, feature-major copies of
+//                   activations for the structured-sparse path and the CUDA-core kernels (same rule).
 //   MST_WS_ATTENTION  per-row dot products of the attention backward pass (same rule).
-//   MST_WS_IMAGE    dense bf16 image of W.M of the layer being multiplied, for layers without value tracking
-//                   (same rule).
+//   MST_WS_IMAGE    dense image of W.M (bf16, or the three pieces) of the layer being multiplied, for layers without
+//                   value tracking (same rule).
 mst_status_t mst_workspace_kind(int kind, size_t bytes, void** ptr) {
   constexpr int MAX_DEVICES = 64;
   static void* buf[MST_WS_KINDS][MAX_DEVICES] = {};

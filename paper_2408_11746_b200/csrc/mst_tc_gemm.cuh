@@ -86,7 +86,7 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
                              cudaStream_t s);
 
 // Returns MST_ERR_SHAPE when the operands cannot be described to the TMA unit (leading dimension or base address
-// not 16-byte aligned); the caller then falls back to the CUDA-core kernel.
+// not 16-byte aligned); callers pass aligned copies of such rows (mst_prepare).
 mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s);
 bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb);
 
@@ -102,6 +102,6 @@ int mst_tc_pick_splits(int64_t tiles, int64_t slots, int64_t kblocks, double out
 // Process-wide scratch buffer for handle-less entry points (grows on demand; growing synchronises the device).
 // Calls that use it must not overlap on the GPU.
 mst_status_t mst_workspace(size_t bytes, void** ptr);
-// The same per purpose: split partial sums, feature-major activation columns of the structured-sparse path.
+// The same per purpose (mst_tc_gemm.cu).
 enum { MST_WS_SPLIT = 0, MST_WS_COLUMNS = 1, MST_WS_ATTENTION = 2, MST_WS_IMAGE = 3, MST_WS_KINDS = 4 };
 mst_status_t mst_workspace_kind(int kind, size_t bytes, void** ptr);

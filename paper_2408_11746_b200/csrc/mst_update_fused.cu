@@ -383,7 +383,7 @@ __device__ void u_sweep(const ULayer& L, uint32_t lo_w, int nloc, bool fastA, bo
     // A lane takes four neighbouring columns, eight lanes a mask word: one 16-byte load and one test of the four magnitudes
     // against the bracket's outer edge settle most groups.
     const int pad = L.wpr * 32 - L.I;
-    const uint32_t gl = sh.lo[1], gw = sh.hi[1] - sh.lo[1], outer = UKEY_END - sh.hi[1];   // |g| bits at or above it: inside or sure
+    const uint32_t gl = sh.lo[1], outer = UKEY_END - sh.hi[1];   // |g| bits at or above it: inside or sure
     const uint32_t wpr = (uint32_t)L.wpr;
     const int I = L.I;
     const float* __restrict__ G = L.G;

@@ -38,10 +38,8 @@ def _run(p, stride, want_lse=True, pad=0):
     (3, 256, 2, 256, 8),       # stride = n: plain causal attention inside one window; padded leading dimensions
     (2, 128, 1, 128, 0),       # a single query block
     (1, 1024, 1, 128, 0),      # seven strided positions
-    (1, 2048, 2, 256, 0)])     # the longest sequence the tensor-memory kernel takes for l = 256: six positions outside the tile
-@pytest.mark.parametrize("kernel", ["warp", "tcgen05"])
-def test_forward_matches_oracle(batch, seq, heads, stride, pad, kernel, monkeypatch):
-    monkeypatch.setenv("MST_ATTN_FWD", kernel)
+    (1, 2048, 2, 256, 0)])     # six strided positions outside the window
+def test_forward_matches_oracle(batch, seq, heads, stride, pad):
     _check_forward(batch, seq, heads, stride, pad)
 
 
@@ -52,7 +50,7 @@ def test_forward_matches_oracle(batch, seq, heads, stride, pad, kernel, monkeypa
     (1, 1024, 1, 512, 0),      # window longer than a block's span
     (2, 256, 2, 1024, 0),      # stride beyond the sequence: plain causal attention
     (1, 4096, 1, 128, 0)])     # 31 strided positions
-def test_forward_strides_of_the_warp_level_kernel(batch, seq, heads, stride, pad):
+def test_forward_odd_short_and_long_strides(batch, seq, heads, stride, pad):
     _check_forward(batch, seq, heads, stride, pad)
 
 
@@ -77,9 +75,7 @@ def _check_forward(batch, seq, heads, stride, pad, seed=None):
     np.testing.assert_array_equal(out[:, :, 0], V[:, :, 0])
 
 
-@pytest.mark.parametrize("kernel", ["warp", "tcgen05"])
-def test_larger_scores_and_run_to_run_identity(kernel, monkeypatch):
-    monkeypatch.setenv("MST_ATTN_FWD", kernel)
+def test_larger_scores_and_run_to_run_identity():
     p = mst_inputs.attention_problem(2, 512, 2, 64, seed=77, std=2.0)      # scaled scores of variance 16: peaked rows
     a, _ = _run(p, 256, want_lse=False)
     b, _ = _run(p, 256, want_lse=False)
@@ -89,10 +85,8 @@ def test_larger_scores_and_run_to_run_identity(kernel, monkeypatch):
     assert rel_err(a, ref) <= TOL["bf16"]
 
 
-@pytest.mark.parametrize("kernel", ["warp", "tcgen05"])
 @pytest.mark.parametrize("stride", [256, 128])
-def test_gpt2_small_full_size_sampled(stride, kernel, monkeypatch):
-    monkeypatch.setenv("MST_ATTN_FWD", kernel)
+def test_gpt2_small_full_size_sampled(stride):
     # 16 sequences of 1024 tokens, 12 heads: the attention input of the benchmark's 16384-token batch
     rng = np.random.default_rng(12 + stride)
     p = mst_inputs.attention_problem(16, 1024, 12, 64)

@@ -675,7 +675,7 @@ def test_path_in_use_reports_the_resolved_path():
     L.close()
     q = _problem(64, 64, 8, "f32", 0.1, 1)
     L = make_layer(q)
-    assert L.path_in_use() == mst.MST_PATH_CUDA_CORE             # fp32 layers never leave the CUDA cores
+    assert L.path_in_use() == mst.MST_PATH_CUDA_CORE             # of the bf16 families none: the value says nothing more
     L.close()
 
 

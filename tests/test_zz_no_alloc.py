@@ -6,6 +6,8 @@ them from a fixed work area inside the library.  Because that area is shared and
 left in it, the check is made on two calls in a row with different layers: the second must not be disturbed by the
 leftovers of the first.  The file name sorts last so that it runs after every other test.
 """
+import gc
+
 import numpy as np
 import pytest
 
@@ -35,6 +37,7 @@ def _noalloc_csr(p, capacity):
         _warmed.append(True)
     # the call's contract: no device memory is allocated or freed, neither through torch's allocator nor around it
     torch.cuda.synchronize()
+    gc.collect()     # tensors that earlier tests left in reference cycles are not freed between the two readings
     free0, _ = torch.cuda.mem_get_info()
     stats0 = torch.cuda.memory_stats()
     mst.mst_mask_to_csr_noalloc(O, I, mdtype(p), W, I, M, capacity, rp, ci, vv)
