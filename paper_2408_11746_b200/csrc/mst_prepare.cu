@@ -185,6 +185,11 @@ mst_status_t mst_prepare(mst_dtype_t dtype, const mst_image_job* image, const ms
   if (blocks == 0) return MST_OK;
   MST_CUDA_TRY(dtype == MST_F32 ? mst_launch_overlapped(prepare_kernel<float>, dim3(blocks), dim3(256), 0, s, im, part[0], part[1])
                                 : mst_launch_overlapped(prepare_kernel<uint16_t>, dim3(blocks), dim3(256), 0, s, im, part[0], part[1]));
+  // only now: a call that fails before its launch (no memory for its rows, say) must not leave an unbuilt image behind as valid
+  if (image && image->out && image->out == image->layer->dense_w) {
+    image->layer->dense_version = image->layer->version;
+    image->layer->dense_epoch = image->layer->values_epoch;
+  }
   return MST_OK;
 }
 
@@ -205,8 +210,6 @@ mst_status_t mst_image(const mst_layer* L, mst_image_job* job, const uint16_t** 
     MST_TRY(mst_alloc_dense(const_cast<mst_layer*>(L)));
     *image = L->dense_w;
     if (L->dense_version == L->version && L->dense_epoch == L->values_epoch) return MST_OK;
-    L->dense_version = L->version;
-    L->dense_epoch = L->values_epoch;
     job->out = L->dense_w;
   } else {
     void* ws = nullptr;

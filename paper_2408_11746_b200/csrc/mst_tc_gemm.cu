@@ -1068,7 +1068,9 @@ mst_status_t mst_workspace_kind(int kind, size_t bytes, void** ptr) {
       cap[kind][dev] = 0;
     }
     const size_t want = (bytes + ((size_t)1 << 20)) & ~(((size_t)1 << 20) - 1);
-    MST_CUDA_TRY(cudaMalloc(&buf[kind][dev], want));
+    const cudaError_t got = cudaMalloc(&buf[kind][dev], want);
+    if (got != cudaSuccess) cudaGetLastError();   // reported by the status: a later call must not find it again
+    MST_CUDA_TRY(got);
     cap[kind][dev] = want;
   }
   *ptr = buf[kind][dev];

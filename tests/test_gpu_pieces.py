@@ -198,3 +198,25 @@ def test_activation_rows_of_a_partial_tile(O, I, T):
     p = pre.double().requires_grad_(True)
     torch.nn.functional.gelu(p).sum().backward()
     assert _rel(Y, product) < 4e-3 and _rel(H, torch.nn.functional.gelu(product)) < 4e-3 and _rel(D, product * p.grad) < 4e-3
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_a_call_without_memory_leaves_no_image_behind(dtype):
+    # the first call of a layer with value tracking asks for more scratch than the GPU has and is refused; the next one builds the
+    # image all the same
+    O, I, T = 96, 65, 50
+    dt, mdt = (torch.float32, mst.MST_F32) if dtype == "f32" else (torch.bfloat16, mst.MST_BF16)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X, W = torch.randn(T, I, generator=g, device="cuda").to(dt), torch.randn(O, I, generator=g, device="cuda").to(dt)
+    M = (torch.rand(O, I, generator=g, device="cuda") < 0.3).to(torch.uint8)
+    Y = torch.zeros(T, O, device="cuda", dtype=dt)
+    L = mst.Layer(0, O, I, mdt)
+    L.pack(W, M)
+    L.track_values(True)
+    with pytest.raises(mst.MstError) as e:
+        L.fwd(X, Y, 1 << 36)
+    assert e.value.status == 8     # MST_ERR_CUDA
+    del e
+    L.fwd(X, Y, T)
+    assert _rel(Y, X.double() @ (W * M).double().T) <= (5e-7 if dtype == "f32" else 4e-3)
+    L.close()
