@@ -136,8 +136,8 @@ struct mst_layer {
   uint16_t* col_idx[2];  // [cap]
   void* vals[2];         // [cap] layer dtype
 
-  // CSC view of the live structure.  Pack and the update build it for layers on the CUDA-core path only (the tensor paths read
-  // the dense image); otherwise it is built, and allocated (mst_alloc_csc), on first use.
+  // CSC view of the live structure.  Pack builds it for layers on the CUDA-core path, the update only in its kernel-per-phase
+  // form (the tensor paths read the dense image); otherwise it is built, and allocated (mst_alloc_csc), on first use.
   mutable int csc_valid;
   unsigned char* csc_base;  // the view's own allocation, nullptr until it is needed
   uint32_t* bitsT;       // [nwordsT]
