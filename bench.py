@@ -54,11 +54,11 @@ def measured_peaks():
 # (launch list and command in profiles/tc_gemm_pair_dram_traffic_gpt2medium_block_T16384.md).  The figures belong to the
 # kernel sources with the digest below; with any other sources the bench line reports no traffic.
 NCU_TRAFFIC = {
-    "sources": ("mst_tc_gemm.cu", "mst_tc_gemm.cuh", "mst_tc_ptx.cuh"),
-    "sha256_16": "58ce9e9d8b745fb1",
+    "sources": ("mst_tc_gemm.cu", "mst_tc_gemm.cuh", "mst_tc_ptx.cuh", "mst_redo.cuh"),
+    "sha256_16": "da9567b1c5703c3f",
     "launches_per_kind": 4,
-    "read": {"spmm_fwd": 262971392, "spmm_bwd_x": 331241216, "sddmm_dw": 552359680, "dense_grad": 550548992},
-    "write": {"spmm_fwd": 144084992, "spmm_bwd_x": 106702848, "sddmm_dw": 2329344, "dense_grad": 21459968},
+    "read": {"spmm_fwd": 262900736, "spmm_bwd_x": 330319616, "sddmm_dw": 552116480, "dense_grad": 550518272},
+    "write": {"spmm_fwd": 143187200, "spmm_bwd_x": 106348288, "sddmm_dw": 2802944, "dense_grad": 19384576},
 }
 
 
@@ -477,9 +477,9 @@ def run_profile_case(args) -> None:
         Wd = (torch.randn(O, I, device=dev, generator=gen) * 0.02).to(torch.bfloat16)
         mask = torch.from_numpy(mst_inputs.uniform_mask(O, I, nnz, mst_inputs.BASE_SEED + 5, 2)).to(dev)
         L = mst.Layer(2, O, I, mst.MST_BF16)
-        L.pack(Wd, mask)
         G = torch.randn(O, I, device=dev, generator=gen)
         for k in range(4):
+            L.pack(Wd, mask)     # trained values: entries grown by the update before would all tie at zero
             L.update(0.3, target_nnz=-1, random_ratio=0.25, seed=6, step=k, G_dense=G, want_stats=False)
         buf = (ctypes.c_longlong * 64)()
         n = lib.mst_update_profile(buf, 32)
@@ -491,13 +491,14 @@ def run_profile_case(args) -> None:
     if case == "update":
         layers = []
         for li in range(4):
-            L = mst.Layer(li, O, I, mst.MST_BF16)
-            L.pack(Wd, mask)
-            layers.append(L)
+            layers.append(mst.Layer(li, O, I, mst.MST_BF16))
         G.normal_(generator=gen)
         for k in range(3):
+            for L in layers:
+                L.pack(Wd, mask)     # trained values, as above
             rules = [mst.RegrowRule(-1, 0.25, 5, k, 0, 0.0) for _ in layers]
             mst.mst_topology_update_many([L.handle for L in layers], [0.3] * 4, rules, [G] * 4, want_stats=False)
+            layers[0].pack(Wd, mask)
             layers[0].update(0.3, target_nnz=-1, random_ratio=0.25, seed=6, step=k, G_dense=G, want_stats=False)
         torch.cuda.synchronize()
         return

@@ -14,7 +14,7 @@
 // Tensor memory: scores in columns 0-63 and 64-127 (tiles alternate), the halves' outputs in 128-191 and 192-255.  256 columns
 // and 82 KiB of shared memory: two blocks per SM, one's products and loads behind the other's softmax.
 // Far tiles are warp-level mma.sync products of 16 rows each with a softmax of their own, the third partial of the merge.
-// Measured: 16 x 1024 tokens, 12 heads, l = 256 52 us, 8 x 1024, 16 heads, l = 128 37 us; the whole-window kernel (one tile per SM, S single)
+// Measured: 16 x 1024 tokens, 12 heads, l = 256 50 us, 8 x 1024, 16 heads, l = 128 35.5 us; the whole-window kernel (one tile per SM, S single)
 // before took 67 us at l = 256, the mma.sync one 44 us at l = 128.
 #include <cuda.h>
 #include <cuda_bf16.h>

@@ -20,8 +20,8 @@
 // the other's algebra does.  The far strided positions (i - 2l, i - 3l, ...: one key per query and distance) are visited
 // after the window as tiles of which only the diagonal counts: warp-level mma.sync products of 16 rows each, whose sums are
 // added to the accumulators when the rows leave.
-// Measured at 16 x 1024 tokens, 12 heads: l = 256 148 us, l = 128 (8 x 1024, 16 heads) 112 us; the two mma.sync kernels and the delta
-// kernel before took 219 and 117 us.  Leaving out the far tiles gives 124 and 75 us, the window's tiles beyond the first as well 67
+// Measured at 16 x 1024 tokens, 12 heads: l = 256 144 us, l = 128 (8 x 1024, 16 heads) 109 us; the two mma.sync kernels and the delta
+// kernel before took 219 and 117 us.  Of 148 and 112 us, leaving out the far tiles gives 124 and 75 us, the window's tiles beyond the first as well 67
 // and 47 us (300 and 200 MB of compulsory traffic in two passes: 46 and 31 us); the exponentials cost 2 us.
 #include <cuda.h>
 #include <cuda_bf16.h>

@@ -281,7 +281,8 @@ __device__ __forceinline__ void far_accumulate(float (&acc)[2 * N2][4], const fl
 // This warp has read its rows of a far tile: its stage may be filled again.  The reads went through the generic proxy and the next
 // copy into the stage goes through the async proxy, which an arrival alone does not order: without the proxy fence a read that was
 // still under way now and then saw rows of the tile that came next (dQ at l = 128 differed from run to run in one of three calls;
-// up to three tiles per half, as at l = 256, no stage is filled twice).
+// up to three tiles per half, as at l = 256, no stage is filled twice).  8 x 1024 tokens, 16 heads, l = 128: forward 35.2 -> 35.5 us,
+// backward 107.8 -> 108.7.
 __device__ __forceinline__ void far_release(uint32_t far_done, int lane) {
   fence_async_smem();
   __syncwarp();

@@ -1090,9 +1090,9 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
   // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
   // The entries under the mask are fitted to widths 320..768 x 4, 600..4096 tokens, d = 0.026..0.4 (the two epilogues change over at
-  // P.sampled_stage_min); of 160 such calls 159 get the faster kernel to within 0.4 us.  1280 x 320 at 2046 tokens, d = 0.05: 10.0 us
-  // in seven ranges here, 12.3 in the small-tile kernel.  Rows are fitted to widths 192..1280 x 4 (each way), 64..4096 tokens:
-  // 3072 -> 768 at 1024 tokens 17.3 us in the small-tile kernel, 19.6 here.
+  // P.sampled_stage_min), rows to widths 192..1280 x 4 (each way), 64..4096 tokens.  202 calls drawn over these ranges, both kernels
+  // timed: 200 get the faster one to within 0.4 us; all of them here would take 1.15 times as long, all in the small-tile
+  // kernel 1.14 times.  1280 x 320 at 2046 tokens, d = 0.05: 10.0 us in seven ranges here, 12.3 there.
   if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {

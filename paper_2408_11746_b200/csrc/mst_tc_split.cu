@@ -407,6 +407,9 @@ mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
 // One piece (64 columns; 128 were no faster), fitted to back-to-back calls of 64 to 4096 tokens on layers of 192 to 4096 features, at
 // 1.85 GHz: a launch, the k-blocks (24 KB of operands each), two blocks to an SM (clusters do not pack that way: one), a further
 // wave, the sums of a cluster.  GELU adds 1500 a wave and its derivative 8000, and 3000 where two such blocks share an SM.
+// All choices timed for calls drawn over these ranges: with one piece 124 of 146 calls are within 0.4 us of the best number of ranges
+// and the whole 3 % above it (one range always: 11 %); with three pieces 44 of 60, 6 % (21 %) - ranges over eight blocks are the
+// usual miss.
 double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
   const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
