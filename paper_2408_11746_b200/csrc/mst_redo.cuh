@@ -7,8 +7,11 @@
 // is formed again, term by term in fp32, over the stored entries (products) or over the tokens (gradients).  Sums that are finite
 // had only finite terms and are left as they are.
 // The test is one multiply-add per sum by the thread that holds it (2051 x 1023 bf16 at 1999 tokens, all three
-// products: 57.1 -> 57.9 us; 3072 x 768 fp32 step at 256 tokens, with the scaled pieces: 131.8 -> 135.0).  What follows a find is far slower than the tensor cores (one
-// warp per 32 x 32 square, from global memory) and bounded by the work of the CUDA-core kernels times a small factor.
+// products: 57.1 -> 57.9 us; 3072 x 768 fp32 step at 256 tokens, with the scaled pieces: 131.8 -> 135.0).  What follows a find is for
+// runs that have gone wrong and is slower than the CUDA-core kernels (one warp per 32 x 32 square, from global memory): forward of the
+// 3072 x 768 fp32 layer at 256 tokens 0.40 ms with one infinite activation and 0.47 with all NaN (CUDA cores 0.08), of a 769 x 3073 bf16
+// layer at 8192 tokens 3.7 and 7.8 ms (0.57); column by column it was 1.1 and 1.8, 10.6 and 57 ms.  Operands in flight: four of each; eight
+// left the contraction kernels' epilogues with spilled registers, 2 % of the fused activation.
 #pragma once
 #include <stdint.h>
 
@@ -26,59 +29,82 @@ template <typename V>
 static __device__ __noinline__ void mst_redo_square(const mst_redo R, float* v, int64_t row, bool mine, int64_t n, int64_t N) {
   const int lane = threadIdx.x & 31;
   if (R.kind == MST_REDO_GRADIENT) {
-    const V* A = (const V*)R.A + row;
-    const V* B = (const V*)R.B + n + lane;
+    // loads are never conditional (lanes without a row or column read the first, tokens past the last repeat it): four of each fly together
     const bool col = n + lane < N;
+    const V* A = (const V*)R.A + (mine ? row : 0);
+    const V* B = (const V*)R.B + (col ? n + lane : 0);
     float acc[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-    for (int64_t t = 0; t < R.K; ++t) {
-      const float a = mine ? mst_redo_f32(A[t * R.lda]) : 0.f, b = col ? mst_redo_f32(B[t * R.ldb]) : 0.f;
+#pragma unroll 1
+    for (int64_t t0 = 0; t0 < R.K; t0 += 4) {
+      V a[4], b[4];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = fmaf(a, __shfl_sync(0xffffffffu, b, j), acc[j]);
+      for (int u = 0; u < 4; ++u) {
+        const int64_t t = t0 + u < R.K ? t0 + u : R.K - 1;
+        a[u] = A[t * R.lda];
+        b[u] = B[t * R.ldb];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool in = t0 + u < R.K;                               // otherwise 0 * 0
+        const float av = in ? mst_redo_f32(a[u]) : 0.f, bv = in ? mst_redo_f32(b[u]) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = fmaf(av, __shfl_sync(0xffffffffu, bv, j), acc[j]);
+      }
     }
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (mine && mst_redo_needed(v[j])) v[j] = acc[j];
     return;
   }
-  const V* A = (const V*)R.A + row * R.lda;
+  const V* A = (const V*)R.A + (mine ? row : 0) * R.lda;
   const V* vals = (const V*)R.B;
-  for (int j = 0; j < 32 && n + j < N; ++j) {
-    const int64_t c = n + j;
-    const bool need = mine && mst_redo_needed(v[j]);
-    if (!__any_sync(0xffffffffu, need)) continue;
-    float acc = 0.f;
-    for (int64_t k0 = 0; k0 < R.K; k0 += 32) {
-      // a lane per contraction index: is (row, column) of the weight stored, and where
-      const int64_t k = k0 + lane;
-      const int64_t o = R.kind == MST_REDO_FORWARD ? c : k, i = R.kind == MST_REDO_FORWARD ? k : c;
-      float w = 0.f;
-      bool has = false;
-      if (k < R.K) {
-        const uint32_t word = R.bits[o * R.wpr + (i >> 5)], below = (1u << (i & 31)) - 1u;
-        has = (word >> (i & 31)) & 1u;
-        if (has) w = mst_redo_f32(vals[R.wscan[o * R.wpr + (i >> 5)] + __popc(word & below)]);
+  const bool forward = R.kind == MST_REDO_FORWARD;
+  float acc[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+  for (int64_t k0 = 0; k0 < R.K; k0 += 32) {
+    const int count = R.K - k0 < 32 ? (int)(R.K - k0) : 32;
+    // forward: a lane keeps its column's mask word over these contraction indices; input gradient: a lane keeps an index's word
+    // over the columns (n is a multiple of 32)
+    const int64_t o = forward ? n + lane : k0 + lane, wi = o * R.wpr + ((forward ? k0 : n) >> 5);
+    uint32_t word = 0;
+    int32_t first = 0;
+    if (forward ? o < N : lane < count) {
+      word = R.bits[wi];
+      first = R.wscan[wi];
+    }
+#pragma unroll 1
+    for (int e0 = 0; e0 < count; e0 += 4) {
+      V w[4], x[4];
+      uint32_t stored = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u;                                       // at most 31: beyond `count` nothing is stored
+        const uint32_t mask = forward ? word : __shfl_sync(0xffffffffu, word, e);
+        const int32_t at = forward ? first : __shfl_sync(0xffffffffu, first, e);
+        const int bit = forward ? e : lane;
+        const bool has = (mask >> bit) & 1u;                        // (index k0 + e, column n + lane) is stored
+        w[u] = vals[has ? at + __popc(mask & ((1u << bit) - 1u)) : 0];
+        x[u] = A[k0 + (e < count ? e : 0)];
+        stored |= has ? 1u << u : 0u;
       }
-      const uint32_t m = __ballot_sync(0xffffffffu, has);
 #pragma unroll
-      for (int g = 0; g < 32; g += 8) {
-        if (!((m >> g) & 0xFFu)) continue;   // uniform
-        float x[8];
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t columns = __ballot_sync(0xffffffffu, (stored >> u) & 1u);
+        const float wv = mst_redo_f32(w[u]), xv = mst_redo_f32(x[u]);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          x[e] = 0.f;
-          if (need && ((m >> (g + e)) & 1u)) x[e] = mst_redo_f32(A[k0 + g + e]);
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float ww = __shfl_sync(0xffffffffu, w, g + e);
-          if ((m >> (g + e)) & 1u) acc = fmaf(ww, x[e], acc);
+        for (int j = 0; j < 32; ++j) {
+          const float sum = fmaf(__shfl_sync(0xffffffffu, wv, j), xv, acc[j]);
+          acc[j] = (columns >> j) & 1u ? sum : acc[j];
         }
       }
     }
-    if (need) v[j] = acc;
   }
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (mine && n + j < N && mst_redo_needed(v[j])) v[j] = acc[j];
 }
 
 // One thread: one output of a forward product
