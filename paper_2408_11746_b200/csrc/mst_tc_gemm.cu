@@ -46,8 +46,8 @@ struct Params {
   int splits;
   int m_tiles, n_tiles;
   uint32_t full, cut; // pair kernel: whole jobs, and how many each later one is cut into (rows: two halves; gradients: K ranges)
-  int a_mn, b_mn;
   int epilogue;
+  int major;
   void* out;
   int64_t ldc;
   float* partial;
@@ -61,6 +61,20 @@ struct Params {
   int tma_out;  // rows leave through shared memory and TMA stores (tensor map tmC) instead of per-thread stores
   mst_redo redo;          // rows of bf16: sums that are not finite are formed again
   int sampled_stage_min;  // sampled output: a 32 x 32 chunk with at least this many kept entries leaves row by row
+};
+
+// How the accumulators leave: a kernel each, and the operands' majors are constants of the pair kernel too.  What a launch does not
+// run costs it all the same: with one kernel for everything (168 registers where rows of bf16 alone need 62, and cold branches
+// between the hot ones) each product paid 0.4 us a launch and 20 clocks a k-block for it.  8192 tokens, forward / input gradient:
+// 768 x 768 13.3 / 13.2 -> 11.6 / 11.5 us, 3072 x 768 32.4 / 36.4 -> 29.7 / 32.5, 768 x 3072 36.5 / 32.2 -> 32.3 / 29.7; entries under
+// the mask 17.9 -> 16.1, 32.8 -> 32.0, 34.2 -> 32.6.  A training pass that alternates between them gains as much.
+// Which operands are MN-major: none (activations x image), the second (gradients x image), both (gradients x activations)
+enum { M_FORWARD, M_INPUT, M_GRADIENT };
+enum {
+  K_BF16, K_F32, K_SAMPLED,
+  K_ACT,    // bf16 with an activation
+  K_REDO,   // bf16, with or without one, where sums that are not finite are formed again
+  K_ROWS    // whatever the TMA unit cannot describe
 };
 
 // PTX wrappers live in mst_tc_ptx.cuh; waits in this file report to g_tc_error
@@ -84,26 +98,39 @@ __device__ __forceinline__ float ex2_approx(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ void phi_fast(float x, float& cdf, float& e) {
-  const float z = fabsf(x) * 0.70710678118654752f;
-  const float t = rcp_approx(fmaf(0.3275911f, z, 1.0f));
-  e = ex2_approx(x * x * -0.72134752044448170f);  // exp(-x^2 / 2)
-  float poly = fmaf(t, 1.061405429f, -1.453152027f);
-  poly = fmaf(poly, t, 1.421413741f);
-  poly = fmaf(poly, t, -0.284496736f);
-  poly = fmaf(poly, t, 0.254829592f);
-  const float q = 0.5f * poly * t * e;  // Phi(-|x|)
-  cdf = x >= 0.0f ? 1.0f - q : q;
+// Two values at a time: the fp32 pipe takes a register pair per instruction, which halves the issue slots of everything but the
+// reciprocals and exponentials (10 a value against 17; times at epilogue_tile_act).
+// -Phi(-|x|) and exp(-x^2 / 2) of a pair; the five coefficients carry the factor -1/2
+__device__ __forceinline__ void phi_pair(float x0, float x1, uint64_t& nq, uint64_t& e) {
+  const uint64_t t_arg = fma2(pack2(fabsf(x0), fabsf(x1)), pack2(0.3275911f * 0.70710678118654752f, 0.3275911f * 0.70710678118654752f), pack2(1.0f, 1.0f));
+  float t0, t1, y0, y1;
+  unpack2(t_arg, t0, t1);
+  const uint64_t t = pack2(rcp_approx(t0), rcp_approx(t1)), x = pack2(x0, x1);
+  unpack2(mul2(mul2(x, x), pack2(-0.72134752044448170f, -0.72134752044448170f)), y0, y1);
+  e = pack2(ex2_approx(y0), ex2_approx(y1));   // exp(-x^2 / 2)
+  uint64_t poly = fma2(t, pack2(-0.5f * 1.061405429f, -0.5f * 1.061405429f), pack2(0.5f * 1.453152027f, 0.5f * 1.453152027f));
+  poly = fma2(poly, t, pack2(-0.5f * 1.421413741f, -0.5f * 1.421413741f));
+  poly = fma2(poly, t, pack2(0.5f * 0.284496736f, 0.5f * 0.284496736f));
+  poly = fma2(poly, t, pack2(-0.5f * 0.254829592f, -0.5f * 0.254829592f));
+  nq = mul2(mul2(poly, t), e);
 }
-__device__ __forceinline__ float gelu_fast(float x) {
-  float cdf, e;
-  phi_fast(x, cdf, e);
-  return x * cdf;
+// x Phi(x) = max(x, 0) - |x| Phi(-|x|).  The factor of the vanishing term stays finite for x = +inf (the result is +inf); -inf gives
+// NaN, as the product x Phi(x) does.
+__device__ __forceinline__ void gelu_pair(float& x0, float& x1) {
+  uint64_t nq, e;
+  phi_pair(x0, x1, nq, e);
+  const uint64_t ax = pack2(fabsf(fminf(x0, 3.4028235e38f)), fabsf(fminf(x1, 3.4028235e38f)));
+  unpack2(fma2(ax, nq, pack2(fmaxf(x0, 0.f), fmaxf(x1, 0.f))), x0, x1);
 }
-__device__ __forceinline__ float gelu_grad_fast(float x) {
-  float cdf, e;
-  phi_fast(x, cdf, e);
-  return fmaf(x * 0.39894228040143268f, e, cdf);
+// d/dx x Phi(x) = Phi(x) + x phi(x): with u = |x| phi(x) - Phi(-|x|) it is 1 + u right of zero and -u left of it (by the sign bit)
+__device__ __forceinline__ uint64_t gelu_grad_pair(float x0, float x1) {
+  uint64_t nq, e;
+  phi_pair(x0, x1, nq, e);
+  float u0, u1;
+  unpack2(fma2(mul2(pack2(fabsf(x0), fabsf(x1)), pack2(0.39894228040143268f, 0.39894228040143268f)), e, nq), u0, u1);
+  const uint32_t s0 = __float_as_uint(x0) & 0x80000000u, s1 = __float_as_uint(x1) & 0x80000000u;
+  const uint64_t step = add2(pack2(__uint_as_float(s0 | 0x3F000000u), __uint_as_float(s1 | 0x3F000000u)), pack2(0.5f, 0.5f));   // 1 or 0
+  return add2(step, pack2(__uint_as_float(__float_as_uint(u0) ^ s0), __uint_as_float(__float_as_uint(u1) ^ s1)));
 }
 
 // For calls that want sums that are not finite formed again: this warp's share of the accumulator, ahead of the epilogue that stores it
@@ -133,47 +160,31 @@ __device__ __forceinline__ void redo_tile(const Params& P, uint32_t tmem_base, i
   }
 }
 
-// Activation step of one 32-column chunk held in registers (row m, columns n..n+31).  GELU: r <- gelu(r), the
-// pre-activation going to P.pre when given; GELU_GRAD: r <- r * gelu'(pre), pre already fetched into p4 when pre_vec.
-__device__ __forceinline__ void act_chunk(const Params& P, uint32_t (&r)[32], uint16_t* pre, bool pre_vec, const uint4 (&p4)[4],
-                                          int n) {
+// Activation step of one 32-column chunk held in registers (row m, columns n..n+31) for rows that TMA does not take.  GELU: r <-
+// gelu(r), the pre-activation going to `pre` when the caller keeps one; GELU_GRAD: r <- r * gelu'(pre).
+__device__ __forceinline__ void act_chunk(const Params& P, uint32_t (&r)[32], uint16_t* pre, int n) {
+  const int left = P.N - n < 32 ? (int)(P.N - n) : 32;
   if (P.act == MST_ACT_GELU) {
-    if (P.pre) {  // keep the pre-activation for the backward pass
-      if (pre_vec) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          uint4 o;
-          o.x = pack_bf16(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1]));
-          o.y = pack_bf16(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3]));
-          o.z = pack_bf16(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5]));
-          o.w = pack_bf16(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7]));
-          reinterpret_cast<uint4*>(pre)[v] = o;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (n + j < P.N) pre[j] = (uint16_t)(pack_bf16(__uint_as_float(r[j]), 0.f) & 0xFFFFu);
+    for (int j = 0; j < 32; j += 2) {
+      float x0 = __uint_as_float(r[j]), x1 = __uint_as_float(r[j + 1]);
+      if (P.pre) {  // keep the pre-activation for the backward pass
+        const uint32_t w = pack_bf16(x0, x1);
+        if (j < left) pre[j] = (uint16_t)(w & 0xFFFFu);
+        if (j + 1 < left) pre[j + 1] = (uint16_t)(w >> 16);
       }
+      gelu_pair(x0, x1);
+      r[j] = __float_as_uint(x0);
+      r[j + 1] = __float_as_uint(x1);
     }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(gelu_fast(__uint_as_float(r[j])));
   } else {  // multiply by the derivative at the stored pre-activation
-    if (pre_vec) {
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const uint32_t pw[4] = {p4[v].x, p4[v].y, p4[v].z, p4[v].w};
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const float lo = __uint_as_float(pw[h] << 16), hi = __uint_as_float(pw[h] & 0xFFFF0000u);
-          r[8 * v + 2 * h] = __float_as_uint(__uint_as_float(r[8 * v + 2 * h]) * gelu_grad_fast(lo));
-          r[8 * v + 2 * h + 1] = __float_as_uint(__uint_as_float(r[8 * v + 2 * h + 1]) * gelu_grad_fast(hi));
-        }
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (n + j < P.N)
-          r[j] = __float_as_uint(__uint_as_float(r[j]) * gelu_grad_fast(__uint_as_float((uint32_t)pre[j] << 16)));
+    for (int j = 0; j < 32; j += 2) {
+      const float x0 = j < left ? __uint_as_float((uint32_t)pre[j] << 16) : 0.f, x1 = j + 1 < left ? __uint_as_float((uint32_t)pre[j + 1] << 16) : 0.f;
+      float v0, v1;
+      unpack2(mul2(pack2(r[j], r[j + 1]), gelu_grad_pair(x0, x1)), v0, v1);
+      r[j] = __float_as_uint(v0);
+      r[j + 1] = __float_as_uint(v1);
     }
   }
 }
@@ -196,16 +207,8 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
     const int n = n0 + c * 32;
     if (n >= P.N) break;  // uniform
     uint32_t r[32];
-    // derivative mode: the stored pre-activation of this chunk is fetched ahead of the tensor-memory read
-    uint16_t* pre = reinterpret_cast<uint16_t*>(P.pre) + m * P.ldpre + n;
-    const bool pre_vec = n + 32 <= P.N && ((P.ldpre & 7) == 0) && ((reinterpret_cast<uintptr_t>(P.pre) & 15u) == 0);
-    uint4 p4[4];
-    if (P.act == MST_ACT_GELU_GRAD && pre_vec && row_ok) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) p4[v] = __ldg(reinterpret_cast<const uint4*>(pre) + v);
-    }
     tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
-    if (P.act && row_ok) act_chunk(P, r, pre, pre_vec, p4, n);
+    if (P.act && row_ok) act_chunk(P, r, reinterpret_cast<uint16_t*>(P.pre) + m * P.ldpre + n, n);
     __syncwarp();  // the previous chunk has been read out of the box
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
@@ -336,20 +339,29 @@ __device__ __forceinline__ void epilogue_tile_sampled(const Params& P, SampledWo
   }
 }
 
+// eight fp32 values r[j..j+7] as bf16 into 16-byte piece `piece` of this lane's row of a staging box
+__device__ __forceinline__ void stage_bf16(uint32_t my_row, uint32_t piece, const uint32_t (&r)[32], int j) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(my_row + piece * 16u),
+               "r"(pack_bf16(__uint_as_float(r[j + 0]), __uint_as_float(r[j + 1]))),
+               "r"(pack_bf16(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]))),
+               "r"(pack_bf16(__uint_as_float(r[j + 4]), __uint_as_float(r[j + 5]))),
+               "r"(pack_bf16(__uint_as_float(r[j + 6]), __uint_as_float(r[j + 7])))
+               : "memory");
+}
+
 // The same accumulator leaving through shared memory: each warp owns a 32-row x 128-byte staging box (128-byte
 // swizzle: 16-byte piece j of row r sits at piece j ^ (r & 7), so the 32 row-owning lanes write without bank
 // conflicts), fills it from its registers and one lane hands it to the TMA unit, which writes whole lines and clips
 // rows >= M and columns >= N.  bf16: 64 columns per box (two tensor-memory reads); fp32: 32 columns per box, the
 // K-range index as third coordinate.  Per-thread stores of a row-per-lane layout touch 32 lines per instruction and
 // were measured to slow the concurrent main loop by about 15 %.
+template <int KIND>
 __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtensorMap* tmC, uint32_t stage, uint32_t tmem_base,
                                                   int acc, int q, int c0, int lane, int64_t m0, int n0, int split, int cols) {
   const int64_t row0 = (int64_t)m0 + q * 32;
-  const int64_t m = row0 + lane;
-  const bool row_ok = m < P.M;
   const uint32_t my_row = stage + (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
-  if (P.epilogue == MST_TC_OUT_BF16) {
+  if (KIND != K_F32) {
 #pragma unroll 1
     for (int g = c0; g < cols / 64; g += EPI_WARPS / 4) {
       const int n = n0 + g * 64;
@@ -361,25 +373,9 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
         const int nn = n + h * 32;
         if (nn >= P.N) break;  // uniform; the TMA store clips these columns
         uint32_t r[32];
-        uint16_t* pre = reinterpret_cast<uint16_t*>(P.pre) + m * P.ldpre + nn;
-        const bool pre_vec = nn + 32 <= P.N && ((P.ldpre & 7) == 0) && ((reinterpret_cast<uintptr_t>(P.pre) & 15u) == 0);
-        uint4 p4[4];
-        if (P.act == MST_ACT_GELU_GRAD && pre_vec && row_ok) {
-#pragma unroll
-          for (int v = 0; v < 4; ++v) p4[v] = __ldg(reinterpret_cast<const uint4*>(pre) + v);
-        }
         tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + g * 64 + h * 32), r);
-        if (P.act && row_ok) act_chunk(P, r, pre, pre_vec, p4, nn);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const uint32_t piece = (uint32_t)(h * 4 + v) ^ sw;
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(my_row + piece * 16u),
-                       "r"(pack_bf16(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1]))),
-                       "r"(pack_bf16(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3]))),
-                       "r"(pack_bf16(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5]))),
-                       "r"(pack_bf16(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7])))
-                       : "memory");
-        }
+        for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r, 8 * v);
       }
       fence_async_smem();
       __syncwarp();
@@ -414,18 +410,93 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
   }
 }
 
+// The bf16 accumulator with an activation.  Each warp has two boxes, so the pre-activation travels as whole lines too.  GELU: the
+// accumulator goes to `box0` and, activated, to `box1`; both leave by TMA.  GELU_GRAD: the pre-activation of the warp's (at most
+// two) 64-column groups has been fetched into the two boxes while the products ran (fetch_pre), and each box turns into the result
+// where it lies.
+// The second box takes the place of one ring stage.  GPT-2 small at 8192 tokens: fc1 with GELU and the pre-activation kept 47.0 ->
+// 39.1 us (30.1 without the activation), fc2's input gradient with the derivative 53.5 -> 44.6 (30.2); row by row, a value at a time before.
+__device__ __forceinline__ void epilogue_tile_act(const Params& P, const CUtensorMap* tmC, const CUtensorMap* tmP, uint32_t box0, uint32_t box1,
+                                                  uint32_t tmem_base, int acc, int q, int c0, int lane, int64_t m0, int n0, int cols) {
+  const int64_t row0 = m0 + q * 32;
+  const uint32_t sw = (uint32_t)(lane & 7);
+  const bool grad = P.act == MST_ACT_GELU_GRAD;
+#pragma unroll 1
+  for (int g = c0; g < cols / 64; g += EPI_WARPS / 4) {
+    const int n = n0 + g * 64;
+    if (n >= P.N) break;  // uniform
+    const uint32_t out = !grad || g != c0 ? box1 : box0;
+    const uint32_t out_row = out + (uint32_t)lane * 128u, pre_row = (grad ? out : box0) + (uint32_t)lane * 128u;
+    if (!grad) {
+      if (lane == 0) bulk_wait_read();  // the boxes' previous contents have left shared memory
+      __syncwarp();
+    }
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      uint32_t r[32];
+      tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + g * 64 + h * 32), r);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const uint32_t piece = (uint32_t)(h * 4 + v) ^ sw;
+        if (grad) {
+          uint32_t pw[4];
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3]) : "r"(pre_row + piece * 16u));
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint64_t d = gelu_grad_pair(__uint_as_float(pw[k] << 16), __uint_as_float(pw[k] & 0xFFFF0000u));
+            float v0, v1;
+            unpack2(mul2(pack2(r[8 * v + 2 * k], r[8 * v + 2 * k + 1]), d), v0, v1);
+            r[8 * v + 2 * k] = __float_as_uint(v0);
+            r[8 * v + 2 * k + 1] = __float_as_uint(v1);
+          }
+        } else {
+          if (P.pre) stage_bf16(pre_row, piece, r, 8 * v);   // kept for the backward pass
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float x0 = __uint_as_float(r[8 * v + 2 * k]), x1 = __uint_as_float(r[8 * v + 2 * k + 1]);
+            gelu_pair(x0, x1);
+            r[8 * v + 2 * k] = __float_as_uint(x0);
+            r[8 * v + 2 * k + 1] = __float_as_uint(x1);
+          }
+        }
+        stage_bf16(out_row, piece, r, 8 * v);
+      }
+    }
+    fence_async_smem();
+    __syncwarp();
+    if (lane == 0 && row0 < P.M) {
+      if (!grad && P.pre) tma_store_2d(tmP, box0, n, (int)row0);
+      tma_store_2d(tmC, out, n, (int)row0);
+      bulk_commit();
+    }
+  }
+}
+// GELU_GRAD: one lane fetches the pre-activation of the warp's groups of a tile once the boxes' previous contents have left
+__device__ __forceinline__ void fetch_pre(const Params& P, const CUtensorMap* tmP, uint32_t box0, uint32_t box1, uint32_t bar, int q, int c0,
+                                          int64_t m0, int n0, int cols) {
+  const int n1 = n0 + c0 * 64, n2 = n1 + EPI_WARPS / 4 * 64;
+  const bool one = n1 < P.N && c0 < cols / 64, two = n2 < P.N && c0 + EPI_WARPS / 4 < cols / 64;
+  bulk_wait_read();
+  mbar_expect_tx(bar, (one ? OUT_BOX_BYTES : 0) + (two ? OUT_BOX_BYTES : 0));
+  if (one) tma_load_2d(box0, tmP, n1, (int)m0 + q * 32, bar);
+  if (two) tma_load_2d(box1, tmP, n2, (int)m0 + q * 32, bar);
+}
+
 // ------------------------------------------------------------------------------------------- kernel
+template <int KIND>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmC, const Params P) {
+               const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmP, const Params P) {
+  const bool A_MN = P.major == M_GRADIENT, B_MN = P.major != M_FORWARD;
+  constexpr int RING = STAGES - (KIND == K_ACT || KIND == K_REDO ? 1 : 0);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;  // swizzled tiles need 1024-byte alignment
   const uint32_t out_base = tiles_base + STAGES * STAGE_BYTES;  // epilogue staging boxes (1024-byte aligned)
   const uint32_t bar_base = out_base + EPI_WARPS * OUT_BOX_BYTES;
-  // barrier slots (8 bytes each): full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2]
+  // barrier slots (8 bytes each): full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], pre_full[EPI_WARPS]
   const uint32_t full0 = bar_base, empty0 = bar_base + 8 * STAGES, tfull0 = bar_base + 16 * STAGES,
-                 tempty0 = tfull0 + 16;
+                 tempty0 = tfull0 + 16, pre0 = tempty0 + 16;
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_sh;
   volatile int* abort_flag = &abort_sh;
@@ -441,6 +512,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       mbar_init(tfull0 + 8 * a, 1);
       mbar_init(tempty0 + 8 * a, EPI_WARPS);
     }
+    for (int e = 0; e < EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -473,17 +545,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const uint32_t fb = full0 + 8 * s;
           const uint32_t sa = tiles_base + s * STAGE_BYTES, sb = sa + A_BYTES;
           mbar_expect_tx(fb, STAGE_BYTES);
-          if (P.a_mn) {
+          if (A_MN) {
             for (int j = 0; j < BM / 64; ++j) tma_load_2d(sa + j * BOX_BYTES, &tmA, m0 + j * 64, kb * BK, fb);
           } else {
             tma_load_2d(sa, &tmA, kb * BK, m0, fb);
           }
-          if (P.b_mn) {
+          if (B_MN) {
             for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * BOX_BYTES, &tmB, n0 + j * 64, kb * BK, fb);
           } else {
             tma_load_2d(sb, &tmB, kb * BK, n0, fb);
           }
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+          if (++s == RING) { s = 0; ph ^= 1u; }
         }
       }
     }
@@ -491,15 +563,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       // instruction descriptor: fp32 accumulate, bf16 x bf16, M = 128, N = 256, operand majors
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
-                             ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(A_MN ? 1 : 0) << 15) |
+                             ((uint32_t)(B_MN ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       // The issue loop is one thread's serial instruction stream; everything that does not depend on the stage is
       // formed once here.  K-major: 16 K-elements = 32 bytes further along the swizzled row; MN-major: 16 rows of
       // 128 bytes.
-      const uint64_t adesc0 = smem_desc(tiles_base, P.a_mn ? BOX_BYTES : 16, 1024);
-      const uint64_t bdesc0 = smem_desc(tiles_base + A_BYTES, P.b_mn ? BOX_BYTES : 16, 1024);
-      const uint32_t a_kstep = (uint32_t)(P.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
-      const uint32_t b_kstep = (uint32_t)(P.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint64_t adesc0 = smem_desc(tiles_base, A_MN ? BOX_BYTES : 16, 1024);
+      const uint64_t bdesc0 = smem_desc(tiles_base + A_BYTES, B_MN ? BOX_BYTES : 16, 1024);
+      const uint32_t a_kstep = (uint32_t)(A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint32_t b_kstep = (uint32_t)(B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
       for (int64_t w = blockIdx.x; w < works && !*abort_flag; w += gridDim.x) {
@@ -519,7 +591,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
           for (int k = 1; k < BK / UMMA_K; ++k) tc_mma(d_tmem, ad + (uint64_t)(k * a_kstep), bd + (uint64_t)(k * b_kstep), idesc, 1u);
           tc_commit(empty0 + 8 * s);  // the smem stage is free once these MMAs have read it
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+          if (++s == RING) { s = 0; ph ^= 1u; }
         }
         if (!ok) break;
         tc_commit(tfull0 + 8 * acc);  // accumulator complete
@@ -529,17 +601,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;  // tensor-memory lane quarter this warp may read
-    const bool use_tma = P.tma_out && P.epilogue != MST_TC_OUT_SAMPLED;
+    const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
+    const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
+    const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((STAGES - 1) * STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
+    uint32_t tile_ph = 0;
     int acc = 0;
     uint32_t acc_ph = 0;
     for (int64_t w = blockIdx.x; w < works; w += gridDim.x) {
       const int split = (int)(w / tiles), t = (int)(w % tiles);
       const int m0 = (t / P.n_tiles) * BM, n0 = (t % P.n_tiles) * BN;
-      if (P.epilogue == MST_TC_OUT_SAMPLED) {
-        const SampledWords W(P, q, (warp - 2) >> 2, lane, m0, n0);
+      if (KIND == K_SAMPLED) {
+        const SampledWords W(P, q, c0, lane, m0, n0);
         if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
         tc_fence_after();
-        epilogue_tile_sampled(P, W, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, n0,
+        epilogue_tile_sampled(P, W, box, tmem_base, acc, q, c0, lane, n0,
                               P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
         tc_fence_before();
         __syncwarp();
@@ -547,23 +622,29 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         continue;
       }
+      if (fetch && lane == 0) fetch_pre(P, &tmP, box, box1, pre0 + 8 * (warp - 2), q, c0, m0, n0, BN);
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (P.redo.kind) {   // the chunks this warp stores: pairs of them through the bf16 box
-        const int c0 = (warp - 2) >> 2, pairs = use_tma ? 2 : 1;
-        for (int h = 0; h < pairs; ++h) redo_tile(P, tmem_base, acc, q, c0 * pairs + h, EPI_WARPS / 4 * pairs, lane, m0, n0, BN);
+      if (fetch && !mbar_wait(pre0 + 8 * (warp - 2), tile_ph, abort_flag)) break;
+      tile_ph ^= 1u;
+      if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
+        redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, BN);
+        redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, BN);
       }
-      if (use_tma)
-        epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                          n0, split, BN);
-      else
-        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, BN);
+      if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
+        epilogue_tile_act(P, &tmC, &tmP, box, box1, tmem_base, acc, q, c0, lane, m0, n0, BN);
+      } else if (KIND != K_ROWS) {
+        epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+      } else {
+        if (P.redo.kind) redo_tile(P, tmem_base, acc, q, c0, EPI_WARPS / 4, lane, m0, n0, BN);
+        epilogue_tile(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-    if (use_tma && lane == 0) bulk_wait_all();  // this warp's stores have landed before shared memory is given back
+    if (KIND != K_SAMPLED && KIND != K_ROWS && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
   }
 
   // ------------------------------------------------------------------ teardown
@@ -599,8 +680,7 @@ constexpr size_t P_SMEM_BYTES = (size_t)P_STAGES * P_STAGE_BYTES + EPI_WARPS * O
 //   gradients                                  parts of the job's K range, with sums (`split`) of their own.
 // (The k-blocks of all tiles shared out evenly were slower, 34 -> 40 us for 2304 x 768 at 8192 tokens and 108 -> 144 for 4096 x 1024
 // at 16384: pairs at different places of the K range read the activations at different times, and L2 does not hold them.)
-// One kernel serves all of these: a training step alternates between them, and a second instantiation cost every launch
-// about 2 us more.
+template <int KIND>
 struct PairJobs {
   uint32_t w, end, step, tiles;
   int split, m0, n0, cols, kb0, kb1;
@@ -630,7 +710,7 @@ struct PairJobs {
       const uint32_t row = tile / (uint32_t)P.n_tiles;
       m0 = (int)row * (2 * BM);
       n0 = (int)(tile - row * (uint32_t)P.n_tiles) * BN;
-      if (P.epilogue == MST_TC_OUT_BF16) {
+      if (KIND == K_BF16 || KIND == K_ACT || KIND == K_REDO || (KIND == K_ROWS && P.epilogue == MST_TC_OUT_BF16)) {
         n0 += (int)part * (BN / 2);
         cols = cut || P.N - n0 <= BN / 2 ? BN / 2 : BN;
         if (n0 >= P.N) continue;   // that half lies outside the output
@@ -694,16 +774,20 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
                : "memory");
 }
 
+template <int KIND, int MAJOR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmBn, const __grid_constant__ CUtensorMap tmC, const Params P) {
+                    const __grid_constant__ CUtensorMap tmBn, const __grid_constant__ CUtensorMap tmC,
+                    const __grid_constant__ CUtensorMap tmP, const Params P) {
+  constexpr bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
+  constexpr int RING = P_STAGES - (KIND == K_ACT || KIND == K_REDO ? 1 : 0);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
   const uint32_t out_base = tiles_base + P_STAGES * P_STAGE_BYTES;
   const uint32_t bar_base = out_base + EPI_WARPS * OUT_BOX_BYTES;
   const uint32_t full0 = bar_base, empty0 = bar_base + 8 * P_STAGES, tfull0 = bar_base + 16 * P_STAGES,
-                 tempty0 = tfull0 + 16;
+                 tempty0 = tfull0 + 16, pre0 = tempty0 + 16;
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_sh;
   volatile int* abort_flag = &abort_sh;
@@ -720,6 +804,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       mbar_init(tfull0 + 8 * a, 1);
       mbar_init(tempty0 + 8 * a, 2 * EPI_WARPS);
     }
+    for (int e = 0; e < EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0 && lane < 4)   // the maps are parameters: fetched while the predecessor drains
@@ -745,7 +830,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      PairJobs J(P, pair, npairs);
+      PairJobs<KIND> J(P, pair, npairs);
       while (J.next(P) && !*abort_flag) {
         const int m0 = J.m0 + (int)rank * BM;              // this block's rows
         const int n0 = J.n0 + (int)rank * (J.cols / 2);    // this block's half of B
@@ -756,33 +841,33 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           const uint32_t fb = in_even_block(full0 + 8 * s);  // the even block's barrier collects both blocks' bytes
           const uint32_t sa = tiles_base + s * P_STAGE_BYTES, sb = sa + A_BYTES;
           mbar_expect_tx_cluster(fb, bytes);
-          if (P.a_mn) {
+          if (A_MN) {
             for (int j = 0; j < BM / 64; ++j) tma_load_2d_pair(sa + j * BOX_BYTES, &tmA, m0 + j * 64, kb * BK, fb);
           } else {
             tma_load_2d_pair(sa, &tmA, kb * BK, m0, fb);
           }
-          if (P.b_mn) {
+          if (B_MN) {
             tma_load_2d_pair(sb, &tmB, n0, kb * BK, fb);
             if (J.cols == BN) tma_load_2d_pair(sb + BOX_BYTES, &tmB, n0 + 64, kb * BK, fb);
           } else {
             tma_load_2d_pair(sb, J.cols == BN ? &tmB : &tmBn, kb * BK, n0, fb);
           }
-          if (++s == P_STAGES) { s = 0; ph ^= 1u; }
+          if (++s == RING) { s = 0; ph ^= 1u; }
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (even block only)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
-                              ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)((2 * BM) >> 4) << 24);
-      const uint64_t adesc0 = smem_desc(tiles_base, P.a_mn ? BOX_BYTES : 16, 1024);
-      const uint64_t bdesc0 = smem_desc(tiles_base + A_BYTES, P.b_mn ? BOX_BYTES : 16, 1024);
-      const uint32_t a_kstep = (uint32_t)(P.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
-      const uint32_t b_kstep = (uint32_t)(P.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(A_MN ? 1 : 0) << 15) |
+                              ((uint32_t)(B_MN ? 1 : 0) << 16) | ((uint32_t)((2 * BM) >> 4) << 24);
+      const uint64_t adesc0 = smem_desc(tiles_base, A_MN ? BOX_BYTES : 16, 1024);
+      const uint64_t bdesc0 = smem_desc(tiles_base + A_BYTES, B_MN ? BOX_BYTES : 16, 1024);
+      const uint32_t a_kstep = (uint32_t)(A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint32_t b_kstep = (uint32_t)(B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
-      PairJobs J(P, pair, npairs);
+      PairJobs<KIND> J(P, pair, npairs);
       while (J.next(P) && !*abort_flag) {
         const uint32_t idesc = idesc0 | ((uint32_t)(J.cols >> 3) << 17);
         const int kb0 = J.kb0, kb1 = J.kb1;
@@ -800,7 +885,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
           for (int k = 1; k < BK / UMMA_K; ++k) tc_mma_pair(d_tmem, ad + (uint64_t)(k * a_kstep), bd + (uint64_t)(k * b_kstep), idesc, 1u);
           tc_commit_pair(empty0 + 8 * s);  // frees this stage in both blocks
-          if (++s == P_STAGES) { s = 0; ph ^= 1u; }
+          if (++s == RING) { s = 0; ph ^= 1u; }
         }
         if (!ok) break;
         tc_commit_pair(tfull0 + 8 * acc);  // both blocks' halves of the accumulator are complete
@@ -810,18 +895,21 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else {
     // ------------------------------------------------------------------ epilogue (both blocks, own 128 rows)
     const int q = warp & 3;
-    const bool use_tma = P.tma_out && P.epilogue != MST_TC_OUT_SAMPLED;
+    const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
+    const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
+    const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((P_STAGES - 1) * P_STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
+    uint32_t tile_ph = 0;
     int acc = 0;
     uint32_t acc_ph = 0;
-    PairJobs J(P, pair, npairs);
+    PairJobs<KIND> J(P, pair, npairs);
     while (J.next(P)) {
       const int m0 = J.m0 + (int)rank * BM, n0 = J.n0;
       const int split = J.split;
-      if (P.epilogue == MST_TC_OUT_SAMPLED) {
-        const SampledWords W(P, q, (warp - 2) >> 2, lane, m0, n0);
+      if (KIND == K_SAMPLED) {
+        const SampledWords W(P, q, c0, lane, m0, n0);
         if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
         tc_fence_after();
-        epilogue_tile_sampled(P, W, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, n0,
+        epilogue_tile_sampled(P, W, box, tmem_base, acc, q, c0, lane, n0,
                               P.partial ? P.partial + (int64_t)split * P.nnz : reinterpret_cast<float*>(P.out));
         tc_fence_before();
         __syncwarp();
@@ -829,23 +917,29 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         continue;
       }
+      if (fetch && lane == 0) fetch_pre(P, &tmP, box, box1, pre0 + 8 * (warp - 2), q, c0, m0, n0, J.cols);
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (P.redo.kind) {   // the chunks this warp stores: pairs of them through the bf16 box
-        const int c0 = (warp - 2) >> 2, pairs = use_tma ? 2 : 1;
-        for (int h = 0; h < pairs; ++h) redo_tile(P, tmem_base, acc, q, c0 * pairs + h, EPI_WARPS / 4 * pairs, lane, m0, n0, J.cols);
+      if (fetch && !mbar_wait(pre0 + 8 * (warp - 2), tile_ph, abort_flag)) break;
+      tile_ph ^= 1u;
+      if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
+        redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, J.cols);
+        redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, J.cols);
       }
-      if (use_tma)
-        epilogue_tile_tma(P, &tmC, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0,
-                          n0, split, J.cols);
-      else
-        epilogue_tile(P, out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, tmem_base, acc, q, (warp - 2) >> 2, lane, m0, n0, split, J.cols);
+      if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
+        epilogue_tile_act(P, &tmC, &tmP, box, box1, tmem_base, acc, q, c0, lane, m0, n0, J.cols);
+      } else if (KIND != K_ROWS) {
+        epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
+      } else {
+        if (P.redo.kind) redo_tile(P, tmem_base, acc, q, c0, EPI_WARPS / 4, lane, m0, n0, J.cols);
+        epilogue_tile(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(in_even_block(tempty0 + 8 * acc));
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-    if (use_tma && lane == 0) bulk_wait_all();  // this warp's stores have landed before shared memory is given back
+    if (KIND != K_SAMPLED && KIND != K_ROWS && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1130,9 +1224,8 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   int sums = 1;   // partial sums kept for one output at most
   P.m_tiles = (int)((a.M + BM - 1) / BM);
   P.n_tiles = (int)((a.N + BN - 1) / BN);
-  P.a_mn = a.a_mn_major;
-  P.b_mn = a.b_mn_major;
   P.epilogue = a.epilogue;
+  P.major = a.a_mn_major ? M_GRADIENT : a.b_mn_major ? M_INPUT : M_FORWARD;
   P.out = a.out;
   P.ldc = a.ldc;
   P.partial = nullptr;
@@ -1168,11 +1261,11 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       P.partial = (float*)ws;
     }
   }
-  // staged epilogue when the output can be described to the TMA unit (MST_TC_TMA_OUT=0 keeps per-thread stores)
-  CUtensorMap tmC = tmA;
+  // staged epilogue when the output (and the pre-activation) can be described to the TMA unit (MST_TC_TMA_OUT=0 keeps per-thread stores)
+  CUtensorMap tmC = tmA, tmP = tmA;
   P.tma_out = 0;
   if (a.epilogue == MST_TC_OUT_BF16) {
-    P.tma_out = make_out_map_bf16(&tmC, a.out, a.M, a.N, a.ldc) ? 1 : 0;
+    P.tma_out = make_out_map_bf16(&tmC, a.out, a.M, a.N, a.ldc) && (!P.act || !P.pre || make_out_map_bf16(&tmP, P.pre, a.M, a.N, P.ldpre)) ? 1 : 0;
   } else if (a.epilogue == MST_TC_OUT_F32) {
     P.tma_out = (sums > 1 ? make_out_map_f32(&tmC, P.partial, a.M, a.N, a.N, a.M * a.N, sums)
                               : make_out_map_f32(&tmC, a.out, a.M, a.N, a.ldc, a.M * a.ldc, 1))
@@ -1182,6 +1275,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (const char* e = mst_getenv(env, "MST_TC_TMA_OUT")) {
     if (e[0] == '0') P.tma_out = 0;
   }
+  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !P.tma_out ? K_ROWS : P.redo.kind ? K_REDO : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
   if (pair) {
     const int64_t jobs = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits, max_pairs = mst_sm_count() / 2, rest = jobs % max_pairs;
     CUtensorMap tmBn = tmB;
@@ -1193,14 +1287,44 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
     P.full = (uint32_t)(P.cut > 1 ? jobs - rest : jobs);
     const int64_t works = (int64_t)P.full + (int64_t)P.cut * (jobs - (int64_t)P.full);
     if (works > 0x7FFFFFFF) return MST_ERR_SHAPE;
-    MST_SMEM_LIMIT((tc_gemm_pair_kernel), P_SMEM_BYTES);
-    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel, dim3(2 * (unsigned)(works < max_pairs ? works : max_pairs)), dim3(NUM_THREADS),
-                                       P_SMEM_BYTES, s, tmA, tmB, tmBn, tmC, P));
+    const dim3 grid(2 * (unsigned)(works < max_pairs ? works : max_pairs));
+#define MST_LAUNCH_KIND(K, M)                                                                                         \
+  case 8 * M + K:                                                                                                     \
+    MST_SMEM_LIMIT((tc_gemm_pair_kernel<K, M>), P_SMEM_BYTES);                                                        \
+    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_pair_kernel<K, M>, grid, dim3(NUM_THREADS), P_SMEM_BYTES, s, tmA, tmB, tmBn, tmC, tmP, P)); \
+    break
+    switch (8 * P.major + kind) {
+      MST_LAUNCH_KIND(K_BF16, M_FORWARD);
+      MST_LAUNCH_KIND(K_ACT, M_FORWARD);
+      MST_LAUNCH_KIND(K_REDO, M_FORWARD);
+      MST_LAUNCH_KIND(K_ROWS, M_FORWARD);
+      MST_LAUNCH_KIND(K_BF16, M_INPUT);
+      MST_LAUNCH_KIND(K_ACT, M_INPUT);
+      MST_LAUNCH_KIND(K_REDO, M_INPUT);
+      MST_LAUNCH_KIND(K_ROWS, M_INPUT);
+      MST_LAUNCH_KIND(K_F32, M_GRADIENT);
+      MST_LAUNCH_KIND(K_SAMPLED, M_GRADIENT);
+      MST_LAUNCH_KIND(K_ROWS, M_GRADIENT);
+      default: return MST_ERR_INVALID_ARG;
+    }
+#undef MST_LAUNCH_KIND
   } else {
-    MST_SMEM_LIMIT((tc_gemm_kernel), SMEM_BYTES);
     const int64_t works = (int64_t)P.m_tiles * P.n_tiles * P.splits;
     const int grid = (int)(works < mst_sm_count() ? works : mst_sm_count());
-    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_kernel, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, s, tmA, tmB, tmC, P));
+#define MST_LAUNCH_KIND(K)                                                                                            \
+  case K:                                                                                                             \
+    MST_SMEM_LIMIT((tc_gemm_kernel<K>), SMEM_BYTES);                                                                  \
+    MST_CUDA_TRY(mst_launch_overlapped(tc_gemm_kernel<K>, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, s, tmA, tmB, tmC, tmP, P)); \
+    break
+    switch (kind) {
+      MST_LAUNCH_KIND(K_BF16);
+      MST_LAUNCH_KIND(K_F32);
+      MST_LAUNCH_KIND(K_SAMPLED);
+      MST_LAUNCH_KIND(K_ACT);
+      MST_LAUNCH_KIND(K_REDO);
+      MST_LAUNCH_KIND(K_ROWS);
+    }
+#undef MST_LAUNCH_KIND
   }
   MST_CUDA_TRY(cudaGetLastError());
   if (a.also_sampled && pair && sums > 1 && a.epilogue == MST_TC_OUT_F32 && a.N % 4 == 0 && a.ldc % 4 == 0 &&

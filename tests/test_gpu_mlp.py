@@ -127,3 +127,42 @@ def test_mlp_pair_gpt2_small_full_size():
     assert rel_err(host(dPre[ti, oi]), ref) <= TOL["bf16"]
     L1.close(); L2.close()
     assert mst.mst_device_error_flags() == 0
+
+
+@pytest.mark.parametrize("T,d,hid", [(257, 64, 64), (300, 72, 136), (384, 136, 200), (513, 64, 328), (1000, 264, 776)])
+def test_activation_boxes_at_tile_edges(monkeypatch, T, d, hid):
+    """The 256-row kernel's activation: groups of 64 columns cut by the matrix, half-wide tiles, rows past the last box.
+    Tolerance: one bf16 rounding (2^-9) of each stored value plus the operand sums' 2^-24 a term, under 2e-2 of the largest."""
+    monkeypatch.setenv("MST_TC_PAIR", "1")
+    m1 = mst_inputs.uniform_mask(hid, d, mst_inputs.exact_nnz(hid, d, 0.3), 902, 1)
+    m2 = mst_inputs.uniform_mask(d, hid, mst_inputs.exact_nnz(d, hid, 0.3), 902, 2)
+    p1 = mst_inputs.make_layer("fc1", 1, hid, d, T, "bf16", m1, 902, w_std=0.25)
+    p2 = mst_inputs.make_layer("fc2", 2, d, hid, T, "bf16", m2, 902, w_std=0.05)
+    L1, L2 = make_layer(p1), make_layer(p2)
+    X, dY = to_dev(p1, "X"), to_dev(p2, "dY")
+    H, Ypre, H_only, dPre = (torch.full((T + 1, hid), float("nan"), dtype=torch.bfloat16, device=dev()) for _ in range(4))
+    L1.fwd_gelu(X, H, T, Y_pre=Ypre)
+    L1.fwd_gelu(X, H_only, T)
+    pre_host, pre_dev = _pre_activation(T, hid, "bf16", 35)
+    L2.bwd_x_gelu(dY, pre_dev, dPre, T)
+    torch.cuda.synchronize()
+    Y1 = oracle.fwd(p1.X, p1.W, p1.mask)
+    assert rel_err(host(Ypre[:T]), Y1) <= TOL["bf16"]
+    assert rel_err(host(H[:T]), act.gelu(Y1)) <= TOL["bf16"]
+    assert torch.equal(H_only[:T], H[:T])
+    assert rel_err(host(dPre[:T]), oracle.bwd_x(p2.dY, p2.W, p2.mask) * act.gelu_grad(pre_host)) <= TOL["bf16"]
+    for t in (H, Ypre, H_only, dPre):
+        assert torch.isnan(t[T]).all()                # the row after the last is untouched
+    # sums that overflow: x Phi(x) is +inf at +inf and NaN at -inf
+    big = torch.zeros((T, d), dtype=torch.bfloat16, device=dev())
+    row = int(np.argmax((np.abs(p1.W) * p1.mask).max(1)))
+    col = int(np.argmax(np.abs(p1.W[row]) * p1.mask[row]))
+    big[0, col] = 3.0e38 * float(np.sign(p1.W[row, col]))
+    big[1, col] = -big[0, col]
+    one = mst.Layer(3, hid, d, mst.MST_BF16)
+    one.pack(to_dev(p1, "W") * 1e3, torch.from_numpy(p1.mask).to(dev()))
+    one.fwd_gelu(big, H, T)
+    torch.cuda.synchronize()
+    assert torch.isposinf(H[0, row]) and torch.isnan(H[1, row]) and bool((H[2:T] == 0).all())
+    one.close(); L1.close(); L2.close()
+    assert mst.mst_device_error_flags() == 0
