@@ -60,10 +60,7 @@ struct SplitCfg {
 struct SplitParams {
   int64_t M, N;
   int kblocks, splits, m_tiles, n_tiles;
-  int a_mn, b_mn;
-  int epilogue;
   void* out;
-  int act;
   uint16_t* pre;
   int64_t ldpre;
   int64_t ldc;
@@ -133,11 +130,21 @@ __device__ __forceinline__ void box_rows(const float* box, int rr0, int end, int
   for (; r < end; ++r) store(r, box[r * 33 + lane]);
 }
 
-template <int BN, int PIECES>
+// What a launch does not run costs it all the same (see the large tiles' kernel): the kind of output and the operands' majors are
+// constants.  SPLIT_NOTE
+enum {
+  S_F32, S_SAMPLED, S_BF16,
+  S_REDO,   // bf16, where sums that are not finite are formed again (three pieces: always)
+  S_ACT     // bf16 with an activation, with or without such sums
+};
+enum { M_FORWARD, M_INPUT, M_GRADIENT };   // MN-major operands: none, the second, both
+
+template <int BN, int PIECES, int KIND, int MAJOR>
 __global__ void __launch_bounds__(S_THREADS, PIECES == 1 ? 2 : 1)
 tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
   typedef SplitCfg<BN, PIECES> C;
   constexpr int CHUNK_KB = C::CHUNK_KB;
+  constexpr bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -189,12 +196,12 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, &g_split_error)) break;
         const uint32_t fb = full0 + 8 * s, sa = tiles_base + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
         mbar_expect_tx(fb, C::STAGE_BYTES);
-        if (P.a_mn) {
+        if (A_MN) {
           for (int j = 0; j < SBM / 64; ++j) tma_load_3d(sa + j * PIECES * BOX64, &tmA, m0 + j * 64, kb * SBK, 0, fb);
         } else {
           tma_load_3d(sa, &tmA, kb * SBK, m0, 0, fb);
         }
-        if (P.b_mn) {
+        if (B_MN) {
           for (int j = 0; j < BN / 64; ++j) tma_load_3d(sb + j * PIECES * BOX64, &tmB, n0 + j * 64, kb * SBK, 0, fb);
         } else {
           tma_load_3d(sb, &tmB, kb * SBK, n0, 0, fb);
@@ -204,13 +211,13 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.a_mn ? 1 : 0) << 15) |
-                             ((uint32_t)(P.b_mn ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(A_MN ? 1 : 0) << 15) |
+                             ((uint32_t)(B_MN ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
       // K-major: the three pieces of a stage lie one after the other; MN-major: 64-wide blocks, each with its three pieces
-      const uint64_t ad0 = smem_desc(tiles_base, P.a_mn ? PIECES * BOX64 : 16, 1024);
-      const uint64_t bd0 = smem_desc(tiles_base + C::A_BYTES, P.b_mn ? PIECES * BOX64 : 16, 1024);
-      const uint32_t a_piece = (uint32_t)(P.a_mn ? BOX64 : SBM * SBK * 2) >> 4, b_piece = (uint32_t)(P.b_mn ? BOX64 : BN * SBK * 2) >> 4;
-      const uint32_t a_k = (uint32_t)(P.a_mn ? 16 * 128 : 32) >> 4, b_k = (uint32_t)(P.b_mn ? 16 * 128 : 32) >> 4;
+      const uint64_t ad0 = smem_desc(tiles_base, A_MN ? PIECES * BOX64 : 16, 1024);
+      const uint64_t bd0 = smem_desc(tiles_base + C::A_BYTES, B_MN ? PIECES * BOX64 : 16, 1024);
+      const uint32_t a_piece = (uint32_t)(A_MN ? BOX64 : SBM * SBK * 2) >> 4, b_piece = (uint32_t)(B_MN ? BOX64 : BN * SBK * 2) >> 4;
+      const uint32_t a_k = (uint32_t)(A_MN ? 16 * 128 : 32) >> 4, b_k = (uint32_t)(B_MN ? 16 * 128 : 32) >> 4;
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -308,14 +315,14 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
-        if (P.redo.kind && __any_sync(0xffffffffu, zero != 0.f)) {
+        if ((PIECES == 3 || KIND == S_REDO || (KIND == S_ACT && P.redo.kind)) && __any_sync(0xffffffffu, zero != 0.f)) {
           const bool mine = lane >= rr0 && lane < rr1 && row0 + lane < P.M;
           if (PIECES == 3) mst_redo_square<float>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
           else mst_redo_square<uint16_t>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
           __syncwarp();
         }
         const int end = n + lane >= P.N ? 0 : (int)(P.M - row0 < rr1 ? P.M - row0 : rr1);   // rows of this lane's column
-        if (P.epilogue == MST_TC_OUT_SAMPLED) {
+        if (KIND == S_SAMPLED) {
           uint32_t word = 0;
           int32_t at = 0;
           if (row0 + lane < P.M) {
@@ -329,13 +336,13 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int32_t base = __shfl_sync(0xffffffffu, at, rr);
             if ((w >> lane) & 1u) out[base + __popc(w & lt)] = v;
           });
-        } else if (PIECES == 1 && P.epilogue == MST_TC_OUT_BF16) {
+        } else if (KIND != S_F32) {
           uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + row0 * P.ldc + n + lane;
           uint16_t* pre = P.pre + row0 * P.ldpre + n + lane;
-          if (P.act == MST_ACT_NONE)
+          if (KIND != S_ACT)
             box_rows(box, rr0, end, lane,
                      [&](int rr, float v) { out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu); });
-          else if (P.act == MST_ACT_GELU_GRAD) {
+          else if (MAJOR == M_INPUT) {   // the derivative at the stored pre-activation
             // sixteen rows' inputs at a time, before any of their results leaves: row by row each waits out its load (64 tokens,
             // 192 x 768: 11.6 us).  Rows past the end repeat the last one, so that only the stores are conditional and the sixteen
             // derivatives overlap.
@@ -392,13 +399,20 @@ bool make_piece_map(CUtensorMap* tm, const void* base, int pieces, int64_t rows,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int PIECES>
+template <int BN, int PIECES, int KIND, int MAJOR>
 mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
   typedef SplitCfg<BN, PIECES> C;
-  MST_SMEM_LIMIT((tc_split_kernel<BN, PIECES>), C::SMEM);
-  MST_CUDA_TRY(mst_launch_overlapped_cluster(tc_split_kernel<BN, PIECES>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)), dim3(S_THREADS),
-                                             P.splits, C::SMEM, s, tmA, tmB, P));
+  MST_SMEM_LIMIT((tc_split_kernel<BN, PIECES, KIND, MAJOR>), C::SMEM);
+  MST_CUDA_TRY(mst_launch_overlapped_cluster(tc_split_kernel<BN, PIECES, KIND, MAJOR>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)),
+                                             dim3(S_THREADS), P.splits, C::SMEM, s, tmA, tmB, P));
   return MST_OK;
+}
+template <int BN>
+mst_status_t launch_pieces(int epilogue, int major, const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
+  if (epilogue == MST_TC_OUT_SAMPLED) return launch_split<BN, 3, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
+  if (major == M_FORWARD) return launch_split<BN, 3, S_F32, M_FORWARD>(tmA, tmB, P, s);
+  if (major == M_INPUT) return launch_split<BN, 3, S_F32, M_INPUT>(tmA, tmB, P, s);
+  return launch_split<BN, 3, S_F32, M_GRADIENT>(tmA, tmB, P, s);
 }
 
 // Tile width and number of K ranges from a time model in SM clocks.
@@ -446,25 +460,32 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
   P.m_tiles = (int)((a.M + SBM - 1) / SBM);
   P.n_tiles = (int)((a.N + bn - 1) / bn);
   P.splits = splits;
-  P.a_mn = a.a_mn_major;
-  P.b_mn = a.b_mn_major;
-  P.epilogue = a.epilogue;
   P.out = a.out;
   P.ldc = a.ldc;
-  P.act = a.epilogue == MST_TC_OUT_BF16 ? a.act : 0;
   P.pre = (uint16_t*)a.pre;
   P.ldpre = a.ldpre;
   P.bits = a.bits;
   P.wscan = a.wscan;
   P.wpr = a.wpr;
   P.redo = a.redo;
-  if (P.act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
+  const int act = a.epilogue == MST_TC_OUT_BF16 ? a.act : 0, major = a.a_mn_major ? M_GRADIENT : a.b_mn_major ? M_INPUT : M_FORWARD;
+  if (act == MST_ACT_GELU_GRAD && !P.pre) return MST_ERR_INVALID_ARG;
+  // the forms that the entry points have: GELU forward and its derivative backward; one piece: products in bf16, gradients in fp32
+  if (act && (act == MST_ACT_GELU_GRAD) != (major == M_INPUT)) return MST_ERR_INVALID_ARG;
+  if (pieces == 1 && (a.epilogue == MST_TC_OUT_BF16) == (major == M_GRADIENT)) return MST_ERR_INVALID_ARG;
+  if (a.epilogue == MST_TC_OUT_SAMPLED && major != M_GRADIENT) return MST_ERR_INVALID_ARG;
   CUtensorMap tmA, tmB;
   const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, pieces, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, pieces, a.M, a.K, a.lda, SBM);
   const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, pieces, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, pieces, a.N, a.K, a.ldb, bn);
   if (!okA || !okB) return MST_ERR_SHAPE;
-  if (pieces == 3) return bn == 64 ? launch_split<64, 3>(tmA, tmB, P, s) : launch_split<128, 3>(tmA, tmB, P, s);
-  return launch_split<64, 1>(tmA, tmB, P, s);
+  if (pieces == 3) return bn == 64 ? launch_pieces<64>(a.epilogue, major, tmA, tmB, P, s) : launch_pieces<128>(a.epilogue, major, tmA, tmB, P, s);
+  if (a.epilogue == MST_TC_OUT_SAMPLED) return launch_split<64, 1, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
+  if (a.epilogue == MST_TC_OUT_F32) return launch_split<64, 1, S_F32, M_GRADIENT>(tmA, tmB, P, s);
+  if (major == M_FORWARD)
+    return act ? launch_split<64, 1, S_ACT, M_FORWARD>(tmA, tmB, P, s)
+           : P.redo.kind ? launch_split<64, 1, S_REDO, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_FORWARD>(tmA, tmB, P, s);
+  return act ? launch_split<64, 1, S_ACT, M_INPUT>(tmA, tmB, P, s)
+         : P.redo.kind ? launch_split<64, 1, S_REDO, M_INPUT>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_INPUT>(tmA, tmB, P, s);
 }
 
 }  // namespace
