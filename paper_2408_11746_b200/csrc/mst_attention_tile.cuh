@@ -23,8 +23,9 @@ constexpr int D = 64;                      // head dimension
 constexpr int ROWS = 128;                  // a block's own rows = tensor-memory lanes
 constexpr int TS = 64;                     // rows of a streamed tile
 constexpr int TILE_BYTES = TS * D * 2;     // 8 KiB
-constexpr int LDF = 68;                    // row pitch of staged fp32 accumulators (floats)
-constexpr int LDO = 72;                    // row pitch of staged bf16 results (elements)
+constexpr int SLOT_BYTES = 2 * TILE_BYTES; // a ring slot: a tile of each of two operands, or 128 rows of results on their way out
+constexpr int CW = 8;                      // algebra warps: thread = row, the two warps of a lane quarter share a tile's columns
+constexpr int THREADS = 32 * (CW + 2);     // and the lane that loads, the lane that issues the products
 constexpr float SCALE = 0.125f;            // 1 / sqrt(64)
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr float SCALE_LOG2E = SCALE * LOG2E;   // exp(s / sqrt(d) - lse) = 2^(s * SCALE_LOG2E - lse * log2(e))
@@ -61,10 +62,59 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                "r"(bar)
                : "memory");
 }
-// the block's compute warps only (the producer and issuer lanes never join)
-template <int THREADS>
-__device__ __forceinline__ void compute_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+}
+
+// ---------------------------------------------------------------------------------------------- one block after another
+// A block that runs takes over blocks of its own grid that have not started (cluster launch control), so that the next one's
+// operands are on their way while this one's last products and results are.  The request goes out at a block's start, its answer (16 bytes
+// by the async proxy) is read by every role at the block's end; a proxy fence of the reader's, before it lets go of the next block's own
+// rows, orders that ahead of the answer after next, which comes to the same place.  No request follows one that found nothing left.
+// Grids that run at once leave all of this out (template argument MORE): its instructions alone cost a launch 0.4 us.
+// Grid: heads, batch, blocks of a sequence, those with the most tiles first.  (Blocks fastest, as their keys and values are then found in
+// L2, left the SMs idle for a quarter of the time at the end: 8 x 1024 tokens, 16 heads, l = 128 have 3.5 blocks for each of the
+// 296 that run at once; 16 x 1024 tokens, 12 heads, l = 256 backward 153.6 -> 132.6 us by the order.)  Where four operands exceed L2
+// the batch is gone through in equal parts that do not, or far tiles and the next kernel's rows come from DRAM (9 x 1792
+// tokens, 20 heads, forward and backward 338 -> 321 us in three parts; 16 x 1024, 12 heads, which fit: 169 in one part, 174 in two, 177 in four).
+// Sequences of more blocks than the grid's third dimension holds have them in its first.
+struct Place { int h, b, block; };
+constexpr int GRID_Z = 65535;
+constexpr double L2_BYTES = 126e6;
+__device__ __forceinline__ Place place(int x, int y, int z, int blocks) {
+  if (blocks > GRID_Z) return Place{y, z, x};
+  while (z >= blocks) {
+    z -= blocks;
+    y += (int)gridDim.y;
+  }
+  return Place{x, y, z};
+}
+inline dim3 place_grid(int heads, int batch, int blocks) {
+  if (blocks > GRID_Z) return dim3((unsigned)blocks, (unsigned)heads, (unsigned)batch);
+  const double bytes = 4.0 * 2.0 * (double)blocks * ROWS * heads * D;   // of one sequence
+  int parts = 1;
+  while (parts < batch && (batch % parts || bytes * (batch / parts) > L2_BYTES)) ++parts;
+  if ((int64_t)blocks * parts > GRID_Z) parts = 1;
+  return dim3((unsigned)heads, (unsigned)(batch / parts), (unsigned)(blocks * parts));
+}
+__device__ __forceinline__ void take_over(uint32_t answer, uint32_t bar) {
+  mbar_expect_tx(bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
+}
+__device__ __forceinline__ bool taken_over(uint32_t answer, Place& p, int blocks) {
+  uint32_t ok, x, y, z;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%4];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "selp.u32 %3, 1, 0, p;\n\t"
+      "mov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, %1, %2, _}, r;\n\t}"
+      : "=r"(x), "=r"(y), "=r"(z), "=r"(ok)
+      : "r"(answer)
+      : "memory");
+  p = place((int)x, (int)y, (int)z, blocks);
+  return ok != 0;
 }
 
 // ---------------------------------------------------------------------------------------------- tcgen05 products
@@ -125,8 +175,9 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 
 // ---------------------------------------------------------------------------------------------- the tiles a block walks
 // Own rows r0 .. r0 + 127 of a sequence.  LOOK_BACK: queries looking at keys; otherwise keys looking at the queries that see
-// them.  First the `near` tiles (every pair at distance 0 .. l, so the first strided position too), then the far ones: tile
-// (half, m) pairs the own rows r0 + 64 half + r with the rows m l away, row r with row r only, m >= 2.
+// them.  First the far tiles: tile (half, m) pairs the own rows r0 + 64 half + r with the rows m l away, row r with row r only,
+// m >= 2; their sums become the start of the tensor-memory accumulators.  Then the `near` tiles: every pair at distance 0 .. l, so
+// the first strided position too.
 // All quotients are of multiples of 64; `magic` = 2^32 / (l / 64) rounded up divides exactly while both sides are below 2^16 (0:
 // plain division).  Four integer divisions were a tenth of a block's life.
 __host__ __device__ inline uint32_t stride_magic(int l, int seq) {
@@ -162,44 +213,45 @@ struct Walk {
     total = near + far0 + far1;
   }
   // far tile f: which half of the own rows, and where the tile starts.  The halves take turns while both have tiles left, the one
-  // with more of them first: the ring has an even number of stages, so each half keeps to stages of its own, sees every filling
-  // of those and cannot take one for the next but one.
+  // with more of them first, and the ring has an even number of slots: each half's tiles come in slots of its own.
+  __device__ __forceinline__ int far() const { return far0 + far1; }
   __device__ __forceinline__ int far_half(int f) const {
     const int longer = far1 > far0 ? 1 : 0;
     return f < both ? (f & 1) ^ longer : longer;
   }
-  // one half's far tiles: first, first + step, .. below far0 + far1
+  // one half's far tiles: far_first, far_first + far_step, .. below far()
   __device__ __forceinline__ int far_step() const { return both > 0 ? 2 : 1; }
   __device__ __forceinline__ int far_first(int half) const {
     const int longer = far1 > far0 ? 1 : 0;
-    return both > 0 ? half ^ longer : half == longer ? 0 : far0 + far1;
+    return both > 0 ? half ^ longer : half == longer ? 0 : far();
   }
   __device__ __forceinline__ int far_start(int f) const {
     const int m = f < both ? (f >> 1) + 2 : (both >> 1) + (f - both) + 2;
     const int own = r0 + TS * far_half(f);
     return LOOK_BACK ? own - m * l : own + m * l;
   }
-  __device__ __forceinline__ int start(int j) const { return j < near ? first + j * TS : far_start(j - near); }
+  __device__ __forceinline__ int start(int j) const { return j < far() ? far_start(j) : first + (j - far()) * TS; }
 };
 
-// The lane that feeds the ring.  A stage is given back by the commit behind the products of a near tile, or by the four warps that
-// a far tile concerns (a barrier of its own: those warps cannot come to it again before the stage has been filled again).
-template <int STAGES, typename W, typename Load, typename Wait>
-__device__ __forceinline__ void feed_ring(const W& walk, uint32_t ring, uint32_t full, uint32_t empty, uint32_t far_done, Load load, Wait wait) {
+// A running position in the ring.  Slots are used in one order: far tiles, near tiles, slots for the results, block after block.  A
+// parity cannot tell a filling from the next but one, so nobody may wait for a slot whose last filling he cannot know to be over:
+// the warps of a half meet their own far tiles only, in slots of their own; then everybody meets (far_over), and what is not waited
+// for after that is known by the scores or by the results.  A slot is given back by eight arrivals: two from each of the four warps
+// that a far tile concerns, seven of the issuing lane's and the commit behind a near tile's last product, one from each warp for results.
+constexpr uint32_t SLOT_ARRIVALS = CW;
+template <int STAGES>
+struct Ring {
   static_assert(STAGES % 2 == 0, "the halves' far tiles take turns");
-  int s = 0;
-  uint32_t lap = 0;
-  for (int j = 0; j < walk.total; ++j) {
-    const int before = j - STAGES;   // what the stage held one lap ago
-    if (before >= 0) {
-      const bool far = before >= walk.near;
-      const uint32_t use = far ? (uint32_t)((before - walk.near) / STAGES) : lap - 1;
-      if (!wait((far ? far_done : empty) + 8 * s, use & 1u)) return;
-    }
-    load(s, walk.start(j), ring + (uint32_t)(s * 2 * TILE_BYTES), full + 8 * s);
+  uint32_t s = 0, lap = 0;
+  __device__ __forceinline__ void next() {
     if (++s == STAGES) { s = 0; ++lap; }
   }
-}
+  __device__ __forceinline__ void skip(int n) {
+    s += (uint32_t)n;
+    lap += s / STAGES;
+    s %= STAGES;
+  }
+};
 
 // ---------------------------------------------------------------------------------------------- warp-level products (far tiles)
 // mma.sync m16n8k16 with the published fragment layouts: with g = lane / 4 and t = lane % 4, an accumulator tile (16 x 8) holds
@@ -251,68 +303,101 @@ __device__ __forceinline__ void far_accumulate(float (&acc)[2 * N2][4], const fl
     mma_bf16(acc[2 * n2 + 1], a, b[2], b[3]);
   }
 }
+// sums of a warp-level product (16 rows x 64 columns, eight 16 x 8 accumulator tiles) -> sixteen lanes from taddr's on, 64 columns
+__device__ __forceinline__ void tmem_st_tiles(uint32_t taddr, const float (&a)[8][4]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"f"(a[0][0]),
+      "f"(a[0][1]), "f"(a[0][2]), "f"(a[0][3]), "f"(a[1][0]), "f"(a[1][1]), "f"(a[1][2]), "f"(a[1][3]), "f"(a[2][0]), "f"(a[2][1]),
+      "f"(a[2][2]), "f"(a[2][3]), "f"(a[3][0]), "f"(a[3][1]), "f"(a[3][2]), "f"(a[3][3]), "f"(a[4][0]), "f"(a[4][1]), "f"(a[4][2]),
+      "f"(a[4][3]), "f"(a[5][0]), "f"(a[5][1]), "f"(a[5][2]), "f"(a[5][3]), "f"(a[6][0]), "f"(a[6][1]), "f"(a[6][2]), "f"(a[6][3]),
+      "f"(a[7][0]), "f"(a[7][1]), "f"(a[7][2]), "f"(a[7][3]), "r"(taddr)
+      : "memory");
+}
+// ---------------------------------------------------------------------------------------------- far tiles: two lanes a row
+// Row r of the own rows meets row r % 64 of the tile and no other, so a far tile is 64 dot products and 64 scaled rows.  A warp takes
+// sixteen rows, lanes i and i + 16 the two halves of row i's 64 columns: every byte is read from shared memory once.  fp32 sums of
+// exact bf16 products (the mixed-precision FMA of sm_100); weights are rounded to bf16 like those of the near tiles. 8 x 1024 tokens,
+// 16 heads, l = 128 forward: 28.4 us, and 30.6 with mma.sync products as in the backward kernels.
+__device__ __forceinline__ void fma_bf16(float& acc, uint16_t a, uint16_t b) { asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(acc) : "h"(a), "h"(b)); }
+__device__ __forceinline__ void halves(uint32_t w, uint16_t& lo, uint16_t& hi) { asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(w)); }
+struct FarRow { uint32_t w[16]; };   // 32 columns
+__device__ __forceinline__ FarRow far_row(uint32_t tile, int row, int lane) {
+  FarRow x;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const uint4 v = lds128(piece_addr(tile, row, (lane >> 4) * 4 + p));
+    x.w[4 * p] = v.x; x.w[4 * p + 1] = v.y; x.w[4 * p + 2] = v.z; x.w[4 * p + 3] = v.w;
+  }
+  return x;
+}
+// the whole row's dot product, in both of its lanes
+__device__ __forceinline__ float far_dot(const FarRow& a, const FarRow& b) {
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    uint16_t al, ah, bl, bh;
+    halves(a.w[e], al, ah);
+    halves(b.w[e], bl, bh);
+    fma_bf16(s[e & 1], al, bl);
+    fma_bf16(s[2 + (e & 1)], ah, bh);
+  }
+  const float x = (s[0] + s[1]) + (s[2] + s[3]);
+  return x + __shfl_xor_sync(0xffffffffu, x, 16);
+}
+__device__ __forceinline__ void far_add(float (&acc)[32], float weight, const FarRow& b) {
+  uint16_t w, dummy;
+  halves(pack_bf16(weight, 0.f), w, dummy);
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    uint16_t lo, hi;
+    halves(b.w[e], lo, hi);
+    fma_bf16(acc[2 * e], w, lo);
+    fma_bf16(acc[2 * e + 1], w, hi);
+  }
+}
+// the sums -> sixteen tensor-memory lanes from taddr's on, 64 columns: the start of an accumulator
+__device__ __forceinline__ void far_start_sums(uint32_t taddr, const float (&a)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x32bx2.x32.b32 [%32], 32, "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"f"(a[0]),
+      "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(a[4]), "f"(a[5]), "f"(a[6]), "f"(a[7]), "f"(a[8]), "f"(a[9]), "f"(a[10]), "f"(a[11]),
+      "f"(a[12]), "f"(a[13]), "f"(a[14]), "f"(a[15]), "f"(a[16]), "f"(a[17]), "f"(a[18]), "f"(a[19]), "f"(a[20]), "f"(a[21]),
+      "f"(a[22]), "f"(a[23]), "f"(a[24]), "f"(a[25]), "f"(a[26]), "f"(a[27]), "f"(a[28]), "f"(a[29]), "f"(a[30]), "f"(a[31]), "r"(taddr)
+      : "memory");
+}
 // This warp has read its rows of a far tile: its stage may be filled again.  The reads went through the generic proxy and the next
 // copy into the stage goes through the async proxy, which an arrival alone does not order: without the proxy fence a read that was
 // still under way now and then saw rows of the tile that came next (dQ at l = 128 differed from run to run in one of three calls;
 // up to three tiles per half, as at l = 256, no stage is filled twice).  8 x 1024 tokens, 16 heads, l = 128: forward 35.2 -> 35.5 us,
 // backward 107.8 -> 108.7.
-__device__ __forceinline__ void far_release(uint32_t far_done, int lane) {
+__device__ __forceinline__ void far_release(uint32_t empty, int lane) {
   fence_async_smem();
   __syncwarp();
-  if (lane == 0) mbar_arrive(far_done);
-}
-// this strip's accumulators -> fp32 rows r0 .. r0 + 15, columns d0 .., in shared memory (pitch LDF)
-template <int NB>
-__device__ __forceinline__ void far_stage(float* out, const float (&acc)[NB][4], int r0, int d0, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int nb = 0; nb < NB; ++nb) {
-    *reinterpret_cast<float2*>(out + (r0 + g) * LDF + d0 + nb * 8 + 2 * t) = make_float2(acc[nb][0], acc[nb][1]);
-    *reinterpret_cast<float2*>(out + (r0 + g + 8) * LDF + d0 + nb * 8 + 2 * t) = make_float2(acc[nb][2], acc[nb][3]);
-  }
+  if (lane == 0) mbar_arrive_n(empty, SLOT_ARRIVALS / 4);
 }
 
 // ---------------------------------------------------------------------------------------------- results
-// sixteen columns of one row: the accumulator, the far tiles' share of it if there is one, scaled, as bf16 into the staged
-// result tile (pitch LDO)
-__device__ __forceinline__ void stage_row(__nv_bfloat16* out, int row, int col, const uint32_t (&v)[16], const float* sums, float scale) {
-  float x[16];
-#pragma unroll
-  for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
-  if (sums) {
-#pragma unroll
-    for (int e = 0; e < 16; e += 4) {
-      const float4 y = *reinterpret_cast<const float4*>(sums + row * LDF + col + e);
-      x[e] += y.x; x[e + 1] += y.y; x[e + 2] += y.z; x[e + 3] += y.w;
-    }
-  }
+// sixteen columns of one row, scaled, as bf16 into a slot that holds 128 result rows (swizzled like a tile)
+__device__ __forceinline__ void stage_row(uint32_t slot, int row, int col, const uint32_t (&v)[16], float scale) {
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
-    uint4 w;
-    w.x = pack_bf16(x[8 * g + 0] * scale, x[8 * g + 1] * scale);
-    w.y = pack_bf16(x[8 * g + 2] * scale, x[8 * g + 3] * scale);
-    w.z = pack_bf16(x[8 * g + 4] * scale, x[8 * g + 5] * scale);
-    w.w = pack_bf16(x[8 * g + 6] * scale, x[8 * g + 7] * scale);
-    *reinterpret_cast<uint4*>(out + row * LDO + col + 8 * g) = w;
-  }
-}
-// rows first .. first + N - 1 of the staged tile -> global rows, eight lanes per row of 128 bytes
-template <int N>
-__device__ __forceinline__ void write_rows(const __nv_bfloat16* staged, int first, __nv_bfloat16* out, int64_t row, int64_t ld, int lane) {
+    uint32_t w[4];
 #pragma unroll
-  for (int it = 0; it < N / 4; ++it) {
-    const int r = first + it * 4 + (lane >> 3), piece = lane & 7;
-    *reinterpret_cast<uint4*>(out + (row + r) * ld + piece * 8) = *reinterpret_cast<const uint4*>(staged + r * LDO + piece * 8);
+    for (int e = 0; e < 4; ++e) w[e] = pack_bf16(__uint_as_float(v[8 * g + 2 * e]) * scale, __uint_as_float(v[8 * g + 2 * e + 1]) * scale);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(piece_addr(slot, row, col / 8 + g)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                 : "memory");
   }
 }
-
-// [rows x cols] bf16, ld elements between rows; box = 64 rows x 64 columns (one head of 64 tokens)
-inline bool tile_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld) {
+// [rows x cols] bf16, ld elements between rows; box = 64 rows x 64 columns (one head of 64 tokens), or the 32 rows of a lane quarter's results
+inline bool tile_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows = TS) {
   mst_encode_tiled_fn fn = mst_encode_tiled();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)D, (cuuint32_t)TS};
+  cuuint32_t box[2] = {(cuuint32_t)D, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1u, 1u};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
