@@ -5,12 +5,12 @@
 //   0  samples    4096 keys of the prune candidates (|w| of the active entries) and of the growth candidates (|g| of the
 //                 inactive ones) at jittered, evenly spaced positions
 //   -- barrier 0; every block finds, from the sample's order statistics, a bracket [lo, hi) of keys that holds the exact
-//                 threshold (six standard deviations of the sample rank on either side)
+//                 threshold (four standard deviations of the sample rank on either side)
 //                 while barrier 0 fills up: the hash keys of the slice's inactive entries
 //   1  sweep      one pass over the gradients and values of the slice: an entry below its bracket is taken, one inside goes to a
 //                 list in shared memory (3 to 10 % of the candidates), the rest is never looked at again; the listed keys are
-//                 counted in 256 bins over the bracket
-//   -- barrier 1; every block finds the bin of the threshold; the entries of that bin (a few hundred) go to a global list
+//                 counted in 2048 bins over the bracket
+//   -- barrier 1; every block finds the bin of the threshold; the entries of that bin (some tens) go to a global list
 //   -- barrier 2; every block finds the entry of the wanted rank by (key, position) in that list: the threshold, ties resolved by
 //                 the smaller index.  The random growth's threshold is found the same way among the hash keys inside its planned
 //                 bracket; entries whose growth by gradient was still open in phase 1 carry their gradient key along
@@ -25,8 +25,8 @@
 // What bounds it: instruction issue in the two sweeps (an inactive entry costs one SplitMix64 hash, two 64-bit products and about
 // twenty shifts and logic operations, and 4 bytes of gradient) and, around them, a chain of about fifteen block-wide steps and
 // L2 round trips of 1-2 us each that several layers in one launch share.  Four layers of a GPT-2-medium block (12.6 M entries,
-// d = 0.1, zeta = 0.3, R = 0.25): 78 us, of which the hashes 14, the gradient and value sweep 21; one of its layers alone
-// (4.2 M): 51 us.  The form before, one launch per layer with every key in shared memory and five sweeps between six
+// d = 0.1, zeta = 0.3, R = 0.25): 76 us, of which the hashes 14, the gradient and value sweep 20; one of its layers alone
+// (4.2 M): 50 us, a layer of 0.6 M 36.  (256 bins over the bracket and a third pass over the bin of some hundred entries: 2 us more.)  The form before, one launch per layer with every key in shared memory and five sweeps between six
 // grid-wide barriers, took 238 us for the block.
 #include <cmath>
 #include <cstdlib>
@@ -59,7 +59,8 @@ __device__ int g_upd_nstamps;
 constexpr int UT = 1024, UW = UT / 32;     // threads and warps of a block; one block per SM
 constexpr int UBINS = 2048;                // bins of a block's own histograms and of the radix select
 constexpr int USAMPLES = 4096;             // per selection
-constexpr int UCOARSE = 256;               // bins over a bracket that the blocks of a layer sum up
+constexpr int UCOARSE = UBINS;             // bins over a bracket that the blocks of a layer sum up: so many that the threshold's holds a few tens of entries
+constexpr int UFEW = 128;                  // entries of the threshold's bin that the warps rank directly
 constexpr int UBIN_LIST = 4 * UT;          // entries of the threshold's bin, four per thread
 constexpr int UNARROW = UBINS / 2;         // of them, entries that are compared one by one
 constexpr int URAND_LOCAL = 1024;          // random candidates inside the bracket, per block
@@ -220,7 +221,8 @@ __device__ __forceinline__ void u_write_samples(const ULayer& L, int blk, bool w
   }
 }
 
-// Brackets of both selections from the samples (every block, same result) into sh.lo / sh.hi: order statistics from 8192 bins on
+// Brackets of both selections from the samples (every block, same result) into sh.lo / sh.hi, four standard deviations of the sample
+// rank on either side (a threshold outside, once in 10000 updates, costs the radix select; six list half as many entries again): order statistics from 8192 bins on
 // the leading 13 key bits (a step of 1/32 octave), prune counts in the low and gradient counts in the high half of a word; the
 // lower edge is rounded down, the upper edge up.  `bins`: 8192 words of shared memory, all zero.
 constexpr int USTAT_BINS = 8192, USTAT_SHIFT = 18;
@@ -267,7 +269,7 @@ __device__ void u_brackets(const ULayer& L, bool wantA, bool wantB, uint32_t* bi
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const float n = (float)n_valid[s], q = s ? qB : qA;
-    const int at = (int)(n * q), m = (int)(6.0f * sqrtf(fmaxf(n * q * (1.0f - q), 0.f))) + 6;
+    const int at = (int)(n * q), m = (int)(4.0f * sqrtf(fmaxf(n * q * (1.0f - q), 0.f))) + 4;
     rank[2 * s] = at - m;
     rank[2 * s + 1] = at + m + 1;
   }
@@ -303,12 +305,13 @@ __device__ void u_brackets(const ULayer& L, bool wantA, bool wantB, uint32_t* bi
 // spread over bins.
 struct UBinMap {
   uint32_t lo, hi;
-  int shift, sub;      // inner bin = ((key - lo) >> shift) * sub + position * sub / positions
+  uint32_t kscale;     // inner bin = (key - lo) * kscale / 2^32, or, where there are fewer distinct keys than bins (0),
+  int shift, sub;      // ((key - lo) >> shift) * sub + position * sub / positions
   uint32_t scale;
   __device__ __forceinline__ uint32_t bin(uint32_t key, uint32_t pos) const {
     if (key < lo) return 0u;
     if (key >= hi) return UCOARSE - 1;
-    return 1u + ((key - lo) >> shift) * (uint32_t)sub + __umulhi(pos, scale);
+    return 1u + (kscale ? __umulhi(key - lo, kscale) : ((key - lo) >> shift) * (uint32_t)sub + __umulhi(pos, scale));
   }
 };
 __device__ __forceinline__ UBinMap u_bin_map(uint32_t lo, uint32_t hi, uint32_t kmin, uint32_t kmax, int low_zero,
@@ -319,14 +322,17 @@ __device__ __forceinline__ UBinMap u_bin_map(uint32_t lo, uint32_t hi, uint32_t 
   m.lo = (lo >> low_zero) << low_zero;
   m.hi = hi;
   const uint32_t span = hi > m.lo ? hi - 1u - m.lo : 0u;
-  const int bits = 32 - __clz((int)(span >> low_zero));   // of (distinct keys - 1); 0 when there is a single key
-  m.shift = low_zero + (bits > 8 ? bits - 8 : 0);
-  if ((span >> m.shift) + 1u > UCOARSE - 2) ++m.shift;
-  const uint32_t groups = (span >> m.shift) + 1u;          // at most UCOARSE - 2
-  uint32_t sub = (UCOARSE - 2) / groups;
-  if (positions < 2) sub = 1;
-  else if ((unsigned long long)sub >= positions) sub = (uint32_t)(positions - 1);
-  if (m.shift > low_zero || sub < 1u) sub = 1;   // several keys share a group: their order goes before the position
+  m.shift = low_zero;
+  m.kscale = 0u;
+  uint32_t sub = 1;
+  if (span >> low_zero >= UCOARSE - 2) {
+    m.kscale = (uint32_t)(((unsigned long long)(UCOARSE - 2) << 32) / ((unsigned long long)span + 1ULL));
+  } else {
+    sub = (UCOARSE - 2) / ((span >> low_zero) + 1u);
+    if (positions < 2) sub = 1;
+    else if ((unsigned long long)sub >= positions) sub = (uint32_t)(positions - 1);
+    if (sub < 1u) sub = 1;
+  }
   m.sub = (int)sub;
   m.scale = positions < 2 ? 0u : (uint32_t)(((unsigned long long)m.sub << 32) / positions);
   return m;
@@ -597,11 +603,8 @@ __device__ bool u_radix_select(const ULayer& L, int blk, uint32_t lo_w, int nloc
 __device__ void u_pick_bins(const ULayer& L, const bool (&want)[2], const UBinMap& mapA, const UBinMap& mapB, const int (&cnt)[2], int cap, const USlice& S,
                             UShared& sh) {
   const int b0 = 2 * (int)threadIdx.x;
-  unsigned int a0 = 0, a1 = 0, c0 = 0, c1 = 0;
-  if (b0 < UCOARSE) {
-    a0 = __ldcg(L.hist + b0); a1 = __ldcg(L.hist + b0 + 1);
-    c0 = __ldcg(L.hist + UCOARSE + b0); c1 = __ldcg(L.hist + UCOARSE + b0 + 1);
-  }
+  const uint2 a = __ldcg(reinterpret_cast<const uint2*>(L.hist) + threadIdx.x), c = __ldcg(reinterpret_cast<const uint2*>(L.hist + UCOARSE) + threadIdx.x);
+  const unsigned int a0 = a.x, a1 = a.y, c0 = c.x, c1 = c.y;
   const unsigned int overflow = __ldcg(L.ctr + C_OVERFLOW), below[2] = {__ldcg(L.ctr + C_BELOW), __ldcg(L.ctr + C_BELOW + 1)};
   unsigned int eA, eB;
   u_scan2(a0 + a1, c0 + c1, eA, eB, sh);
@@ -646,6 +649,37 @@ __device__ void u_pick_bins(const ULayer& L, const bool (&want)[2], const UBinMa
 }
 
 // ---- behind barrier 2: exact thresholds of the selections whose bin was listed ------------------------------------------------
+// Few entries, as the bins are made for: every warp holds all of them, four a lane, and ranks up to four.  False if there are more.
+__device__ __forceinline__ bool u_rank_few(const ULayer& L, UShared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned int overflow = __ldcg(L.ctr + C_OVERFLOW), count[2] = {__ldcg(L.ctr + C_LIST), __ldcg(L.ctr + C_LIST + 1)};
+  constexpr int PER = UFEW / 32;
+  unsigned long long v[2][PER];   // the places exist whatever the counts
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int h = 0; h < PER; ++h) v[s][h] = __ldcg(L.bin_list + s * UBIN_LIST + 32 * h + lane);
+  if ((overflow & 3u) || (sh.fast[0] && count[0] > UFEW) || (sh.fast[1] && count[1] > UFEW)) return false;   // uniform over the layer's blocks
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int n = sh.fast[s] ? (int)count[s] : 0;
+#pragma unroll
+    for (int h = 0; h < PER; ++h)
+      if (lane + 32 * h >= n) v[s][h] = ~0ULL;
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      if (warp + 32 * h >= n) break;
+      const unsigned long long x = __shfl_sync(0xffffffffu, v[s][h], warp);
+      int rank = 0;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) rank += __popc(__ballot_sync(0xffffffffu, v[s][j] < x));
+      if (rank + 1 == (int)sh.bin_rank[s] && lane == 0) sh.tau[s] = x;
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
 // The bin's entries (at most four per thread, in registers) are binned once more between their extremes, by key or, when they all
 // have the same key, by position; the entries of the resulting bin are compared with one another.
 __device__ void u_rank_bins(const ULayer& L, UShared& sh) {
@@ -926,7 +960,7 @@ __global__ void __launch_bounds__(UT, 1) mg_update_kernel(const __grid_constant_
     __syncthreads();
     if (alive) {
       u_sweep(L, lo_w, nloc, tryA, tryB, tryR, list_cap, S, sh, cnt);
-      if (threadIdx.x < 2 * UCOARSE) sh.hist[threadIdx.x / UCOARSE][threadIdx.x % UCOARSE] = 0u;
+      for (int b = threadIdx.x; b < 2 * UCOARSE; b += UT) (&sh.hist[0][0])[b] = 0u;
       __syncthreads();
       UPD_STAMP(5);
     }
@@ -964,9 +998,9 @@ __global__ void __launch_bounds__(UT, 1) mg_update_kernel(const __grid_constant_
         atomicOr(&L.ctr[C_OVERFLOW], 3u);   // both selections then take the radix select
       }
       __syncthreads();
-      if (threadIdx.x < 2 * UCOARSE) {
-        const unsigned int v = sh.hist[threadIdx.x / UCOARSE][threadIdx.x % UCOARSE];
-        if (v) atomicAdd(&L.hist[threadIdx.x], v);
+      for (int b = threadIdx.x; b < 2 * UCOARSE; b += UT) {
+        const unsigned int v = (&sh.hist[0][0])[b];
+        if (v) atomicAdd(&L.hist[b], v);
       }
       if (!(sh.overflow & 4u)) {
         const size_t at = (size_t)sh.r_n;
@@ -983,7 +1017,7 @@ __global__ void __launch_bounds__(UT, 1) mg_update_kernel(const __grid_constant_
       UPD_STAMP(9);
     }
     if (alive) {
-      u_rank_bins(L, sh);
+      if (!u_rank_few(L, sh)) u_rank_bins(L, sh);
       UPD_STAMP(10);
       if (tryR && (!wantB || sh.fast[1])) okR = u_rank_random(L, wantB, sh);
       UPD_STAMP(11);

@@ -83,3 +83,27 @@ def test_more_layers_than_one_launch_takes():
         mst.mst_topology_update_many([L.handle for L in layers], [0.3] * len(probs), rules, [torch.from_numpy(g).to(dev()) for g in Gs],
                                      want_stats=False)
         state = [_check(L, p, W, M, G, 0.3, -1, 0.25, step) for L, p, (W, M), G in zip(layers, probs, state, Gs)]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("tied", [2, 100, 128, 130, 1000, 1100, 5000])
+def test_threshold_among_equal_gradients(tied, dtype):
+    """The threshold's bin holds as many entries as the warps rank directly (128), one or a few more, more than are compared one by one
+    (1024), more than the list takes (4096): the same selection, ties by position."""
+    O, I, zeta, R = 600, 768, 0.3, 0.25
+    p = _problem(O, I, dtype, 0.2, 7100 + tied)
+    rng = np.random.default_rng(tied)
+    L = make_layer(p)
+    W, M = np.where(p.mask == 1, p.W, np.float32(0)).astype(np.float32), p.mask.copy()
+    for step in range(2):
+        _, _, _, n_grad = oracle.mg_counts(zeta, int(M.sum()), -1, M.size, R)
+        G = rng.standard_normal((O, I)).astype(np.float32)
+        free = np.flatnonzero(M.reshape(-1) == 0)
+        order = free[np.argsort(-np.abs(G.reshape(-1)[free]), kind="stable")]
+        plateau = order[max(0, n_grad - tied // 2): n_grad + (tied + 1) // 2]
+        flat = G.reshape(-1)
+        flat[plateau] = np.abs(flat[order[n_grad]]) * np.where(rng.random(plateau.size) < 0.5, -1, 1)
+        mst.mst_topology_update(L.handle, zeta, -1, R, 11, step, False, torch.from_numpy(G).to(dev()), want_stats=False)
+        W, M = _check(L, p, W, M, G, zeta, -1, R, step)
+    L.close()
+    assert mst.mst_device_error_flags() == 0
