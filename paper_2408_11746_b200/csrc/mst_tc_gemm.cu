@@ -410,76 +410,117 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
   }
 }
 
-// The bf16 accumulator with an activation.  Each warp has two boxes, so the pre-activation travels as whole lines too.  GELU: the
-// accumulator goes to `box0` and, activated, to `box1`; both leave by TMA.  GELU_GRAD: the pre-activation of the warp's (at most
-// two) 64-column groups has been fetched into the two boxes while the products ran (fetch_pre), and each box turns into the result
-// where it lies.
-// The second box takes the place of one ring stage.  GPT-2 small at 8192 tokens: fc1 with GELU and the pre-activation kept 47.0 ->
-// 39.1 us (30.1 without the activation), fc2's input gradient with the derivative 53.5 -> 44.6 (30.2); row by row, a value at a time before.
-__device__ __forceinline__ void epilogue_tile_act(const Params& P, const CUtensorMap* tmC, const CUtensorMap* tmP, uint32_t box0, uint32_t box1,
-                                                  uint32_t tmem_base, int acc, int q, int c0, int lane, int64_t m0, int n0, int cols) {
+// The bf16 accumulator with an activation.  Each warp has two boxes, so the pre-activation travels as whole lines too, and the two
+// alternate: a box is filled while the other one's copy is on its way.  GELU: the accumulator goes to `box0` and, activated, to
+// `box1`.  GELU_GRAD: the pre-activation of the warp's (at most two) 64-column groups is fetched into a box each, as soon as the
+// tile before has left it, and each box turns into the result where it lies.
+// The second box takes the place of one ring stage (0.8 us of 30).  GPT-2 small at 8192 tokens: fc1 with GELU and the pre-activation kept
+// 47.0 -> 38.0 us (30.2 without the activation), fc2's input gradient with the derivative 53.5 -> 40.6 (30.2); a value at a time and the
+// pre-activation row by row before.  Without the arithmetic the two take as long: what is left is the pre-activation's 50 MB.
+struct ActBoxes {
+  uint32_t box[2], bar[2];
+  uint32_t phase;   // bit i: parity of the next filling of box i
+};
+__device__ __forceinline__ bool act_group(const Params& P, int c0, int i, int n0, int cols) {   // does the tile have the warp's group i?
+  const int g = c0 + i * (EPI_WARPS / 4);
+  return g < cols / 64 && n0 + g * 64 < P.N;
+}
+// one lane: the pre-activation of group i of a tile
+__device__ __forceinline__ void fetch_pre(const Params& P, const CUtensorMap* tmP, const ActBoxes& A, int i, int q, int c0, int m0, int n0, int cols) {
+  if (!act_group(P, c0, i, n0, cols)) return;
+  mbar_expect_tx(A.bar[i], OUT_BOX_BYTES);
+  tma_load_2d(A.box[i], tmP, n0 + (c0 + i * (EPI_WARPS / 4)) * 64, m0 + q * 32, A.bar[i]);
+}
+template <bool GRAD>
+__device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtensorMap* tmC, const CUtensorMap* tmP, ActBoxes& A, uint32_t tmem_base, int acc,
+                                                  int q, int c0, int lane, int64_t m0, int n0, int cols, volatile int* abort_flag) {
   const int64_t row0 = m0 + q * 32;
   const uint32_t sw = (uint32_t)(lane & 7);
-  const bool grad = P.act == MST_ACT_GELU_GRAD;
 #pragma unroll 1
-  for (int g = c0; g < cols / 64; g += EPI_WARPS / 4) {
-    const int n = n0 + g * 64;
-    if (n >= P.N) break;  // uniform
-    const uint32_t out = !grad || g != c0 ? box1 : box0;
-    const uint32_t out_row = out + (uint32_t)lane * 128u, pre_row = (grad ? out : box0) + (uint32_t)lane * 128u;
-    if (!grad) {
-      if (lane == 0) bulk_wait_read();  // the boxes' previous contents have left shared memory
-      __syncwarp();
-    }
+  for (int i = 0; i < 2; ++i) {
+    if (!act_group(P, c0, i, n0, cols)) break;  // uniform
+    const int g = c0 + i * (EPI_WARPS / 4), n = n0 + g * 64;
+    const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + g * 64);
+    if (GRAD) {
+      const uint32_t my_row = (i ? A.box[1] : A.box[0]) + (uint32_t)lane * 128u;
+      if (!mbar_wait(i ? A.bar[1] : A.bar[0], (A.phase >> i) & 1u, abort_flag)) return false;
+      A.phase ^= 1u << i;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      uint32_t r[32];
-      tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + g * 64 + h * 32), r);
+      for (int h = 0; h < 2; ++h) {
+        uint32_t r[32], pw[16];
+        tmem_ld32_nowait(at + (uint32_t)(h * 32), r);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const uint32_t piece = (uint32_t)(h * 4 + v) ^ sw;
-        if (grad) {
-          uint32_t pw[4];
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3]) : "r"(pre_row + piece * 16u));
+        for (int v = 0; v < 4; ++v)
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pw[4 * v]), "=r"(pw[4 * v + 1]), "=r"(pw[4 * v + 2]), "=r"(pw[4 * v + 3])
+                       : "r"(my_row + (((uint32_t)(h * 4 + v)) ^ sw) * 16u));
+        tmem_ld_wait(r);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint64_t d = gelu_grad_pair(__uint_as_float(pw[k] << 16), __uint_as_float(pw[k] & 0xFFFF0000u));
-            float v0, v1;
-            unpack2(mul2(pack2(r[8 * v + 2 * k], r[8 * v + 2 * k + 1]), d), v0, v1);
-            r[8 * v + 2 * k] = __float_as_uint(v0);
-            r[8 * v + 2 * k + 1] = __float_as_uint(v1);
-          }
-        } else {
-          if (P.pre) stage_bf16(pre_row, piece, r, 8 * v);   // kept for the backward pass
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            float x0 = __uint_as_float(r[8 * v + 2 * k]), x1 = __uint_as_float(r[8 * v + 2 * k + 1]);
-            gelu_pair(x0, x1);
-            r[8 * v + 2 * k] = __float_as_uint(x0);
-            r[8 * v + 2 * k + 1] = __float_as_uint(x1);
-          }
+        for (int k = 0; k < 16; ++k) {
+          const uint64_t d = gelu_grad_pair(__uint_as_float(pw[k] << 16), __uint_as_float(pw[k] & 0xFFFF0000u));
+          float v0, v1;
+          unpack2(mul2(pack2(r[2 * k], r[2 * k + 1]), d), v0, v1);
+          r[2 * k] = __float_as_uint(v0);
+          r[2 * k + 1] = __float_as_uint(v1);
         }
-        stage_bf16(out_row, piece, r, 8 * v);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r, 8 * v);
+      }
+    } else {
+      const uint32_t pre_row = A.box[0] + (uint32_t)lane * 128u, my_row = A.box[1] + (uint32_t)lane * 128u;
+      uint32_t r[2][32];
+      tmem_ld32_nowait(at, r[0]);
+      tmem_ld32_nowait(at + 32u, r[1]);
+      if (P.pre && lane == 0) bulk_wait_read_but_last();   // the pre-activations of the group before have left their box
+      __syncwarp();
+      tmem_ld_wait(r[0]);
+      tmem_ld_wait(r[1]);
+      if (P.pre) {                                         // kept for the backward pass
+#pragma unroll
+        for (int v = 0; v < 8; ++v) stage_bf16(pre_row, (uint32_t)v ^ sw, r[v >> 2], 8 * (v & 3));
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (row0 < P.M) tma_store_2d(tmP, A.box[0], n, (int)row0);
+          bulk_commit();
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          float x0 = __uint_as_float(r[h][2 * k]), x1 = __uint_as_float(r[h][2 * k + 1]);
+          gelu_pair(x0, x1);
+          r[h][2 * k] = __float_as_uint(x0);
+          r[h][2 * k + 1] = __float_as_uint(x1);
+        }
+        if (h == 0) {
+          if (lane == 0) {
+            if (P.pre) bulk_wait_read_but_last();          // the activations of the group before have
+            else bulk_wait_read();
+          }
+          __syncwarp();
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r[h], 8 * v);
       }
     }
     fence_async_smem();
     __syncwarp();
-    if (lane == 0 && row0 < P.M) {
-      if (!grad && P.pre) tma_store_2d(tmP, box0, n, (int)row0);
-      tma_store_2d(tmC, out, n, (int)row0);
+    if (lane == 0) {
+      if (row0 < P.M) tma_store_2d(tmC, GRAD && i == 0 ? A.box[0] : A.box[1], n, (int)row0);
       bulk_commit();
     }
   }
+  return true;
 }
-// GELU_GRAD: one lane fetches the pre-activation of the warp's groups of a tile once the boxes' previous contents have left
-__device__ __forceinline__ void fetch_pre(const Params& P, const CUtensorMap* tmP, uint32_t box0, uint32_t box1, uint32_t bar, int q, int c0,
-                                          int64_t m0, int n0, int cols) {
-  const int n1 = n0 + c0 * 64, n2 = n1 + EPI_WARPS / 4 * 64;
-  const bool one = n1 < P.N && c0 < cols / 64, two = n2 < P.N && c0 + EPI_WARPS / 4 < cols / 64;
+// GELU_GRAD, one lane: the next tile's pre-activations, each into its box when this tile's copy has read it
+__device__ __forceinline__ void fetch_next(const Params& P, const CUtensorMap* tmP, const ActBoxes& A, int q, int c0, int n0, int cols, int next_m0, int next_n0,
+                                           int next_cols) {
+  if (act_group(P, c0, 1, n0, cols)) bulk_wait_read_but_last();
+  else bulk_wait_read();
+  fetch_pre(P, tmP, A, 0, q, c0, next_m0, next_n0, next_cols);
   bulk_wait_read();
-  mbar_expect_tx(bar, (one ? OUT_BOX_BYTES : 0) + (two ? OUT_BOX_BYTES : 0));
-  if (one) tma_load_2d(box0, tmP, n1, (int)m0 + q * 32, bar);
-  if (two) tma_load_2d(box1, tmP, n2, (int)m0 + q * 32, bar);
+  fetch_pre(P, tmP, A, 1, q, c0, next_m0, next_n0, next_cols);
 }
 
 // ------------------------------------------------------------------------------------------- kernel
@@ -494,7 +535,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;  // swizzled tiles need 1024-byte alignment
   const uint32_t out_base = tiles_base + STAGES * STAGE_BYTES;  // epilogue staging boxes (1024-byte aligned)
   const uint32_t bar_base = out_base + EPI_WARPS * OUT_BOX_BYTES;
-  // barrier slots (8 bytes each): full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], pre_full[EPI_WARPS]
+  // barrier slots (8 bytes each): full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], pre_full[2 * EPI_WARPS]
   const uint32_t full0 = bar_base, empty0 = bar_base + 8 * STAGES, tfull0 = bar_base + 16 * STAGES,
                  tempty0 = tfull0 + 16, pre0 = tempty0 + 16;
   __shared__ uint32_t tmem_base_holder;
@@ -512,7 +553,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       mbar_init(tfull0 + 8 * a, 1);
       mbar_init(tempty0 + 8 * a, EPI_WARPS);
     }
-    for (int e = 0; e < EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
+    for (int e = 0; e < 2 * EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -604,7 +645,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
     const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
     const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((STAGES - 1) * STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
-    uint32_t tile_ph = 0;
+    ActBoxes A = {{box, box1}, {pre0 + 16 * (warp - 2), pre0 + 16 * (warp - 2) + 8}, 0};
     int acc = 0;
     uint32_t acc_ph = 0;
     for (int64_t w = blockIdx.x; w < works; w += gridDim.x) {
@@ -622,17 +663,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         continue;
       }
-      if (fetch && lane == 0) fetch_pre(P, &tmP, box, box1, pre0 + 8 * (warp - 2), q, c0, m0, n0, BN);
+      if (fetch && lane == 0 && w == blockIdx.x) {
+        fetch_pre(P, &tmP, A, 0, q, c0, m0, n0, BN);
+        fetch_pre(P, &tmP, A, 1, q, c0, m0, n0, BN);
+      }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (fetch && !mbar_wait(pre0 + 8 * (warp - 2), tile_ph, abort_flag)) break;
-      tile_ph ^= 1u;
       if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, BN);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, BN);
       }
       if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
-        epilogue_tile_act(P, &tmC, &tmP, box, box1, tmem_base, acc, q, c0, lane, m0, n0, BN);
+        if (!(P.major == M_INPUT ? epilogue_tile_act<true>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)
+                                 : epilogue_tile_act<false>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)))
+          break;
+        if (fetch && lane == 0 && w + gridDim.x < works) {
+          const int tn = (int)((w + gridDim.x) % tiles);
+          fetch_next(P, &tmP, A, q, c0, n0, BN, (tn / P.n_tiles) * BM, (tn % P.n_tiles) * BN, BN);
+        }
       } else if (KIND != K_ROWS) {
         epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
       } else {
@@ -804,7 +852,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       mbar_init(tfull0 + 8 * a, 1);
       mbar_init(tempty0 + 8 * a, 2 * EPI_WARPS);
     }
-    for (int e = 0; e < EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
+    for (int e = 0; e < 2 * EPI_WARPS; ++e) mbar_init(pre0 + 8 * e, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0 && lane < 4)   // the maps are parameters: fetched while the predecessor drains
@@ -898,10 +946,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
     const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
     const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((P_STAGES - 1) * P_STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
-    uint32_t tile_ph = 0;
+    ActBoxes A = {{box, box1}, {pre0 + 16 * (warp - 2), pre0 + 16 * (warp - 2) + 8}, 0};
     int acc = 0;
     uint32_t acc_ph = 0;
     PairJobs<KIND> J(P, pair, npairs);
+    bool first = true;
     while (J.next(P)) {
       const int m0 = J.m0 + (int)rank * BM, n0 = J.n0;
       const int split = J.split;
@@ -917,17 +966,23 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         continue;
       }
-      if (fetch && lane == 0) fetch_pre(P, &tmP, box, box1, pre0 + 8 * (warp - 2), q, c0, m0, n0, J.cols);
+      if (fetch && lane == 0 && first) {
+        fetch_pre(P, &tmP, A, 0, q, c0, m0, n0, J.cols);
+        fetch_pre(P, &tmP, A, 1, q, c0, m0, n0, J.cols);
+      }
+      first = false;
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (fetch && !mbar_wait(pre0 + 8 * (warp - 2), tile_ph, abort_flag)) break;
-      tile_ph ^= 1u;
       if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, J.cols);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, J.cols);
       }
       if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
-        epilogue_tile_act(P, &tmC, &tmP, box, box1, tmem_base, acc, q, c0, lane, m0, n0, J.cols);
+        if (!epilogue_tile_act<MAJOR == M_INPUT>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, J.cols, abort_flag)) break;
+        if (fetch) {
+          PairJobs<KIND> N = J;
+          if (N.next(P) && lane == 0) fetch_next(P, &tmP, A, q, c0, n0, J.cols, N.m0 + (int)rank * BM, N.n0, N.cols);
+        }
       } else if (KIND != K_ROWS) {
         epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
       } else {
