@@ -595,13 +595,14 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     } else {
       MST_TRY(mst_prepare(L->dtype, &job, nullptr, 0, s));
     }
-    // A few tokens: the latency kernel (16 tokens: 3 us a layer of GPT-2-small width against 5 for the smallest tiles; at 32 its
-    // blocks read the activations too often and it loses).  Columns beyond the row must be zero in the activations too.
-    if (!transpose && T <= MST_SMALL_FWD_TOKENS && (cols % 8 == 0 || a.A != in))
-      return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, a.redo, s);
     a.epilogue = MST_TC_OUT_BF16;
     a.splits = 1;
     a.act = act; a.pre = pre; a.ldpre = ldpre;
+    // A few tokens: the latency kernel.  Columns beyond the row must be zero in the activations too.
+    if (!transpose && (cols % 8 == 0 || a.A != in) &&
+        (T <= MST_SMALL_FWD_TOKENS ||
+         (T <= MST_SMALL_FWD_MOST && mst_small_fwd_clocks(T, rows, cols) < mst_tc_small_clocks(a) && !mst_getenv(mst_env_any(), "MST_TC_PAIR"))))
+      return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, a.redo, s);
     return mst_tc_gemm(a, s);
   }
   // CUDA cores: the product lands in the pre-activation buffer when the caller keeps one, else in the output

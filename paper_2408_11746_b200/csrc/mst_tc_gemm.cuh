@@ -75,8 +75,10 @@ mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s);
 // The same kernel for bf16 operands and outputs of few tiles, all epilogues, and its estimated time in SM clocks
 mst_status_t mst_tc_small(const mst_tc_gemm_args& a, cudaStream_t s);
 double mst_tc_small_clocks(const mst_tc_gemm_args& a);
-// forward product for at most MST_SMALL_FWD_TOKENS tokens (mst_small_fwd.cu)
-constexpr int64_t MST_SMALL_FWD_TOKENS = 16;
+// forward product of a few tokens (mst_small_fwd.cu): always up to MST_SMALL_FWD_TOKENS, up to MST_SMALL_FWD_MOST where its estimated time,
+// in SM clocks as above, is shorter than the small tiles'
+constexpr int64_t MST_SMALL_FWD_TOKENS = 16, MST_SMALL_FWD_MOST = 1024;
+double mst_small_fwd_clocks(int64_t T, int O, int K);
 mst_status_t mst_small_fwd(const void* X, int64_t ldx, int64_t T, const uint16_t* image, int64_t ldimage, int O, int K, void* Y, int64_t ldy,
                            int act, void* pre, int64_t ldpre, const mst_redo& redo, cudaStream_t s);
 

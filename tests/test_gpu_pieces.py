@@ -102,6 +102,15 @@ def test_bf16_products_of_few_tiles(O, I, T):
     assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
 
 
+@pytest.mark.parametrize("O,I,T,pad", [
+    (96, 96, 1024, 0), (96, 96, 1025, 0),      # the most tokens the latency kernel takes, and one more
+    (200, 136, 600, 0), (2304, 768, 33, 0), (5120, 1280, 17, 0), (300, 4096, 31, 0), (17, 40, 257, 0), (333, 777, 250, 3), (1280, 1288, 64, 0)])
+def test_forward_of_a_few_hundred_tokens(O, I, T, pad):
+    # the latency kernel or the small tiles, by their estimates
+    y, dx, dw, g = _layer_case(O, I, T, "bf16", 0.2, O + I + T, pad)
+    assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
+
+
 @pytest.mark.parametrize("O,I,T,density", [
     (5120, 1280, 8190, 0.1),     # 100 tiles on 74 pairs: 26 cut in two
     (3840, 1250, 8000, 0.3),     # 75 tiles: one cut, the others whole; ragged columns
