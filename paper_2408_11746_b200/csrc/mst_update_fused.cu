@@ -60,7 +60,7 @@ constexpr int UT = 1024, UW = UT / 32;     // threads and warps of a block; one 
 constexpr int UBINS = 2048;                // bins of a block's own histograms and of the radix select
 constexpr int USAMPLES = 4096;             // per selection
 constexpr int UCOARSE = UBINS;             // bins over a bracket that the blocks of a layer sum up: so many that the threshold's holds a few tens of entries
-constexpr int UFEW = 128;                  // entries of the threshold's bin that the warps rank directly
+constexpr int UFEW = 256;                  // entries of the threshold's bin that the warps rank directly
 constexpr int UBIN_LIST = 4 * UT;          // entries of the threshold's bin, four per thread
 constexpr int UNARROW = UBINS / 2;         // of them, entries that are compared one by one
 constexpr int URAND_LOCAL = 1024;          // random candidates inside the bracket, per block
@@ -649,31 +649,31 @@ __device__ void u_pick_bins(const ULayer& L, const bool (&want)[2], const UBinMa
 }
 
 // ---- behind barrier 2: exact thresholds of the selections whose bin was listed ------------------------------------------------
-// Few entries, as the bins are made for: every warp holds all of them, four a lane, and ranks up to four.  False if there are more.
+// Few entries, as the bins are made for: half of the warps see to each selection, every one of them holds all of its entries, up to eight a
+// lane, and ranks each sixteenth by ballots.  False if there are more.
 __device__ __forceinline__ bool u_rank_few(const ULayer& L, UShared& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, s = threadIdx.x >> 9, warp = (threadIdx.x >> 5) & 15;
   const unsigned int overflow = __ldcg(L.ctr + C_OVERFLOW), count[2] = {__ldcg(L.ctr + C_LIST), __ldcg(L.ctr + C_LIST + 1)};
   constexpr int PER = UFEW / 32;
-  unsigned long long v[2][PER];   // the places exist whatever the counts
+  unsigned long long v[PER];   // the places exist whatever the count
 #pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int h = 0; h < PER; ++h) v[s][h] = __ldcg(L.bin_list + s * UBIN_LIST + 32 * h + lane);
+  for (int h = 0; h < PER; ++h) v[h] = __ldcg(L.bin_list + s * UBIN_LIST + 32 * h + lane);
   if ((overflow & 3u) || (sh.fast[0] && count[0] > UFEW) || (sh.fast[1] && count[1] > UFEW)) return false;   // uniform over the layer's blocks
+  const int n = sh.fast[s] ? (int)count[s] : 0, want = (int)sh.bin_rank[s] - 1;
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const int n = sh.fast[s] ? (int)count[s] : 0;
+  for (int h = 0; h < PER; ++h)
+    if (lane + 32 * h >= n) v[h] = ~0ULL;
 #pragma unroll
-    for (int h = 0; h < PER; ++h)
-      if (lane + 32 * h >= n) v[s][h] = ~0ULL;
+  for (int h = 0; h < PER; ++h) {
 #pragma unroll
-    for (int h = 0; h < PER; ++h) {
-      if (warp + 32 * h >= n) break;
-      const unsigned long long x = __shfl_sync(0xffffffffu, v[s][h], warp);
+    for (int half = 0; half < 32; half += 16) {
+      if (warp + half + 32 * h >= n) break;
+      const unsigned long long x = __shfl_sync(0xffffffffu, v[h], warp + half);
       int rank = 0;
 #pragma unroll
-      for (int j = 0; j < PER; ++j) rank += __popc(__ballot_sync(0xffffffffu, v[s][j] < x));
-      if (rank + 1 == (int)sh.bin_rank[s] && lane == 0) sh.tau[s] = x;
+      for (int j = 0; j < PER; ++j)
+        if (32 * j < n) rank += __popc(__ballot_sync(0xffffffffu, v[j] < x));
+      if (rank == want && lane == 0) sh.tau[s] = x;
     }
   }
   __syncthreads();

@@ -86,9 +86,9 @@ def test_more_layers_than_one_launch_takes():
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
-@pytest.mark.parametrize("tied", [2, 100, 128, 130, 1000, 1100, 5000])
+@pytest.mark.parametrize("tied", [2, 100, 256, 258, 1000, 1100, 5000])
 def test_threshold_among_equal_gradients(tied, dtype):
-    """The threshold's bin holds as many entries as the warps rank directly (128), one or a few more, more than are compared one by one
+    """The threshold's bin holds as many entries as the warps rank directly (256), one or a few more, more than are compared one by one
     (1024), more than the list takes (4096): the same selection, ties by position."""
     O, I, zeta, R = 600, 768, 0.3, 0.25
     p = _problem(O, I, dtype, 0.2, 7100 + tied)
