@@ -1238,24 +1238,30 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   const bool env = mst_env_any();
   // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
   // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
-  // The entries under the mask are fitted to widths 320..768 x 4, 600..4096 tokens, d = 0.026..0.4 (the two epilogues change over at
-  // P.sampled_stage_min), rows to widths 192..1280 x 4 (each way), 64..4096 tokens.  202 calls drawn over these ranges, both kernels
-  // timed: 200 get the faster one to within 0.4 us; all of them here would take 1.15 times as long, all in the small-tile
-  // kernel 1.14 times.  1280 x 320 at 2046 tokens, d = 0.05: 10.0 us in seven ranges here, 12.3 there.
+  // Fitted to 130 layers drawn over 96..4096 features (at most 4096 x 2048), 130..4096 tokens, d = 0.02..0.5, up to seven calls each, both
+  // kernels timed, once for sizes of whole 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in
+  // partial words and squares.  The choices are 1.4 % (even) and 0.2 % (odd) above the better kernel of each call; with one set of
+  // figures for both, from before the kernels were cut into kinds, 3.8 and 3.2 %.
   if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
-      double here = (!a.act ? 9100.0 : a.M > BM ? 13000.0 : 18000.0) + (double)kb * 564.0;   // one token tile: single blocks
-      if (a.epilogue != MST_TC_OUT_BF16) {
-        const bool entries = a.epilogue == MST_TC_OUT_SAMPLED;
+      double here;
+      if (a.epilogue == MST_TC_OUT_BF16) {
+        const bool even = a.ldc % 8 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0 &&
+                          (!a.act || !a.pre || (a.ldpre % 8 == 0 && (reinterpret_cast<uintptr_t>(a.pre) & 15u) == 0));
+        const double setup = !a.act ? 9600.0 : a.act == MST_ACT_GELU ? (even ? 11100.0 : 13600.0) : (even ? 13000.0 : 20300.0);
+        here = (a.act && a.M <= BM ? 18000.0 : setup) + (double)kb * (even ? 450.0 : 560.0);   // one token tile: single blocks
+      } else {
+        const bool entries = a.epilogue == MST_TC_OUT_SAMPLED, even = a.M % 8 == 0 && a.N % 8 == 0;
         const double out_bytes = entries ? 4.0 * (double)a.nnz : 4.0 * (double)a.M * (double)a.N;
         int cut;
         const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes, &cut), per = (kb + sp - 1) / sp;
         if (entries) {
-          here = ((double)a.nnz * 1024.0 < SAMPLED_STAGE_MIN * (double)a.M * (double)a.N ? 12000.0 : 14000.0) + (double)per * 574.0;
-          if (sp > 1) here += 3500.0 + (double)sp * out_bytes * 7.4e-4;   // written and read, 5 TB/s at 1.85 GHz
+          const bool few = (double)a.nnz * 1024.0 < SAMPLED_STAGE_MIN * (double)a.M * (double)a.N;
+          here = even ? (few ? 10800.0 : 13300.0) + (double)per * 400.0 : (few ? 12000.0 : 14000.0) + (double)per * 574.0;
+          if (sp > 1) here += (even ? 2800.0 : 3500.0) + (double)sp * out_bytes * 7.4e-4;   // written and read, 5 TB/s at 1.85 GHz
         } else {
-          here = 17100.0 + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0);
+          here = (even ? 10300.0 : 17100.0) + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0);
         }
       }
       if (mst_tc_small_clocks(a) < here) return mst_tc_small(a, s);
