@@ -64,7 +64,7 @@ struct mst_tc_gemm_args {
   void* pre;             // GELU: optional bf16 output for the pre-activation (may be NULL);
                          // GELU_GRAD: bf16 input holding the pre-activation the derivative is taken at
   int64_t ldpre;
-  float* also_sampled;   // F32: the entries under the mask (bits, wscan, wpr) as well, where partial sums are added up anyway;
+  float* also_sampled;   // F32: the entries under the mask (bits, wscan, wpr) as well, where partial sums are added up anyway or tiles are small;
   bool* sampled;         //      set to true when that was done
   mst_redo redo;         // BF16 epilogue and mst_tc_split: sums that are not finite are formed again
 };

@@ -102,6 +102,28 @@ def test_bf16_products_of_few_tiles(O, I, T):
     assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
 
 
+@pytest.mark.parametrize("O,I,T,dtype", [(1, 1, 1, "f32"), (65, 63, 129, "f32"), (128, 33, 64, "f32"), (300, 40, 1000, "f32"), (2051, 130, 257, "f32"),
+                                         (1, 3, 1, "bf16"), (129, 31, 65, "bf16"), (255, 257, 300, "bf16"), (513, 96, 1500, "bf16")])
+def test_dense_gradient_of_small_tiles_with_its_entries(O, I, T, dtype):
+    # the entries under the mask leave with the tile: the very values of the matrix, which are those without entries
+    g = torch.Generator(device="cuda").manual_seed(O + I)
+    dt, mdt = (torch.float32, mst.MST_F32) if dtype == "f32" else (torch.bfloat16, mst.MST_BF16)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda").to(dt)
+    X, dY, W = n(T, I), n(T, O), n(O, I)
+    M = (torch.rand(O, I, generator=g, device="cuda") < 0.3).to(torch.uint8)
+    M[0, 0] = 1
+    L = mst.Layer(0, O, I, mdt)
+    L.pack(W, M)
+    G, both = torch.full((O, I), float("nan"), device="cuda"), torch.full((O, I), float("nan"), device="cuda")
+    dW = torch.full((L.nnz,), float("nan"), device="cuda")
+    L.dense_grad(dY, X, T, G)
+    L.dense_grad_dw(dY, X, T, both, dW)
+    assert mst.mst_device_error_flags() == 0
+    assert torch.equal(G, both) and torch.equal(dW, both[M.bool()])
+    assert _rel(G, dY.double().T @ X.double()) <= 1e-5
+    L.close()
+
+
 @pytest.mark.parametrize("O,I,T,pad", [
     (96, 96, 1024, 0), (96, 96, 1025, 0),      # the most tokens the latency kernel takes, and one more
     (200, 136, 600, 0), (2304, 768, 33, 0), (5120, 1280, 17, 0), (300, 4096, 31, 0), (17, 40, 257, 0), (333, 777, 250, 3), (1280, 1288, 64, 0)])
