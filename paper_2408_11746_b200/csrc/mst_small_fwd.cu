@@ -109,12 +109,16 @@ mst_status_t launch_small(const void* X, int64_t ldx, int64_t T, const uint16_t*
 
 }  // namespace
 
-// A launch with its trip to memory, and the 64 K bytes that each block of 16 tokens and 16 features reads, at what L2 delivers to all SMs
-// (8.5 TB/s).  124 forward calls drawn over 96..5120 features and 17..600 tokens, both kernels timed: the choice against the
-// small tiles is 0.3 % above the better one of each; small tiles from 17 tokens on, as before, 42 % (a GPT-2-small block at 17, 32, 64
-// tokens: 29.6 -> 16.3 us, 30.3 -> 16.1, 30.4 -> 23.0; at GPT-2-large width and 64 tokens the tiles win, 40 against 50).
+// A launch with its trip to memory, and the 64 K bytes that each block of 16 tokens and 16 features reads, at what L2 delivers to all SMs, with
+// what a block costs beside them; figures for each number of warps (launch_small).  Fitted to 212 forward calls without copies, drawn over
+// 96..5120 features and 17..1024 tokens, 5 to 9 % off their times; one figure for all (15 % off) had 717 x 114 -> 3712 take 33 us here
+// instead of 10 in small tiles.  Small tiles from 17 tokens on, as they once were: 42 % above the better kernel (a GPT-2-small block
+// at 17, 32, 64 tokens: 29.6 -> 16.3 us, 30.3 -> 16.1, 30.4 -> 23.0; at GPT-2-large width and 64 tokens the tiles win, 40 against 50).
 double mst_small_fwd_clocks(int64_t T, int O, int K) {
-  return 6100.0 + (double)((O + 15) / 16) * (double)((T + 15) / 16) * 64.0 * (double)K / 4600.0;
+  const double bytes = (double)((O + 15) / 16) * (double)((T + 15) / 16) * 64.0;   // per index of the contraction range
+  if (K <= 1024) return 6200.0 + bytes * (double)(K + 404) / 8980.0;
+  if (K <= 2048) return 5700.0 + bytes * (double)(K + 3060) / 16330.0;
+  return 5500.0 + bytes * (double)(K + 1040) / 5600.0;
 }
 
 // X rows 16-byte aligned, columns K .. multiple of 8 zero in X and in the image; act NONE or GELU

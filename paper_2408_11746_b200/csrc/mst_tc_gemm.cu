@@ -1238,10 +1238,10 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   const bool env = mst_env_any();
   // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
   // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
-  // Fitted to 130 layers drawn over 96..4096 features (at most 4096 x 2048), 130..4096 tokens, d = 0.02..0.5, up to seven calls each, both
-  // kernels timed, once for sizes of whole 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in
-  // partial words and squares.  The choices are 1.4 % (even) and 0.2 % (odd) above the better kernel of each call; with one set of
-  // figures for both, from before the kernels were cut into kinds, 3.8 and 3.2 %.
+  // Fitted to layers drawn over 96..4096 features (at most 4096 x 2048) and 17..4096 tokens, both kernels timed, once for sizes of whole
+  // 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in partial words and squares.  Gradients:
+  // 130 layers, d = 0.02..0.5, the choices 1.4 % (even) and 0.2 % (odd) above the better kernel of each call.  Products: 190 layers,
+  // figures of the calls whose operands need no copies (3 to 8 % off the measured times, 7 to 33 before).
   if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
@@ -1249,8 +1249,12 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       if (a.epilogue == MST_TC_OUT_BF16) {
         const bool even = a.ldc % 8 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0 &&
                           (!a.act || !a.pre || (a.ldpre % 8 == 0 && (reinterpret_cast<uintptr_t>(a.pre) & 15u) == 0));
-        const double setup = !a.act ? 9600.0 : a.act == MST_ACT_GELU ? (even ? 11100.0 : 13600.0) : (even ? 13000.0 : 20300.0);
-        here = (a.act && a.M <= BM ? 18000.0 : setup) + (double)kb * (even ? 450.0 : 560.0);   // one token tile: single blocks
+        const double k = (double)kb;
+        if (a.M <= BM) here = a.act ? (even ? 12900.0 : 28000.0) + k * 603.0 : 8350.0 + k * 606.0;   // one token tile: single blocks
+        else if (!a.act) here = even ? 8350.0 + k * 460.0 : 10400.0 + k * 552.0;
+        else if (a.act == MST_ACT_GELU_GRAD) here = even ? 10800.0 + k * 462.0 : 19000.0 + k * 505.0;
+        else here = even ? 10750.0 + k * 478.0 : 13600.0 + k * 560.0;
+        if (a.act == MST_ACT_GELU && !even) here += 0.024 * (double)a.M * (double)a.N;   // pre-activations value by value: 1390 x 2346, 56 us
       } else {
         const bool entries = a.epilogue == MST_TC_OUT_SAMPLED, even = a.M % 8 == 0 && a.N % 8 == 0;
         const double out_bytes = entries ? 4.0 * (double)a.nnz : 4.0 * (double)a.M * (double)a.N;

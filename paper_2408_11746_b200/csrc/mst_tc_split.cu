@@ -25,6 +25,8 @@
 // warp 1 issues the MMAs, warps 2-9 own the sums (one row and BN / 2 columns per thread).  Every wait is bounded.
 #include <cuda.h>
 
+#include <atomic>
+
 #include "mst_bits.cuh"
 #include "mst_internal.cuh"
 #include "mst_redo.cuh"
@@ -421,16 +423,52 @@ mst_status_t launch_pieces(int epilogue, int major, const CUtensorMap& tmA, cons
   return launch_split<BN, 3, S_F32, M_GRADIENT>(tmA, tmB, P, s);
 }
 
+// Blocks that run at once, one to an SM, in clusters of `size`: the groups of SMs that a cluster must fit into are no multiples of it (148
+// SMs hold 148, 148, 132 and 120 blocks in clusters of 1, 2, 4 and 8).  Asked once per device.
+int cluster_slots(int size) {
+  static std::atomic<int> known[64][9];
+  const int sms = mst_sm_count();
+  int dev = 0;
+  if (size <= 1 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sms;
+  int n = known[dev][size].load(std::memory_order_relaxed);
+  if (n == 0) {
+    typedef SplitCfg<128, 3> C;   // one block to an SM
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * sms));
+    cfg.blockDim = dim3(S_THREADS);
+    cfg.dynamicSmemBytes = C::SMEM;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_F32, M_GRADIENT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_F32, M_GRADIENT>, &cfg) != cudaSuccess || clusters <= 0) {
+      cudaGetLastError();   // reported by the launch, if it matters there
+      return sms;
+    }
+    n = clusters * size < sms ? clusters * size : sms;
+    known[dev][size].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // Tile width and number of K ranges from a time model in SM clocks.
 // Three pieces: 24 MMAs per k-block (64 clocks each at 128 columns, 40 at 64, where the A operand's shared-memory reads dominate),
-// about 4000 for launch, fill and drain of a block, and 1500 for the sums of a cluster.
-// One piece (64 columns; 128 were no faster), fitted to back-to-back calls of 64 to 4096 tokens on layers of 192 to 4096 features, at
-// 1.85 GHz: a launch, the k-blocks (24 KB of operands each), two blocks to an SM (clusters do not pack that way: one), a further
-// wave, the sums of a cluster.  GELU adds 1500 a wave and its derivative 8000, and 3000 where two such blocks share an SM.
-// All choices timed for calls drawn over these ranges: with one piece 124 of 146 calls are within 0.4 us of the best number of ranges
-// and the whole 3 % above it (one range always: 11 %); with three pieces 44 of 60, 6 % (21 %) - ranges over eight blocks are the
-// usual miss.
+// about 10000 for launch, fill and drain of a wave, and 1500 for the sums of a cluster.
+// One piece (64 columns; 128 were no faster), at 1.85 GHz: a launch, the k-blocks (24 KB of operands each), a further wave, the sums of
+// a cluster; two blocks share an SM, in clusters as well, each then a little slower.
+// All choices timed for 138 fp32 and 190 bf16 layers drawn over 96..4096 x 96..2048 features and the widths of a block up to 1280, 64..1024
+// (fp32) and 17..4096 tokens; 138 and 189 further ones for the check.  With 148 blocks assumed at any cluster size and one of a cluster to
+// an SM, ranges over eight blocks were taken where two or four are faster: fp32 calls 4.5 % above the best choice of each, now 0.6;
+// the further ones take 0.965 of that time, bf16 products of few tiles 0.96 (1024 x 1024 at 162 tokens, fp32: 21.9 -> 13.7 us; bf16 input
+// gradient 4352 -> 1088 at 710 tokens 21.8 -> 16.8).
 double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
+  struct Figures { double launch, wave, k_shared, shared, cluster; };
+  static const Figures plain = {7160.0, 0.0, 483.0, 1490.0, 5940.0}, gelu = {10700.0, 1550.0, 515.0, 1640.0, 2440.0},
+                       grad = {13000.0, 2500.0, 512.0, 1980.0, 1700.0};
   const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
   double best = 1e30;
@@ -439,18 +477,20 @@ double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
   for (int w = 64; w <= (pieces == 3 ? 128 : 64); w += 64) {
     const int64_t tiles = m_tiles * ((a.N + w - 1) / w);
     for (int sp = 1; sp <= 8 && sp <= kblocks; sp *= 2) {   // cluster sizes
-      const int kb = (kblocks + sp - 1) / sp;
+      const int kb = (kblocks + sp - 1) / sp, fit = cluster_slots(sp);
       double t;
       if (pieces == 3) {
-        const int64_t waves = (tiles * sp + sms - 1) / sms;
-        t = (double)waves * (kb * (w == 64 ? 960.0 : 1536.0) + 4000.0) + (sp > 1 ? 1500.0 : 0.0);
+        const int64_t waves = (tiles * sp + fit - 1) / fit;
+        t = (double)waves * (kb * (w == 64 ? 960.0 : 1620.0) + 10000.0) + (sp > 1 ? 1500.0 : 0.0);
+      } else if (a.epilogue == MST_TC_OUT_BF16) {
+        const Figures& F = a.act == MST_ACT_GELU_GRAD ? grad : a.act ? gelu : plain;
+        const int64_t waves = (tiles * sp + 2 * fit - 1) / (2 * fit);
+        const double pair = kb * F.k_shared;
+        t = F.launch + F.wave * (double)waves + (double)(waves - 1) * (11500.0 + pair) + (tiles * sp > fit ? pair + F.shared : kb * 471.0) +
+            (sp > 1 ? F.cluster : 0.0);
       } else {
         const int64_t slots = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + slots - 1) / slots;
-        if (a.epilogue == MST_TC_OUT_BF16)
-          t = 9300.0 + (double)waves * (kb * 480.0 + (a.act == MST_ACT_GELU_GRAD ? 8000.0 : a.act ? 1500.0 : 0.0)) +
-              (double)(waves - 1) * 8000.0 + (sp > 1 ? 5000.0 : a.act && tiles > sms ? 3000.0 : 0.0);
-        else
-          t = 9000.0 + (double)waves * kb * 555.0 + (double)(waves - 1) * 10000.0 + (sp > 1 ? 5000.0 : 0.0);
+        t = 9000.0 + (double)waves * kb * 555.0 + (double)(waves - 1) * 10000.0 + (sp > 1 ? 5000.0 : 0.0);
       }
       if (t < best * 0.97) { best = t; *bn = w; *splits = sp; }
     }
