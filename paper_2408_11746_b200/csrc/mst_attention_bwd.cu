@@ -227,9 +227,13 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       for (int it = 0; ok; ++it) {
         const Walk<true> walk((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
         const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
+        const int skip = (MORE ? 1 : 0) + walk.far();        // the forward output, the far tiles
         ok = wait_on(S.own_full, (uint32_t)it & 1u, abort_flag);
-        ok = ok && wait_on(S.far_over, (uint32_t)it & 1u, abort_flag);
-        k.skip((MORE ? 1 : 0) + walk.far());                 // the forward output, the far tiles
+        // A slot's parity tells one filling from the next only if the one before is known to be over.  The slots skipped here are filled once the
+        // far tiles are over; the first two tiles' scores go ahead of that, beside delta and the far tiles, where their slots are filled for
+        // the first time.  Everything later waits for weights of all warps, and these come after the far tiles' sums.
+        if (it > 0 || skip + 2 > STAGES) ok = ok && wait_on(S.far_over, (uint32_t)it & 1u, abort_flag);
+        k.skip(skip);
         uint32_t sp = 0;
         for (int j = 0; j <= walk.near && ok; ++j) {
           const uint32_t s = k.s;
@@ -499,7 +503,7 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const Walk<false> walk(at.block * ROWS, l, P.seq, P.magic);
         const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
         ok = wait_on(S.own_full, (uint32_t)it & 1u, abort_flag);
-        ok = ok && wait_on(S.far_over, (uint32_t)it & 1u, abort_flag);
+        if (it > 0 || walk.far() + 1 > STAGES) ok = ok && wait_on(S.far_over, (uint32_t)it & 1u, abort_flag);   // as in dQ, for one tile
         k.skip(walk.far());
         ok = ok && filled();
         for (int j = 0; j < walk.near && ok; ++j, ++t) {
