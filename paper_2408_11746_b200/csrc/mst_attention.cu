@@ -149,8 +149,9 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
         const int near = walk.near;
         const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
         ok = wait_on(own_full, (uint32_t)it & 1u, abort_flag);
-        // the first two tiles' scores need not wait for the far tiles where their slots are filled for the first time (see dQ)
-        if (it > 0 || walk.far() + 2 > STAGES) ok = ok && wait_on(far_over, (uint32_t)it & 1u, abort_flag);
+        // in a block without successors the first two tiles' scores need not wait for the far tiles where their slots are filled for the
+        // first time (see dQ)
+        if (MORE || walk.far() + 2 > STAGES) ok = ok && wait_on(far_over, (uint32_t)it & 1u, abort_flag);
         k.skip(walk.far());
         Ring<STAGES> kv = k;             // the tile whose weights are ready next
         // scores of tile j, in issue order behind the product that read the weights of the tile two before there

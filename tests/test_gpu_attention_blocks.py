@@ -25,7 +25,9 @@ def _forward_reference(qkv, B, n, H, stride):
     (16, 256, 20, 192),    # 640
     (8, 448, 19, 64),      # an odd number of 64-row tiles: the last block has half its rows, its second half no far tiles
     (6, 704, 17, 192),     # the same, far tiles in odd and even numbers
-    (5, 1152, 12, 128)])   # up to sixteen far tiles, 540 blocks
+    (5, 1152, 12, 128),    # up to sixteen far tiles, 540 blocks
+    (2, 1152, 6, 128),     # none to sixteen of them in blocks without successors: slots filled for the first time and again
+    (1, 832, 7, 192)])     # the same, odd numbers
 def test_blocks_that_take_over_others(B, n, H, stride):
     gen = torch.Generator(device="cuda").manual_seed(n + stride)
     C = 64 * H
