@@ -99,7 +99,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
 
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);
   Ring<STAGES> k;
   // the next block, if there is one (block `it` of this one's life is at its end)
   auto next = [&](int it) { return MORE && wait_on(next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(answers + 16 * (it & 1), at, P.blocks); };
@@ -432,7 +432,7 @@ extern "C" mst_status_t mst_strided_attention_fwd(const void* Q, const void* K, 
   P.magic = stride_magic(P.stride, seq_len);
   MST_SMEM_LIMIT((strided_attention_fwd_kernel<false>), SMEM_BYTES);
   MST_SMEM_LIMIT((strided_attention_fwd_kernel<true>), SMEM_BYTES);
-  MST_CUDA_TRY(mst_launch_overlapped(more ? strided_attention_fwd_kernel<true> : strided_attention_fwd_kernel<false>, place_grid(heads, batch, P.blocks), dim3(THREADS),
+  MST_CUDA_TRY(mst_launch_overlapped(more ? strided_attention_fwd_kernel<true> : strided_attention_fwd_kernel<false>, place_grid(heads, batch, P.blocks, !more && P.stride < P.seq), dim3(THREADS),
                                      SMEM_BYTES, (cudaStream_t)stream, tmQ, tmK, tmV, tmO, P));
   MST_CUDA_TRY(cudaGetLastError());
   return MST_OK;

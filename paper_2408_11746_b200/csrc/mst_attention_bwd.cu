@@ -212,7 +212,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);
 
   if (warp == CW) {
     if (lane == 0) feed<true, 1, MORE>(S, P, at, &tmQ, &tmG, &tmK, &tmV, &tmO, abort_flag);
@@ -489,7 +489,7 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks);   // early keys have the most tiles
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);   // early keys have the most tiles
 
   if (warp == CW) {
     if (lane == 0) feed<false, 2, MORE>(S, P, at, &tmK, &tmV, &tmQ, &tmG, nullptr, abort_flag);
@@ -773,7 +773,7 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
   MST_SMEM_LIMIT((attn_bwd_dq_kernel<true>), SMEM_BYTES);
   MST_SMEM_LIMIT((attn_bwd_dkv_kernel<false>), SMEM_BYTES);
   MST_SMEM_LIMIT((attn_bwd_dkv_kernel<true>), SMEM_BYTES);
-  const dim3 grid = place_grid(heads, batch, P.blocks);
+  const dim3 grid = place_grid(heads, batch, P.blocks, !more && P.stride < P.seq);
   MST_CUDA_TRY(mst_launch_overlapped(more ? attn_bwd_dq_kernel<true> : attn_bwd_dq_kernel<false>, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, tmO, tmDQ, P));
   MST_CUDA_TRY(mst_launch_overlapped(more ? attn_bwd_dkv_kernel<true> : attn_bwd_dkv_kernel<false>, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, tmDK, tmDV, P));
   MST_CUDA_TRY(cudaGetLastError());

@@ -77,20 +77,23 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
 // 296 that run at once; 16 x 1024 tokens, 12 heads, l = 256 backward 153.6 -> 132.6 us by the order.)  Where four operands exceed L2
 // the batch is gone through in equal parts that do not, or far tiles and the next kernel's rows come from DRAM (9 x 1792
 // tokens, 20 heads, forward and backward 338 -> 321 us in three parts; 16 x 1024, 12 heads, which fit: 169 in one part, 174 in two, 177 in four).
+// Grids that run at once (no last wave to fill) have a sequence's blocks first where the window is shorter than the sequence, so that blocks with
+// tiles in common are neighbours: forward and backward 1 x 1024 tokens, 6 heads, l = 128 43.3 -> 39.6 us, 2 x 1024, 9 heads, l = 256 42.5 -> 40.2; windows
+// of the whole sequence lose by it (3 x 512, 10 heads 39.3 -> 41.9, 2 x 256, 20 heads 26.8 -> 28.4).
 // Sequences of more blocks than the grid's third dimension holds have them in its first.
 struct Place { int h, b, block; };
 constexpr int GRID_Z = 65535;
 constexpr double L2_BYTES = 126e6;
-__device__ __forceinline__ Place place(int x, int y, int z, int blocks) {
-  if (blocks > GRID_Z) return Place{y, z, x};
+__device__ __forceinline__ Place place(int x, int y, int z, int blocks, bool blocks_first) {
+  if (blocks_first || blocks > GRID_Z) return Place{y, z, x};
   while (z >= blocks) {
     z -= blocks;
     y += (int)gridDim.y;
   }
   return Place{x, y, z};
 }
-inline dim3 place_grid(int heads, int batch, int blocks) {
-  if (blocks > GRID_Z) return dim3((unsigned)blocks, (unsigned)heads, (unsigned)batch);
+inline dim3 place_grid(int heads, int batch, int blocks, bool blocks_first) {
+  if (blocks_first || blocks > GRID_Z) return dim3((unsigned)blocks, (unsigned)heads, (unsigned)batch);
   const double bytes = 4.0 * 2.0 * (double)blocks * ROWS * heads * D;   // of one sequence
   int parts = 1;
   while (parts < batch && (batch % parts || bytes * (batch / parts) > L2_BYTES)) ++parts;
@@ -113,7 +116,7 @@ __device__ __forceinline__ bool taken_over(uint32_t answer, Place& p, int blocks
       : "=r"(x), "=r"(y), "=r"(z), "=r"(ok)
       : "r"(answer)
       : "memory");
-  p = place((int)x, (int)y, (int)z, blocks);
+  p = place((int)x, (int)y, (int)z, blocks, false);
   return ok != 0;
 }
 
