@@ -16,7 +16,7 @@
 // Tensor memory: scores in columns 0-63 and 64-127 (tiles alternate), the halves' outputs in 128-191 and 192-255.  256 columns
 // and 83 KiB of shared memory: two blocks per SM, one's products and loads behind the other's softmax.
 // The far tiles' softmax (two lanes a row, 16 rows a warp) is where the first half starts: reference and sum through shared memory, outputs in tensor memory.
-// Results leave by TMA from a slot of the ring.
+// Results leave by TMA from a slot of the ring, or, in a block without successors, as whole rows from where the own rows were.
 // Bound: the chain of a tile through its warps (scores, exponentials, weights: about 1000 clocks for a block, two of them at
 // work on an SM); the SM issues in half of its cycles, DRAM is busy for a quarter of the time.  16 x 1024 tokens, 12 heads, l = 256 50.2 -> 40 us,
 // 8 x 1024, 16 heads, l = 128 35.5 -> 28.4 (one block after the other, heads last in the grid, far tiles at the end, on mma.sync).
@@ -40,8 +40,10 @@ constexpr size_t SMEM_BYTES = 2 * TILE_BYTES + RING_BYTES + STAT_FLOATS * 4 + 32
 __device__ int g_attn_error = 0;
 
 struct FwdParams {
+  __nv_bfloat16* Out;
+  int64_t ldo;
   float* lse;          // [batch, heads, seq] or NULL
-  int seq, heads, stride, blocks;
+  int seq, heads, stride, blocks, blocks_first;
   uint32_t magic;
 };
 
@@ -52,7 +54,7 @@ __device__ __forceinline__ bool wait_on(uint32_t bar, uint32_t parity, volatile 
 // The exponents of a row are taken against m; a row that has seen nothing keeps m = -inf and takes them against 0
 __device__ __forceinline__ float reference(float m) { return m == -INFINITY ? 0.f : m; }
 
-template <bool MORE>   // the grid has more blocks than run at once
+template <bool MORE, bool FAR>   // see mst_attention_tile.cuh
 __global__ void __launch_bounds__(THREADS, 2)
 strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const FwdParams P) {
@@ -87,7 +89,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
     mbar_init(far_over, CW);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == CW && lane < 4) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : &tmO);
+  if (warp == CW && lane < (MORE ? 4 : 3)) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : &tmO);
   if (warp == CW + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&holder)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -96,10 +98,12 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = holder;
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);
+  Walk<true> first((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
+  if (!MORE) first.now();
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
 
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);
   Ring<STAGES> k;
   // the next block, if there is one (block `it` of this one's life is at its end)
   auto next = [&](int it) { return MORE && wait_on(next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(answers + 16 * (it & 1), at, P.blocks); };
@@ -115,7 +119,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
       auto slot = [&]() { return k.lap == 0 || wait_on(empty + 8 * k.s, (k.lap - 1) & 1u, abort_flag); };
       for (int it = 0; ok; ++it) {
         const int col = at.h * D, row0 = at.b * P.seq, q0 = (P.blocks - 1 - at.block) * ROWS;   // late queries have the most tiles
-        const Walk<true> walk(q0, l, P.seq, P.magic);
+        const Walk<true> walk = MORE ? Walk<true>(q0, l, P.seq, P.magic) : first;
         if (it > 0 && !wait_on(own_free, (uint32_t)(it - 1) & 1u, abort_flag)) break;
         mbar_expect_tx(own_full, 2 * TILE_BYTES);
         tma_load_2d(own, &tmQ, col, row0 + q0, own_full);
@@ -130,7 +134,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
           tma_load_2d(dst + TILE_BYTES, &tmV, col, row0 + walk.start(j), bar);
           k.next();
         }
-        ok = ok && slot();               // a slot for the results
+        ok = ok && MORE && slot();       // a slot for the results
         if (!ok) break;
         mbar_arrive(full + 8 * k.s);
         k.next();
@@ -145,9 +149,9 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
       bool ok = true;
       auto filled = [&]() { return wait_on(full + 8 * k.s, k.lap & 1u, abort_flag); };
       for (int it = 0; ok; ++it) {
-        const Walk<true> walk((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
+        const Walk<true> walk = MORE ? Walk<true>((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic) : first;
         const int near = walk.near;
-        const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
+        const uint32_t from_far = FAR && walk.far() > 0 ? 1u : 0u;
         ok = wait_on(own_full, (uint32_t)it & 1u, abort_flag);
         // in a block without successors the first two tiles' scores need not wait for the far tiles where their slots are filled for the
         // first time (see dQ)
@@ -214,8 +218,8 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
     for (int it = 0; ok; ++it) {
       const int h = at.h, b = at.b, q0 = (P.blocks - 1 - at.block) * ROWS, row0 = b * P.seq;
       const int i = q0 + r, i_lo = q0 + quarter * 32;        // this thread's query, this warp's: i_lo .. i_lo + 31
-      const Walk<true> walk(q0, l, P.seq, P.magic);
-      const int far = walk.far();
+      const Walk<true> walk = MORE ? Walk<true>(q0, l, P.seq, P.magic) : first;
+      const int far = FAR ? walk.far() : 0;
       float m = -INFINITY;                                   // reference of this half's softmax, base 2
       uint64_t sum2 = 0ULL;
       ok = wait_on(own_full, (uint32_t)it & 1u, abort_flag);
@@ -351,10 +355,10 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
       const float inv = 1.f / total;
       a0 *= inv;
       a1 *= inv;
-      ok = ok && wait_on(full + 8 * k.s, k.lap & 1u, abort_flag) && wait_on(acc_full, (uint32_t)it & 1u, abort_flag);
+      ok = ok && (!MORE || wait_on(full + 8 * k.s, k.lap & 1u, abort_flag)) && wait_on(acc_full, (uint32_t)it & 1u, abort_flag);
       tc_fence_after();
       if (P.lse && half == 0 && ok) P.lse[((int64_t)b * P.heads + h) * P.seq + i] = (mm + log2f(total)) * 0.6931471805599453f;
-      const uint32_t res = ring + k.s * SLOT_BYTES;
+      const uint32_t res = MORE ? ring + k.s * SLOT_BYTES : own;   // without successors the own rows have been read for good
 #pragma unroll
       for (int pc = 0; pc < 2; ++pc) {
         const int c = half * 32 + pc * 16;
@@ -366,6 +370,11 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
 #pragma unroll
         for (int e = 0; e < 16; ++e) u[e] = __float_as_uint(fmaf(a0, __uint_as_float(u[e]), a1 * __uint_as_float(v[e])));
         stage_row(res, r, c, u, 1.f);
+      }
+      if (!MORE) {
+        ok = meet() && ok;
+        if (ok) write_rows(res, rs, P.Out + ((int64_t)row0 + q0) * P.ldo + h * D, P.ldo, lane);
+        break;
       }
       fence_async_smem();
       tc_fence_before();                                     // the accumulators have been read
@@ -383,7 +392,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
       k.next();
       ok = ok && next(it);
     }
-    if (half == 0 && lane == 0) bulk_wait_read();            // shared memory outlives the copies
+    if (MORE && half == 0 && lane == 0) bulk_wait_read();    // shared memory outlives the copies
   }
   if (*abort_flag) {
     for (int t = 0; t < 2000; ++t) __nanosleep(1000);   // let copies and products in flight land
@@ -394,6 +403,14 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
+}
+
+template <bool MORE, bool FAR>
+mst_status_t launch(dim3 grid, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmO, const FwdParams& P,
+                    cudaStream_t s) {
+  MST_SMEM_LIMIT((strided_attention_fwd_kernel<MORE, FAR>), SMEM_BYTES);
+  MST_CUDA_TRY(mst_launch_overlapped(strided_attention_fwd_kernel<MORE, FAR>, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmO, P));
+  return MST_OK;
 }
 
 }  // namespace
@@ -420,20 +437,21 @@ extern "C" mst_status_t mst_strided_attention_fwd(const void* Q, const void* K, 
   if (batch == 0) return MST_OK;
   const int64_t rows = (int64_t)batch * seq_len;
   if (rows > 0x7FFFFFFF || heads > 65535 || batch > 65535) return MST_ERR_SHAPE;
-  CUtensorMap tmQ, tmK, tmV, tmO;
-  if (!tile_map(&tmQ, Q, rows, width, ld) || !tile_map(&tmK, K, rows, width, ld) || !tile_map(&tmV, V, rows, width, ld) ||
-      !tile_map(&tmO, Out, rows, width, ldo, ROWS / 4))
-    return MST_ERR_SHAPE;
   FwdParams P;
+  P.Out = (__nv_bfloat16*)Out;
+  P.ldo = ldo;
   P.lse = lse;
   P.seq = seq_len; P.heads = heads; P.blocks = seq_len / ROWS;
-  const bool more = (int64_t)P.blocks * heads * batch > 2 * (int64_t)mst_sm_count();
   P.stride = stride < seq_len ? stride : seq_len;   // from there on the same pairs: all earlier positions
   P.magic = stride_magic(P.stride, seq_len);
-  MST_SMEM_LIMIT((strided_attention_fwd_kernel<false>), SMEM_BYTES);
-  MST_SMEM_LIMIT((strided_attention_fwd_kernel<true>), SMEM_BYTES);
-  MST_CUDA_TRY(mst_launch_overlapped(more ? strided_attention_fwd_kernel<true> : strided_attention_fwd_kernel<false>, place_grid(heads, batch, P.blocks, !more && P.stride < P.seq), dim3(THREADS),
-                                     SMEM_BYTES, (cudaStream_t)stream, tmQ, tmK, tmV, tmO, P));
+  const Form form = form_of(batch, heads, P.blocks, P.stride, seq_len);
+  P.blocks_first = form.blocks_first;
+  CUtensorMap tmQ, tmK, tmV, tmO = {};
+  if (!tile_map(&tmQ, Q, rows, width, ld) || !tile_map(&tmK, K, rows, width, ld) || !tile_map(&tmV, V, rows, width, ld) ||
+      (form.more && !tile_map(&tmO, Out, rows, width, ldo, ROWS / 4)))
+    return MST_ERR_SHAPE;
+  const dim3 grid = place_grid(heads, batch, P.blocks, form.blocks_first);
+  MST_TRY((form.more ? launch<true, true> : form.far ? launch<false, true> : launch<false, false>)(grid, tmQ, tmK, tmV, tmO, P, (cudaStream_t)stream));
   MST_CUDA_TRY(cudaGetLastError());
   return MST_OK;
 }

@@ -21,7 +21,8 @@
 // of which only the diagonal counts: warp-level mma.sync products of 16 rows each, whose sums are where the tensor-memory accumulators
 // start (formed row by row on the FMA pipe, as the forward kernel does it, they take a third more instructions here: 128.4 us against 126.6 at l = 256).
 // A block that is done takes over one that has not started; its own rows, the forward output and the first tiles are then in
-// shared memory or on their way.  Results leave by TMA from slots of the ring.
+// shared memory or on their way.  Results leave by TMA from slots of the ring, or, in a block without
+// successors, as whole rows from where the own rows were.
 // Bound: as forward, the chain of a tile through its warps; tensor pipe and issue slots are half busy, DRAM a third.
 // 16 x 1024 tokens, 12 heads, l = 256 144.7 -> 124.2 us, 8 x 1024, 16 heads, l = 128 108.7 -> 87.8.
 #include <cuda.h>
@@ -47,7 +48,9 @@ struct BwdParams {
   int64_t ldo;
   const float* lse;    // [batch, heads, seq]
   float* stat;         // [batch, heads, seq / 64][2][64]: -lse log2 e, -delta
-  int seq, heads, stride, blocks;
+  __nv_bfloat16 *dQ, *dK, *dV;
+  int64_t ldg;
+  int seq, heads, stride, blocks, blocks_first;
   uint32_t magic;
 };
 
@@ -149,14 +152,14 @@ __device__ __forceinline__ bool meet(const Smem& S, int quarter, uint32_t parity
 // The lane that loads: the block's own rows of two operands (and, for the queries' pass, their forward output, in a slot), then tile after tile of two others (and, for the keys' pass, the
 // statistics of the tile's queries), then RESULTS slots that the results leave through.
 template <bool LOOK_BACK, int RESULTS, bool MORE>
-__device__ __forceinline__ void feed(const Smem& S, const BwdParams& P, Place at, const CUtensorMap* own_a, const CUtensorMap* own_b,
+__device__ __forceinline__ void feed(const Smem& S, const BwdParams& P, Place at, const Walk<LOOK_BACK>& first, const CUtensorMap* own_a, const CUtensorMap* own_b,
                                      const CUtensorMap* tile_a, const CUtensorMap* tile_b, const CUtensorMap* own_out, volatile int* abort_flag) {
   Ring<STAGES> k;
   bool ok = true;
   auto slot = [&]() { return k.lap == 0 || wait_on(S.empty + 8 * k.s, (k.lap - 1) & 1u, abort_flag); };
   for (int it = 0; ok; ++it) {
     const int col = at.h * D, row0 = at.b * P.seq;
-    const Walk<LOOK_BACK> walk((LOOK_BACK ? P.blocks - 1 - at.block : at.block) * ROWS, P.stride, P.seq, P.magic);
+    const Walk<LOOK_BACK> walk = MORE ? Walk<LOOK_BACK>((LOOK_BACK ? P.blocks - 1 - at.block : at.block) * ROWS, P.stride, P.seq, P.magic) : first;
     const float* stat = LOOK_BACK ? nullptr : P.stat + 2 * ((int64_t)at.b * P.heads + at.h) * P.seq;
     if (it > 0 && !wait_on(S.own_free, (uint32_t)(it - 1) & 1u, abort_flag)) return;
     mbar_expect_tx(S.own_full, 4 * TILE_BYTES);
@@ -183,6 +186,7 @@ __device__ __forceinline__ void feed(const Smem& S, const BwdParams& P, Place at
       if (!LOOK_BACK) bulk_load(S.stat + k.s * STAT_BYTES, stat + 2 * from, STAT_BYTES, bar);
       k.next();
     }
+    if (!MORE) return;
     for (int e = 0; e < RESULTS; ++e) {
       if (!slot()) return;
       mbar_arrive(S.full + 8 * k.s);
@@ -196,7 +200,7 @@ __device__ __forceinline__ void feed(const Smem& S, const BwdParams& P, Place at
 // ------------------------------------------------------------------------------------------- dQ
 // Tensor memory: S in columns 0-63, dP 64-127, dQ 128-191, dS (bf16) 192-223.  S and dP are free as soon as they are in
 // registers, so the next tile's scores are formed during this tile's algebra.
-template <bool MORE>   // the grid has more blocks than run at once
+template <bool MORE, bool FAR>   // see mst_attention_tile.cuh
 __global__ void __launch_bounds__(THREADS, 2)
 attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmO,
@@ -208,14 +212,16 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   volatile int* abort_flag = &abort_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = P.stride;
-  if (warp == CW && lane < 6) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmO : &tmD);
+  if (warp == CW && lane < (MORE ? 6 : 4)) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmO : &tmD);
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);
+  Walk<true> first((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
+  if (!MORE) first.now();
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);
 
   if (warp == CW) {
-    if (lane == 0) feed<true, 1, MORE>(S, P, at, &tmQ, &tmG, &tmK, &tmV, &tmO, abort_flag);
+    if (lane == 0) feed<true, 1, MORE>(S, P, at, first, &tmQ, &tmG, &tmK, &tmV, &tmO, abort_flag);
   } else if (warp == CW + 1) {
     if (lane == 0) {
       const uint64_t qd = smem_desc(S.own0, 16, 1024), gd = smem_desc(S.own1, 16, 1024), kd0 = smem_desc(S.ring, 16, 1024);
@@ -225,8 +231,8 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       bool ok = true;
       auto filled = [&]() { return wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag); };
       for (int it = 0; ok; ++it) {
-        const Walk<true> walk((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
-        const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
+        const Walk<true> walk = MORE ? Walk<true>((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic) : first;
+        const uint32_t from_far = FAR && walk.far() > 0 ? 1u : 0u;
         const int skip = (MORE ? 1 : 0) + walk.far();        // the forward output, the far tiles
         ok = wait_on(S.own_full, (uint32_t)it & 1u, abort_flag);
         // A slot's parity tells one filling from the next only if the one before is known to be over.  The slots skipped here are filled once the
@@ -301,8 +307,8 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     for (int it = 0; ok; ++it) {
       const int h = at.h, b = at.b, q0 = (P.blocks - 1 - at.block) * ROWS, row0 = b * P.seq;
       const int i = q0 + r;
-      const Walk<true> walk(q0, l, P.seq, P.magic);
-      const int far = walk.far();
+      const Walk<true> walk = MORE ? Walk<true>(q0, l, P.seq, P.magic) : first;
+      const int far = FAR ? walk.far() : 0;
       // delta of this row: the threads of a row take COLS dimensions each
       const bool row_ok = i < P.seq;
       nl *= -LOG2E;
@@ -438,9 +444,9 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       k.skip(walk.near);
       const bool more = ok && next_block<MORE>(S, P, it, at, abort_flag);
       if (more) fetch_row(at);
-      ok = ok && wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag) && wait_on(S.acc_full, (uint32_t)it & 1u, abort_flag);
+      ok = ok && (!MORE || wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag)) && wait_on(S.acc_full, (uint32_t)it & 1u, abort_flag);
       tc_fence_after();
-      const uint32_t res = S.ring + k.s * SLOT_BYTES;
+      const uint32_t res = MORE ? S.ring + k.s * SLOT_BYTES : S.own0;   // without successors the own rows have been read for good
       uint32_t v[PIECES][16];
 #pragma unroll
       for (int pc = 0; pc < PIECES; ++pc) tmem_ld16_nowait(t_row + (uint32_t)(128 + c + pc * 16), v[pc]);
@@ -448,6 +454,11 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       for (int pc = 0; pc < PIECES; ++pc) {
         tmem_ld16_wait(v[pc]);
         stage_row(res, r, c + pc * 16, v[pc], SCALE);
+      }
+      if (!MORE) {
+        ok = meet(S, quarter, 1u, lane, abort_flag) && ok;
+        if (ok && q0 + quarter * 32 < P.seq) write_rows(res, rs, P.dQ + ((int64_t)row0 + q0) * P.ldg + h * D, P.ldg, lane);
+        break;
       }
       fence_async_smem();
       tc_fence_before();                                     // the accumulator has been read
@@ -465,7 +476,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       k.next();
       ok = ok && more;
     }
-    if (c == 0 && lane == 0) bulk_wait_read();               // shared memory outlives the copies
+    if (MORE && c == 0 && lane == 0) bulk_wait_read();       // shared memory outlives the copies
   }
   block_teardown(tmem, warp, abort_flag);
 }
@@ -473,7 +484,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 // ------------------------------------------------------------------------------------------- dK, dV
 // Tensor memory: S^T in columns 0-63, dP^T 64-127, dK 128-191, dV 192-255; each warp writes P^T over the scores it has
 // read (eight columns at its sixteen's start) and dS^T over its dP.
-template <bool MORE>   // the grid has more blocks than run at once
+template <bool MORE, bool FAR>   // see mst_attention_tile.cuh
 __global__ void __launch_bounds__(THREADS, 2)
 attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmDK,
@@ -485,14 +496,16 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   volatile int* abort_flag = &abort_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = P.stride;
-  if (warp == CW && lane < 6) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmDK : &tmDV);
+  if (warp == CW && lane < (MORE ? 6 : 4)) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmDK : &tmDV);
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);   // early keys have the most tiles
+  Walk<false> first(at.block * ROWS, l, P.seq, P.magic);
+  if (!MORE) first.now();
   mst_grid_launch_dependents();
   mst_grid_dependency_wait();
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.stride < P.seq);   // early keys have the most tiles
 
   if (warp == CW) {
-    if (lane == 0) feed<false, 2, MORE>(S, P, at, &tmK, &tmV, &tmQ, &tmG, nullptr, abort_flag);
+    if (lane == 0) feed<false, 2, MORE>(S, P, at, first, &tmK, &tmV, &tmQ, &tmG, nullptr, abort_flag);
   } else if (warp == CW + 1) {
     if (lane == 0) {
       const uint64_t kd = smem_desc(S.own0, 16, 1024), vd = smem_desc(S.own1, 16, 1024), qd0 = smem_desc(S.ring, 16, 1024);
@@ -502,8 +515,8 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       bool ok = true;
       auto filled = [&]() { return wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag); };
       for (int it = 0; ok; ++it) {
-        const Walk<false> walk(at.block * ROWS, l, P.seq, P.magic);
-        const uint32_t from_far = walk.far() > 0 ? 1u : 0u;
+        const Walk<false> walk = MORE ? Walk<false>(at.block * ROWS, l, P.seq, P.magic) : first;
+        const uint32_t from_far = FAR && walk.far() > 0 ? 1u : 0u;
         ok = wait_on(S.own_full, (uint32_t)it & 1u, abort_flag);
         if (MORE || walk.far() + 1 > STAGES) ok = ok && wait_on(S.far_over, (uint32_t)it & 1u, abort_flag);   // as in dQ, for one tile
         k.skip(walk.far());
@@ -555,8 +568,8 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     for (int it = 0; ok; ++it) {
       const int h = at.h, k0 = at.block * ROWS, row0 = at.b * P.seq;
       const int jk = k0 + r, j_lo = k0 + quarter * 32;       // this thread's key, this warp's: j_lo .. j_lo + 31
-      const Walk<false> walk(k0, l, P.seq, P.magic);
-      const int far = walk.far();
+      const Walk<false> walk = MORE ? Walk<false>(k0, l, P.seq, P.magic) : first;
+      const int far = FAR ? walk.far() : 0;
       if (it > 0 && c == 0 && lane == 0) {                   // the copies of the last results have read them, long since: their slots may be filled again
         bulk_wait_read();
         mbar_arrive(S.empty + 8 * ((k.s + STAGES - 2) % STAGES));
@@ -692,8 +705,8 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       uint32_t at_slot[2];
 #pragma unroll
       for (int which = 0; which < 2; ++which) {              // dK and dV, through a slot each
-        ok = ok && wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag);
-        at_slot[which] = k.s;
+        ok = ok && (!MORE || wait_on(S.full + 8 * k.s, k.lap & 1u, abort_flag));
+        at_slot[which] = MORE ? S.ring + k.s * SLOT_BYTES : which ? S.own1 : S.own0;
         k.next();
         uint32_t v[PIECES][16];
 #pragma unroll
@@ -701,8 +714,16 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int pc = 0; pc < PIECES; ++pc) {
           tmem_ld16_wait(v[pc]);
-          stage_row(S.ring + at_slot[which] * SLOT_BYTES, r, c + pc * 16, v[pc], which ? 1.f : SCALE);
+          stage_row(at_slot[which], r, c + pc * 16, v[pc], which ? 1.f : SCALE);
         }
+      }
+      if (!MORE) {
+        ok = meet(S, quarter, 0u, lane, abort_flag) && ok;
+        if (ok && k0 + quarter * 32 < P.seq) {
+          write_rows(at_slot[0], rs, P.dK + ((int64_t)row0 + k0) * P.ldg + h * D, P.ldg, lane);
+          write_rows(at_slot[1], rs, P.dV + ((int64_t)row0 + k0) * P.ldg + h * D, P.ldg, lane);
+        }
+        break;
       }
       fence_async_smem();
       tc_fence_before();                                     // the accumulators have been read
@@ -711,20 +732,30 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (lane == 0) {
         if (c == 0) {
           if (ok && k0 + quarter * 32 < P.seq) {
-            tma_store_2d(&tmDK, S.ring + at_slot[0] * SLOT_BYTES + (uint32_t)quarter * 32u * 128u, h * D, row0 + k0 + quarter * 32);
-            tma_store_2d(&tmDV, S.ring + at_slot[1] * SLOT_BYTES + (uint32_t)quarter * 32u * 128u, h * D, row0 + k0 + quarter * 32);
+            tma_store_2d(&tmDK, at_slot[0] + (uint32_t)quarter * 32u * 128u, h * D, row0 + k0 + quarter * 32);
+            tma_store_2d(&tmDV, at_slot[1] + (uint32_t)quarter * 32u * 128u, h * D, row0 + k0 + quarter * 32);
           }
           bulk_commit();
         } else {
-          mbar_arrive(S.empty + 8 * at_slot[0]);
-          mbar_arrive(S.empty + 8 * at_slot[1]);
+          mbar_arrive(S.empty + 8 * ((k.s + STAGES - 2) % STAGES));
+          mbar_arrive(S.empty + 8 * ((k.s + STAGES - 1) % STAGES));
         }
       }
       ok = ok && next_block<MORE>(S, P, it, at, abort_flag);
     }
-    if (c == 0 && lane == 0) bulk_wait_read();               // shared memory outlives the copies
+    if (MORE && c == 0 && lane == 0) bulk_wait_read();       // shared memory outlives the copies
   }
   block_teardown(tmem, warp, abort_flag);
+}
+
+struct Maps { CUtensorMap Q, K, V, G, O, dQ, dK, dV; };
+template <bool MORE, bool FAR>
+mst_status_t launch(dim3 grid, const Maps& m, const BwdParams& P, cudaStream_t s) {
+  MST_SMEM_LIMIT((attn_bwd_dq_kernel<MORE, FAR>), SMEM_BYTES);
+  MST_SMEM_LIMIT((attn_bwd_dkv_kernel<MORE, FAR>), SMEM_BYTES);
+  MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dq_kernel<MORE, FAR>, grid, dim3(THREADS), SMEM_BYTES, s, m.Q, m.K, m.V, m.G, m.O, m.dQ, P));
+  MST_CUDA_TRY(mst_launch_overlapped(attn_bwd_dkv_kernel<MORE, FAR>, grid, dim3(THREADS), SMEM_BYTES, s, m.Q, m.K, m.V, m.G, m.dK, m.dV, P));
+  return MST_OK;
 }
 
 }  // namespace
@@ -754,10 +785,14 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
   const int64_t rows = (int64_t)batch * seq_len;
   if (rows > 0x7FFFFFFF || heads > 65535 || batch > 65535) return MST_ERR_SHAPE;
   cudaStream_t s = (cudaStream_t)stream;
-  CUtensorMap tmQ, tmK, tmV, tmG, tmO, tmDQ, tmDK, tmDV;
-  if (!tile_map(&tmQ, Q, rows, width, ld) || !tile_map(&tmK, K, rows, width, ld) || !tile_map(&tmV, V, rows, width, ld) ||
-      !tile_map(&tmG, dOut, rows, width, lddo) || !tile_map(&tmO, Out, rows, width, ldo) || !tile_map(&tmDQ, dQ, rows, width, ldg, ROWS / 4) ||
-      !tile_map(&tmDK, dK, rows, width, ldg, ROWS / 4) || !tile_map(&tmDV, dV, rows, width, ldg, ROWS / 4))
+  const int blocks = (seq_len + ROWS - 1) / ROWS, l = stride < seq_len ? stride : seq_len;   // from there on the same pairs: all earlier positions
+  const Form form = form_of(batch, heads, blocks, l, seq_len);
+  Maps m = {};
+  if (!tile_map(&m.Q, Q, rows, width, ld) || !tile_map(&m.K, K, rows, width, ld) || !tile_map(&m.V, V, rows, width, ld) ||
+      !tile_map(&m.G, dOut, rows, width, lddo))
+    return MST_ERR_SHAPE;
+  if (form.more && (!tile_map(&m.O, Out, rows, width, ldo) || !tile_map(&m.dQ, dQ, rows, width, ldg, ROWS / 4) ||
+                    !tile_map(&m.dK, dK, rows, width, ldg, ROWS / 4) || !tile_map(&m.dV, dV, rows, width, ldg, ROWS / 4)))
     return MST_ERR_SHAPE;
   void* ws = nullptr;
   MST_TRY(mst_workspace_kind(MST_WS_ATTENTION, 2 * sizeof(float) * (size_t)rows * heads, &ws));
@@ -765,17 +800,13 @@ extern "C" mst_status_t mst_strided_attention_bwd(const void* Q, const void* K, 
   P.Out = (const __nv_bfloat16*)Out;
   P.ldo = ldo;
   P.lse = lse; P.stat = (float*)ws;
-  P.seq = seq_len; P.heads = heads; P.blocks = (seq_len + ROWS - 1) / ROWS;
-  const bool more = (int64_t)P.blocks * heads * batch > 2 * (int64_t)mst_sm_count();
-  P.stride = stride < seq_len ? stride : seq_len;   // from there on the same pairs: all earlier positions
-  P.magic = stride_magic(P.stride, seq_len);
-  MST_SMEM_LIMIT((attn_bwd_dq_kernel<false>), SMEM_BYTES);
-  MST_SMEM_LIMIT((attn_bwd_dq_kernel<true>), SMEM_BYTES);
-  MST_SMEM_LIMIT((attn_bwd_dkv_kernel<false>), SMEM_BYTES);
-  MST_SMEM_LIMIT((attn_bwd_dkv_kernel<true>), SMEM_BYTES);
-  const dim3 grid = place_grid(heads, batch, P.blocks, !more && P.stride < P.seq);
-  MST_CUDA_TRY(mst_launch_overlapped(more ? attn_bwd_dq_kernel<true> : attn_bwd_dq_kernel<false>, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, tmO, tmDQ, P));
-  MST_CUDA_TRY(mst_launch_overlapped(more ? attn_bwd_dkv_kernel<true> : attn_bwd_dkv_kernel<false>, grid, dim3(THREADS), SMEM_BYTES, s, tmQ, tmK, tmV, tmG, tmDK, tmDV, P));
+  P.dQ = (__nv_bfloat16*)dQ; P.dK = (__nv_bfloat16*)dK; P.dV = (__nv_bfloat16*)dV;
+  P.ldg = ldg;
+  P.seq = seq_len; P.heads = heads; P.blocks = blocks; P.blocks_first = form.blocks_first;
+  P.stride = l;
+  P.magic = stride_magic(l, seq_len);
+  const dim3 grid = place_grid(heads, batch, blocks, form.blocks_first);
+  MST_TRY((form.more ? launch<true, true> : form.far ? launch<false, true> : launch<false, false>)(grid, m, P, s));
   MST_CUDA_TRY(cudaGetLastError());
   return MST_OK;
 }

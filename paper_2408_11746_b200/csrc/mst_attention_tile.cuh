@@ -71,13 +71,19 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
 // operands are on their way while this one's last products and results are.  The request goes out at a block's start, its answer (16 bytes
 // by the async proxy) is read by every role at the block's end; a proxy fence of the reader's, before it lets go of the next block's own
 // rows, orders that ahead of the answer after next, which comes to the same place.  No request follows one that found nothing left.
-// Grids that run at once leave all of this out (template argument MORE): its instructions alone cost a launch 0.4 us.
+// Grids that run at once leave all of this out (template argument MORE): its instructions alone cost a launch 0.4 us.  Their results
+// leave as whole rows by the warps, which nothing follows: through a ring slot and the TMA unit they took 0.3 us a kernel longer.  What a block
+// walks is worked out ahead of the wait for the kernel before, and windows that reach back half of the sequence or more, so that
+// there are no far tiles, have kernels without them (FAR: 0.4 us a kernel for code that is only jumped over, as the kernels of a pass take turns in the
+// instruction cache).  Forward and backward, before / after each of these: 1 x 256 tokens, 6 heads, l = 256 23.3 / 21.8 / 22.0 / 21.6 us,
+// 2 x 512, 12 heads, l = 256 33.8 / 33.0 / 32.2 / 31.9, 3 x 768, 15 heads, l = 512 49.6 / 49.6 / 49.3 / 48.6; with far tiles 3 x 640, 9 heads, l = 128
+// 38.3 / 37.3 / 37.1.  (Rows stored straight from the registers, 16 bytes of each at a time: 1 to 3 us longer.)
 // Grid: heads, batch, blocks of a sequence, those with the most tiles first.  (Blocks fastest, as their keys and values are then found in
 // L2, left the SMs idle for a quarter of the time at the end: 8 x 1024 tokens, 16 heads, l = 128 have 3.5 blocks for each of the
 // 296 that run at once; 16 x 1024 tokens, 12 heads, l = 256 backward 153.6 -> 132.6 us by the order.)  Where four operands exceed L2
 // the batch is gone through in equal parts that do not, or far tiles and the next kernel's rows come from DRAM (9 x 1792
 // tokens, 20 heads, forward and backward 338 -> 321 us in three parts; 16 x 1024, 12 heads, which fit: 169 in one part, 174 in two, 177 in four).
-// Grids that run at once (no last wave to fill) have a sequence's blocks first where the window is shorter than the sequence, so that blocks with
+// Grids that run at once (two blocks to an SM, no last wave to fill) have a sequence's blocks first where the window is shorter than the sequence, so that blocks with
 // tiles in common are neighbours: forward and backward 1 x 1024 tokens, 6 heads, l = 128 43.3 -> 39.6 us, 2 x 1024, 9 heads, l = 256 42.5 -> 40.2; windows
 // of the whole sequence lose by it (3 x 512, 10 heads 39.3 -> 41.9, 2 x 256, 20 heads 26.8 -> 28.4).
 // Sequences of more blocks than the grid's third dimension holds have them in its first.
@@ -99,6 +105,11 @@ inline dim3 place_grid(int heads, int batch, int blocks, bool blocks_first) {
   while (parts < batch && (batch % parts || bytes * (batch / parts) > L2_BYTES)) ++parts;
   if ((int64_t)blocks * parts > GRID_Z) parts = 1;
   return dim3((unsigned)heads, (unsigned)(batch / parts), (unsigned)(blocks * parts));
+}
+struct Form { bool more, far, blocks_first; };
+inline Form form_of(int batch, int heads, int blocks, int stride, int seq) {
+  const int64_t all = (int64_t)batch * heads * blocks, at_once = 2 * (int64_t)mst_sm_count();
+  return Form{all > at_once, seq - stride > stride, all <= at_once && stride < seq};
 }
 __device__ __forceinline__ void take_over(uint32_t answer, uint32_t bar) {
   mbar_expect_tx(bar, 16);
@@ -215,6 +226,8 @@ struct Walk {
     both = 2 * (far0 < far1 ? far0 : far1);
     total = near + far0 + far1;
   }
+  // worked out here, not where it is first used
+  __device__ __forceinline__ void now() { asm volatile("" : "+r"(first), "+r"(near), "+r"(far0), "+r"(far1), "+r"(both), "+r"(total)); }
   // far tile f: which half of the own rows, and where the tile starts.  The halves take turns while both have tiles left, the one
   // with more of them first, and the ring has an even number of slots: each half's tiles come in slots of its own.
   __device__ __forceinline__ int far() const { return far0 + far1; }
@@ -392,6 +405,14 @@ __device__ __forceinline__ void stage_row(uint32_t slot, int row, int col, const
     for (int e = 0; e < 4; ++e) w[e] = pack_bf16(__uint_as_float(v[8 * g + 2 * e]) * scale, __uint_as_float(v[8 * g + 2 * e + 1]) * scale);
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(piece_addr(slot, row, col / 8 + g)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
                  : "memory");
+  }
+}
+// sixteen rows of the slot from `first` on -> the caller's rows, eight lanes per row of 128 bytes
+__device__ __forceinline__ void write_rows(uint32_t slot, int first, __nv_bfloat16* out, int64_t ld, int lane) {
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int r = first + it * 4 + (lane >> 3);
+    *reinterpret_cast<uint4*>(out + r * ld + (lane & 7) * 8) = lds128(piece_addr(slot, r, lane & 7));
   }
 }
 // [rows x cols] bf16, ld elements between rows; box = 64 rows x 64 columns (one head of 64 tokens), or the 32 rows of a lane quarter's results

@@ -27,7 +27,11 @@ def _forward_reference(qkv, B, n, H, stride):
     (6, 704, 17, 192),     # the same, far tiles in odd and even numbers
     (5, 1152, 12, 128),    # up to sixteen far tiles, 540 blocks
     (2, 1152, 6, 128),     # none to sixteen of them in blocks without successors: slots filled for the first time and again
-    (1, 832, 7, 192)])     # the same, odd numbers
+    (1, 832, 7, 192),      # the same, odd numbers
+    (1, 256, 6, 256),      # windows of the whole sequence: kernels without far tiles
+    (2, 768, 5, 384),      # windows of half of it
+    (3, 320, 5, 192),      # the same with half a block at the end
+    (2, 64, 3, 64)])       # nothing but half a block
 def test_blocks_that_take_over_others(B, n, H, stride):
     gen = torch.Generator(device="cuda").manual_seed(n + stride)
     C = 64 * H
