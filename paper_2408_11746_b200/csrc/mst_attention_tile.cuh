@@ -71,7 +71,11 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
 // operands are on their way while this one's last products and results are.  The request goes out at a block's start, its answer (16 bytes
 // by the async proxy) is read by every role at the block's end; a proxy fence of the reader's, before it lets go of the next block's own
 // rows, orders that ahead of the answer after next, which comes to the same place.  No request follows one that found nothing left.
-// Grids that run at once leave all of this out (template argument MORE): its instructions alone cost a launch 0.4 us.  Their results
+// The block to come is claimed when its predecessor starts, not by whoever is done first, so it pays where each of those that run at once has more
+// than two to see to (MORE): at 297 of 296 blocks 9 x 384 tokens, 11 heads, l = 128 took 40.0 us with it, 33.9 without, 3 x 1536, 9 heads, l = 192 (324) 63.7
+// and 50.0, 5 x 1152, 13 heads, l = 256 (585) 75.1 and 71.9, 3 x 2048, 14 heads, l = 128 (672) 114.0 and 118.2, 6 x 1024, 17 heads, l = 256 (816) 97.3
+// and 101.1.
+// Fewer blocks leave all of this out: its instructions alone cost a launch 0.4 us.  Their results
 // leave as whole rows by the warps, which nothing follows: through a ring slot and the TMA unit they took 0.3 us a kernel longer.  What a block
 // walks is worked out ahead of the wait for the kernel before, and windows that reach back half of the sequence or more, so that
 // there are no far tiles, have kernels without them (FAR: 0.4 us a kernel for code that is only jumped over, as the kernels of a pass take turns in the
@@ -109,7 +113,7 @@ inline dim3 place_grid(int heads, int batch, int blocks, bool blocks_first) {
 struct Form { bool more, far, blocks_first; };
 inline Form form_of(int batch, int heads, int blocks, int stride, int seq) {
   const int64_t all = (int64_t)batch * heads * blocks, at_once = 2 * (int64_t)mst_sm_count();
-  return Form{all > at_once, seq - stride > stride, all <= at_once && stride < seq};
+  return Form{all > 2 * at_once, seq - stride > stride, all <= at_once && stride < seq};
 }
 __device__ __forceinline__ void take_over(uint32_t answer, uint32_t bar) {
   mbar_expect_tx(bar, 16);

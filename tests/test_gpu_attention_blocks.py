@@ -21,11 +21,12 @@ def _forward_reference(qkv, B, n, H, stride):
 
 @pytest.mark.parametrize("B,n,H,stride", [
     (8, 128, 37, 64),      # 296 blocks: all of them run at once on 148 SMs
-    (9, 384, 11, 128),     # 297: one is taken over
+    (9, 384, 11, 128),     # 297: one starts when another is done
+    (8, 256, 37, 64),      # 592: the most of which none is taken over
     (16, 256, 20, 192),    # 640
     (8, 448, 19, 64),      # an odd number of 64-row tiles: the last block has half its rows, its second half no far tiles
     (6, 704, 17, 192),     # the same, far tiles in odd and even numbers
-    (5, 1152, 12, 128),    # up to sixteen far tiles, 540 blocks
+    (6, 1152, 12, 128),    # up to sixteen far tiles, 648 blocks
     (2, 1152, 6, 128),     # none to sixteen of them in blocks without successors: slots filled for the first time and again
     (1, 832, 7, 192),      # the same, odd numbers
     (1, 256, 6, 256),      # windows of the whole sequence: kernels without far tiles
