@@ -98,7 +98,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = holder;
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, P.heads, !MORE && P.blocks_first);
   Walk<true> first((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
   if (!MORE) first.now();
   mst_grid_launch_dependents();
@@ -106,7 +106,7 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
 
   Ring<STAGES> k;
   // the next block, if there is one (block `it` of this one's life is at its end)
-  auto next = [&](int it) { return MORE && wait_on(next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(answers + 16 * (it & 1), at, P.blocks); };
+  auto next = [&](int it) { return MORE && wait_on(next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(answers + 16 * (it & 1), at, P.blocks, P.heads); };
   auto next_fenced = [&](int it) {   // for the lanes that have no other fence ahead of their part in the own rows' release
     const bool more = next(it);
     fence_async_smem();

@@ -140,7 +140,7 @@ __device__ __forceinline__ void block_teardown(uint32_t tmem, int warp, volatile
 // block `it` of this one's life is at its end: the next one, if there is one (the warps' fence comes with the own rows' release)
 template <bool MORE>
 __device__ __forceinline__ bool next_block(const Smem& S, const BwdParams& P, int it, Place& at, volatile int* abort_flag) {
-  return MORE && wait_on(S.next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(S.answers + 16 * (it & 1), at, P.blocks);
+  return MORE && wait_on(S.next_full + 8 * (it & 1), (uint32_t)(it >> 1) & 1u, abort_flag) && taken_over(S.answers + 16 * (it & 1), at, P.blocks, P.heads);
 }
 // the two warps of a lane quarter meet
 __device__ __forceinline__ bool meet(const Smem& S, int quarter, uint32_t parity, int lane, volatile int* abort_flag) {
@@ -214,7 +214,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   const int l = P.stride;
   if (warp == CW && lane < (MORE ? 6 : 4)) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmO : &tmD);
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, P.heads, !MORE && P.blocks_first);
   Walk<true> first((P.blocks - 1 - at.block) * ROWS, l, P.seq, P.magic);
   if (!MORE) first.now();
   mst_grid_launch_dependents();
@@ -498,7 +498,7 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const int l = P.stride;
   if (warp == CW && lane < (MORE ? 6 : 4)) prefetch_map(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmG : lane == 4 ? &tmDK : &tmDV);
   const uint32_t tmem = block_setup(S, &holder, &abort_sh, warp);
-  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, !MORE && P.blocks_first);   // early keys have the most tiles
+  Place at = place((int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, P.blocks, P.heads, !MORE && P.blocks_first);   // early keys have the most tiles
   Walk<false> first(at.block * ROWS, l, P.seq, P.magic);
   if (!MORE) first.now();
   mst_grid_launch_dependents();

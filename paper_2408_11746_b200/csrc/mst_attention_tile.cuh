@@ -9,7 +9,9 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <cmath>
 #include <cstdint>
+#include <numeric>
 
 #include "mst_internal.cuh"
 #include "mst_tc_gemm.cuh"
@@ -85,8 +87,11 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
 // Grid: heads, batch, blocks of a sequence, those with the most tiles first.  (Blocks fastest, as their keys and values are then found in
 // L2, left the SMs idle for a quarter of the time at the end: 8 x 1024 tokens, 16 heads, l = 128 have 3.5 blocks for each of the
 // 296 that run at once; 16 x 1024 tokens, 12 heads, l = 256 backward 153.6 -> 132.6 us by the order.)  Where four operands exceed L2
-// the batch is gone through in equal parts that do not, or far tiles and the next kernel's rows come from DRAM (9 x 1792
-// tokens, 20 heads, forward and backward 338 -> 321 us in three parts; 16 x 1024, 12 heads, which fit: 169 in one part, 174 in two, 177 in four).
+// it is gone through in equal parts that do not, as few as possible, of the batch or of the heads or of both, or far tiles and the
+// next kernel's rows come from DRAM (9 x 1792 tokens, 20 heads, forward and backward 338 -> 321 us in three parts, 16 x 2048, 20 heads, l = 128 922 -> 737;
+// 16 x 1024, 12 heads, which fit: 169 in one part, 174 in two, 177 in four.  Each part starts with its heaviest blocks again, so many small parts cost as
+// well: 13 x 1024 tokens, 20 heads, l = 128 246 us in thirteen parts of the batch, 229 in two of the heads; 13 x 1664, 13 heads, l = 512, where thirteen is
+// the least, 348 in them and 339 in one, with a seventh more than L2 holds.)
 // Grids that run at once (two blocks to an SM, no last wave to fill) have a sequence's blocks first where the window is shorter than the sequence, so that blocks with
 // tiles in common are neighbours: forward and backward 1 x 1024 tokens, 6 heads, l = 128 43.3 -> 39.6 us, 2 x 1024, 9 heads, l = 256 42.5 -> 40.2; windows
 // of the whole sequence lose by it (3 x 512, 10 heads 39.3 -> 41.9, 2 x 256, 20 heads 26.8 -> 28.4).
@@ -94,21 +99,33 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
 struct Place { int h, b, block; };
 constexpr int GRID_Z = 65535;
 constexpr double L2_BYTES = 126e6;
-__device__ __forceinline__ Place place(int x, int y, int z, int blocks, bool blocks_first) {
+__device__ __forceinline__ Place place(int x, int y, int z, int blocks, int heads, bool blocks_first) {
   if (blocks_first || blocks > GRID_Z) return Place{y, z, x};
-  while (z >= blocks) {
+  while (z >= blocks) {   // the next part
     z -= blocks;
-    y += (int)gridDim.y;
+    x += (int)gridDim.x;
+    if (x >= heads) {
+      x -= heads;
+      y += (int)gridDim.y;
+    }
   }
   return Place{x, y, z};
 }
 inline dim3 place_grid(int heads, int batch, int blocks, bool blocks_first) {
   if (blocks_first || blocks > GRID_Z) return dim3((unsigned)blocks, (unsigned)heads, (unsigned)batch);
-  const double bytes = 4.0 * 2.0 * (double)blocks * ROWS * heads * D;   // of one sequence
-  int parts = 1;
-  while (parts < batch && (batch % parts || bytes * (batch / parts) > L2_BYTES)) ++parts;
-  if ((int64_t)blocks * parts > GRID_Z) parts = 1;
-  return dim3((unsigned)heads, (unsigned)(batch / parts), (unsigned)(blocks * parts));
+  const double share = 4.0 * 2.0 * (double)blocks * ROWS * heads * D * batch / L2_BYTES;
+  int of_batch = 1, of_heads = 1;
+  const int64_t least = (int64_t)ceil(share);
+  for (int64_t parts = least; least > 1 && parts <= 8 * least; ++parts) {
+    const int64_t g = std::gcd(parts, (int64_t)batch);
+    if (heads % (parts / g) == 0) {
+      of_batch = (int)g;
+      of_heads = (int)(parts / g);
+      break;
+    }
+  }
+  if ((int64_t)blocks * of_batch * of_heads > GRID_Z || (share < 1.3 && of_batch * of_heads > 4)) of_batch = of_heads = 1;
+  return dim3((unsigned)(heads / of_heads), (unsigned)(batch / of_batch), (unsigned)(blocks * of_batch * of_heads));
 }
 struct Form { bool more, far, blocks_first; };
 inline Form form_of(int batch, int heads, int blocks, int stride, int seq) {
@@ -119,7 +136,7 @@ __device__ __forceinline__ void take_over(uint32_t answer, uint32_t bar) {
   mbar_expect_tx(bar, 16);
   asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
 }
-__device__ __forceinline__ bool taken_over(uint32_t answer, Place& p, int blocks) {
+__device__ __forceinline__ bool taken_over(uint32_t answer, Place& p, int blocks, int heads) {
   uint32_t ok, x, y, z;
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
@@ -131,7 +148,7 @@ __device__ __forceinline__ bool taken_over(uint32_t answer, Place& p, int blocks
       : "=r"(x), "=r"(y), "=r"(z), "=r"(ok)
       : "r"(answer)
       : "memory");
-  p = place((int)x, (int)y, (int)z, blocks, false);
+  p = place((int)x, (int)y, (int)z, blocks, heads, false);
   return ok != 0;
 }
 

@@ -27,6 +27,10 @@ def _forward_reference(qkv, B, n, H, stride):
     (8, 448, 19, 64),      # an odd number of 64-row tiles: the last block has half its rows, its second half no far tiles
     (6, 704, 17, 192),     # the same, far tiles in odd and even numbers
     (6, 1152, 12, 128),    # up to sixteen far tiles, 648 blocks
+    (34, 384, 19, 128),    # more than L2 holds: the batch in two parts
+    (37, 384, 18, 192),    # the heads in two, as nothing divides the batch
+    (98, 256, 20, 128),    # both in two
+    (23, 512, 23, 256),    # one part, as the least number would be twenty-three
     (2, 1152, 6, 128),     # none to sixteen of them in blocks without successors: slots filled for the first time and again
     (1, 832, 7, 192),      # the same, odd numbers
     (1, 256, 6, 256),      # windows of the whole sequence: kernels without far tiles
