@@ -73,7 +73,8 @@ enum { M_FORWARD, M_INPUT, M_GRADIENT };
 enum {
   K_BF16, K_F32, K_SAMPLED,
   K_ACT,    // bf16 with an activation
-  K_REDO,   // bf16, with or without one, where sums that are not finite are formed again
+  K_REDO, K_REDO_ACT,   // bf16 without and with one, where sums that are not finite are formed again (one kernel for both, a ring stage short: 770 -> 3072 at
+                        // 8192 tokens 38.3 -> 37.3 us, its input gradient 37.1 -> 36.3)
   K_ROWS    // whatever the TMA unit cannot describe
 };
 
@@ -134,7 +135,7 @@ __device__ __forceinline__ uint64_t gelu_grad_pair(float x0, float x1) {
 }
 
 // For calls that want sums that are not finite formed again: this warp's share of the accumulator, ahead of the epilogue that stores it
-// and into the same places.  A pass of its own (a launch with such rows pays 0.1-1.2 us for it: 770 -> 3072 at 8192 tokens 38.8 -> 39.9): the test inside the epilogues cost the
+// and into the same places.  A pass of its own (a launch with such rows pays 0.1-1.2 us for it): the test inside the epilogues cost the
 // fused activation of calls that have no use for it 2 %, and sending these calls through the row-by-row epilogue cost them 14 %.
 __device__ __forceinline__ void redo_tile(const Params& P, uint32_t tmem_base, int acc, int q, int c0, int step, int lane, int64_t m0, int n0, int cols) {
   const int64_t row0 = m0 + q * 32;
@@ -529,7 +530,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmP, const Params P) {
   const bool A_MN = P.major == M_GRADIENT, B_MN = P.major != M_FORWARD;
-  constexpr int RING = STAGES - (KIND == K_ACT || KIND == K_REDO ? 1 : 0);
+  constexpr bool ACT = KIND == K_ACT || KIND == K_REDO_ACT, REDO = KIND == K_REDO || KIND == K_REDO_ACT;
+  constexpr int RING = STAGES - (ACT ? 1 : 0);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;  // swizzled tiles need 1024-byte alignment
@@ -642,7 +644,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;  // tensor-memory lane quarter this warp may read
-    const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
+    const bool fetch = ACT && P.act == MST_ACT_GELU_GRAD;
     const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
     const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((STAGES - 1) * STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
     ActBoxes A = {{box, box1}, {pre0 + 16 * (warp - 2), pre0 + 16 * (warp - 2) + 8}, 0};
@@ -669,11 +671,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
+      if (REDO) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, BN);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, BN);
       }
-      if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
+      if (ACT) {
         if (!(P.major == M_INPUT ? epilogue_tile_act<true>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)
                                  : epilogue_tile_act<false>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)))
           break;
@@ -758,7 +760,7 @@ struct PairJobs {
       const uint32_t row = tile / (uint32_t)P.n_tiles;
       m0 = (int)row * (2 * BM);
       n0 = (int)(tile - row * (uint32_t)P.n_tiles) * BN;
-      if (KIND == K_BF16 || KIND == K_ACT || KIND == K_REDO || (KIND == K_ROWS && P.epilogue == MST_TC_OUT_BF16)) {
+      if (KIND == K_BF16 || KIND == K_ACT || KIND == K_REDO || KIND == K_REDO_ACT || (KIND == K_ROWS && P.epilogue == MST_TC_OUT_BF16)) {
         n0 += (int)part * (BN / 2);
         cols = cut || P.N - n0 <= BN / 2 ? BN / 2 : BN;
         if (n0 >= P.N) continue;   // that half lies outside the output
@@ -828,7 +830,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     const __grid_constant__ CUtensorMap tmBn, const __grid_constant__ CUtensorMap tmC,
                     const __grid_constant__ CUtensorMap tmP, const Params P) {
   constexpr bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
-  constexpr int RING = P_STAGES - (KIND == K_ACT || KIND == K_REDO ? 1 : 0);
+  constexpr bool ACT = KIND == K_ACT || KIND == K_REDO_ACT, REDO = KIND == K_REDO || KIND == K_REDO_ACT;
+  constexpr int RING = P_STAGES - (ACT ? 1 : 0);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -943,7 +946,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else {
     // ------------------------------------------------------------------ epilogue (both blocks, own 128 rows)
     const int q = warp & 3;
-    const bool fetch = (KIND == K_ACT || KIND == K_REDO) && P.act == MST_ACT_GELU_GRAD;
+    const bool fetch = ACT && P.act == MST_ACT_GELU_GRAD;
     const int c0 = (warp - 2) >> 2;   // the warps of a lane quarter interleave their chunks
     const uint32_t box = out_base + (uint32_t)(warp - 2) * OUT_BOX_BYTES, box1 = tiles_base + (uint32_t)((P_STAGES - 1) * P_STAGE_BYTES + (warp - 2) * OUT_BOX_BYTES);
     ActBoxes A = {{box, box1}, {pre0 + 16 * (warp - 2), pre0 + 16 * (warp - 2) + 8}, 0};
@@ -973,11 +976,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       first = false;
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (KIND == K_REDO) {   // the chunks this warp stores: pairs of them
+      if (REDO) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, J.cols);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, J.cols);
       }
-      if (KIND == K_ACT || (KIND == K_REDO && P.act)) {
+      if (ACT) {
         if (!epilogue_tile_act<MAJOR == M_INPUT>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, J.cols, abort_flag)) break;
         if (fetch) {
           PairJobs<KIND> N = J;
@@ -1340,7 +1343,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (const char* e = mst_getenv(env, "MST_TC_TMA_OUT")) {
     if (e[0] == '0') P.tma_out = 0;
   }
-  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !P.tma_out ? K_ROWS : P.redo.kind ? K_REDO : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
+  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !P.tma_out ? K_ROWS : P.redo.kind ? (P.act ? K_REDO_ACT : K_REDO) : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
   if (pair) {
     const int64_t jobs = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits, max_pairs = mst_sm_count() / 2, rest = jobs % max_pairs;
     CUtensorMap tmBn = tmB;
@@ -1362,10 +1365,12 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       MST_LAUNCH_KIND(K_BF16, M_FORWARD);
       MST_LAUNCH_KIND(K_ACT, M_FORWARD);
       MST_LAUNCH_KIND(K_REDO, M_FORWARD);
+      MST_LAUNCH_KIND(K_REDO_ACT, M_FORWARD);
       MST_LAUNCH_KIND(K_ROWS, M_FORWARD);
       MST_LAUNCH_KIND(K_BF16, M_INPUT);
       MST_LAUNCH_KIND(K_ACT, M_INPUT);
       MST_LAUNCH_KIND(K_REDO, M_INPUT);
+      MST_LAUNCH_KIND(K_REDO_ACT, M_INPUT);
       MST_LAUNCH_KIND(K_ROWS, M_INPUT);
       MST_LAUNCH_KIND(K_F32, M_GRADIENT);
       MST_LAUNCH_KIND(K_SAMPLED, M_GRADIENT);
@@ -1387,6 +1392,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       MST_LAUNCH_KIND(K_SAMPLED);
       MST_LAUNCH_KIND(K_ACT);
       MST_LAUNCH_KIND(K_REDO);
+      MST_LAUNCH_KIND(K_REDO_ACT);
       MST_LAUNCH_KIND(K_ROWS);
     }
 #undef MST_LAUNCH_KIND

@@ -117,7 +117,9 @@ def test_fp32_gradients(O, I, T):
     (519, 520, 7),       # rows of the output start anywhere
     (130, 91, 100),      # small tiles
     (515, 136, 300),
-    (1100, 515, 6000)])  # block pairs, results by TMA (input gradient: row by row)
+    (1100, 515, 6000),   # block pairs, rows of both results start anywhere
+    (1104, 515, 6000),   # forward: copied rows, results by TMA
+    (515, 1104, 6000)])  # input gradient: the same
 def test_bf16_rows_that_start_anywhere(O, I, T):
     _products(O, I, T, "bf16", 1e-2, O)
 
