@@ -58,7 +58,7 @@ struct Params {
   int act;
   void* pre;
   int64_t ldpre;
-  int tma_out;  // rows leave through shared memory and TMA stores (tensor map tmC) instead of per-thread stores
+  int whole;    // bf16 rows by TMA: columns up to here, the last whole 16 bytes of a row, are in the map; the others leave by the lanes
   mst_redo redo;          // rows of bf16: sums that are not finite are formed again
   int sampled_stage_min;  // sampled output: a 32 x 32 chunk with at least this many kept entries leaves row by row
 };
@@ -350,6 +350,20 @@ __device__ __forceinline__ void stage_bf16(uint32_t my_row, uint32_t piece, cons
                : "memory");
 }
 
+// The TMA unit writes whole 16-byte pieces: of a row that ends inside one it would overwrite up to seven columns beyond, which are
+// the caller's.  This lane's row of a box of 64 columns from n on: those behind the last whole piece.  Ahead of the fence that lets the box go.
+__device__ __forceinline__ void store_tail(const Params& P, uint32_t my_row, uint32_t sw, void* out, int64_t ld, int64_t m, int n) {
+  if (P.whole == P.N || P.whole >= n + 64 || m >= P.M) return;
+  uint16_t* to = reinterpret_cast<uint16_t*>(out) + m * ld;
+#pragma unroll 1
+  for (int c = P.whole; c < P.N; ++c) {
+    const uint32_t j = (uint32_t)(c - n);
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(my_row + ((j >> 3) ^ sw) * 16u + (j & 7u) * 2u) : "memory");
+    to[c] = v;
+  }
+}
+
 // The same accumulator leaving through shared memory: each warp owns a 32-row x 128-byte staging box (128-byte
 // swizzle: 16-byte piece j of row r sits at piece j ^ (r & 7), so the 32 row-owning lanes write without bank
 // conflicts), fills it from its registers and one lane hands it to the TMA unit, which writes whole lines and clips
@@ -378,9 +392,10 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
 #pragma unroll
         for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r, 8 * v);
       }
+      store_tail(P, my_row, sw, P.out, P.ldc, row0 + lane, n);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0 && row0 < P.M) {
+      if (lane == 0 && row0 < P.M && n < P.whole) {
         tma_store_2d(tmC, stage, n, (int)row0);
         bulk_commit();
       }
@@ -478,10 +493,11 @@ __device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtenso
       if (P.pre) {                                         // kept for the backward pass
 #pragma unroll
         for (int v = 0; v < 8; ++v) stage_bf16(pre_row, (uint32_t)v ^ sw, r[v >> 2], 8 * (v & 3));
+        store_tail(P, pre_row, sw, P.pre, P.ldpre, row0 + lane, n);
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          if (row0 < P.M) tma_store_2d(tmP, A.box[0], n, (int)row0);
+          if (row0 < P.M && n < P.whole) tma_store_2d(tmP, A.box[0], n, (int)row0);
           bulk_commit();
         }
       }
@@ -505,10 +521,11 @@ __device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtenso
         for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r[h], 8 * v);
       }
     }
+    store_tail(P, (GRAD && i == 0 ? A.box[0] : A.box[1]) + (uint32_t)lane * 128u, sw, P.out, P.ldc, row0 + lane, n);
     fence_async_smem();
     __syncwarp();
     if (lane == 0) {
-      if (row0 < P.M) tma_store_2d(tmC, GRAD && i == 0 ? A.box[0] : A.box[1], n, (int)row0);
+      if (row0 < P.M && n < P.whole) tma_store_2d(tmC, GRAD && i == 0 ? A.box[0] : A.box[1], n, (int)row0);
       bulk_commit();
     }
   }
@@ -1331,19 +1348,20 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   }
   // staged epilogue when the output (and the pre-activation) can be described to the TMA unit (MST_TC_TMA_OUT=0 keeps per-thread stores)
   CUtensorMap tmC = tmA, tmP = tmA;
-  P.tma_out = 0;
+  bool tma_out = false;
+  P.whole = (int)a.N & ~7;
   if (a.epilogue == MST_TC_OUT_BF16) {
-    P.tma_out = make_out_map_bf16(&tmC, a.out, a.M, a.N, a.ldc) && (!P.act || !P.pre || make_out_map_bf16(&tmP, P.pre, a.M, a.N, P.ldpre)) ? 1 : 0;
+    // pre-activations that are read may end anywhere
+    tma_out = P.whole > 0 && make_out_map_bf16(&tmC, a.out, a.M, P.whole, a.ldc) &&
+              (!P.act || !P.pre || make_out_map_bf16(&tmP, P.pre, a.M, P.act == MST_ACT_GELU ? P.whole : a.N, P.ldpre));
   } else if (a.epilogue == MST_TC_OUT_F32) {
-    P.tma_out = (sums > 1 ? make_out_map_f32(&tmC, P.partial, a.M, a.N, a.N, a.M * a.N, sums)
-                              : make_out_map_f32(&tmC, a.out, a.M, a.N, a.ldc, a.M * a.ldc, 1))
-                    ? 1
-                    : 0;
+    tma_out = a.N % 4 == 0 && (sums > 1 ? make_out_map_f32(&tmC, P.partial, a.M, a.N, a.N, a.M * a.N, sums)
+                                        : make_out_map_f32(&tmC, a.out, a.M, a.N, a.ldc, a.M * a.ldc, 1));
   }
   if (const char* e = mst_getenv(env, "MST_TC_TMA_OUT")) {
-    if (e[0] == '0') P.tma_out = 0;
+    if (e[0] == '0') tma_out = false;
   }
-  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !P.tma_out ? K_ROWS : P.redo.kind ? (P.act ? K_REDO_ACT : K_REDO) : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
+  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !tma_out ? K_ROWS : P.redo.kind ? (P.act ? K_REDO_ACT : K_REDO) : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
   if (pair) {
     const int64_t jobs = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits, max_pairs = mst_sm_count() / 2, rest = jobs % max_pairs;
     CUtensorMap tmBn = tmB;

@@ -4,6 +4,7 @@ import pytest
 
 import mst_inputs
 import oracle
+from oracle import activation
 
 pytestmark = pytest.mark.gpu
 
@@ -744,4 +745,45 @@ def test_pack_of_a_large_layer(O, I):
     assert L.nnz == nnz and int(rp[0]) == 0
     assert torch.equal(rp[1:].long(), M.sum(1, dtype=torch.int64).cumsum(0))
     assert torch.equal(ci.long(), at[:, 1]) and torch.equal(vv, W[at[:, 0], at[:, 1]])
+    L.close()
+
+
+@pytest.mark.parametrize("path,pairs", [("MST_PATH_AUTO", None), ("MST_PATH_AUTO", "1"), ("MST_PATH_AUTO", "0"), ("MST_PATH_CUDA_CORE", None),
+                                        ("MST_PATH_SPARSE_TC", None)])
+@pytest.mark.parametrize("O,I,T", [(33, 40, 77), (199, 64, 300), (64, 199, 300), (5, 130, 40), (33, 40, 12), (1025, 136, 700), (520, 1031, 270), (65, 7, 1)])
+def test_columns_beyond_the_row_are_the_callers(monkeypatch, path, pairs, O, I, T):
+    # rows that start on 16-byte boundaries and end inside one: what lies behind them stays as it is
+    if pairs is not None:
+        monkeypatch.setenv("MST_TC_PAIR", pairs)
+    p = _problem(O, I, T, "bf16", 0.2, 8200 + O + I + T)
+    L = make_layer(p)
+    L.set_path(getattr(mst, path))
+    pitch = lambda n: (n + 7) // 8 * 8
+    ldo, ldi = pitch(O), pitch(I)
+
+    def wide(C, ld, fill=None):
+        t = torch.full((T + 1, ld), float("nan"), dtype=torch.bfloat16, device=dev())
+        if fill is not None:
+            t[:T, :C] = fill
+        return t
+    X, dY = wide(I, ldi, to_dev(p, "X")), wide(O, ldo, to_dev(p, "dY"))
+    at = wide(I, ldi, to_dev(p, "X"))
+    Y, H, H_only, pre = (wide(O, ldo) for _ in range(4))
+    dX, dP = wide(I, ldi), wide(I, ldi)
+    mst.mst_spmm_fwd(L.handle, X, ldi, T, Y, ldo)
+    mst.mst_spmm_fwd_gelu(L.handle, X, ldi, T, pre, ldo, H, ldo)
+    mst.mst_spmm_fwd_gelu(L.handle, X, ldi, T, 0, ldo, H_only, ldo)
+    mst.mst_spmm_bwd_x(L.handle, dY, ldo, T, dX, ldi)
+    mst.mst_spmm_bwd_x_gelu(L.handle, dY, ldo, T, at, ldi, dP, ldi)
+    torch.cuda.synchronize()
+    assert mst.mst_device_error_flags() == 0
+    for t, C in ((Y, O), (H, O), (H_only, O), (pre, O), (dX, I), (dP, I)):
+        assert torch.isnan(t[:T, C:]).all() and torch.isnan(t[T]).all() and not torch.isnan(t[:T, :C]).any()
+    Wm = np.where(p.mask == 1, p.W, np.float32(0))
+    y, dx = oracle.fwd(p.X, Wm, p.mask), oracle.bwd_x(p.dY, Wm, p.mask)
+    assert rel_err(host(Y[:T, :O]), y) <= TOL["bf16"] and rel_err(host(pre[:T, :O]), y) <= TOL["bf16"]
+    assert rel_err(host(dX[:T, :I]), dx) <= TOL["bf16"]
+    assert torch.equal(H[:T, :O], H_only[:T, :O])
+    a, b = activation.gelu(y), dx * activation.gelu_grad(p.X.astype(np.float64))
+    assert rel_err(host(H[:T, :O]), a) <= TOL["bf16"] and rel_err(host(dP[:T, :I]), b) <= TOL["bf16"]
     L.close()
