@@ -73,9 +73,11 @@ enum { M_FORWARD, M_INPUT, M_GRADIENT };
 enum {
   K_BF16, K_F32, K_SAMPLED,
   K_ACT,    // bf16 with an activation
-  K_REDO, K_REDO_ACT,   // bf16 without and with one, where sums that are not finite are formed again (one kernel for both, a ring stage short: 770 -> 3072 at
-                        // 8192 tokens 38.3 -> 37.3 us, its input gradient 37.1 -> 36.3)
-  K_ROWS    // whatever the TMA unit cannot describe
+  // bf16 without and with one, where sums that are not finite are formed again or rows end inside a 16-byte piece.  (One kernel for both, a ring
+  // stage short: 770 -> 3072 at 8192 tokens 38.3 -> 37.3 us, its input gradient 37.1 -> 36.3.  The ends of rows seen to in the kernels above: 1 to 2 %
+  // of theirs.)
+  K_REDO, K_REDO_ACT,
+  K_ROWS, K_ROWS_ACT    // whatever the TMA unit cannot describe, without and with an activation
 };
 
 // PTX wrappers live in mst_tc_ptx.cuh; waits in this file report to g_tc_error
@@ -161,55 +163,41 @@ __device__ __forceinline__ void redo_tile(const Params& P, uint32_t tmem_base, i
   }
 }
 
-// Activation step of one 32-column chunk held in registers (row m, columns n..n+31) for rows that TMA does not take.  GELU: r <-
-// gelu(r), the pre-activation going to `pre` when the caller keeps one; GELU_GRAD: r <- r * gelu'(pre).
-__device__ __forceinline__ void act_chunk(const Params& P, uint32_t (&r)[32], uint16_t* pre, int n) {
-  const int left = P.N - n < 32 ? (int)(P.N - n) : 32;
-  if (P.act == MST_ACT_GELU) {
-#pragma unroll
-    for (int j = 0; j < 32; j += 2) {
-      float x0 = __uint_as_float(r[j]), x1 = __uint_as_float(r[j + 1]);
-      if (P.pre) {  // keep the pre-activation for the backward pass
-        const uint32_t w = pack_bf16(x0, x1);
-        if (j < left) pre[j] = (uint16_t)(w & 0xFFFFu);
-        if (j + 1 < left) pre[j + 1] = (uint16_t)(w >> 16);
-      }
-      gelu_pair(x0, x1);
-      r[j] = __float_as_uint(x0);
-      r[j + 1] = __float_as_uint(x1);
-    }
-  } else {  // multiply by the derivative at the stored pre-activation
-#pragma unroll
-    for (int j = 0; j < 32; j += 2) {
-      const float x0 = j < left ? __uint_as_float((uint32_t)pre[j] << 16) : 0.f, x1 = j + 1 < left ? __uint_as_float((uint32_t)pre[j + 1] << 16) : 0.f;
-      float v0, v1;
-      unpack2(mul2(pack2(r[j], r[j + 1]), gelu_grad_pair(x0, x1)), v0, v1);
-      r[j] = __float_as_uint(v0);
-      r[j + 1] = __float_as_uint(v1);
-    }
-  }
-}
-
 // One 128 x BN accumulator (tensor-memory lanes = rows) -> rows of any leading dimension and alignment, for outputs the TMA
 // unit cannot describe.  q = lane quarter this warp may read, m0/n0 = first row / column of this block's tile, c0 = first
 // 32-column chunk this warp takes (the warps of one lane quarter interleave their chunks).  A chunk goes through the warp's
 // staging box, so that a store instruction writes 32 neighbours of one row; stores by the row-owning lanes touch 32 lines
 // each (2051 x 1999 bf16 outputs: 4.1 M two-byte stores to as many sectors).
+// Activations (ACT) are taken behind the box too, so that the pre-activations travel as neighbours of one row.  By the row-owning lanes, two bytes to
+// a line, 768 -> 3072 at 8192 tokens with pre-activations of odd pitch took 256 us for GELU and 99 for its derivative; now 49 and 69.  The
+// derivative's are fetched a chunk ahead, a group of eight rows when the chunk before has used its own (eight rows ahead: 144 us).
+template <int ACT, bool BF16>
 __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, uint32_t tmem_base, int acc, int q, int c0, int lane,
                                               int64_t m0, int n0, int split, int cols) {
+  constexpr bool GRAD = ACT == MST_ACT_GELU_GRAD;
+  constexpr int STEP = EPI_WARPS / 4;
   const int64_t row0 = (int64_t)m0 + q * 32;
-  const int64_t m = row0 + lane;
-  const bool row_ok = m < P.M;
   const uint32_t my_row = stage + (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
   const int rows = P.M - row0 < 32 ? (int)(P.M - row0) : 32;
+  uint16_t* const pre0 = reinterpret_cast<uint16_t*>(P.pre) + row0 * P.ldpre + lane;
+  uint16_t x[GRAD ? 32 : 1];
+  auto fetch = [&](int c, int r8) {
+    const int n = n0 + c * 32;
+    const bool any = c < cols / 32 && n + lane < P.N;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[r8 + k] = any && r8 + k < rows ? pre0[n + (r8 + k) * P.ldpre] : (uint16_t)0;
+  };
+  if (GRAD) {
+#pragma unroll
+    for (int r8 = 0; r8 < 32; r8 += 8) fetch(c0, r8);
+  }
 #pragma unroll 1
-  for (int c = c0; c < cols / 32; c += EPI_WARPS / 4) {
+  for (int c = c0; c < cols / 32; c += STEP) {
     const int n = n0 + c * 32;
     if (n >= P.N) break;  // uniform
     uint32_t r[32];
     tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
-    if (P.act && row_ok) act_chunk(P, r, reinterpret_cast<uint16_t*>(P.pre) + m * P.ldpre + n, n);
     __syncwarp();  // the previous chunk has been read out of the box
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
@@ -220,30 +208,42 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
     }
     __syncwarp();
     const bool col_ok = n + lane < P.N;
-    const bool bf16 = P.epilogue == MST_TC_OUT_BF16;
-    float* f32 = P.partial ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
-    const int64_t ld = bf16 || !P.partial ? P.ldc : P.N;
     // A square inside the output is stored without a test per row (the branches and 64-bit addresses cost four times the stores).
     const bool inside = rows == 32 && n + 32 <= P.N;
+    float* f32 = P.partial ? P.partial + (int64_t)split * P.M * P.N : reinterpret_cast<float*>(P.out);
+    const int64_t ld = BF16 || !P.partial ? P.ldc : P.N;
     const int64_t at0 = row0 * ld + n + lane;
-#pragma unroll 1
-    for (int r8 = 0; r8 < rows; r8 += 8) {
+    auto group = [&](int r8) {
       float v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {   // eight rows are read back before the first is stored
         const uint32_t piece = (uint32_t)(lane >> 2) ^ (uint32_t)k;
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[k]) : "r"(stage + (uint32_t)(r8 + k) * 128u + piece * 16u + (uint32_t)(lane & 3) * 4u) : "memory");
       }
-      if (bf16) {
-        uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + at0 + r8 * ld;
+      auto put = [&](uint16_t* to, int64_t pitch) {
         if (inside) {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) out[k * ld] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
+          for (int k = 0; k < 8; ++k) to[k * pitch] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
         } else if (col_ok) {
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            if (r8 + k < rows) out[k * ld] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
+            if (r8 + k < rows) to[k * pitch] = (uint16_t)(pack_bf16(v[k], 0.f) & 0xFFFFu);
         }
+      };
+      if (GRAD) {
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+          const uint64_t d = gelu_grad_pair(__uint_as_float((uint32_t)x[r8 + k] << 16), __uint_as_float((uint32_t)x[r8 + k + 1] << 16));
+          unpack2(mul2(pack2(v[k], v[k + 1]), d), v[k], v[k + 1]);
+        }
+        fetch(c + STEP, r8);
+      } else if (ACT == MST_ACT_GELU) {
+        if (P.pre) put(pre0 + n + r8 * P.ldpre, P.ldpre);   // kept for the backward pass
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) gelu_pair(v[k], v[k + 1]);
+      }
+      if (BF16) {
+        put(reinterpret_cast<uint16_t*>(P.out) + at0 + r8 * ld, ld);
       } else {
         float* out = f32 + at0 + r8 * ld;
         if (inside) {
@@ -255,6 +255,13 @@ __device__ __forceinline__ void epilogue_tile(const Params& P, uint32_t stage, u
             if (r8 + k < rows) out[k * ld] = v[k];
         }
       }
+    };
+    if (GRAD) {
+#pragma unroll
+      for (int r8 = 0; r8 < 32; r8 += 8) group(r8);
+    } else {
+#pragma unroll 1
+      for (int r8 = 0; r8 < rows; r8 += 8) group(r8);
     }
   }
 }
@@ -392,10 +399,10 @@ __device__ __forceinline__ void epilogue_tile_tma(const Params& P, const CUtenso
 #pragma unroll
         for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r, 8 * v);
       }
-      store_tail(P, my_row, sw, P.out, P.ldc, row0 + lane, n);
+      if (KIND == K_REDO) store_tail(P, my_row, sw, P.out, P.ldc, row0 + lane, n);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0 && row0 < P.M && n < P.whole) {
+      if (lane == 0 && row0 < P.M && (KIND != K_REDO || n < P.whole)) {
         tma_store_2d(tmC, stage, n, (int)row0);
         bulk_commit();
       }
@@ -447,7 +454,7 @@ __device__ __forceinline__ void fetch_pre(const Params& P, const CUtensorMap* tm
   mbar_expect_tx(A.bar[i], OUT_BOX_BYTES);
   tma_load_2d(A.box[i], tmP, n0 + (c0 + i * (EPI_WARPS / 4)) * 64, m0 + q * 32, A.bar[i]);
 }
-template <bool GRAD>
+template <bool GRAD, bool TAIL>
 __device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtensorMap* tmC, const CUtensorMap* tmP, ActBoxes& A, uint32_t tmem_base, int acc,
                                                   int q, int c0, int lane, int64_t m0, int n0, int cols, volatile int* abort_flag) {
   const int64_t row0 = m0 + q * 32;
@@ -493,11 +500,11 @@ __device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtenso
       if (P.pre) {                                         // kept for the backward pass
 #pragma unroll
         for (int v = 0; v < 8; ++v) stage_bf16(pre_row, (uint32_t)v ^ sw, r[v >> 2], 8 * (v & 3));
-        store_tail(P, pre_row, sw, P.pre, P.ldpre, row0 + lane, n);
+        if (TAIL) store_tail(P, pre_row, sw, P.pre, P.ldpre, row0 + lane, n);
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          if (row0 < P.M && n < P.whole) tma_store_2d(tmP, A.box[0], n, (int)row0);
+          if (row0 < P.M && (!TAIL || n < P.whole)) tma_store_2d(tmP, A.box[0], n, (int)row0);
           bulk_commit();
         }
       }
@@ -521,11 +528,11 @@ __device__ __forceinline__ bool epilogue_tile_act(const Params& P, const CUtenso
         for (int v = 0; v < 4; ++v) stage_bf16(my_row, (uint32_t)(h * 4 + v) ^ sw, r[h], 8 * v);
       }
     }
-    store_tail(P, (GRAD && i == 0 ? A.box[0] : A.box[1]) + (uint32_t)lane * 128u, sw, P.out, P.ldc, row0 + lane, n);
+    if (TAIL) store_tail(P, (GRAD && i == 0 ? A.box[0] : A.box[1]) + (uint32_t)lane * 128u, sw, P.out, P.ldc, row0 + lane, n);
     fence_async_smem();
     __syncwarp();
     if (lane == 0) {
-      if (row0 < P.M && n < P.whole) tma_store_2d(tmC, GRAD && i == 0 ? A.box[0] : A.box[1], n, (int)row0);
+      if (row0 < P.M && (!TAIL || n < P.whole)) tma_store_2d(tmC, GRAD && i == 0 ? A.box[0] : A.box[1], n, (int)row0);
       bulk_commit();
     }
   }
@@ -688,30 +695,33 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (REDO) {   // the chunks this warp stores: pairs of them
+      if (REDO && P.redo.kind) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, BN);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, BN);
       }
       if (ACT) {
-        if (!(P.major == M_INPUT ? epilogue_tile_act<true>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)
-                                 : epilogue_tile_act<false>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)))
+        if (!(P.major == M_INPUT ? epilogue_tile_act<true, REDO>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)
+                                 : epilogue_tile_act<false, REDO>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, BN, abort_flag)))
           break;
         if (fetch && lane == 0 && w + gridDim.x < works) {
           const int tn = (int)((w + gridDim.x) % tiles);
           fetch_next(P, &tmP, A, q, c0, n0, BN, (tn / P.n_tiles) * BM, (tn % P.n_tiles) * BN, BN);
         }
-      } else if (KIND != K_ROWS) {
+      } else if (KIND != K_ROWS && KIND != K_ROWS_ACT) {
         epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
       } else {
         if (P.redo.kind) redo_tile(P, tmem_base, acc, q, c0, EPI_WARPS / 4, lane, m0, n0, BN);
-        epilogue_tile(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+        if (KIND == K_ROWS && P.major == M_GRADIENT) epilogue_tile<MST_ACT_NONE, false>(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+        else if (KIND == K_ROWS) epilogue_tile<MST_ACT_NONE, true>(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+        else if (P.major == M_INPUT) epilogue_tile<MST_ACT_GELU_GRAD, true>(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
+        else epilogue_tile<MST_ACT_GELU, true>(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, BN);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-    if (KIND != K_SAMPLED && KIND != K_ROWS && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
+    if (KIND != K_SAMPLED && KIND != K_ROWS && KIND != K_ROWS_ACT && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
   }
 
   // ------------------------------------------------------------------ teardown
@@ -777,7 +787,7 @@ struct PairJobs {
       const uint32_t row = tile / (uint32_t)P.n_tiles;
       m0 = (int)row * (2 * BM);
       n0 = (int)(tile - row * (uint32_t)P.n_tiles) * BN;
-      if (KIND == K_BF16 || KIND == K_ACT || KIND == K_REDO || KIND == K_REDO_ACT || (KIND == K_ROWS && P.epilogue == MST_TC_OUT_BF16)) {
+      if (KIND == K_BF16 || KIND == K_ACT || KIND == K_REDO || KIND == K_REDO_ACT || KIND == K_ROWS_ACT || (KIND == K_ROWS && P.epilogue == MST_TC_OUT_BF16)) {
         n0 += (int)part * (BN / 2);
         cols = cut || P.N - n0 <= BN / 2 ? BN / 2 : BN;
         if (n0 >= P.N) continue;   // that half lies outside the output
@@ -993,28 +1003,28 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       first = false;
       if (!mbar_wait(tfull0 + 8 * acc, acc_ph, abort_flag)) break;
       tc_fence_after();
-      if (REDO) {   // the chunks this warp stores: pairs of them
+      if (REDO && P.redo.kind) {   // the chunks this warp stores: pairs of them
         redo_tile(P, tmem_base, acc, q, 2 * c0, EPI_WARPS / 2, lane, m0, n0, J.cols);
         redo_tile(P, tmem_base, acc, q, 2 * c0 + 1, EPI_WARPS / 2, lane, m0, n0, J.cols);
       }
       if (ACT) {
-        if (!epilogue_tile_act<MAJOR == M_INPUT>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, J.cols, abort_flag)) break;
+        if (!epilogue_tile_act<MAJOR == M_INPUT, REDO>(P, &tmC, &tmP, A, tmem_base, acc, q, c0, lane, m0, n0, J.cols, abort_flag)) break;
         if (fetch) {
           PairJobs<KIND> N = J;
           if (N.next(P) && lane == 0) fetch_next(P, &tmP, A, q, c0, n0, J.cols, N.m0 + (int)rank * BM, N.n0, N.cols);
         }
-      } else if (KIND != K_ROWS) {
+      } else if (KIND != K_ROWS && KIND != K_ROWS_ACT) {
         epilogue_tile_tma<KIND>(P, &tmC, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
       } else {
         if (P.redo.kind) redo_tile(P, tmem_base, acc, q, c0, EPI_WARPS / 4, lane, m0, n0, J.cols);
-        epilogue_tile(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
+        epilogue_tile<KIND == K_ROWS ? MST_ACT_NONE : MAJOR == M_INPUT ? MST_ACT_GELU_GRAD : MST_ACT_GELU, MAJOR != M_GRADIENT>(P, box, tmem_base, acc, q, c0, lane, m0, n0, split, J.cols);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(in_even_block(tempty0 + 8 * acc));
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-    if (KIND != K_SAMPLED && KIND != K_ROWS && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
+    if (KIND != K_SAMPLED && KIND != K_ROWS && KIND != K_ROWS_ACT && lane == 0) bulk_wait_read();  // this warp's stores have left shared memory; the end of the grid waits for their arrival
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1361,7 +1371,8 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
   if (const char* e = mst_getenv(env, "MST_TC_TMA_OUT")) {
     if (e[0] == '0') tma_out = false;
   }
-  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !tma_out ? K_ROWS : P.redo.kind ? (P.act ? K_REDO_ACT : K_REDO) : a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.act ? K_ACT : K_BF16;
+  const int kind = a.epilogue == MST_TC_OUT_SAMPLED ? K_SAMPLED : !tma_out ? (P.act ? K_ROWS_ACT : K_ROWS) : 
+                   a.epilogue == MST_TC_OUT_F32 ? K_F32 : P.redo.kind || P.whole != a.N ? (P.act ? K_REDO_ACT : K_REDO) : P.act ? K_ACT : K_BF16;
   if (pair) {
     const int64_t jobs = (int64_t)((P.m_tiles + 1) / 2) * P.n_tiles * P.splits, max_pairs = mst_sm_count() / 2, rest = jobs % max_pairs;
     CUtensorMap tmBn = tmB;
@@ -1385,11 +1396,13 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       MST_LAUNCH_KIND(K_REDO, M_FORWARD);
       MST_LAUNCH_KIND(K_REDO_ACT, M_FORWARD);
       MST_LAUNCH_KIND(K_ROWS, M_FORWARD);
+      MST_LAUNCH_KIND(K_ROWS_ACT, M_FORWARD);
       MST_LAUNCH_KIND(K_BF16, M_INPUT);
       MST_LAUNCH_KIND(K_ACT, M_INPUT);
       MST_LAUNCH_KIND(K_REDO, M_INPUT);
       MST_LAUNCH_KIND(K_REDO_ACT, M_INPUT);
       MST_LAUNCH_KIND(K_ROWS, M_INPUT);
+      MST_LAUNCH_KIND(K_ROWS_ACT, M_INPUT);
       MST_LAUNCH_KIND(K_F32, M_GRADIENT);
       MST_LAUNCH_KIND(K_SAMPLED, M_GRADIENT);
       MST_LAUNCH_KIND(K_ROWS, M_GRADIENT);
@@ -1412,6 +1425,7 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
       MST_LAUNCH_KIND(K_REDO);
       MST_LAUNCH_KIND(K_REDO_ACT);
       MST_LAUNCH_KIND(K_ROWS);
+      MST_LAUNCH_KIND(K_ROWS_ACT);
     }
 #undef MST_LAUNCH_KIND
   }

@@ -166,3 +166,39 @@ def test_activation_boxes_at_tile_edges(monkeypatch, T, d, hid):
     assert torch.isposinf(H[0, row]) and torch.isnan(H[1, row]) and bool((H[2:T] == 0).all())
     one.close(); L1.close(); L2.close()
     assert mst.mst_device_error_flags() == 0
+
+
+@pytest.mark.parametrize("pairs", ["1", "0"])
+@pytest.mark.parametrize("T,O,I,pad,shift", [(300, 200, 136, 1, 0), (257, 328, 64, 2, 1), (513, 72, 72, 0, 4), (77, 33, 40, 0, 0)])
+def test_pre_activation_of_any_pitch(monkeypatch, pairs, T, O, I, pad, shift):
+    """Pre-activations that TMA does not take: the very values of the call whose rows it does, and the derivative in place."""
+    monkeypatch.setenv("MST_TC_PAIR", pairs)
+    g = torch.Generator(device="cuda").manual_seed(O + T)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()
+    X, dY, W1, W2 = n(T, I), n(T, I), n(O, I), n(I, O)
+    M1, M2 = ((torch.rand(s, generator=g, device="cuda") < 0.4).to(torch.uint8) for s in ((O, I), (I, O)))
+    L1, L2 = mst.Layer(0, O, I, mst.MST_BF16), mst.Layer(1, I, O, mst.MST_BF16)
+    L1.pack(W1, M1)
+    L2.pack(W2, M2)
+    even = (O + 7) // 8 * 8
+    outs = []
+    for ld, off in ((even, 0), (O + pad, shift)):
+        whole = torch.full((T * ld + off + 8,), float("nan"), dtype=torch.bfloat16, device="cuda")
+        pre = whole[off:off + T * ld].view(T, ld)
+        H, dP = (torch.full((T, even), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        mst.mst_spmm_fwd_gelu(L1.handle, X, I, T, pre, ld, H, even)
+        kept = pre[:, :O].clone()
+        mst.mst_spmm_bwd_x_gelu(L2.handle, dY, I, T, pre, ld, dP, even)
+        assert torch.equal(pre[:, :O], kept) and bool(torch.isnan(pre[:, O:]).all()) and bool(torch.isnan(whole[off + T * ld:]).all())
+        mst.mst_spmm_bwd_x_gelu(L2.handle, dY, I, T, pre, ld, pre, ld)
+        torch.cuda.synchronize()
+        outs.append((H[:, :O].clone(), kept, dP[:, :O].clone(), pre[:, :O].clone()))
+        assert bool(torch.isnan(H[:, O:]).all()) and bool(torch.isnan(dP[:, O:]).all())
+    assert mst.mst_device_error_flags() == 0
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+    assert torch.equal(outs[1][2], outs[1][3])
+    x = X.double() @ (W1.double() * M1).T
+    assert float((outs[1][0].double() - x * 0.5 * (1 + torch.erf(x / 2 ** 0.5))).norm()) <= 1e-2 * float(x.norm())
+    L1.close()
+    L2.close()
