@@ -599,11 +599,12 @@ mst_status_t mst_launch_spmm(const mst_layer* L, bool transpose, const void* in,
     a.splits = 1;
     a.act = act; a.pre = pre; a.ldpre = ldpre;
     // A few tokens: the latency kernel.  Columns beyond the row must be zero in the activations too.
-    if (!transpose && (cols % 8 == 0 || a.A != in) &&
-        (T <= MST_SMALL_FWD_TOKENS ||
-         (T <= MST_SMALL_FWD_MOST && mst_small_fwd_clocks(T, rows, cols) < mst_tc_small_clocks(a) && !mst_getenv(mst_env_any(), "MST_TC_PAIR"))))
+    const bool latency = !transpose && (cols % 8 == 0 || a.A != in);
+    mst_tc_choice choice;
+    if (!latency || T > MST_SMALL_FWD_TOKENS) choice = mst_tc_choose(a);
+    if (latency && (T <= MST_SMALL_FWD_TOKENS || (T <= MST_SMALL_FWD_MOST && mst_small_fwd_clocks(T, rows, cols) < choice.clocks)))
       return mst_small_fwd(a.A, a.lda, T, image, ldimage, rows, cols, out, ldout, act, pre, ldpre, a.redo, s);
-    return mst_tc_gemm(a, s);
+    return mst_tc_gemm(a, choice, s);
   }
   // CUDA cores: the product lands in the pre-activation buffer when the caller keeps one, else in the output
   void* prod = (act == MST_ACT_GELU && pre) ? pre : out;

@@ -1262,17 +1262,15 @@ bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb) 
          ((reinterpret_cast<uintptr_t>(B) & 15u) == 0) && mst_encode_tiled() != nullptr;
 }
 
-mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
-  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
-  if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
-  const bool env = mst_env_any();
+mst_tc_choice mst_tc_choose(const mst_tc_gemm_args& a) {
+  mst_tc_choice c = {false, mst_env_any(), 0.0, {0, 0, 0.0}};
   // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
   // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
   // Fitted to layers drawn over 96..4096 features (at most 4096 x 2048) and 17..4096 tokens, both kernels timed, once for sizes of whole
   // 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in partial words and squares.  Gradients:
   // 130 layers, d = 0.02..0.5, the choices 1.4 % (even) and 0.2 % (odd) above the better kernel of each call.  Products: 190 layers,
   // figures of the calls whose operands need no copies (3 to 8 % off the measured times, 7 to 33 before).
-  if (!mst_getenv(env, "MST_TC_PAIR") && !mst_getenv(env, "MST_TC_SPLITS") && a.splits <= 1) {
+  if (!mst_getenv(c.env, "MST_TC_PAIR") && !mst_getenv(c.env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
       double here;
@@ -1298,9 +1296,19 @@ mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) {
           here = (even ? 10300.0 : 17100.0) + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0);
         }
       }
-      if (mst_tc_small_clocks(a) < here) return mst_tc_small(a, s);
+      c.plan = mst_tc_small_plan(a);
+      c.small = c.plan.clocks < here;
+      c.clocks = c.small ? c.plan.clocks : here;
     }
   }
+  return c;
+}
+
+mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, const mst_tc_choice& choice, cudaStream_t s) {
+  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return MST_ERR_INVALID_ARG;
+  if (!mst_tc_gemm_usable(a.A, a.lda, a.B, a.ldb)) return MST_ERR_SHAPE;
+  if (choice.small) return mst_tc_small(a, choice.plan, s);
+  const bool env = choice.env;
   CUtensorMap tmA, tmB;
   // Block pairs (256-row tiles) pay off once there are at least two row tiles; MST_TC_PAIR=0/1 overrides.
   bool pair = a.M > BM;

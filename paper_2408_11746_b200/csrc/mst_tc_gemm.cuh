@@ -72,9 +72,11 @@ struct mst_tc_gemm_args {
 // C = A * B with fp32 accuracy from operands given as three bf16 pieces each (mst_prepare.cu; lda / ldb are the pieces'
 // leading dimensions, M / N / K the matrix sizes).  Epilogues F32 (rows) and SAMPLED.
 mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s);
-// The same kernel for bf16 operands and outputs of few tiles, all epilogues, and its estimated time in SM clocks
-mst_status_t mst_tc_small(const mst_tc_gemm_args& a, cudaStream_t s);
-double mst_tc_small_clocks(const mst_tc_gemm_args& a);
+// The same kernel for bf16 operands and outputs of few tiles, all epilogues: tile width and K ranges with their estimated time in SM clocks,
+// and the call with them
+struct mst_small_plan { int bn, splits; double clocks; };
+mst_small_plan mst_tc_small_plan(const mst_tc_gemm_args& a);
+mst_status_t mst_tc_small(const mst_tc_gemm_args& a, const mst_small_plan& plan, cudaStream_t s);
 // forward product of a few tokens (mst_small_fwd.cu): always up to MST_SMALL_FWD_TOKENS, up to MST_SMALL_FWD_MOST where its estimated time,
 // in SM clocks as above, is shorter than the small tiles'
 constexpr int64_t MST_SMALL_FWD_TOKENS = 16, MST_SMALL_FWD_MOST = 1024;
@@ -89,7 +91,11 @@ mst_status_t mst_tc_gradient(mst_tc_gemm_args a, mst_dtype_t dtype, const void* 
 
 // Returns MST_ERR_SHAPE when the operands cannot be described to the TMA unit (leading dimension or base address
 // not 16-byte aligned); callers pass aligned copies of such rows (mst_prepare).
-mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s);
+// The choice of its kernel is made once a call; `clocks` is the chosen one's estimate where one was made, else 0.
+struct mst_tc_choice { bool small, env; double clocks; mst_small_plan plan; };
+mst_tc_choice mst_tc_choose(const mst_tc_gemm_args& a);
+mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, const mst_tc_choice& choice, cudaStream_t s);
+inline mst_status_t mst_tc_gemm(const mst_tc_gemm_args& a, cudaStream_t s) { return mst_tc_gemm(a, mst_tc_choose(a), s); }
 bool mst_tc_gemm_usable(const void* A, int64_t lda, const void* B, int64_t ldb);
 
 // cuTensorMapEncodeTiled of the loaded driver (nullptr when it has none) and the SM count of the current device

@@ -423,36 +423,46 @@ mst_status_t launch_pieces(int epilogue, int major, const CUtensorMap& tmA, cons
   return launch_split<BN, 3, S_F32, M_GRADIENT>(tmA, tmB, P, s);
 }
 
-// Blocks that run at once, one to an SM, in clusters of `size`: the groups of SMs that a cluster must fit into are no multiples of it (148
-// SMs hold 148, 148, 132 and 120 blocks in clusters of 1, 2, 4 and 8).  Asked once per device.
-int cluster_slots(int size) {
+// Blocks that run at once, one to an SM, in clusters of 1 .. 8: the groups of SMs that a cluster must fit into are no multiples of it (148
+// SMs hold 148, 148, 132 and 120 blocks in clusters of 1, 2, 4 and 8).  Asked once per device, and for the device once a plan: asked for every width and
+// number of ranges the plans of a forward call cost it 0.5 us.
+struct Slots { int in[9]; };
+Slots cluster_slots() {
   static std::atomic<int> known[64][9];
-  const int sms = mst_sm_count();
+  Slots found;
   int dev = 0;
-  if (size <= 1 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sms;
-  int n = known[dev][size].load(std::memory_order_relaxed);
-  if (n == 0) {
-    typedef SplitCfg<128, 3> C;   // one block to an SM
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(size * sms));
-    cfg.blockDim = dim3(S_THREADS);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)size;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_F32, M_GRADIENT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_F32, M_GRADIENT>, &cfg) != cudaSuccess || clusters <= 0) {
-      cudaGetLastError();   // reported by the launch, if it matters there
-      return sms;
+  const bool here = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  int sms = here ? known[dev][1].load(std::memory_order_relaxed) : 0;
+  if (sms == 0) sms = mst_sm_count();
+  for (int& n : found.in) n = sms;
+  if (!here) return found;
+  known[dev][1].store(sms, std::memory_order_relaxed);
+  for (int size = 2; size <= 8; size *= 2) {
+    int n = known[dev][size].load(std::memory_order_relaxed);
+    if (n == 0) {
+      typedef SplitCfg<128, 3> C;   // one block to an SM
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(size * sms));
+      cfg.blockDim = dim3(S_THREADS);
+      cfg.dynamicSmemBytes = C::SMEM;
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = (unsigned)size;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int clusters = 0;
+      if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_F32, M_GRADIENT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_F32, M_GRADIENT>, &cfg) != cudaSuccess || clusters <= 0) {
+        cudaGetLastError();   // reported by the launch, if it matters there
+        continue;
+      }
+      n = clusters * size < sms ? clusters * size : sms;
+      known[dev][size].store(n, std::memory_order_relaxed);
     }
-    n = clusters * size < sms ? clusters * size : sms;
-    known[dev][size].store(n, std::memory_order_relaxed);
+    found.in[size] = n;
   }
-  return n;
+  return found;
 }
 
 // Tile width and number of K ranges from a time model in SM clocks.
@@ -465,19 +475,18 @@ int cluster_slots(int size) {
 // an SM, ranges over eight blocks were taken where two or four are faster: fp32 calls 4.5 % above the best choice of each, now 0.6;
 // the further ones take 0.965 of that time, bf16 products of few tiles 0.96 (1024 x 1024 at 162 tokens, fp32: 21.9 -> 13.7 us; bf16 input
 // gradient 4352 -> 1088 at 710 tokens 21.8 -> 16.8).
-double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
+mst_small_plan plan_split(const mst_tc_gemm_args& a, int pieces) {
   struct Figures { double launch, wave, k_shared, shared, cluster; };
   static const Figures plain = {7160.0, 0.0, 483.0, 1490.0, 5940.0}, gelu = {10700.0, 1550.0, 515.0, 1640.0, 2440.0},
                        grad = {13000.0, 2500.0, 512.0, 1980.0, 1700.0};
-  const int sms = mst_sm_count(), kblocks = (int)((a.K + SBK - 1) / SBK);
+  const Slots slots = cluster_slots();
+  const int sms = slots.in[1], kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
-  double best = 1e30;
-  *bn = pieces == 3 ? 128 : 64;
-  *splits = 1;
+  mst_small_plan best = {64, 1, 1e30};
   for (int w = 64; w <= (pieces == 3 ? 128 : 64); w += 64) {
     const int64_t tiles = m_tiles * ((a.N + w - 1) / w);
     for (int sp = 1; sp <= 8 && sp <= kblocks; sp *= 2) {   // cluster sizes
-      const int kb = (kblocks + sp - 1) / sp, fit = cluster_slots(sp);
+      const int kb = (kblocks + sp - 1) / sp, fit = slots.in[sp];
       double t;
       if (pieces == 3) {
         const int64_t waves = (tiles * sp + fit - 1) / fit;
@@ -489,10 +498,10 @@ double plan_split(const mst_tc_gemm_args& a, int pieces, int* bn, int* splits) {
         t = F.launch + F.wave * (double)waves + (double)(waves - 1) * (11500.0 + pair) + (tiles * sp > fit ? pair + F.shared : kb * 471.0) +
             (sp > 1 ? F.cluster : 0.0);
       } else {
-        const int64_t slots = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + slots - 1) / slots;
+        const int64_t most = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + most - 1) / most;
         t = 9000.0 + (double)waves * kb * 555.0 + (double)(waves - 1) * 10000.0 + (sp > 1 ? 5000.0 : 0.0);
       }
-      if (t < best * 0.97) { best = t; *bn = w; *splits = sp; }
+      if (t < best.clocks * 0.97) best = {w, sp, t};
     }
   }
   return best;
@@ -544,21 +553,13 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
 }  // namespace
 
 mst_status_t mst_tc_split(const mst_tc_gemm_args& a, cudaStream_t s) {
-  int bn, splits;
-  plan_split(a, 3, &bn, &splits);
-  return run_split(a, 3, bn, splits, s);
+  const mst_small_plan plan = plan_split(a, 3);
+  return run_split(a, 3, plan.bn, plan.splits, s);
 }
 
-double mst_tc_small_clocks(const mst_tc_gemm_args& a) {
-  int bn, splits;
-  return plan_split(a, 1, &bn, &splits);
-}
+mst_small_plan mst_tc_small_plan(const mst_tc_gemm_args& a) { return plan_split(a, 1); }
 
-mst_status_t mst_tc_small(const mst_tc_gemm_args& a, cudaStream_t s) {
-  int bn, splits;
-  plan_split(a, 1, &bn, &splits);
-  return run_split(a, 1, bn, splits, s);
-}
+mst_status_t mst_tc_small(const mst_tc_gemm_args& a, const mst_small_plan& plan, cudaStream_t s) { return run_split(a, 1, plan.bn, plan.splits, s); }
 
 mst_status_t mst_split_error_flags(int32_t* flags) {
   int v = 0;
