@@ -1266,10 +1266,14 @@ mst_tc_choice mst_tc_choose(const mst_tc_gemm_args& a) {
   mst_tc_choice c = {false, mst_env_any(), 0.0, {0, 0, 0.0}};
   // Few tiles: compare one wave of this kernel with the small-tile kernel's estimate, in SM clocks as there: a launch, the k-blocks of
   // a pair's tile, an epilogue that nothing overlaps in a single wave, and a second launch that adds the ranges and moves their sums.
-  // Fitted to layers drawn over 96..4096 features (at most 4096 x 2048) and 17..4096 tokens, both kernels timed, once for sizes of whole
-  // 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in partial words and squares.  Gradients:
-  // 130 layers, d = 0.02..0.5, the choices 1.4 % (even) and 0.2 % (odd) above the better kernel of each call.  Products: 190 layers,
-  // figures of the calls whose operands need no copies (3 to 8 % off the measured times, 7 to 33 before).
+  // Fitted to layers drawn over 96..4096 features (at most 4096 x 2048), or a block's of width 320..1280, and 17..4096 tokens, both kernels timed,
+  // once for sizes of whole 16-byte pieces and once for odd ones, whose rows leave one by one and whose entries end in partial words and
+  // squares.  Products: 190 layers, figures of the calls whose operands need no copies (3 to 8 % off the measured times, 7 to 33 before); activations
+  // of odd rows, which travel 32 neighbours at a time: 169 and 168 calls, 1.1 and 1.9 % above the best of each (2.3 and 2.1 with the figures from before
+  // they did); the derivative in one token tile 3.5 % above it (5.8 with 12900 + 603 a k-block).  Gradients: 511 layers, d = 0.02..0.5, with everything a call launches: where the entries do not leave with the contraction
+  // or its sums, a sweep over the finished matrix follows.  Above the best kernel and number of ranges of each call, even / odd: entries 0.6 / 1.4 %, dense
+  // 0.4 / 1.1, dense with entries 0.7 / 1.2; 1.1 / 1.4, 2.7 / 1.5 and 3.2 / 1.9 with the sweep left out and 148 blocks in clusters of any size
+  // (2304 x 768, 1817 tokens, dense with entries: 18.7 us here, 14.3 in small tiles).
   if (!mst_getenv(c.env, "MST_TC_PAIR") && !mst_getenv(c.env, "MST_TC_SPLITS") && a.splits <= 1) {
     const int64_t tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), kb = (a.K + BK - 1) / BK, pairs = mst_sm_count() / 2;
     if (tiles <= pairs) {
@@ -1278,22 +1282,27 @@ mst_tc_choice mst_tc_choose(const mst_tc_gemm_args& a) {
         const bool even = a.ldc % 8 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0 &&
                           (!a.act || !a.pre || (a.ldpre % 8 == 0 && (reinterpret_cast<uintptr_t>(a.pre) & 15u) == 0));
         const double k = (double)kb;
-        if (a.M <= BM) here = a.act ? (even ? 12900.0 : 28000.0) + k * 603.0 : 8350.0 + k * 606.0;   // one token tile: single blocks
-        else if (!a.act) here = even ? 8350.0 + k * 460.0 : 10400.0 + k * 552.0;
-        else if (a.act == MST_ACT_GELU_GRAD) here = even ? 10800.0 + k * 462.0 : 19000.0 + k * 505.0;
-        else here = even ? 10750.0 + k * 478.0 : 13600.0 + k * 560.0;
-        if (a.act == MST_ACT_GELU && !even) here += 0.024 * (double)a.M * (double)a.N;   // pre-activations value by value: 1390 x 2346, 56 us
+        const bool grad = a.act == MST_ACT_GELU_GRAD;
+        if (!a.act) here = a.M <= BM ? 8350.0 + k * 606.0 : even ? 8350.0 + k * 460.0 : 10400.0 + k * 552.0;   // one token tile: single blocks
+        else if (a.M <= BM) here = even ? (grad ? 16000.0 + k * 500.0 : 12900.0 + k * 603.0) : grad ? 26500.0 + k * 570.0 : 20000.0 + k * 579.0;
+        else if (even) here = grad ? 10800.0 + k * 462.0 : 10750.0 + k * 478.0;
+        else here = (grad ? 17000.0 + k * 450.0 : 13600.0 + k * 560.0) + (grad ? 0.0030 : 0.0025) * (double)a.M * (double)a.N;
       } else {
         const bool entries = a.epilogue == MST_TC_OUT_SAMPLED, even = a.M % 8 == 0 && a.N % 8 == 0;
         const double out_bytes = entries ? 4.0 * (double)a.nnz : 4.0 * (double)a.M * (double)a.N;
         int cut;
         const int64_t sp = mst_tc_pick_splits(tiles, pairs, kb, out_bytes, &cut), per = (kb + sp - 1) / sp;
+        // the entries come with the sums of several ranges, or from the finished matrix
+        const bool sweep = a.also_sampled && !(a.M > BM && sp > 1 && a.N % 4 == 0);
         if (entries) {
           const bool few = (double)a.nnz * 1024.0 < SAMPLED_STAGE_MIN * (double)a.M * (double)a.N;
-          here = even ? (few ? 10800.0 : 13300.0) + (double)per * 400.0 : (few ? 12000.0 : 14000.0) + (double)per * 574.0;
-          if (sp > 1) here += (even ? 2800.0 : 3500.0) + (double)sp * out_bytes * 7.4e-4;   // written and read, 5 TB/s at 1.85 GHz
+          here = even ? (few ? 10500.0 : 12900.0) + (double)per * 588.0 : (few ? 12000.0 : 14000.0) + (double)per * 574.0;
+          if (sp > 1) here += even ? 3330.0 + (double)sp * out_bytes * 1.17e-3 : 3500.0 + (double)sp * out_bytes * 7.4e-4;   // written and read
+        } else if (even) {
+          here = a.also_sampled ? 13900.0 + (double)per * 548.0 + (sweep ? 4780.0 : 0.0) : 11500.0 + (double)per * 568.0;
+          if (sp > 1) here += (a.also_sampled ? -150.0 : 2020.0) + (double)sp * out_bytes * (a.also_sampled ? 5.1e-4 : 4.0e-4);
         } else {
-          here = (even ? 10300.0 : 17100.0) + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0);
+          here = 17100.0 + (double)per * 510.0 + (sp > 1 ? 5700.0 : 0.0) + (sweep ? 5000.0 : 0.0);
         }
       }
       c.plan = mst_tc_small_plan(a);

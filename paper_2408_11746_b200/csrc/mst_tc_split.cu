@@ -474,14 +474,16 @@ Slots cluster_slots() {
 // (fp32) and 17..4096 tokens; 138 and 189 further ones for the check.  With 148 blocks assumed at any cluster size and one of a cluster to
 // an SM, ranges over eight blocks were taken where two or four are faster: fp32 calls 4.5 % above the best choice of each, now 0.6;
 // the further ones take 0.965 of that time, bf16 products of few tiles 0.96 (1024 x 1024 at 162 tokens, fp32: 21.9 -> 13.7 us; bf16 input
-// gradient 4352 -> 1088 at 710 tokens 21.8 -> 16.8).
+// gradient 4352 -> 1088 at 710 tokens 21.8 -> 16.8).  Gradients of one piece: see mst_tc_choose.
 mst_small_plan plan_split(const mst_tc_gemm_args& a, int pieces) {
   struct Figures { double launch, wave, k_shared, shared, cluster; };
   static const Figures plain = {7160.0, 0.0, 483.0, 1490.0, 5940.0}, gelu = {10700.0, 1550.0, 515.0, 1640.0, 2440.0},
-                       grad = {13000.0, 2500.0, 512.0, 1980.0, 1700.0};
+                       grad = {13000.0, 2500.0, 512.0, 1980.0, 1700.0},
+                       sampled = {9070.0, 0.0, 496.0, 1620.0, 3690.0}, f32 = {9290.0, 0.0, 450.0, 850.0, 3510.0}, both = {9670.0, 0.0, 481.0, 2680.0, 3460.0};
   const Slots slots = cluster_slots();
   const int sms = slots.in[1], kblocks = (int)((a.K + SBK - 1) / SBK);
   const int64_t m_tiles = (a.M + SBM - 1) / SBM;
+  const bool gradient = a.epilogue != MST_TC_OUT_BF16, even = a.M % 8 == 0 && a.N % 8 == 0;
   mst_small_plan best = {64, 1, 1e30};
   for (int w = 64; w <= (pieces == 3 ? 128 : 64); w += 64) {
     const int64_t tiles = m_tiles * ((a.N + w - 1) / w);
@@ -491,14 +493,15 @@ mst_small_plan plan_split(const mst_tc_gemm_args& a, int pieces) {
       if (pieces == 3) {
         const int64_t waves = (tiles * sp + fit - 1) / fit;
         t = (double)waves * (kb * (w == 64 ? 960.0 : 1620.0) + 10000.0) + (sp > 1 ? 1500.0 : 0.0);
-      } else if (a.epilogue == MST_TC_OUT_BF16) {
-        const Figures& F = a.act == MST_ACT_GELU_GRAD ? grad : a.act ? gelu : plain;
+      } else if (!gradient || even) {
+        const Figures& F = a.epilogue == MST_TC_OUT_SAMPLED ? sampled : gradient ? (a.also_sampled ? both : f32) : a.act == MST_ACT_GELU_GRAD ? grad : a.act ? gelu : plain;
         const int64_t waves = (tiles * sp + 2 * fit - 1) / (2 * fit);
-        const double pair = kb * F.k_shared;
-        t = F.launch + F.wave * (double)waves + (double)(waves - 1) * (11500.0 + pair) + (tiles * sp > fit ? pair + F.shared : kb * 471.0) +
-            (sp > 1 ? F.cluster : 0.0);
+        const double pair = kb * F.k_shared, alone = kb * (!gradient ? 471.0 : a.epilogue == MST_TC_OUT_SAMPLED ? 432.0 : a.also_sampled ? 478.0 : 389.0);
+        t = F.launch + F.wave * (double)waves + (double)(waves - 1) * (11500.0 + pair) + (tiles * sp > fit ? pair + F.shared : alone) + (sp > 1 ? F.cluster : 0.0);
       } else {
-        const int64_t most = sp > 1 ? sms : 2 * sms, waves = (tiles * sp + most - 1) / most;
+        // gradients of odd sizes: copies ahead, partial squares.  Entries are nearer to the best with one block of a cluster to an SM (1.4 % above it
+        // against 1.7), dense ones with two (1.1 against 1.5).
+        const int64_t most = a.epilogue != MST_TC_OUT_SAMPLED || sp == 1 ? 2 * fit : sms, waves = (tiles * sp + most - 1) / most;
         t = 9000.0 + (double)waves * kb * 555.0 + (double)(waves - 1) * 10000.0 + (sp > 1 ? 5000.0 : 0.0);
       }
       if (t < best.clocks * 0.97) best = {w, sp, t};
