@@ -202,3 +202,38 @@ def test_pre_activation_of_any_pitch(monkeypatch, pairs, T, O, I, pad, shift):
     assert float((outs[1][0].double() - x * 0.5 * (1 + torch.erf(x / 2 ** 0.5))).norm()) <= 1e-2 * float(x.norm())
     L1.close()
     L2.close()
+
+
+@pytest.mark.parametrize("pairs", ["1", "0"])
+@pytest.mark.parametrize("T,hid,pitch", [(5000, 1288, 1288), (4993, 1283, 1288), (5000, 1283, 1283)])
+def test_activation_of_later_tiles(monkeypatch, pairs, T, hid, pitch):
+    """More tiles than run at once, so that a block goes on to a second one, whose pre-activations are on their way by then: last columns of 8,
+    of 3 behind whole pieces, and rows that TMA does not take.  Every element: the sum's bf16 operands are exact and its fp32 terms lose 2^-24
+    each of their magnitudes (64 terms, 2^-18 of their sum), the published erf form 2^-19 absolute and the unit's exponential and reciprocal
+    less; one bf16 rounding, 2^-8 of the value."""
+    monkeypatch.setenv("MST_TC_PAIR", pairs)
+    I = 64
+    g = torch.Generator(device="cuda").manual_seed(T + hid)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()
+    X, dY, W1, W2 = n(T, I), n(T, I), n(hid, I), n(I, hid)
+    M1, M2 = ((torch.rand(s, generator=g, device="cuda") < 0.3).to(torch.uint8) for s in ((hid, I), (I, hid)))
+    L1, L2 = mst.Layer(0, hid, I, mst.MST_BF16), mst.Layer(1, I, hid, mst.MST_BF16)
+    L1.pack(W1, M1)
+    L2.pack(W2, M2)
+    H, pre, at, dP = (torch.full((T, pitch), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    at[:, :hid] = n(T, hid) * 2
+    mst.mst_spmm_fwd_gelu(L1.handle, X, I, T, pre, pitch, H, pitch)
+    mst.mst_spmm_bwd_x_gelu(L2.handle, dY, I, T, at, pitch, dP, pitch)
+    torch.cuda.synchronize()
+    assert mst.mst_device_error_flags() == 0
+    phi = lambda x: 0.5 * (1 + torch.erf(x / 2 ** 0.5))
+    w1, w2, a = W1.double() * M1, W2.double() * M2, at[:, :hid].double()
+    y, size = X.double() @ w1.T, X.double().abs() @ w1.abs().T
+    d, dsize = dY.double() @ w2, dY.double().abs() @ w2.abs()
+    slope = phi(a) + a * torch.exp(-a * a / 2) / (2 * torch.pi) ** 0.5
+    for got, ref, magnitude in ((pre, y, size), (H, y * phi(y), size * 1.13 + y.abs()), (dP, d * slope, dsize * slope.abs() + d.abs())):
+        over = (got[:, :hid].double() - ref).abs() - (ref.abs() * 2.0 ** -8 + magnitude * 2.0 ** -18)
+        assert float(over.max()) <= 0, (float(over.max()), int(over.argmax()))
+        assert torch.isnan(got[:, hid:]).all()
+    L1.close()
+    L2.close()
