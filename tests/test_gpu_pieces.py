@@ -133,6 +133,26 @@ def test_forward_of_a_few_hundred_tokens(O, I, T, pad):
     assert y <= 4e-3 and dx <= 4e-3 and dw <= 1e-5 and g <= 1e-5
 
 
+@pytest.mark.parametrize("O,I,T,kernel", [
+    (768, 768, 16, "small_fwd_kernel"), (768, 768, 64, "small_fwd_kernel"), (300, 4096, 31, "small_fwd_kernel"), (17, 40, 257, "small_fwd_kernel"),
+    (1280, 1288, 512, "tc_split_kernel"), (3712, 114, 717, "tc_gemm_pair_kernel"), (96, 96, 1025, "tc_split_kernel"), (2048, 2048, 4000, "tc_gemm_pair_kernel")])
+def test_kernel_of_a_forward_call(O, I, T, kernel):
+    # sizes for which the estimates lie a factor 1.2 or more apart, or that are outside of a kernel's range
+    from torch.profiler import ProfilerActivity, profile
+    n = lambda *s: torch.randn(*s, device="cuda").bfloat16()
+    L = mst.Layer(0, O, I, mst.MST_BF16)
+    L.pack(n(O, I), (torch.rand(O, I, device="cuda") < 0.2).to(torch.uint8))
+    X, Y = n(T, I), torch.empty(T, O, dtype=torch.bfloat16, device="cuda")
+    L.fwd(X, Y, T)
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as seen:
+        L.fwd(X, Y, T)
+        torch.cuda.synchronize()
+    names = [e.name for e in seen.events() if "_kernel" in e.name and "prepare" not in e.name]
+    assert len(names) == 1 and kernel in names[0], names
+    L.close()
+
+
 @pytest.mark.parametrize("O,I,T,density", [
     (5120, 1280, 8190, 0.1),     # 100 tiles on 74 pairs: 26 cut in two
     (3840, 1250, 8000, 0.3),     # 75 tiles: one cut, the others whole; ragged columns
