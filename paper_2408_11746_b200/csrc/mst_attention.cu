@@ -236,21 +236,21 @@ strided_attention_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __gr
           ok = wait_on(full + 8 * kf.s, kf.lap & 1u, abort_flag);
           if (!ok) break;
           const uint32_t kt = ring + kf.s * SLOT_BYTES;
-            const int row = (rs + (lane & 15)) & (TS - 1);
-            const FarRow v = far_row(kt + TILE_BYTES, row, lane);
-            const float x = far_dot(mine, far_row(kt, row, lane)) * SCALE_LOG2E;
-            const bool up = x > fm + LAZY;
-            if (__any_sync(0xffffffffu, up)) {
-              const float c = up ? ex2(fm - x) : 1.f;
-              if (up) fm = x;
-              fs *= c;
+          const int row = (rs + (lane & 15)) & (TS - 1);
+          const FarRow v = far_row(kt + TILE_BYTES, row, lane);
+          const float x = far_dot(mine, far_row(kt, row, lane)) * SCALE_LOG2E;
+          const bool up = x > fm + LAZY;
+          if (__any_sync(0xffffffffu, up)) {
+            const float c = up ? ex2(fm - x) : 1.f;
+            if (up) fm = x;
+            fs *= c;
 #pragma unroll
-              for (int e = 0; e < 32; ++e) acc[e] *= c;
-            }
-            const float w = ex2(x - reference(fm));
-            fs += w;
-            far_add(acc, w, v);
-            far_release(empty + 8 * kf.s, lane);
+            for (int e = 0; e < 32; ++e) acc[e] *= c;
+          }
+          const float w = ex2(x - reference(fm));
+          fs += w;
+          far_add(acc, w, v);
+          far_release(empty + 8 * kf.s, lane);
         }
         k.skip(far);
         far_start_sums(tmem + ((uint32_t)rs << 16) + 128u, acc);

@@ -355,24 +355,24 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           kf.skip(f);
           ok = wait_on(S.full + 8 * kf.s, kf.lap & 1u, abort_flag);
           if (!ok) break;
-            const uint32_t kt = S.ring + kf.s * SLOT_BYTES;
-            float sc[2][4], dp[2][4];
-            far_scores(sc, S.own0, rs, kt, c0, lane);
-            far_scores(dp, S.own1, rs, kt + TILE_BYTES, c0, lane);
+          const uint32_t kt = S.ring + kf.s * SLOT_BYTES;
+          float sc[2][4], dp[2][4];
+          far_scores(sc, S.own0, rs, kt, c0, lane);
+          far_scores(dp, S.own1, rs, kt + TILE_BYTES, c0, lane);
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb) {
+          for (int nb = 0; nb < 2; ++nb) {
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float ds = 0.f;
-                if (g + (e >> 1) * 8 == nb * 8 + 2 * tq + (e & 1)) {
-                  const float p = ex2(fmaf(sc[nb][e], SCALE_LOG2E, (e >> 1) ? st1.x : st0.x));
-                  ds = p * (dp[nb][e] - ((e >> 1) ? st1.y : st0.y));
-                }
-                sc[nb][e] = ds;
+            for (int e = 0; e < 4; ++e) {
+              float ds = 0.f;
+              if (g + (e >> 1) * 8 == nb * 8 + 2 * tq + (e & 1)) {
+                const float p = ex2(fmaf(sc[nb][e], SCALE_LOG2E, (e >> 1) ? st1.x : st0.x));
+                ds = p * (dp[nb][e] - ((e >> 1) ? st1.y : st0.y));
               }
+              sc[nb][e] = ds;
             }
-            far_accumulate<4>(acc, sc, kt, c0, 0, lane);
-            far_release(S.empty + 8 * kf.s, lane);
+          }
+          far_accumulate(acc, sc, kt, c0, lane);
+          far_release(S.empty + 8 * kf.s, lane);
         }
         k.skip(far);
         tmem_st_tiles(tmem + ((uint32_t)rs << 16) + 128u, acc);
@@ -590,28 +590,28 @@ attn_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           kf.skip(f);
           ok = wait_on(S.full + 8 * kf.s, kf.lap & 1u, abort_flag);
           if (!ok) break;
-            const uint32_t qt = S.ring + kf.s * SLOT_BYTES;
-            float st[2][4], dp[2][4];
-            far_scores(st, S.own0, rs, qt, c0, lane);
-            far_scores(dp, S.own1, rs, qt + TILE_BYTES, c0, lane);
+          const uint32_t qt = S.ring + kf.s * SLOT_BYTES;
+          float st[2][4], dp[2][4];
+          far_scores(st, S.own0, rs, qt, c0, lane);
+          far_scores(dp, S.own1, rs, qt + TILE_BYTES, c0, lane);
 #pragma unroll
-            for (int nb = 0; nb < 2; ++nb) {
-              const float* sq = S.at<float>(S.stat + kf.s * STAT_BYTES) + c0 + nb * 8 + 2 * tq;
-              const float2 nl = *reinterpret_cast<const float2*>(sq), nd = *reinterpret_cast<const float2*>(sq + TS);
+          for (int nb = 0; nb < 2; ++nb) {
+            const float* sq = S.at<float>(S.stat + kf.s * STAT_BYTES) + c0 + nb * 8 + 2 * tq;
+            const float2 nl = *reinterpret_cast<const float2*>(sq), nd = *reinterpret_cast<const float2*>(sq + TS);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float p = 0.f, ds = 0.f;
-                if (g + (e >> 1) * 8 == nb * 8 + 2 * tq + (e & 1)) {
-                  p = ex2(fmaf(st[nb][e], SCALE_LOG2E, (e & 1) ? nl.y : nl.x));
-                  ds = p * (dp[nb][e] + ((e & 1) ? nd.y : nd.x));
-                }
-                st[nb][e] = p;
-                dp[nb][e] = ds;
+            for (int e = 0; e < 4; ++e) {
+              float p = 0.f, ds = 0.f;
+              if (g + (e >> 1) * 8 == nb * 8 + 2 * tq + (e & 1)) {
+                p = ex2(fmaf(st[nb][e], SCALE_LOG2E, (e & 1) ? nl.y : nl.x));
+                ds = p * (dp[nb][e] + ((e & 1) ? nd.y : nd.x));
               }
+              st[nb][e] = p;
+              dp[nb][e] = ds;
             }
-            far_accumulate<4>(acc_v, st, qt + TILE_BYTES, c0, 0, lane);
-            far_accumulate<4>(acc_k, dp, qt, c0, 0, lane);
-            far_release(S.empty + 8 * kf.s, lane);
+          }
+          far_accumulate(acc_v, st, qt + TILE_BYTES, c0, lane);
+          far_accumulate(acc_k, dp, qt, c0, lane);
+          far_release(S.empty + 8 * kf.s, lane);
         }
         k.skip(far);
         tmem_st_tiles(tmem + ((uint32_t)rs << 16) + 128u, acc_k);

@@ -328,14 +328,13 @@ __device__ __forceinline__ void far_scores(float (&c)[2][4], uint32_t own, int r
     }
   }
 }
-// acc[16 x 16 N2] += weights (two 16 x 8 score tiles) * columns d0 .. of rows c0 .. c0 + 15 of `tile`
-template <int N2>
-__device__ __forceinline__ void far_accumulate(float (&acc)[2 * N2][4], const float (&w)[2][4], uint32_t tile, int c0, int d0, int lane) {
+// acc[16 x 64] += weights (two 16 x 8 score tiles) * rows c0 .. c0 + 15 of `tile`
+__device__ __forceinline__ void far_accumulate(float (&acc)[8][4], const float (&w)[2][4], uint32_t tile, int c0, int lane) {
   const uint32_t a[4] = {pack_bf16(w[0][0], w[0][1]), pack_bf16(w[0][2], w[0][3]), pack_bf16(w[1][0], w[1][1]), pack_bf16(w[1][2], w[1][3])};
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) {
+  for (int n2 = 0; n2 < 4; ++n2) {
     uint32_t b[4];
-    ldsm_x4_t(b, piece_addr(tile, c0 + (lane & 7) + ((lane >> 3) & 1) * 8, d0 / 8 + n2 * 2 + (lane >> 4)));
+    ldsm_x4_t(b, piece_addr(tile, c0 + (lane & 7) + ((lane >> 3) & 1) * 8, n2 * 2 + (lane >> 4)));
     mma_bf16(acc[2 * n2], a, b[0], b[1]);
     mma_bf16(acc[2 * n2 + 1], a, b[2], b[3]);
   }
