@@ -70,6 +70,7 @@ struct SplitParams {
   const int32_t* wscan;
   int wpr;
   float* entries;   // S_BOTH
+  int kind, major;  // S_ANY, M_ANY
   mst_redo redo;
 };
 
@@ -135,22 +136,28 @@ __device__ __forceinline__ void box_rows(const float* box, int rr0, int end, int
 
 // What a launch does not run costs it all the same (see the large tiles' kernel): the kind of output and the operands' majors are
 // constants.  One kernel for all: 0.3-0.5 us more a launch (1216 x 1216, 534 tokens: forward 9.7 against 9.2 us, weight gradient 8.3
-// against 7.9; fp32 3072 x 768, 256 tokens: 18.2 against 17.8).
+// against 7.9).  But each fetches its instructions anew when a pass comes to it.  In bf16 a block's four layers follow one another in the same kernel: its
+// passes take 1 to 3 % less (width 448, 2227 tokens 125.8 against 127.5 us, 320 at 1100 101.4 against 105.3; four forward calls of width 896 at 120
+// tokens 32.4 against 33.7), and the three products of a single layer 0 to 8 % more (640 x 640 at 640 tokens 26.3 against 24.2).  Pieces, six products
+// to a k-block and mostly one layer a pass, have one kernel of each width (S_ANY, M_ANY): 495 x 96 at 208 tokens 29.8 -> 27.8 us, 208 x 297 at 170
+// 31.2 -> 29.7, 320 x 576 at 75 31.2 -> 29.8, 1114 x 256 at 253 38.4 -> 37.1; 2.4 % over sixty layers of 96..2048 features.
 enum {
   S_F32, S_SAMPLED,
   S_BOTH,   // fp32, and its entries under the mask
   S_BF16,
-  S_REDO,   // bf16, where sums that are not finite are formed again (three pieces: always)
-  S_ACT     // bf16 with an activation, with or without such sums
+  S_REDO,   // bf16, where sums that are not finite are formed again (pieces: always)
+  S_ACT,    // bf16 with an activation, with or without such sums
+  S_ANY     // of the first three, as P.kind says
 };
-enum { M_FORWARD, M_INPUT, M_GRADIENT };   // MN-major operands: none, the second, both
+enum { M_FORWARD, M_INPUT, M_GRADIENT, M_ANY };   // MN-major operands: none, the second, both; as P.major says
 
-template <int BN, int PIECES, int KIND, int MAJOR>
+template <int BN, int PIECES, int KIND_, int MAJOR_>
 __global__ void __launch_bounds__(S_THREADS, PIECES == 1 ? 2 : 1)
 tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
   typedef SplitCfg<BN, PIECES> C;
   constexpr int CHUNK_KB = C::CHUNK_KB;
-  constexpr bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
+  const int KIND = KIND_ == S_ANY ? P.kind : KIND_, MAJOR = MAJOR_ == M_ANY ? P.major : MAJOR_;
+  const bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -343,7 +350,7 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if ((w >> lane) & 1u) out[base + __popc(w & lt)] = v;
           });
         }
-        if (KIND >= S_BF16) {
+        if (PIECES == 1 && KIND >= S_BF16) {
           uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + row0 * P.ldc + n + lane;
           uint16_t* pre = P.pre + row0 * P.ldpre + n + lane;
           if (KIND != S_ACT)
@@ -414,15 +421,6 @@ mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
                                              dim3(S_THREADS), P.splits, C::SMEM, s, tmA, tmB, P));
   return MST_OK;
 }
-template <int BN>
-mst_status_t launch_pieces(int epilogue, int major, const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
-  if (epilogue == MST_TC_OUT_SAMPLED) return launch_split<BN, 3, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
-  if (major == M_FORWARD) return launch_split<BN, 3, S_F32, M_FORWARD>(tmA, tmB, P, s);
-  if (major == M_INPUT) return launch_split<BN, 3, S_F32, M_INPUT>(tmA, tmB, P, s);
-  if (P.entries) return launch_split<BN, 3, S_BOTH, M_GRADIENT>(tmA, tmB, P, s);
-  return launch_split<BN, 3, S_F32, M_GRADIENT>(tmA, tmB, P, s);
-}
-
 // Blocks that run at once, one to an SM, in clusters of 1 .. 8: the groups of SMs that a cluster must fit into are no multiples of it (148
 // SMs hold 148, 148, 132 and 120 blocks in clusters of 1, 2, 4 and 8).  Asked once per device, and for the device once a plan: asked for every width and
 // number of ranges the plans of a forward call cost it 0.5 us.
@@ -452,8 +450,8 @@ Slots cluster_slots() {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int clusters = 0;
-      if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_F32, M_GRADIENT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
-          cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_F32, M_GRADIENT>, &cfg) != cudaSuccess || clusters <= 0) {
+      if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_ANY, M_ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_ANY, M_ANY>, &cfg) != cudaSuccess || clusters <= 0) {
         cudaGetLastError();   // reported by the launch, if it matters there
         continue;
       }
@@ -542,15 +540,18 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
   const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, pieces, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, pieces, a.M, a.K, a.lda, SBM);
   const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, pieces, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, pieces, a.N, a.K, a.ldb, bn);
   if (!okA || !okB) return MST_ERR_SHAPE;
-  if (pieces == 3) return bn == 64 ? launch_pieces<64>(a.epilogue, major, tmA, tmB, P, s) : launch_pieces<128>(a.epilogue, major, tmA, tmB, P, s);
-  if (a.epilogue == MST_TC_OUT_SAMPLED) return launch_split<64, 1, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
-  if (a.epilogue == MST_TC_OUT_F32)
-    return P.entries ? launch_split<64, 1, S_BOTH, M_GRADIENT>(tmA, tmB, P, s) : launch_split<64, 1, S_F32, M_GRADIENT>(tmA, tmB, P, s);
-  if (major == M_FORWARD)
-    return act ? launch_split<64, 1, S_ACT, M_FORWARD>(tmA, tmB, P, s)
-           : P.redo.kind ? launch_split<64, 1, S_REDO, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_FORWARD>(tmA, tmB, P, s);
-  return act ? launch_split<64, 1, S_ACT, M_INPUT>(tmA, tmB, P, s)
-         : P.redo.kind ? launch_split<64, 1, S_REDO, M_INPUT>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_INPUT>(tmA, tmB, P, s);
+  P.major = major;
+  P.kind = a.epilogue == MST_TC_OUT_SAMPLED ? S_SAMPLED : a.epilogue == MST_TC_OUT_F32 ? (P.entries ? S_BOTH : S_F32) : act ? S_ACT : P.redo.kind ? S_REDO : S_BF16;
+  if (pieces == 3) return bn == 64 ? launch_split<64, 3, S_ANY, M_ANY>(tmA, tmB, P, s) : launch_split<128, 3, S_ANY, M_ANY>(tmA, tmB, P, s);
+  const bool forward = major == M_FORWARD;
+  switch (P.kind) {
+    case S_SAMPLED: return launch_split<64, 1, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
+    case S_F32: return launch_split<64, 1, S_F32, M_GRADIENT>(tmA, tmB, P, s);
+    case S_BOTH: return launch_split<64, 1, S_BOTH, M_GRADIENT>(tmA, tmB, P, s);
+    case S_ACT: return forward ? launch_split<64, 1, S_ACT, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_ACT, M_INPUT>(tmA, tmB, P, s);
+    case S_REDO: return forward ? launch_split<64, 1, S_REDO, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_REDO, M_INPUT>(tmA, tmB, P, s);
+    default: return forward ? launch_split<64, 1, S_BF16, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_INPUT>(tmA, tmB, P, s);
+  }
 }
 
 }  // namespace
