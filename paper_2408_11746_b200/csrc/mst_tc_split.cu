@@ -70,6 +70,7 @@ struct SplitParams {
   const int32_t* wscan;
   int wpr;
   float* entries;   // S_BOTH
+  int kind, major;
   mst_redo redo;
 };
 
@@ -133,24 +134,24 @@ __device__ __forceinline__ void box_rows(const float* box, int rr0, int end, int
   for (; r < end; ++r) store(r, box[r * 33 + lane]);
 }
 
-// What a launch does not run costs it all the same (see the large tiles' kernel): the kind of output and the operands' majors are
-// constants.  One kernel for all: 0.3-0.5 us more a launch (1216 x 1216, 534 tokens: forward 9.7 against 9.2 us, weight gradient 8.3
-// against 7.9; fp32 3072 x 768, 256 tokens: 18.2 against 17.8).
+// One kernel for every kind of output and the operands' majors, but for the activations.  A kernel each takes 0.3 to 0.5 us less where one call
+// repeats (3072 x 768 in fp32, 256 tokens: 17.8 against 18.2), but a pass takes turns, and each then fetches its instructions anew: the three
+// products of small layers, a kernel each / one, fp32 495 x 96 at 208 tokens 29.8 / 27.7 us, 320 x 576 at 75 31.2 / 29.7, 1114 x 256 at 253 38.5 / 37.0,
+// bf16 896 x 111 at 925 28.7 / 26.9, 256 x 383 at 785 26.7 / 24.7; 2.4 % over thirty fp32 layers of 96..2048 features, 0.7 % over thirty in bf16.
 enum {
   S_F32, S_SAMPLED,
   S_BOTH,   // fp32, and its entries under the mask
-  S_BF16,
-  S_REDO,   // bf16, where sums that are not finite are formed again (three pieces: always)
-  S_ACT     // bf16 with an activation, with or without such sums
+  S_BF16
 };
 enum { M_FORWARD, M_INPUT, M_GRADIENT };   // MN-major operands: none, the second, both
 
-template <int BN, int PIECES, int KIND, int MAJOR>
+template <int BN, int PIECES, int ACT>
 __global__ void __launch_bounds__(S_THREADS, PIECES == 1 ? 2 : 1)
 tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitParams P) {
   typedef SplitCfg<BN, PIECES> C;
   constexpr int CHUNK_KB = C::CHUNK_KB;
-  constexpr bool A_MN = MAJOR == M_GRADIENT, B_MN = MAJOR != M_FORWARD;
+  const int kind = ACT ? S_BF16 : P.kind;
+  const bool a_mn = !ACT && P.major == M_GRADIENT, b_mn = ACT ? ACT == MST_ACT_GELU_GRAD : P.major != M_FORWARD;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -202,12 +203,12 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, &g_split_error)) break;
         const uint32_t fb = full0 + 8 * s, sa = tiles_base + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
         mbar_expect_tx(fb, C::STAGE_BYTES);
-        if (A_MN) {
+        if (a_mn) {
           for (int j = 0; j < SBM / 64; ++j) tma_load_3d(sa + j * PIECES * BOX64, &tmA, m0 + j * 64, kb * SBK, 0, fb);
         } else {
           tma_load_3d(sa, &tmA, kb * SBK, m0, 0, fb);
         }
-        if (B_MN) {
+        if (b_mn) {
           for (int j = 0; j < BN / 64; ++j) tma_load_3d(sb + j * PIECES * BOX64, &tmB, n0 + j * 64, kb * SBK, 0, fb);
         } else {
           tma_load_3d(sb, &tmB, kb * SBK, n0, 0, fb);
@@ -217,13 +218,13 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(A_MN ? 1 : 0) << 15) |
-                             ((uint32_t)(B_MN ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a_mn ? 1 : 0) << 15) |
+                             ((uint32_t)(b_mn ? 1 : 0) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
       // K-major: the three pieces of a stage lie one after the other; MN-major: 64-wide blocks, each with its three pieces
-      const uint64_t ad0 = smem_desc(tiles_base, A_MN ? PIECES * BOX64 : 16, 1024);
-      const uint64_t bd0 = smem_desc(tiles_base + C::A_BYTES, B_MN ? PIECES * BOX64 : 16, 1024);
-      const uint32_t a_piece = (uint32_t)(A_MN ? BOX64 : SBM * SBK * 2) >> 4, b_piece = (uint32_t)(B_MN ? BOX64 : BN * SBK * 2) >> 4;
-      const uint32_t a_k = (uint32_t)(A_MN ? 16 * 128 : 32) >> 4, b_k = (uint32_t)(B_MN ? 16 * 128 : 32) >> 4;
+      const uint64_t ad0 = smem_desc(tiles_base, a_mn ? PIECES * BOX64 : 16, 1024);
+      const uint64_t bd0 = smem_desc(tiles_base + C::A_BYTES, b_mn ? PIECES * BOX64 : 16, 1024);
+      const uint32_t a_piece = (uint32_t)(a_mn ? BOX64 : SBM * SBK * 2) >> 4, b_piece = (uint32_t)(b_mn ? BOX64 : BN * SBK * 2) >> 4;
+      const uint32_t a_k = (uint32_t)(a_mn ? 16 * 128 : 32) >> 4, b_k = (uint32_t)(b_mn ? 16 * 128 : 32) >> 4;
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -321,14 +322,14 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         __syncwarp();
         const int64_t row0 = (int64_t)m0 + q * 32;
-        if ((PIECES == 3 || KIND == S_REDO || (KIND == S_ACT && P.redo.kind)) && __any_sync(0xffffffffu, zero != 0.f)) {
+        if (P.redo.kind && __any_sync(0xffffffffu, zero != 0.f)) {
           const bool mine = lane >= rr0 && lane < rr1 && row0 + lane < P.M;
           if (PIECES == 3) mst_redo_square<float>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
           else mst_redo_square<uint16_t>(P.redo, box + lane * 33, row0 + lane, mine, n, P.N);
           __syncwarp();
         }
         const int end = n + lane >= P.N ? 0 : (int)(P.M - row0 < rr1 ? P.M - row0 : rr1);   // rows of this lane's column
-        if (KIND == S_SAMPLED || KIND == S_BOTH) {
+        if (kind == S_SAMPLED || kind == S_BOTH) {
           uint32_t word = 0;
           int32_t at = 0;
           if (row0 + lane < P.M) {
@@ -336,20 +337,20 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             word = P.bits[wi];
             at = P.wscan[wi];
           }
-          float* out = KIND == S_BOTH ? P.entries : reinterpret_cast<float*>(P.out);
+          float* out = kind == S_BOTH ? P.entries : reinterpret_cast<float*>(P.out);
           box_rows(box, rr0, rr1, lane, [&](int rr, float v) {   // words beyond the matrix are empty
             const uint32_t w = __shfl_sync(0xffffffffu, word, rr);
             const int32_t base = __shfl_sync(0xffffffffu, at, rr);
             if ((w >> lane) & 1u) out[base + __popc(w & lt)] = v;
           });
         }
-        if (KIND >= S_BF16) {
+        if (PIECES == 1 && kind == S_BF16) {
           uint16_t* out = reinterpret_cast<uint16_t*>(P.out) + row0 * P.ldc + n + lane;
           uint16_t* pre = P.pre + row0 * P.ldpre + n + lane;
-          if (KIND != S_ACT)
+          if (ACT == MST_ACT_NONE)
             box_rows(box, rr0, end, lane,
                      [&](int rr, float v) { out[rr * P.ldc] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu); });
-          else if (MAJOR == M_INPUT) {   // the derivative at the stored pre-activation
+          else if (ACT == MST_ACT_GELU_GRAD) {   // the derivative at the stored pre-activation
             // sixteen rows' inputs at a time, before any of their results leaves: row by row each waits out its load (64 tokens,
             // 192 x 768: 11.6 us).  Rows past the end repeat the last one, so that only the stores are conditional and the sixteen
             // derivatives overlap.
@@ -371,7 +372,7 @@ tc_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
               if (P.pre) pre[rr * P.ldpre] = (uint16_t)(pack_bf16(v, 0.f) & 0xFFFFu);
               out[rr * P.ldc] = (uint16_t)(pack_bf16(mst_gelu(v), 0.f) & 0xFFFFu);
             });
-        } else if (KIND != S_SAMPLED) {
+        } else if (kind != S_SAMPLED) {
           float* out = reinterpret_cast<float*>(P.out) + row0 * P.ldc + n + lane;
           box_rows(box, rr0, end, lane, [&](int rr, float v) { out[rr * P.ldc] = v; });
         }
@@ -406,23 +407,14 @@ bool make_piece_map(CUtensorMap* tm, const void* base, int pieces, int64_t rows,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int PIECES, int KIND, int MAJOR>
+template <int BN, int PIECES, int ACT>
 mst_status_t launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
   typedef SplitCfg<BN, PIECES> C;
-  MST_SMEM_LIMIT((tc_split_kernel<BN, PIECES, KIND, MAJOR>), C::SMEM);
-  MST_CUDA_TRY(mst_launch_overlapped_cluster(tc_split_kernel<BN, PIECES, KIND, MAJOR>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)),
+  MST_SMEM_LIMIT((tc_split_kernel<BN, PIECES, ACT>), C::SMEM);
+  MST_CUDA_TRY(mst_launch_overlapped_cluster(tc_split_kernel<BN, PIECES, ACT>, dim3((unsigned)(P.m_tiles * P.n_tiles * P.splits)),
                                              dim3(S_THREADS), P.splits, C::SMEM, s, tmA, tmB, P));
   return MST_OK;
 }
-template <int BN>
-mst_status_t launch_pieces(int epilogue, int major, const CUtensorMap& tmA, const CUtensorMap& tmB, const SplitParams& P, cudaStream_t s) {
-  if (epilogue == MST_TC_OUT_SAMPLED) return launch_split<BN, 3, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
-  if (major == M_FORWARD) return launch_split<BN, 3, S_F32, M_FORWARD>(tmA, tmB, P, s);
-  if (major == M_INPUT) return launch_split<BN, 3, S_F32, M_INPUT>(tmA, tmB, P, s);
-  if (P.entries) return launch_split<BN, 3, S_BOTH, M_GRADIENT>(tmA, tmB, P, s);
-  return launch_split<BN, 3, S_F32, M_GRADIENT>(tmA, tmB, P, s);
-}
-
 // Blocks that run at once, one to an SM, in clusters of 1 .. 8: the groups of SMs that a cluster must fit into are no multiples of it (148
 // SMs hold 148, 148, 132 and 120 blocks in clusters of 1, 2, 4 and 8).  Asked once per device, and for the device once a plan: asked for every width and
 // number of ranges the plans of a forward call cost it 0.5 us.
@@ -452,8 +444,8 @@ Slots cluster_slots() {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int clusters = 0;
-      if (cudaFuncSetAttribute(tc_split_kernel<128, 3, S_F32, M_GRADIENT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
-          cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, S_F32, M_GRADIENT>, &cfg) != cudaSuccess || clusters <= 0) {
+      if (cudaFuncSetAttribute(tc_split_kernel<128, 3, MST_ACT_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&clusters, tc_split_kernel<128, 3, MST_ACT_NONE>, &cfg) != cudaSuccess || clusters <= 0) {
         cudaGetLastError();   // reported by the launch, if it matters there
         continue;
       }
@@ -542,15 +534,11 @@ mst_status_t run_split(const mst_tc_gemm_args& a, int pieces, int bn, int splits
   const bool okA = a.a_mn_major ? make_piece_map(&tmA, a.A, pieces, a.K, a.M, a.lda, SBK) : make_piece_map(&tmA, a.A, pieces, a.M, a.K, a.lda, SBM);
   const bool okB = a.b_mn_major ? make_piece_map(&tmB, a.B, pieces, a.K, a.N, a.ldb, SBK) : make_piece_map(&tmB, a.B, pieces, a.N, a.K, a.ldb, bn);
   if (!okA || !okB) return MST_ERR_SHAPE;
-  if (pieces == 3) return bn == 64 ? launch_pieces<64>(a.epilogue, major, tmA, tmB, P, s) : launch_pieces<128>(a.epilogue, major, tmA, tmB, P, s);
-  if (a.epilogue == MST_TC_OUT_SAMPLED) return launch_split<64, 1, S_SAMPLED, M_GRADIENT>(tmA, tmB, P, s);
-  if (a.epilogue == MST_TC_OUT_F32)
-    return P.entries ? launch_split<64, 1, S_BOTH, M_GRADIENT>(tmA, tmB, P, s) : launch_split<64, 1, S_F32, M_GRADIENT>(tmA, tmB, P, s);
-  if (major == M_FORWARD)
-    return act ? launch_split<64, 1, S_ACT, M_FORWARD>(tmA, tmB, P, s)
-           : P.redo.kind ? launch_split<64, 1, S_REDO, M_FORWARD>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_FORWARD>(tmA, tmB, P, s);
-  return act ? launch_split<64, 1, S_ACT, M_INPUT>(tmA, tmB, P, s)
-         : P.redo.kind ? launch_split<64, 1, S_REDO, M_INPUT>(tmA, tmB, P, s) : launch_split<64, 1, S_BF16, M_INPUT>(tmA, tmB, P, s);
+  P.major = major;
+  P.kind = a.epilogue == MST_TC_OUT_SAMPLED ? S_SAMPLED : a.epilogue == MST_TC_OUT_BF16 ? S_BF16 : P.entries ? S_BOTH : S_F32;
+  if (pieces == 3) return bn == 64 ? launch_split<64, 3, MST_ACT_NONE>(tmA, tmB, P, s) : launch_split<128, 3, MST_ACT_NONE>(tmA, tmB, P, s);
+  return act == MST_ACT_GELU ? launch_split<64, 1, MST_ACT_GELU>(tmA, tmB, P, s)
+         : act ? launch_split<64, 1, MST_ACT_GELU_GRAD>(tmA, tmB, P, s) : launch_split<64, 1, MST_ACT_NONE>(tmA, tmB, P, s);
 }
 
 }  // namespace
