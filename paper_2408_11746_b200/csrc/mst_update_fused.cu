@@ -25,7 +25,7 @@
 // What bounds it: instruction issue in the two sweeps (an inactive entry costs one SplitMix64 hash, two 64-bit products and about
 // twenty shifts and logic operations, and 4 bytes of gradient) and, around them, a chain of about fifteen block-wide steps and
 // L2 round trips of 1-2 us each that several layers in one launch share.  Four layers of a GPT-2-medium block (12.6 M entries,
-// d = 0.1, zeta = 0.3, R = 0.25): 76 us, of which the hashes 14, the gradient and value sweep 20; one of its layers alone
+// d = 0.1, zeta = 0.3, R = 0.25): 74 us, of which the hashes 14, the gradient and value sweep 20; one of its layers alone
 // (4.2 M): 50 us, a layer of 0.6 M 36.  (256 bins over the bracket and a third pass over the bin of some hundred entries: 2 us more.)  The form before, one launch per layer with every key in shared memory and five sweeps between six
 // grid-wide barriers, took 238 us for the block.
 #include <cmath>
