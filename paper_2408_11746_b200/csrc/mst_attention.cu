@@ -18,7 +18,7 @@
 // The far tiles' softmax (two lanes a row, 16 rows a warp) is where the first half starts: reference and sum through shared memory, outputs in tensor memory.
 // Results leave by TMA from a slot of the ring, or, in a block without successors, as whole rows from where the own rows were.
 // Bound: the chain of a tile through its warps (scores, exponentials, weights: about 1000 clocks for a block, two of them at
-// work on an SM); the SM issues in half of its cycles, DRAM is busy for a quarter of the time.  16 x 1024 tokens, 12 heads, l = 256 50.2 -> 40 us,
+// work on an SM).  16 x 1024 tokens, 12 heads, l = 256 50.2 -> 40 us,
 // 8 x 1024, 16 heads, l = 128 35.5 -> 28.4 (one block after the other, heads last in the grid, far tiles at the end, on mma.sync).
 #include <cuda.h>
 #include <cuda_bf16.h>

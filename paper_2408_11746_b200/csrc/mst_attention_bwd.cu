@@ -23,7 +23,7 @@
 // A block that is done takes over one that has not started; its own rows, the forward output and the first tiles are then in
 // shared memory or on their way.  Results leave by TMA from slots of the ring, or, in a block without
 // successors, as whole rows from where the own rows were.
-// Bound: as forward, the chain of a tile through its warps; tensor pipe and issue slots are half busy, DRAM a third.
+// Bound: as forward, the chain of a tile through its warps.
 // 16 x 1024 tokens, 12 heads, l = 256 144.7 -> 124.2 us, 8 x 1024, 16 heads, l = 128 108.7 -> 87.8.
 #include <cuda.h>
 #include <cuda_bf16.h>
